@@ -100,7 +100,8 @@ enum lbm_status {
 enum lbm_option {
     LBM_OPT_DIAG_EVERY = 0, /* fused diagnostics every K steps (0 = off, the default) */
     LBM_OPT_KERNEL = 1,     /* 0 = auto, 1 = generic one-cell-per-thread kernel,
-                               2 = TMA row-staged kernel (needs Nx * sizeof % 16 == 0) */
+                               2 = TMA row-staged kernel (needs Nx * sizeof % 16 == 0; auto also
+                               takes it for longer ragged rows, which it stores padded) */
     LBM_OPT_USE_GRAPH = 2,  /* 1 = replay steps from a captured CUDA graph (default 0) */
     LBM_OPT_TUNE = 3        /* 1 = time the candidate launch shapes now and keep the best */
 };
@@ -154,8 +155,9 @@ int lbm_set_option(lbm_ctx *ctx, int option, int64_t value);
 int lbm_init_fields(lbm_ctx *ctx, const void *rho, const void *u, int dtype, int on_device);
 
 /*
- * Advance n >= 0 time steps of Eq. (1).  Each step is one launch of the fused
- * stream-collide kernel (AA pattern, in place).  When LBM_OPT_DIAG_EVERY = K > 0 the
+ * Advance n >= 0 time steps of Eq. (1) with the fused stream-collide kernel (AA pattern, in
+ * place): one launch for many steps with the TMA row-staged kernel, one launch per step with
+ * the one-cell kernel and for steps with diagnostics.  When LBM_OPT_DIAG_EVERY = K > 0 the
  * step kernels of steps t with t % K == 0 also reduce the diagnostics of state t; the
  * call then synchronises and returns LBM_ENONFINITE if any of them saw a non-finite
  * cell (the state is kept for inspection).
@@ -203,7 +205,7 @@ int lbm_step_count(lbm_ctx *ctx, int64_t *out);
  * Launch shape of the step kernel chosen for this context: out[0] = kernel (1 generic,
  * 2 TMA row-staged), out[1] = threads per block, out[2] = blocks, out[3] = pipeline
  * stages, out[4] = rows per job, out[5] = cells per row segment, out[6] = dynamic
- * shared memory bytes, out[7] = population storage bytes.
+ * shared memory bytes, out[7] = population storage bytes (with the padding of ragged rows).
  */
 int lbm_launch_info(lbm_ctx *ctx, int64_t out[8]);
 
@@ -211,7 +213,7 @@ int lbm_launch_info(lbm_ctx *ctx, int64_t out[8]);
  * Choose the step kernel's launch shape explicitly.  shape = {kernel, threads, stages,
  * rows, seg, cap}: kernel 1 = generic (threads per block, the rest ignored), 2 = TMA
  * row-staged with `threads` colliding threads per block (a multiple of 32, at most 256,
- * 512 for D2Q9 with binary16 storage; one copy-issuing warp is added), `stages`
+ * 512 for D2Q9 with binary16 storage; two copy-issuing warps are added), `stages`
  * shared-memory stages (2..8), `rows` rows per job when whole rows fit, `seg` cells per
  * row segment (seg >= Nx for whole rows; otherwise a multiple of 16 / sizeof(storage), and
  * never below it) and `cap` bytes per direction buffer (1024, 2048, 4096 or 8192).  The

@@ -78,10 +78,11 @@ struct lbm_ctx {
     int sticky = 0;
     // diagnostics
     int64_t diag_every = 0;
+    int32_t *status = nullptr;   // start of one allocation that holds these five
+    unsigned *sync = nullptr;    // counters of several-step launches
     double *partials = nullptr;  // [kPartialsCap][8]
     double *hist = nullptr;      // [kHistCap][8]
     double *scratch = nullptr;   // one record
-    int32_t *status = nullptr;
     int64_t hist_count = 0;
     // launch
     int kernel_opt = 0;  // 0 auto, 1 generic, 2 tma
@@ -171,6 +172,7 @@ StepArgs step_args(lbm_ctx *c, int odd, int diag) {
     a.diag = diag;
     a.partials = c->partials;
     a.status = c->status;
+    a.sync = c->sync;
     a.timeout_ns = wait_timeout_ns();
     return a;
 }
@@ -179,38 +181,71 @@ int launch_blocks(lbm_ctx *c) { return c->kernel == 2 ? c->tma.blocks : c->gen_b
 
 cudaError_t launch_one(lbm_ctx *c, int odd, int diag, cudaStream_t s) {
     const StepArgs a = step_args(c, odd, diag);
-    if (c->kernel == 2) return step_tma(a, c->tma, s);
+    if (c->kernel == 2) return step_tma(a, c->tma, 1, s);
     return step_generic(a, c->gen_blocks, c->gen_threads, s);
 }
 
-// Default TMA shape, used until the tuner runs: the shape the tuner picks on the large
-// workloads measured so far.  128 colliding threads; direction buffers of 2048 bytes for
-// D3Q27 (4096 when a row is longer, up to 4096 bytes) and 4096 bytes for D2Q9; whole rows
-// filling the buffer when a row fits, otherwise aligned segments; 2 stages for D3Q27 (two
-// blocks per SM) and 3 for D2Q9; as many blocks as fit on the device.
+// n steps without diagnostics from the layout `odd` describes: several to a launch with the
+// TMA kernel, one each with the one-cell kernel.
+cudaError_t launch_steps(lbm_ctx *c, int odd, int64_t n, cudaStream_t s) {
+    int64_t most = 1;
+    if (c->kernel == 2 && n > 1) most = tma_max_steps(c->lat, c->tma);
+    cudaError_t e = cudaSuccess;
+    while (n > 0 && e == cudaSuccess) {
+        const int64_t m = std::min(n, most);
+        if (m == 1) e = launch_one(c, odd, 0, s);
+        else e = step_tma(step_args(c, odd, 0), c->tma, (int)m, s);
+        odd ^= (int)(m & 1);
+        n -= m;
+    }
+    return e;
+}
+
+// Default TMA shape, used until the tuner runs.  128 colliding threads and 2 stages: two
+// blocks per SM for D3Q27 with direction buffers of 2048 bytes (4096 when a row is longer, up
+// to 4096 bytes), three for D2Q9 with 4096 bytes (4096^2 FP32 several steps a launch: 120
+// GLUPS, against 98 with 3 stages and two blocks).  Whole rows filling the buffer when a row
+// fits, otherwise equal aligned segments; as many blocks as fit on the device.
 bool default_tma_shape(lbm_ctx *c, TmaShape &t) {
     const int es = esize_of(c->prec);
-    const int64_t rowb = c->lat.nx * (int64_t)es;
+    const int64_t rowb = c->lat.pitch * (int64_t)es;
     const int U = 16 / es;
     t.threads = 128;
     int cap = c->D == 3 ? 2048 : 4096;
     if (c->D == 3 && rowb > cap && rowb <= 4096) cap = 4096;
+    if (c->lat.pitch != c->lat.nx && rowb > cap) cap = 8192;  // padded rows are copied whole
     t.cap = cap;
     if (rowb <= cap) {
         t.seg = c->lat.nx;
         t.rows = (int)std::max<int64_t>(1, std::min<int64_t>(cap / rowb, c->lat.ny));
     } else {
-        t.seg = (cap / es - 2 * U) / U * U;
+        const int most = (cap / es - 2 * U) / U * U;
+        const int64_t n = (c->lat.nx + most - 1) / most;
+        t.seg = (int)(((c->lat.nx + n - 1) / n + U - 1) / U * U);
         t.rows = 1;
     }
-    t.stages = c->D == 3 ? 2 : 3;
+    t.stages = 2;
     t.smem_bytes = tma_smem_bytes(c->lat, t);
     if (t.smem_bytes < 0) return false;
     const int nb = tma_max_blocks_per_sm(c->lat, c->eq, c->bulk, t);
     if (nb < 1) return false;
     t.blocks = sm_count() * nb;
+    // A lattice of few rows is spread over all blocks, one job each: jobs of full buffers would
+    // leave most SMs without work (64^2 FP64: 8 jobs, 20.5 us a step; 64 jobs, 7.9 us).
+    const int64_t groups = std::max<int64_t>(1, t.blocks / c->lat.nz);  // row groups of a plane
+    t.rows = (int)std::max<int64_t>(1, std::min<int64_t>(t.rows, (c->lat.ny + groups - 1) / groups));
+    // With little more than one job a block, a job's collisions (512 cells: two iterations of
+    // 128 threads over pairs) are the step's critical path: 64^3 binary16 9.3 -> 7.7 us, 512^2
+    // FP32 5.7 -> 5.1 us a step.
+    while (t.rows > 1 && t.rows * c->lat.nx > 512 &&
+           2 * ((c->lat.ny + t.rows - 1) / t.rows) * (int64_t)c->lat.nz < 3 * (int64_t)t.blocks)
+        t.rows = (t.rows + 1) / 2;
     return true;
 }
+
+// Callers may ask for the TMA kernel on unpadded rows only; padded ones use it by the
+// library's own choice (LBM_OPT_KERNEL 0) or the tuner's.
+bool tma_selectable(lbm_ctx *c) { return tma_supported(c->lat) && c->lat.pitch == c->lat.nx; }
 
 void drop_graph(lbm_ctx *c) {
     if (c->graph2) {
@@ -401,7 +436,7 @@ float time_steps(lbm_ctx *c, int64_t step0, int nsteps) {
         return -1;
     }
     bool ok = cudaEventRecord(e0, c->stream) == cudaSuccess;
-    for (int s = 0; s < nsteps && ok; ++s) ok = launch_one(c, (int)((step0 + s) & 1), 0, c->stream) == cudaSuccess;
+    ok = ok && launch_steps(c, (int)(step0 & 1), nsteps, c->stream) == cudaSuccess;
     ok = ok && cudaEventRecord(e1, c->stream) == cudaSuccess;
     float ms = -1;
     if (ok && cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
@@ -464,12 +499,12 @@ int autotune(lbm_ctx *c) {
     // of a 2-D copy)
     for (int i = 0; i < c->Q; ++i)
         CK(cudaMemcpyAsync(static_cast<char *>(p->lat.A) + (size_t)i * p->lat.plane * es,
-                           static_cast<const char *>(c->lat.A) + (size_t)i * c->lat.plane * es, (size_t)p->ncell * es,
+                           static_cast<const char *>(c->lat.A) + (size_t)i * c->lat.plane * es, (size_t)p->lat.pitch * pd[1] * pd[2] * es,
                            cudaMemcpyDeviceToDevice, c->stream),
            "tuning proxy fill");
     std::vector<std::vector<int>> cands;
     const int U = 16 / es;
-    const int64_t rowb = c->lat.nx * (int64_t)es;
+    const int64_t rowb = c->lat.pitch * (int64_t)es;
     for (int th : {128, 256}) {
         int g = (int)std::min<int64_t>((c->ncell + th - 1) / th, (int64_t)sm_count() * 16);
         cands.push_back({1, th, std::max(g, 1), 0, 0, 0, 0, 0});
@@ -481,7 +516,7 @@ int autotune(lbm_ctx *c) {
                 const int rmax = (int)std::min<int64_t>(cap / rowb, c->lat.ny);
                 geo.push_back({rmax, (int)c->lat.nx});
                 if (rmax > 1) geo.push_back({std::max(1, rmax / 2), (int)c->lat.nx});
-            } else {
+            } else if (c->lat.pitch == c->lat.nx) {
                 // the longest segment the buffer holds, and the same number of segments
                 // made equal (no short ragged last segment with a job's full overhead)
                 const int smax = (cap / es - 2 * U) / U * U;
@@ -617,31 +652,46 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
     c->stream = static_cast<cudaStream_t>(cuda_stream);
     const int es = esize_of(precision);
     const int64_t align = 256 / es;
-    const int64_t plane = (ncell + align - 1) / align * align;
-    c->lat.plane = plane;
+    c->lat.pitch = padded_pitch(c->D, precision, dims[0]);
+    int64_t plane = (c->lat.pitch * dims[1] * dims[2] + align - 1) / align * align;
     c->lat.nx = (int)dims[0];
     c->lat.ny = (int)dims[1];
     c->lat.nz = (int)dims[2];
     c->lat.ncell = ncell;
     c->lat.D = c->D;
     c->lat.P = precision;
-    const size_t bytes = (size_t)c->Q * plane * es;
-    if (cudaMalloc(&c->lat.A, bytes) != cudaSuccess) {
+    size_t bytes = (size_t)c->Q * plane * es;
+    cudaError_t em = cudaMalloc(&c->lat.A, bytes);
+    if (em != cudaSuccess && c->lat.pitch != c->lat.nx) {
+        // no room for the padding: unpadded rows (and the one-cell kernel)
+        cudaGetLastError();
+        c->lat.pitch = c->lat.nx;
+        plane = (ncell + align - 1) / align * align;
+        bytes = (size_t)c->Q * plane * es;
+        em = cudaMalloc(&c->lat.A, bytes);
+    }
+    c->lat.plane = plane;
+    if (em != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return fail(LBM_ENOMEM, "population storage of %zu bytes", bytes);
     }
-    bool ok = cudaMalloc(&c->partials, sizeof(double) * kDiagWords * kPartialsCap) == cudaSuccess &&
-              cudaMalloc(&c->hist, sizeof(double) * 8 * kHistCap) == cudaSuccess &&
-              cudaMalloc(&c->scratch, sizeof(double) * 8) == cudaSuccess &&
-              cudaMalloc(&c->status, sizeof(int32_t)) == cudaSuccess;
-    if (!ok) {
+    // one allocation for the small buffers; the status word and the counters start at zero
+    const size_t zeroed = 256 + (sizeof(unsigned) * (kSyncDone + sync_units(c->lat)) + 255) / 256 * 256;
+    const size_t recs = sizeof(double) * kDiagWords * (kPartialsCap + kHistCap + 4);
+    char *aux = nullptr;
+    if (cudaMalloc(&aux, zeroed + recs) != cudaSuccess) {
         cudaGetLastError();
         lbm_destroy(c);
         return fail(LBM_ENOMEM, "diagnostics buffers");
     }
+    c->status = reinterpret_cast<int32_t *>(aux);
+    c->sync = reinterpret_cast<unsigned *>(aux + 256);
+    c->partials = reinterpret_cast<double *>(aux + zeroed);
+    c->hist = c->partials + kDiagWords * kPartialsCap;
+    c->scratch = c->hist + 8 * kHistCap;
     if (cudaMemsetAsync(c->lat.A, 0, bytes, c->stream) != cudaSuccess ||
-        cudaMemsetAsync(c->status, 0, sizeof(int32_t), c->stream) != cudaSuccess) {
+        cudaMemsetAsync(aux, 0, zeroed, c->stream) != cudaSuccess) {
         lbm_destroy(c);
         return cuda_fail("initial memset", cudaGetLastError());
     }
@@ -680,7 +730,7 @@ int lbm_set_option(lbm_ctx *c, int option, int64_t value) {
         return LBM_OK;
     case LBM_OPT_KERNEL:
         if (value < 0 || value > 2) return fail(LBM_EINVAL, "kernel must be 0, 1 or 2");
-        if (value == 2 && !tma_supported(c->lat))
+        if (value == 2 && !tma_selectable(c))
             return fail(LBM_EINVAL, "TMA row kernel needs Nx * sizeof(storage) to be a multiple of 16");
         c->kernel_opt = (int)value;
         if (value == 1) c->kernel = 1;
@@ -772,6 +822,16 @@ int lbm_step(lbm_ctx *c, int64_t n) {
     for (; s < n; ++s) {
         const int odd = (int)(c->step & 1);
         const int diag = c->diag_every > 0 && (c->step % c->diag_every) == 0;
+        if (!diag) {
+            // up to the next diagnostics step
+            int64_t m = n - s;
+            if (c->diag_every > 0) m = std::min(m, c->diag_every - c->step % c->diag_every);
+            cudaError_t e = launch_steps(c, odd, m, c->stream);
+            if (e != cudaSuccess) return ctx_sticky(c, cuda_fail("step launch", e));
+            c->step += m;
+            s += m - 1;
+            continue;
+        }
         cudaError_t e = launch_one(c, odd, diag, c->stream);
         if (e != cudaSuccess) return ctx_sticky(c, cuda_fail("step launch", e));
         if (diag) {
@@ -995,7 +1055,7 @@ int lbm_set_launch_shape(lbm_ctx *c, const int64_t shape[6]) {
         return LBM_OK;
     }
     if (shape[0] != 2) return fail(LBM_EINVAL, "kernel must be 1 or 2");
-    if (!tma_supported(c->lat)) return fail(LBM_EINVAL, "TMA row kernel needs Nx * sizeof(storage) %% 16 == 0");
+    if (!tma_selectable(c)) return fail(LBM_EINVAL, "TMA row kernel needs Nx * sizeof(storage) %% 16 == 0");
     const int tmax = tma_thread_limit(c->lat);
     if (shape[1] < 32 || shape[1] > tmax || shape[1] % 32)
         return fail(LBM_EINVAL, "threads must be a multiple of 32 in [32, %d] for this lattice and storage", tmax);
@@ -1032,10 +1092,7 @@ void lbm_destroy(lbm_ctx *c) {
     cudaStreamSynchronize(c->stream);
     drop_graph(c);
     cudaFree(c->lat.A);
-    cudaFree(c->partials);
-    cudaFree(c->hist);
-    cudaFree(c->scratch);
-    cudaFree(c->status);
+    cudaFree(c->status);  // the start of the small buffers' allocation
     cudaFree(c->stage[0]);
     cudaFree(c->stage[1]);
     cudaGetLastError();

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256) k_step_batch(const lbmh::BatchArgs a) {
                 const int y = (int)(r % ny);
                 const int z = (int)(r / ny);
                 const CellMoments<double> m =
-                    aa_cell_step<D, P_F64, EQ, BULK>(A, ncell, nx, ny, nz, x, y, z, odd, a.rho0, om, sn);
+                    aa_cell_step<D, P_F64, EQ, BULK>(A, ncell, nx, ny, nz, nx, x, y, z, odd, a.rho0, om, sn);
                 if (probe) {
                     // exp(-i k.r) = tw_x[x] tw_y[y] tw_z[z]
                     const double2 tx = tw[x], ty = tw[nx + y];
@@ -135,7 +135,7 @@ __global__ void k_batch_moments(const double *arena, const int64_t *cell_start, 
         const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((int64_t)nx * ny));
         const double *A = arena + (int64_t)Q * c0;
         double f[Q];
-        for (int i = 0; i < Q; ++i) f[i] = A[aa_index<D>(i, x, y, z, nx, ny, nz, n, odd)];
+        for (int i = 0; i < Q; ++i) f[i] = A[aa_index<D>(i, x, y, z, nx, ny, nz, nx, n, odd)];
         const CellMoments<double> m = moments_shifted<D, double>(f, rho0);
         rho[g] = Out(m.rho);
         for (int a = 0; a < D; ++a) u[(int64_t)D * c0 + a * n + c] = Out(m.u[a]);
@@ -154,7 +154,7 @@ __global__ void k_batch_pop(const double *arena, const int64_t *cell_start, cons
         const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((int64_t)nx * ny));
         const double *A = arena + (int64_t)Q * c0;
         for (int i = 0; i < Q; ++i)
-            f[(int64_t)Q * c0 + (int64_t)i * n + c] = Out(A[aa_index<D>(i, x, y, z, nx, ny, nz, n, odd)] + wq<D>(i) * rho0);
+            f[(int64_t)Q * c0 + (int64_t)i * n + c] = Out(A[aa_index<D>(i, x, y, z, nx, ny, nz, nx, n, odd)] + wq<D>(i) * rho0);
     }
 }
 

@@ -35,8 +35,11 @@ __global__ void k_init(lbmh::Lattice lat, double rho0d, const In *__restrict__ r
         R h[Q];
         equilibrium_h<D, EQ, R>(uu, h);
         const R drho = r - rho0;
+        int x, y, z;
+        cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
+        const int64_t cell = x + (int64_t)lat.pitch * (y + (int64_t)lat.ny * z);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) A[(int64_t)i * lat.plane + c] = St::store(R(wq<D>(i)) * fma_r(r, h[i], drho));
+        for (int i = 0; i < Q; ++i) A[(int64_t)i * lat.plane + cell] = St::store(R(wq<D>(i)) * fma_r(r, h[i], drho));
     }
 }
 
@@ -46,13 +49,10 @@ __device__ __forceinline__ void load_canonical(const lbmh::Lattice &lat, int odd
                                                int &y, int &z) {
     using St = Storage<P>;
     const auto *A = static_cast<const typename St::T *>(lat.A);
-    x = (int)(c % lat.nx);
-    const int64_t r = c / lat.nx;
-    y = (int)(r % lat.ny);
-    z = (int)(r / lat.ny);
+    cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
 #pragma unroll
     for (int i = 0; i < qof(D); ++i)
-        f[i] = St::load(A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.plane, odd)]);
+        f[i] = St::load(A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)]);
 }
 
 template <int D, int P, typename Out>
@@ -92,13 +92,12 @@ __global__ void k_set_pop(lbmh::Lattice lat, double rho0, int odd, const In *__r
     auto *A = static_cast<typename St::T *>(lat.A);
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < lat.ncell;
          c += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(c % lat.nx);
-        const int64_t r = c / lat.nx;
-        const int y = (int)(r % lat.ny), z = (int)(r / lat.ny);
+        int x, y, z;
+        cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
 #pragma unroll
         for (int i = 0; i < qof(D); ++i) {
             const double v = (double)f[(int64_t)i * lat.ncell + c] - wq<D>(i) * rho0;
-            A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.plane, odd)] = St::store(R(v));
+            A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)] = St::store(R(v));
         }
     }
 }
@@ -109,12 +108,11 @@ __global__ void k_get_pop_raw(lbmh::Lattice lat, int odd, typename Storage<P>::T
     const auto *A = static_cast<const typename Storage<P>::T *>(lat.A);
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < lat.ncell;
          c += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(c % lat.nx);
-        const int64_t r = c / lat.nx;
-        const int y = (int)(r % lat.ny), z = (int)(r / lat.ny);
+        int x, y, z;
+        cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
 #pragma unroll
         for (int i = 0; i < qof(D); ++i)
-            f[(int64_t)i * lat.ncell + c] = A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.plane, odd)];
+            f[(int64_t)i * lat.ncell + c] = A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)];
     }
 }
 
@@ -123,12 +121,11 @@ __global__ void k_set_pop_raw(lbmh::Lattice lat, int odd, const typename Storage
     auto *A = static_cast<typename Storage<P>::T *>(lat.A);
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < lat.ncell;
          c += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(c % lat.nx);
-        const int64_t r = c / lat.nx;
-        const int y = (int)(r % lat.ny), z = (int)(r / lat.ny);
+        int x, y, z;
+        cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
 #pragma unroll
         for (int i = 0; i < qof(D); ++i)
-            A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.plane, odd)] = f[(int64_t)i * lat.ncell + c];
+            A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)] = f[(int64_t)i * lat.ncell + c];
     }
 }
 

@@ -20,7 +20,7 @@ namespace lbmd {
 // elements at A; returns the cell's pre-collision moments.
 template <int D, int P, int EQ, bool BULK>
 __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
-    typename Storage<P>::T *__restrict__ A, int64_t plane, int nx, int ny, int nz, int x, int y,
+    typename Storage<P>::T *__restrict__ A, int64_t plane, int nx, int ny, int nz, int pitch, int x, int y,
     int z, int odd, typename Storage<P>::R rho0, typename Storage<P>::R omega0,
     typename Storage<P>::R six_nu, int32_t *status = nullptr) {
     using St = Storage<P>;
@@ -29,11 +29,11 @@ __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
     // checked builds: the cell and (through the periodic wrap) all its neighbours lie
     // inside the lattice, so every index below stays inside the Q planes
     if (!LBM_CHECK(x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz &&
-                       (int64_t)nx * ny * nz <= plane, status)) {
+                       (int64_t)pitch * ny * nz <= plane, status)) {
         CellMoments<R> none{};
         return none;
     }
-    const int64_t cell = x + (int64_t)nx * (y + (int64_t)ny * z);
+    const int64_t cell = x + (int64_t)pitch * (y + (int64_t)ny * z);
     const int xs[3] = {wrapi(x - 1, nx), x, wrapi(x + 1, nx)};
     const int ys[3] = {wrapi(y - 1, ny), y, wrapi(y + 1, ny)};
     const int zs[3] = {D == 3 ? wrapi(z - 1, nz) : z, z, D == 3 ? wrapi(z + 1, nz) : z};
@@ -46,11 +46,11 @@ __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
         for (int i = 0; i < Q; ++i) {
             // f_i(r) = A[opp(i)][r - c_i]
             const int64_t src = xs[1 - cxo(i)] +
-                                (int64_t)nx * (ys[1 - cyo(i)] + (int64_t)ny * zs[1 - (D == 3 ? czo(i) : 0)]);
+                                (int64_t)pitch * (ys[1 - cyo(i)] + (int64_t)ny * zs[1 - (D == 3 ? czo(i) : 0)]);
             f[i] = St::load(A[(int64_t)(Q - 1 - i) * plane + src]);
         }
     }
-    const CellMoments<R> m = collide<D, EQ, BULK, R, relax_two_fma<D, P>()>(f, rho0, omega0, six_nu);
+    const CellMoments<R> m = collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
     if (!odd) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) A[(int64_t)(Q - 1 - i) * plane + cell] = St::store(f[i]);
@@ -58,7 +58,7 @@ __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int64_t dst = xs[1 + cxo(i)] +
-                                (int64_t)nx * (ys[1 + cyo(i)] + (int64_t)ny * zs[1 + (D == 3 ? czo(i) : 0)]);
+                                (int64_t)pitch * (ys[1 + cyo(i)] + (int64_t)ny * zs[1 + (D == 3 ? czo(i) : 0)]);
             A[(int64_t)i * plane + dst] = St::store(f[i]);
         }
     }
@@ -77,24 +77,11 @@ __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
     DiagAcc acc;
     DiagLocal<R> loc;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const bool small = a.lat.ncell < ((int64_t)1 << 31);
     for (int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; cell < a.lat.ncell;
          cell += stride) {
         int x, y, z;
-        if (small) {  // 32-bit index arithmetic
-            const unsigned c = (unsigned)cell;
-            const unsigned rowi = c / (unsigned)nx;
-            x = (int)(c - rowi * (unsigned)nx);
-            const unsigned zq = rowi / (unsigned)ny;
-            y = (int)(rowi - zq * (unsigned)ny);
-            z = (int)zq;
-        } else {
-            x = (int)(cell % nx);
-            const int64_t rowi = cell / nx;
-            y = (int)(rowi % ny);
-            z = (int)(rowi / ny);
-        }
-        const CellMoments<R> m = aa_cell_step<D, P, EQ, BULK>(A, a.lat.plane, nx, ny, nz, x, y, z,
+        cell_coords(cell, a.lat.ncell, nx, ny, x, y, z);
+        const CellMoments<R> m = aa_cell_step<D, P, EQ, BULK>(A, a.lat.plane, nx, ny, nz, a.lat.pitch, x, y, z,
                                                               a.odd, rho0, omega0, six_nu, a.status);
         if (a.diag) {
             loc.add(m.rho, m.u, rho0);

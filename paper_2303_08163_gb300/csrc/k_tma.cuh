@@ -13,15 +13,21 @@
 // memory and buffer b is stored back to exactly the global location it was loaded from.
 // Different jobs touch disjoint global locations, so jobs need no ordering.
 //
-// Data movement (warp specialised): the last warp of the block is the producer, the
-// others collide.  Lane b of the producer issues the cp.async.bulk copies of buffer b
-// (global -> shared, completion counted in transaction bytes on the stage's `full`
-// mbarrier) and later the cp.async.bulk stores of the same buffer (shared -> global) in
-// its own bulk async-group, so each lane orders its own store before its own refill of
-// that buffer.  Consumer warps wait on `full`, collide the job in place, fence their
-// shared-memory writes for the async proxy and arrive on the stage's `empty` mbarrier;
-// the producer then stores the stage back and refills it `stages` jobs ahead.  Rows must
-// be 16-byte multiples (Nx * sizeof(storage) % 16 == 0).
+// Data movement (warp specialised): after the colliding (consumer) warps come a loader and a
+// storer warp.  Lane b of the loader issues the cp.async.bulk copies of buffer b (global ->
+// shared, completion counted in transaction bytes on the stage's `full` mbarrier).  Consumer
+// warps wait on `full`, collide the job in place, fence their shared-memory writes for the
+// async proxy and arrive on the stage's `empty` mbarrier.  Lane b of the storer then issues
+// the cp.async.bulk stores of buffer b, and once they have read the stage it arrives on
+// `freed` and the loader refills it.  Two warps, because a loader that waits for another
+// block's step (below) must not hold up the stores that other blocks wait for.  Rows must
+// start on 16-byte boundaries: the row pitch is a multiple of 16 bytes (a ragged row is
+// padded to it, and whole rows are copied with their padding; the cells of the padding are
+// never read by a real cell).
+//
+// One launch advances one step (jobs strided over the blocks, no waits; the diagnostics are
+// reduced here) or several (jobs by ticket, with counters of finished jobs; see
+// decode_chain).
 //
 // Segmented rows (seg < Nx) carry a halo of U = 16 / sizeof(storage) cells on each side.
 // In the odd step the cells of a segment touch positions [X0 - 1, X0 + len - 1) of the
@@ -41,42 +47,124 @@ constexpr int kTmaMaxThreads = 256;  // consumer threads of the D3Q27 kernels; o
 __host__ __device__ constexpr int tma_max_threads(int D, int P) { return D == 2 && P == 2 ? 512 : kTmaMaxThreads; }
 
 // bufstride (elements between direction buffers) equals the compile-time buffer
-// capacity CAPB / sizeof(storage) of the kernel instantiation.
+// capacity CAPB / sizeof(storage) of the kernel instantiation.  rowstride is the distance
+// between the rows of a job in shared memory: the row pitch for whole rows (the copies
+// carry the padding along), the segment with its halos otherwise (rows without padding).
 struct TmaGeom {
     int stages, rows, seg, nseg, ygroups, halo, rowstride, bufstride;
     int64_t njobs;
+    // several steps in one launch (nsteps > 1), see decode_chain
+    int nsteps, npos, ncross, strips, stripw, pjobs, depth, lag;
 };
 
 constexpr int kTmaCaps[4] = {1024, 2048, 4096, 8192};  // bytes per direction buffer
 
 struct JobPos {
     int z, y0, nrows, X0, len;
+    int odd;  // AA parity of the job's step
 };
 
-__device__ __forceinline__ JobPos decode_job(const lbmh::StepArgs &a, const TmaGeom &g, int64_t job) {
+__device__ __forceinline__ JobPos job_at(const lbmh::StepArgs &a, const TmaGeom &g, int z, int yg, int s, int odd) {
     JobPos j;
-    const unsigned jb = (unsigned)job;  // njobs < 2^31 (checked on the host)
-    const unsigned rest = jb / (unsigned)g.nseg;
-    const int s = (int)(jb - rest * (unsigned)g.nseg);
-    const unsigned zq = rest / (unsigned)g.ygroups;
-    const int yg = (int)(rest - zq * (unsigned)g.ygroups);
-    j.z = (int)zq;
+    j.z = z;
     j.y0 = yg * g.rows;
     j.nrows = min(g.rows, a.lat.ny - j.y0);
     j.X0 = s * g.seg;
     j.len = min(g.seg, a.lat.nx - j.X0);
+    j.odd = odd;
     return j;
+}
+
+// One step (nsteps == 1): job number -> rows and segment.
+__device__ __forceinline__ JobPos decode_job(const lbmh::StepArgs &a, const TmaGeom &g, unsigned job) {
+    const unsigned rest = job / (unsigned)g.nseg;
+    const unsigned zq = rest / (unsigned)g.ygroups;
+    return job_at(a, g, (int)zq, (int)(rest - zq * (unsigned)g.ygroups), (int)(job - rest * (unsigned)g.nseg), a.odd);
+}
+
+// Several steps (nsteps > 1).  The units of the lattice are its row groups, at position p of
+// the sweep axis and c across it: (p, c) = (z, row group) in 3-D, (row group, 0) in 2-D.  Job
+// (s, p, c, segment) -- step s -- needs step s - 1 of the units (p +- 1, c +- 1) (periodic) and
+// nothing else: the AA pattern's locations that it reads and writes were last touched by
+// cells of those.  A counter per unit holds its finished jobs.
+//
+// `depth` steps travel along the sweep axis together, each `lag` positions behind the one
+// before, so that a position comes from HBM once for `depth` steps while the positions
+// between the first and the last of them stay in L2.  Where whole positions are too large
+// for that, they are cut across into `strips` swept one after the other; a strip moves down
+// by one row group a step (its lower neighbour is done, its upper one is not), the first
+// one shrinks from both ends and the last one grows into the periodic wrap:
+//   strip k at inner step t covers c in [k H - t, (k + 1) H - t), from t in the first,
+//   to ncross + t in the last.
+// Step s starts at position s, so that its periodic neighbour is among the first that step
+// s - 1 finished:
+//   ticket -> (phase, t, job), phase - lag t = (q strips + k) npos + i, s = q depth + t,
+//   p = (s + i) mod npos.
+// Every job comes after the jobs it needs in ticket order (lag >= 2, npos > lag (depth - 1)
+// + 2), and blocks take tickets from one counter, so whichever blocks are resident, the
+// holder of the smallest unfinished ticket never waits: no deadlock, no need for all blocks
+// to run at once.
+struct ChainJob {
+    JobPos j;
+    int step, p, c;  // step < 0: no job (the ends of the wavefront and of the strips)
+};
+
+__host__ __device__ __forceinline__ void chain_strip(const TmaGeom &g, int k, int t, int &lo, int &hi) {
+    lo = 0;
+    hi = g.ncross;
+    if (g.strips > 1) {
+        lo = k == 0 ? t : k * g.stripw - t;
+        hi = k == g.strips - 1 ? g.ncross + t : (k + 1) * g.stripw - t;
+    }
+}
+
+__device__ __forceinline__ ChainJob decode_chain(const lbmh::StepArgs &a, const TmaGeom &g, unsigned ticket) {
+    ChainJob r;
+    const unsigned slot = ticket / (unsigned)g.pjobs;
+    const unsigned jj = ticket - slot * (unsigned)g.pjobs;
+    const unsigned phase = slot / (unsigned)g.depth;
+    const int t = (int)(slot - phase * (unsigned)g.depth);
+    const int x = (int)phase - g.lag * t;
+    r.step = -1;
+    r.p = r.c = 0;
+    r.j = JobPos{0, 0, 0, 0, 0, 0};
+    if (x < 0) return r;
+    const int qk = x / g.npos, i = x - qk * g.npos, q = qk / g.strips, k = qk - q * g.strips;
+    const int s = q * g.depth + t;
+    if (s >= g.nsteps) return r;
+    int lo, hi;
+    chain_strip(g, k, t, lo, hi);
+    const unsigned row = jj / (unsigned)g.nseg;
+    int c = lo + (int)row;
+    if (c >= hi) return r;
+    if (c >= g.ncross) c -= g.ncross;
+    r.step = s;
+    r.p = (int)(((unsigned)s + (unsigned)i) % (unsigned)g.npos);
+    r.c = c;
+    const bool flat = a.lat.D == 2;
+    r.j = job_at(a, g, flat ? 0 : r.p, flat ? r.p : c, (int)(jj - row * (unsigned)g.nseg), (a.odd + s) & 1);
+    return r;
+}
+
+__host__ __device__ __forceinline__ int64_t chain_tickets(const TmaGeom &g) {
+    const int64_t supers = (g.nsteps + g.depth - 1) / g.depth;
+    return (supers * g.strips * g.npos + (int64_t)g.lag * (g.depth - 1)) * g.depth * g.pjobs;
 }
 
 // Global row (plane, y, z) of buffer b of a job.
 template <int D, typename T>
-__device__ __forceinline__ T *buffer_row(const lbmh::StepArgs &a, int b, int z, int y) {
+__device__ __forceinline__ T *buffer_row(const lbmh::StepArgs &a, int odd, int b, int z, int y) {
     constexpr int Q = qof(D);
-    const int plane = a.odd ? Q - 1 - b : b;
-    const int zz = (D == 3 && a.odd) ? wrapi(z - czo(b), a.lat.nz) : z;
-    const int yy = a.odd ? wrapi(y - cyo(b), a.lat.ny) : y;
+    const int plane = odd ? Q - 1 - b : b;
+    const int zz = (D == 3 && odd) ? wrapi(z - czo(b), a.lat.nz) : z;
+    const int yy = odd ? wrapi(y - cyo(b), a.lat.ny) : y;
     return static_cast<T *>(a.lat.A) + (int64_t)plane * a.lat.plane +
-           ((int64_t)zz * a.lat.ny + yy) * a.lat.nx;
+           ((int64_t)zz * a.lat.ny + yy) * a.lat.pitch;
+}
+
+// Elements one row of a job's copies moves: the whole row with its padding, or the segment.
+__device__ __forceinline__ int copy_len(const TmaGeom &g, const JobPos &j) {
+    return g.nseg == 1 ? g.rowstride : j.len;
 }
 
 // Bytes of one job's loads (all buffers), for the stage's expect-tx.
@@ -84,8 +172,8 @@ template <int D, typename T>
 __device__ __forceinline__ uint32_t tma_job_bytes(const lbmh::StepArgs &a, const TmaGeom &g, const JobPos &j) {
     constexpr int Q = qof(D);
     constexpr int U = 16 / (int)sizeof(T);
-    uint32_t bytes = (uint32_t)(Q * j.nrows * j.len * (int)sizeof(T));
-    if (a.odd && g.nseg > 1) bytes += (uint32_t)((2 * Q / 3) * U * (int)sizeof(T));
+    uint32_t bytes = (uint32_t)(Q * j.nrows * copy_len(g, j) * (int)sizeof(T));
+    if (j.odd && g.nseg > 1) bytes += (uint32_t)((2 * Q / 3) * U * (int)sizeof(T));
     return bytes;
 }
 
@@ -116,16 +204,16 @@ __device__ __forceinline__ void tma_issue_loads(const lbmh::StepArgs &a, const T
     T *sbuf = st + (int64_t)b * g.bufstride;
     int r = 0;
     while (r < j.nrows) {
-        const int ysrc = a.odd ? wrapi(j.y0 + r - cyo(b), ny) : j.y0 + r;
+        const int ysrc = j.odd ? wrapi(j.y0 + r - cyo(b), ny) : j.y0 + r;
         const int run = min(j.nrows - r, ny - ysrc);
-        const T *src = buffer_row<D, T>(a, b, j.z, j.y0 + r) + j.X0;
+        const T *src = buffer_row<D, T>(a, j.odd, b, j.z, j.y0 + r) + j.X0;
         T *dst = sbuf + r * g.rowstride + g.halo;
-        const uint32_t bytes = (uint32_t)(run * j.len * (int)sizeof(T));
+        const uint32_t bytes = (uint32_t)(run * copy_len(g, j) * (int)sizeof(T));
         if (bulk_ok<D, T>(a, g, st, dst, src, bytes)) bulk_g2s(dst, src, bytes, bar);
         r += run;
     }
-    if (a.odd && g.nseg > 1) {
-        const T *grow = buffer_row<D, T>(a, b, j.z, j.y0);
+    if (j.odd && g.nseg > 1) {
+        const T *grow = buffer_row<D, T>(a, j.odd, b, j.z, j.y0);
         if (cxo(b) == 1) {
             const int xs = j.X0 == 0 ? nx - U : j.X0 - U;
             if (bulk_ok<D, T>(a, g, st, sbuf, grow + xs, U * sizeof(T))) bulk_g2s(sbuf, grow + xs, U * sizeof(T), bar);
@@ -144,19 +232,19 @@ __device__ __forceinline__ void tma_issue_stores(const lbmh::StepArgs &a, const 
     constexpr int U = 16 / (int)sizeof(T);
     const int ny = a.lat.ny;
     T *sbuf = st + (int64_t)b * g.bufstride;
-    if (!(a.odd && g.nseg > 1)) {
+    if (!(j.odd && g.nseg > 1)) {
         int r = 0;
         while (r < j.nrows) {
-            const int ysrc = a.odd ? wrapi(j.y0 + r - cyo(b), ny) : j.y0 + r;
+            const int ysrc = j.odd ? wrapi(j.y0 + r - cyo(b), ny) : j.y0 + r;
             const int run = min(j.nrows - r, ny - ysrc);
-            T *dst = buffer_row<D, T>(a, b, j.z, j.y0 + r) + j.X0;
+            T *dst = buffer_row<D, T>(a, j.odd, b, j.z, j.y0 + r) + j.X0;
             const T *src = sbuf + r * g.rowstride + g.halo;
-            const uint32_t bytes = (uint32_t)(run * j.len * (int)sizeof(T));
+            const uint32_t bytes = (uint32_t)(run * copy_len(g, j) * (int)sizeof(T));
             if (bulk_ok<D, T>(a, g, st, src, dst, bytes)) bulk_s2g(dst, src, bytes);
             r += run;
         }
     } else {
-        T *grow = buffer_row<D, T>(a, b, j.z, j.y0);
+        T *grow = buffer_row<D, T>(a, j.odd, b, j.z, j.y0);
         if (cxo(b) == 0) {
             const uint32_t bytes = (uint32_t)(j.len * (int)sizeof(T));
             if (bulk_ok<D, T>(a, g, st, sbuf + g.halo, grow + j.X0, bytes)) bulk_s2g(grow + j.X0, sbuf + g.halo, bytes);
@@ -180,7 +268,7 @@ __device__ __forceinline__ void tma_plain_stores(const lbmh::StepArgs &a, const 
     for (int t = tid; t < NB * U; t += nthr) {
         const int k = t / U, e = t - (t / U) * U;
         const int b = (k >> 1) * 3 + ((k & 1) ? 2 : 0);  // k-th direction with c_x != 0
-        T *grow = buffer_row<D, T>(a, b, j.z, j.y0);
+        T *grow = buffer_row<D, T>(a, j.odd, b, j.z, j.y0);
         const T *srow = st + (int64_t)b * g.bufstride;
         int gx, sx;
         if (cxo(b) == 1) {
@@ -270,9 +358,9 @@ __device__ __forceinline__ void tma_compute(const lbmh::StepArgs &a, const TmaGe
         // checked builds: every position the cell touches lies inside its direction buffer
         if (LBM_CHECK(p.row + min(p.xm, p.x) >= 0 && p.row + max(p.xp, p.x) < g.bufstride, a.status)) {
             R f[Q];
-            tma_load_cell<D, P, CAPB>(st, p, a.odd, f);
-            const CellMoments<R> m = collide<D, EQ, BULK, R, relax_two_fma<D, P>()>(f, rho0, omega0, six_nu);
-            tma_store_cell<D, P, CAPB>(st, p, a.odd, f);
+            tma_load_cell<D, P, CAPB>(st, p, j.odd, f);
+            const CellMoments<R> m = collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
+            tma_store_cell<D, P, CAPB>(st, p, j.odd, f);
             if (a.diag) loc.add(m.rho, m.u, rho0);
         }
         xl += nthr;
@@ -284,39 +372,54 @@ __device__ __forceinline__ void tma_compute(const lbmh::StepArgs &a, const TmaGe
     if (a.diag) loc.flush(acc, a.rho0);
 }
 
-// binary16 storage: the same collision, two neighbouring cells per thread per iteration,
-// so that every buffer position pair the two cells own at an even offset moves as one
-// 32-bit shared-memory access and one paired conversion.  Even step: cells (x, x + 1),
-// x even, own the pair at x in every buffer.  Odd step, whole rows: cells (x, x + 1), x
-// odd (the last pair is (len - 1, 0)), own the pairs at x - 1 and x + 1 in the buffers
-// with c_x != 0; the c_x = 0 buffers go one half at a time.  Odd step, segments (no wrap
-// inside the job): cells (x, x + 1), x even, own the pair at x in the c_x = 0 buffers and
-// go one half at a time elsewhere.  The conversions round exactly as the one-cell path
-// does, so the stored state is the same bit for bit.
-__device__ __forceinline__ float2 ld_pair(const __half *b, int p) {
-    return __half22float2(*reinterpret_cast<const __half2 *>(b + p));
+// FP32 and binary16 storage: two neighbouring cells per thread per iteration, one in each
+// half of the packed FP32 collision (collide32 over f32x2).  Every buffer position pair the
+// two cells own at an even offset moves as one shared-memory access (and for binary16 one
+// paired conversion).  Even step: cells (x, x + 1), x even, own the pair at x in every buffer.
+// Odd step, whole rows: cells (x, x + 1), x odd (the last pair is (len - 1, 0)), own the pairs
+// at x - 1 and x + 1 in the buffers with c_x != 0; the c_x = 0 buffers go one half at a time.
+// Odd step, segments (no wrap inside the job): cells (x, x + 1), x even, own the pair at x in
+// the c_x = 0 buffers and go one half at a time elsewhere.  The operations and conversions
+// round exactly as the one-cell path does, so the stored state is the same bit for bit.  Rows
+// of odd length (padded rows) go one cell at a time: a pairing that wraps has no aligned
+// pairs there.
+__device__ __forceinline__ f32x2 ld_pair(const __half *b, int p) {
+    const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(b + p));
+    return pack2(v.x, v.y);
 }
-__device__ __forceinline__ void st_pair(__half *b, int p, float lo, float hi) {
+__device__ __forceinline__ f32x2 ld_pair(const float *b, int p) {
+    const float2 v = *reinterpret_cast<const float2 *>(b + p);
+    return pack2(v.x, v.y);
+}
+__device__ __forceinline__ void st_pair(__half *b, int p, f32x2 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
     *reinterpret_cast<__half2 *>(b + p) = __floats2half2_rn(lo, hi);
+}
+__device__ __forceinline__ void st_pair(float *b, int p, f32x2 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    *reinterpret_cast<float2 *>(b + p) = make_float2(lo, hi);
 }
 
 // MODE 0: even step; 1: odd step, whole rows; 2: odd step, segments; -1: chosen at run
 // time from the step parity and the job layout (one loop body for all three).
-template <int D, int EQ, bool BULK, int CAPB, int MODE>
+template <int D, int P, int EQ, bool BULK, int CAPB, int MODE>
 __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const TmaGeom &g,
-                                                  const JobPos &j, __half *st, DiagAcc &acc,
+                                                  const JobPos &j, typename Storage<P>::T *st, DiagAcc &acc,
                                                   int tid, int nthr) {
+    using St = Storage<P>;
+    using T = typename St::T;
     constexpr int Q = qof(D);
-    constexpr int bs = CAPB / 2;  // halves between direction buffers
-    const int mode = MODE >= 0 ? MODE : (!a.odd ? 0 : (g.nseg == 1 ? 1 : 2));
-    const float rho0 = a.rho0f, omega0 = a.omega0f, six_nu = a.six_nuf;
-    const int hl = j.len >> 1;  // len is a multiple of 8 cells (16-byte rows)
+    constexpr int bs = CAPB / (int)sizeof(T);  // elements between direction buffers
+    const int mode = MODE >= 0 ? MODE : (!j.odd ? 0 : (g.nseg == 1 ? 1 : 2));
+    const int hl = j.len >> 1;  // len is even here
     const int npairs = j.nrows * hl;
     DiagLocal<float> loc;
     int r = tid / hl;
     int xh = tid - r * hl;
     for (int c = tid; c < npairs; c += nthr) {
-        __half *row = st + r * g.rowstride + g.halo;
+        T *row = st + r * g.rowstride + g.halo;
         // cells xa and xb = xa + 1 (the odd pairing of whole rows wraps its last pair to
         // cell 0); pm = xa - 1 and pp = xb + 1 are the outer neighbours, inside the row for
         // whole rows (xa >= 1 in the odd pairing) and in the halos for segments
@@ -329,78 +432,63 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
         const int lo = mode == 0 ? xa : min(min(pm, xa), xb);
         const int hi = mode == 0 ? xa + 1 : max(max(xb + 1, pp), xa);
         if (LBM_CHECK(row_off + lo >= 0 && row_off + hi < bs, a.status)) {
-            float fa[Q], fb[Q];
+            f32x2 f[Q];
             if (mode == 0) {
     #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    const float2 v = ld_pair(row + i * bs, xa);
-                    fa[i] = v.x;
-                    fb[i] = v.y;
-                }
+                for (int i = 0; i < Q; ++i) f[i] = ld_pair(row + i * bs, xa);
             } else if (mode == 1) {
     #pragma unroll
                 for (int i = 0; i < Q; ++i) {
-                    const __half *b = row + i * bs;
-                    if (cxo(i) == 0) {
-                        fa[i] = __half2float(b[xa]);
-                        fb[i] = __half2float(b[xb]);
-                    } else {
-                        const float2 v = ld_pair(b, cxo(i) == 1 ? pm : xb);
-                        fa[i] = v.x;
-                        fb[i] = v.y;
-                    }
+                    const T *b = row + i * bs;
+                    if (cxo(i) == 0) f[i] = pack2(St::load(b[xa]), St::load(b[xb]));
+                    else f[i] = ld_pair(b, cxo(i) == 1 ? pm : xb);
                 }
             } else {
     #pragma unroll
                 for (int i = 0; i < Q; ++i) {
-                    const __half *b = row + i * bs;
-                    if (cxo(i) == 0) {
-                        const float2 v = ld_pair(b, xa);
-                        fa[i] = v.x;
-                        fb[i] = v.y;
-                    } else if (cxo(i) == 1) {
-                        fa[i] = __half2float(b[pm]);
-                        fb[i] = __half2float(b[xa]);
-                    } else {
-                        fa[i] = __half2float(b[xb]);
-                        fb[i] = __half2float(b[pp]);
-                    }
+                    const T *b = row + i * bs;
+                    if (cxo(i) == 0) f[i] = ld_pair(b, xa);
+                    else if (cxo(i) == 1) f[i] = pack2(St::load(b[pm]), St::load(b[xa]));
+                    else f[i] = pack2(St::load(b[xb]), St::load(b[pp]));
                 }
             }
-            const CellMoments<float> ma = collide<D, EQ, BULK, float, relax_two_fma<D, P_F16S>()>(fa, rho0, omega0, six_nu);
-            const CellMoments<float> mb = collide<D, EQ, BULK, float, relax_two_fma<D, P_F16S>()>(fb, rho0, omega0, six_nu);
+            const Moments32<f32x2> m = collide32<D, P, EQ, BULK, f32x2>(f, a.rho0f, a.omega0f, a.six_nuf);
             if (mode == 0) {
     #pragma unroll
-                for (int i = 0; i < Q; ++i) st_pair(row + (Q - 1 - i) * bs, xa, fa[i], fb[i]);
-            } else if (mode == 1) {
-    #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    __half *b = row + (Q - 1 - i) * bs;
-                    if (cxo(i) == 0) {
-                        b[xa] = __float2half_rn(fa[i]);
-                        b[xb] = __float2half_rn(fb[i]);
-                    } else {
-                        st_pair(b, cxo(i) == 1 ? xb : pm, fa[i], fb[i]);
-                    }
-                }
+                for (int i = 0; i < Q; ++i) st_pair(row + (Q - 1 - i) * bs, xa, f[i]);
             } else {
     #pragma unroll
                 for (int i = 0; i < Q; ++i) {
-                    __half *b = row + (Q - 1 - i) * bs;
-                    if (cxo(i) == 0) {
-                        st_pair(b, xa, fa[i], fb[i]);
-                    } else if (cxo(i) == 1) {
-                        b[xb] = __float2half_rn(fa[i]);
-                        b[pp] = __float2half_rn(fb[i]);
+                    T *b = row + (Q - 1 - i) * bs;
+                    float va, vb;
+                    unpack2(f[i], va, vb);
+                    if (mode == 1) {
+                        if (cxo(i) == 0) {
+                            b[xa] = St::store(va);
+                            b[xb] = St::store(vb);
+                        } else {
+                            st_pair(b, cxo(i) == 1 ? xb : pm, f[i]);
+                        }
                     } else {
-                        b[pm] = __float2half_rn(fa[i]);
-                        b[xa] = __float2half_rn(fb[i]);
+                        if (cxo(i) == 0) {
+                            st_pair(b, xa, f[i]);
+                        } else if (cxo(i) == 1) {
+                            b[xb] = St::store(va);
+                            b[pp] = St::store(vb);
+                        } else {
+                            b[pm] = St::store(va);
+                            b[xa] = St::store(vb);
+                        }
                     }
                 }
             }
             if (a.diag) {
-                loc.add(ma.rho, ma.u, rho0);
-                loc.add(mb.rho, mb.u, rho0);
+                float ra, rb, ua[3], ub[3];
+                unpack2(m.rho, ra, rb);
+    #pragma unroll
+                for (int q = 0; q < 3; ++q) unpack2(m.u[q], ua[q], ub[q]);
+                loc.add(ra, ua, a.rho0f);
+                loc.add(rb, ub, a.rho0f);
             }
         }
         xh += nthr;
@@ -412,120 +500,188 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
     if (a.diag) loc.flush(acc, a.rho0);
 }
 
+// The warps after the consumers: the loader and the storer.
+constexpr int kTmaServiceThreads = 64;
+
 template <int D, int P, int EQ, bool BULK, int CAPB>
-__global__ void __launch_bounds__(tma_max_threads(D, P) + 32) k_step_tma(const lbmh::StepArgs a, const TmaGeom g) {
+__global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_step_tma(const lbmh::StepArgs a, const TmaGeom g) {
     using T = typename Storage<P>::T;
     constexpr int Q = qof(D);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[kTmaMaxStages];
     __shared__ __align__(8) uint64_t empty[kTmaMaxStages];
+    __shared__ __align__(8) uint64_t freed[kTmaMaxStages];
+    __shared__ JobPos jobq[kTmaMaxStages];  // the job in each stage; nrows == 0 ends the block's work
+    __shared__ int unitq[kTmaMaxStages];    // its unit
     T *sm = reinterpret_cast<T *>(smem_raw);
     const int64_t stage_elems = (int64_t)Q * (CAPB / (int)sizeof(T));
     const int S = g.stages;
-    const int64_t G = gridDim.x;
-    const int ncons = (int)blockDim.x - 32;  // consumer threads; the last warp produces
+    const int ncons = (int)blockDim.x - kTmaServiceThreads;
     const int lane = threadIdx.x & 31;
-    const bool producer = (int)threadIdx.x >= ncons;
+    const int role = (int)threadIdx.x < ncons ? 0 : ((int)threadIdx.x < ncons + 32 ? 1 : 2);
+    const bool chain = g.nsteps > 1;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], ncons / 32);
+            mbar_init(&freed[s], 1);
         }
         fence_barrier_init();
     }
     __syncthreads();
     DiagAcc acc;
     bool failed = false;
-    if (producer) {
-        int64_t k = 0;
-        for (;; ++k) {
-            const int64_t job = blockIdx.x + k * G;
-            if (job >= g.njobs) break;
-            const int s = (int)(k % S);
-            const JobPos jp = decode_job(a, g, job);
-            if (k >= S) {
-                // stage s still holds job k - S: wait for its collision, store it back
-                const int64_t q = k - S;
-                const bool ok = mbar_wait_bounded(&empty[s], (uint32_t)((q / S) & 1), a.timeout_ns);
+    if (role == 1) {
+        // loader: takes the jobs, waits for the steps they need, refills the stages
+        const unsigned total = chain ? (unsigned)chain_tickets(g) : (unsigned)g.njobs;
+        unsigned next = blockIdx.x;
+        if (chain && lane == 0) next = atomicAdd(&a.sync[0], 1u);
+        int s = 0;
+        uint32_t phase = 0;
+        bool wrapped = false;
+        for (;;) {
+            JobPos jp{0, 0, 0, 0, 0, 0};
+            unsigned job = chain ? __shfl_sync(0xffffffffu, next, 0) : next;
+            bool end = job >= total;
+            int step = 0, up = 0, uc = 0;
+            if (!end) {
+                if (chain) {
+                    const ChainJob c = decode_chain(a, g, job);
+                    if (lane == 0) next = atomicAdd(&a.sync[0], 1u);  // in flight while this job is set up
+                    if (c.step < 0) continue;
+                    jp = c.j;
+                    step = c.step;
+                    up = c.p;
+                    uc = c.c;
+                } else {
+                    next = job + gridDim.x;
+                    jp = decode_job(a, g, job);
+                }
+            }
+            if (wrapped) {  // the stage's last job has been stored
+                const bool ok = mbar_wait_bounded(&freed[s], phase ^ 1u, a.timeout_ns);
                 if (__any_sync(0xffffffffu, !ok)) {
                     failed = true;
                     break;
                 }
-                const JobPos jq = decode_job(a, g, blockIdx.x + q * G);
-                if (a.odd && g.nseg > 1) {
-                    tma_plain_stores<D, T>(a, g, jq, sm + s * stage_elems, lane, 32);
-                    __syncwarp();  // every lane's plain stores read the stage before any refill
+            }
+            if (!end && step > 0) {
+                bool ok = true;
+                if (lane < (D == 3 ? 9 : 3)) {
+                    const int p = wrapi(up + lane % 3 - 1, g.npos);
+                    const int c = D == 3 ? wrapi(uc + lane / 3 - 1, g.ncross) : 0;
+                    ok = wait_count_bounded(&a.sync[lbmh::kSyncDone + p * g.ncross + c], (unsigned)(step * g.nseg),
+                                            a.status, a.timeout_ns);
                 }
-                if (lane == 0) mbar_arrive_expect_tx(&full[s], tma_job_bytes<D, T>(a, g, jp));
-                if (lane < Q) {
-                    // each lane stores its direction's buffer, waits until that store has
-                    // read shared memory, and refills the same buffer; lanes do not wait
-                    // for one another (the stage's phase completes once all bytes land)
-                    tma_issue_stores<D, T>(a, g, jq, lane, sm + s * stage_elems);
-                    bulk_commit();
-                    bulk_wait_read<0>();
-                    tma_issue_loads<D, T>(a, g, jp, lane, sm + s * stage_elems, &full[s]);
+                if (__any_sync(0xffffffffu, !ok)) {
+                    failed = true;
+                    end = true;
                 }
-            } else {
-                if (lane == 0) mbar_arrive_expect_tx(&full[s], tma_job_bytes<D, T>(a, g, jp));
-                if (lane < Q) tma_issue_loads<D, T>(a, g, jp, lane, sm + s * stage_elems, &full[s]);
+                // what other SMs' copy engines and threads wrote, before this SM's copy engine reads
+                fence_proxy_async();
+            }
+            if (lane == 0) {
+                if (end) jp.nrows = 0;
+                jobq[s] = jp;
+                unitq[s] = up * g.ncross + uc;
+                mbar_arrive_expect_tx(&full[s], end ? 0u : tma_job_bytes<D, T>(a, g, jp));
+            }
+            if (end) break;
+            if (lane < Q) tma_issue_loads<D, T>(a, g, jp, lane, sm + s * stage_elems, &full[s]);
+            if (++s == S) {
+                s = 0;
+                phase ^= 1u;
+                wrapped = true;
             }
         }
-        const int64_t issued = k;
-        if (!failed) {
-            // store back the last stages
-            for (int64_t q = (issued > S ? issued - S : 0); q < issued; ++q) {
-                const int s = (int)(q % S);
-                const bool ok = mbar_wait_bounded(&empty[s], (uint32_t)((q / S) & 1), a.timeout_ns);
-                if (__any_sync(0xffffffffu, !ok)) {
-                    failed = true;
-                    break;
-                }
-                const JobPos jq = decode_job(a, g, blockIdx.x + q * G);
-                if (a.odd && g.nseg > 1) tma_plain_stores<D, T>(a, g, jq, sm + s * stage_elems, lane, 32);
-                if (lane < Q) {
-                    tma_issue_stores<D, T>(a, g, jq, lane, sm + s * stage_elems);
-                    bulk_commit();
-                }
+    } else if (role == 2) {
+        // storer: writes collided stages back, frees them, and reports finished jobs
+        int s = 0;
+        uint32_t phase = 0;
+        for (;;) {
+            const bool ok = mbar_wait_bounded(&empty[s], phase, a.timeout_ns);
+            if (__any_sync(0xffffffffu, !ok)) {
+                failed = true;
+                break;
+            }
+            const JobPos jq = jobq[s];
+            const int unit = unitq[s];
+            if (jq.nrows == 0) break;
+            T *st = sm + s * stage_elems;
+            if (jq.odd && g.nseg > 1) tma_plain_stores<D, T>(a, g, jq, st, lane, 32);
+            if (lane < Q) tma_issue_stores<D, T>(a, g, jq, lane, st);
+            bulk_commit();
+            bulk_wait_read<0>();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cta(&freed[s]);
+            if (chain) {
+                bulk_wait_all();
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) red_release(&a.sync[lbmh::kSyncDone + unit], 1u);
+            }
+            if (++s == S) {
+                s = 0;
+                phase ^= 1u;
             }
         }
         bulk_wait_all();
         if (failed) {
             // let loads still in flight land before the block's shared memory is released
-            for (int64_t q = (issued > S ? issued - S : 0); q < issued; ++q)
-                (void)mbar_wait_bounded(&full[q % S], (uint32_t)((q / S) & 1), a.timeout_ns);
+            for (int q = 0; q < S; ++q) (void)mbar_wait_bounded(&full[(s + q) % S], s + q >= S ? phase ^ 1u : phase, a.timeout_ns);
         }
     } else {
-        for (int64_t k = 0;; ++k) {
-            const int64_t job = blockIdx.x + k * G;
-            if (job >= g.njobs) break;
-            const int s = (int)(k % S);
-            const bool ok = mbar_wait_bounded(&full[s], (uint32_t)((k / S) & 1), a.timeout_ns);
+        int s = 0;
+        uint32_t phase = 0;
+        for (;;) {
+            const bool ok = mbar_wait_bounded(&full[s], phase, a.timeout_ns);
             if (__any_sync(0xffffffffu, !ok)) {
                 failed = true;
                 break;
             }
-            T *st = sm + s * stage_elems;
-            const JobPos jp = decode_job(a, g, job);
-            if constexpr (P == P_F16S && D == 3) {
-                // the D3Q27 pair body is long: one copy serves the three pairings (three
-                // specialised copies measured slower)
-                tma_compute_pairs<D, EQ, BULK, CAPB, -1>(a, g, jp, st, acc, threadIdx.x, ncons);
-            } else if constexpr (P == P_F16S) {
-                if (!a.odd)
-                    tma_compute_pairs<D, EQ, BULK, CAPB, 0>(a, g, jp, st, acc, threadIdx.x, ncons);
-                else if (g.nseg == 1)
-                    tma_compute_pairs<D, EQ, BULK, CAPB, 1>(a, g, jp, st, acc, threadIdx.x, ncons);
-                else
-                    tma_compute_pairs<D, EQ, BULK, CAPB, 2>(a, g, jp, st, acc, threadIdx.x, ncons);
-            } else
-                tma_compute<D, P, EQ, BULK, CAPB>(a, g, jp, st, acc, threadIdx.x, ncons);
-            fence_proxy_async_smem();
-            __syncwarp();
+            const JobPos jp = jobq[s];
+            if (jp.nrows > 0) {
+                T *st = sm + s * stage_elems;
+                if (P == P_F64 || (jp.len & 1)) {
+                    tma_compute<D, P, EQ, BULK, CAPB>(a, g, jp, st, acc, threadIdx.x, ncons);
+                } else if constexpr (P != P_F64 && D == 3) {
+                    // the D3Q27 pair body is long: one copy serves the three pairings (three
+                    // specialised copies measured slower)
+                    tma_compute_pairs<D, P, EQ, BULK, CAPB, -1>(a, g, jp, st, acc, threadIdx.x, ncons);
+                } else if constexpr (P != P_F64) {
+                    if (!jp.odd)
+                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 0>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else if (g.nseg == 1)
+                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 1>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else
+                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 2>(a, g, jp, st, acc, threadIdx.x, ncons);
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+            }
             if (lane == 0) mbar_arrive_cta(&empty[s]);
+            if (jp.nrows == 0) break;
+            if (++s == S) {
+                s = 0;
+                phase ^= 1u;
+            }
         }
     }
     if (failed && lane == 0) report_status(a.status, -5); /* LBM_ETIMEOUT */
+    if (chain) {
+        // the last block to finish clears the counters for the next launch
+        __syncthreads();
+        bool last = false;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            last = atomicAdd(&a.sync[1], 1u) == gridDim.x - 1;
+        }
+        if (__syncthreads_or(last)) {
+            uint4 *w = reinterpret_cast<uint4 *>(a.sync);
+            for (int p = threadIdx.x; p < (lbmh::kSyncDone + g.npos * g.ncross + 3) / 4; p += blockDim.x)
+                w[p] = make_uint4(0, 0, 0, 0);
+        }
+    }
     if (a.diag) diag_block_store(acc, a.partials + (int64_t)blockIdx.x * lbmh::kDiagWords);
 }
 

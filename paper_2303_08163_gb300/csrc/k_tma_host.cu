@@ -1,4 +1,7 @@
 // k_tma_host.cu -- geometry and launch of the TMA row-staged step kernel.
+#include <algorithm>
+
+
 #include "k_tma.cuh"
 
 namespace lbmh {
@@ -37,7 +40,20 @@ static int esize(int P) { return P == lbmd::P_F64 ? 8 : (P == lbmd::P_F32 ? 4 : 
 
 bool tma_supported(const Lattice &lat) {
     const int es = esize(lat.P);
-    return ((int64_t)lat.nx * es) % 16 == 0 && (lat.plane * es) % 16 == 0 && lat.nx >= 16 / es;
+    if (((int64_t)lat.pitch * es) % 16 != 0 || (lat.plane * es) % 16 != 0 || lat.nx < 16 / es) return false;
+    // padded rows are copied whole (a segment's halo would start off a 16-byte boundary)
+    return lat.pitch == lat.nx || lat.pitch * es <= (lat.D == 3 ? 4096 : 8192);
+}
+
+// Rows of a ragged lattice (nx * sizeof % 16 != 0) are padded to whole 16-byte units when
+// the TMA kernel can then copy them whole and the padding stays under an eighth of the row
+// (rows of at least 128 bytes).  FP64 storage is bound by the FP64 pipe, not by how its rows
+// are fetched, and keeps its rows unpadded.
+int padded_pitch(int D, int P, int64_t nx) {
+    const int es = esize(P);
+    const int64_t rowb = nx * es, up = (rowb + 15) / 16 * 16;
+    if (rowb % 16 == 0 || P == lbmd::P_F64 || rowb < 128 || up > (D == 3 ? 4096 : 8192)) return (int)nx;
+    return (int)(up / es);
 }
 
 static lbmd::TmaGeom geom(const Lattice &lat, const TmaShape &t) {
@@ -49,10 +65,70 @@ static lbmd::TmaGeom geom(const Lattice &lat, const TmaShape &t) {
     g.rows = g.nseg > 1 ? 1 : (t.rows < 1 ? 1 : (t.rows > lat.ny ? lat.ny : t.rows));
     g.ygroups = (lat.ny + g.rows - 1) / g.rows;
     g.halo = g.nseg > 1 ? U : 0;
-    g.rowstride = g.seg + 2 * g.halo;
+    g.rowstride = g.nseg > 1 ? g.seg + 2 * g.halo : lat.pitch;
     g.bufstride = t.cap / esize(lat.P);
     g.njobs = (int64_t)lat.nz * g.ygroups * g.nseg;
+    g.nsteps = 1;
+    g.npos = g.ncross = g.strips = g.stripw = g.pjobs = g.depth = g.lag = 0;
     return g;
+}
+
+// The sweep of a several-step launch (see decode_chain).  Returns false when the lattice has
+// more units than counters.
+//
+// Depth: a state that stays in L2 between steps is swept one step after the other.  A larger
+// one is swept `depth` steps at a time, cut into strips where needed, so that what lies between
+// the first and the last of them fits in L2: the jobs in flight (every stage of every block and
+// one ticket more) spread over depth x pjobs jobs a phase, and two positions for the neighbours.
+static bool chain_geom(const Lattice &lat, const TmaShape &t, int nsteps, lbmd::TmaGeom &g) {
+    constexpr int64_t kResident = (int64_t)90 << 20;  // state that stays in the 129 MB L2
+    constexpr int64_t kWindow = (int64_t)60 << 20;    // and the travelling window of a larger one
+    g.nsteps = nsteps;
+    g.npos = lat.D == 3 ? lat.nz : g.ygroups;
+    g.ncross = lat.D == 3 ? g.ygroups : 1;
+    if ((int64_t)g.npos * g.ncross > sync_units(lat)) return false;
+    g.strips = 1;
+    g.stripw = g.ncross;
+    g.pjobs = g.ncross * g.nseg;
+    g.depth = 1;
+    g.lag = 0;
+    const int64_t state = (int64_t)lbmd::qof(lat.D) * lat.plane * esize(lat.P);
+    if (state <= kResident || lat.P == lbmd::P_F64) return true;
+    const int64_t unit = state / ((int64_t)g.npos * g.ncross);
+    const int64_t inflight = (int64_t)t.blocks * (t.stages + 1);
+    for (int d = 3; d >= 2; --d)
+        for (int k = 1; k <= 64; ++k) {
+            const int h = (g.ncross + k - 1) / k, last = g.ncross - (k - 1) * h;
+            if (k > 1 && (last < 1 || h < 8 * (d - 1))) break;
+            const int wide = k == 1 ? h : std::max(h, last + 2 * (d - 1));
+            const int64_t pj = (int64_t)wide * g.nseg;
+            const int64_t lag = 2 + (inflight + d * pj - 1) / (d * pj);
+            if ((lag * (d - 1) + 3) * wide * unit > kWindow) continue;
+            if (lag * (d - 1) + 2 >= g.npos) continue;
+            g.depth = d;
+            g.strips = k;
+            g.stripw = h;
+            g.pjobs = (int)pj;
+            g.lag = (int)lag;
+            return true;
+        }
+    return true;
+}
+
+int64_t sync_units(const Lattice &lat) { return std::min<int64_t>((int64_t)lat.ny * lat.nz, (int64_t)1 << 22); }
+
+int64_t tma_max_steps(const Lattice &lat, const TmaShape &t) {
+    lbmd::TmaGeom g = geom(lat, t);
+    if (!chain_geom(lat, t, 2, g)) return 1;
+    // tickets stay below 2^30, and a launch to some tens of milliseconds
+    const int64_t work = lat.P == lbmd::P_F64 ? (int64_t)1 << 27 : (int64_t)1 << 31;
+    int64_t n = std::max<int64_t>(work / lat.ncell / g.depth, 1) * g.depth;
+    while (n > 1) {
+        g.nsteps = (int)std::min<int64_t>(n, 1 << 28);
+        if (chain_tickets(g) < (int64_t)1 << 30) break;
+        n /= 2;
+    }
+    return n;
 }
 
 // Dynamic shared memory of a shape, or -1 when the shape is invalid: the segment must be
@@ -64,7 +140,7 @@ int tma_smem_bytes(const Lattice &lat, const TmaShape &t) {
     const int U = 16 / esize(lat.P);
     if (t.stages < 2 || t.stages > kTmaMaxStages) return -1;
     if (t.cap != 1024 && t.cap != 2048 && t.cap != 4096 && t.cap != 8192) return -1;
-    if (t.seg < lat.nx && (t.seg % U) != 0) return -1;
+    if (t.seg < lat.nx && ((t.seg % U) != 0 || lat.pitch != lat.nx)) return -1;
     const lbmd::TmaGeom g = geom(lat, t);
     if ((int64_t)g.rows * g.rowstride > g.bufstride) return -1;
     if (g.njobs >= ((int64_t)1 << 31)) return -1;
@@ -87,21 +163,27 @@ int tma_max_blocks_per_sm(const Lattice &lat, int eq, int bulk, const TmaShape &
         cudaGetLastError();
         return 0;
     }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, t.threads + 32, t.smem_bytes) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, t.threads + lbmd::kTmaServiceThreads, t.smem_bytes) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return n;
 }
 
-cudaError_t step_tma(const StepArgs &a, const TmaShape &t, cudaStream_t s) {
+cudaError_t step_tma(const StepArgs &a, const TmaShape &t, int nsteps, cudaStream_t s) {
     const void *fn = tma_kernel(a.lat, a.eq, a.bulk, t.cap);
     if (!fn) return cudaErrorInvalidValue;
     lbmd::TmaGeom g = geom(a.lat, t);
     StepArgs aa = a;
     void *args[] = {(void *)&aa, (void *)&g};
-    // t.threads consumer threads plus the producer warp
-    return cudaLaunchKernel(fn, dim3(t.blocks), dim3(t.threads + 32), args, (size_t)t.smem_bytes, s);
+    int blocks = t.blocks;
+    if (nsteps > 1) {
+        if (!chain_geom(a.lat, t, nsteps, g)) return cudaErrorInvalidValue;
+        // more blocks than jobs of one step would only wait for one another
+        blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, g.njobs));
+    }
+    // t.threads consumer threads plus the loader and the storer warp
+    return cudaLaunchKernel(fn, dim3(blocks), dim3(t.threads + lbmd::kTmaServiceThreads), args, (size_t)t.smem_bytes, s);
 }
 
 }  // namespace lbmh

@@ -36,13 +36,29 @@ template <> __device__ __forceinline__ float step_scalar<float>(double, float f)
 // values in the opposite slot of the sending cell).
 template <int D>
 __device__ __forceinline__ int64_t aa_index(int i, int x, int y, int z, int nx, int ny, int nz,
-                                            int64_t plane, int odd) {
+                                            int pitch, int64_t plane, int odd) {
     constexpr int Q = qof(D);
-    if (!odd) return (int64_t)i * plane + x + (int64_t)nx * (y + (int64_t)ny * z);
+    if (!odd) return (int64_t)i * plane + x + (int64_t)pitch * (y + (int64_t)ny * z);
     const int xs = wrapi(x - cxo(i), nx);
     const int ys = wrapi(y - cyo(i), ny);
     const int zs = (D == 3) ? wrapi(z - czo(i), nz) : z;
-    return (int64_t)(Q - 1 - i) * plane + xs + (int64_t)nx * (ys + (int64_t)ny * zs);
+    return (int64_t)(Q - 1 - i) * plane + xs + (int64_t)pitch * (ys + (int64_t)ny * zs);
+}
+
+// Coordinates of cell c = x + nx (y + ny z), with 32-bit divisions where the index allows
+// (a 64-bit division is a long instruction sequence).
+__device__ __forceinline__ void cell_coords(int64_t c, int64_t ncell, int nx, int ny, int &x, int &y, int &z) {
+    if (ncell < ((int64_t)1 << 31)) {
+        const unsigned u = (unsigned)c, r = u / (unsigned)nx, q = r / (unsigned)ny;
+        x = (int)(u - r * (unsigned)nx);
+        y = (int)(r - q * (unsigned)ny);
+        z = (int)q;
+    } else {
+        const int64_t r = c / nx, q = r / ny;
+        x = (int)(c - r * nx);
+        y = (int)(r - q * ny);
+        z = (int)q;
+    }
 }
 
 struct DiagAcc {

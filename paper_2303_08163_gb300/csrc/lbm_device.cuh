@@ -281,20 +281,10 @@ __host__ __device__ __forceinline__ CellMoments<R> moments_shifted(const R (&f)[
     return m;
 }
 
-// The relaxation f* = (1 - 2beta) f + 2beta w_i (drho + rho h_i) of one direction of
-// weight class c, in one of two forms.  TWO_FMA: two FMAs per direction, with the
-// per-class products 2beta w rho and 2beta w drho formed once per cell (fewest
-// instructions: used where instruction issue is the bound, FP64 and D2Q9 with binary16
-// storage).  Otherwise the factored form 2beta w (rho h + drho) + (1 - 2beta) f, which
-// measured faster for the bandwidth-bound FP32 and D3Q27 binary16 steps (fewer live
-// registers).  Both kernels of a lattice use the same form, so their states agree bit for
-// bit.
-template <int D, int P>
-__host__ __device__ constexpr bool relax_two_fma() {
-    return P == P_F64 || (D == 2 && P == P_F16S);
-}
-
-template <typename R, bool TWO_FMA = (sizeof(R) == 8)> struct Relax {
+// The FP64 relaxation f* = (1 - 2beta) f + 2beta w_i (drho + rho h_i) of one direction of
+// weight class c: two FMAs per direction, with the per-class products 2beta w rho and
+// 2beta w drho formed once per cell (fewest instructions on the FP64 pipe, the bound).
+template <typename R> struct Relax {
     R keep, rho, drho, omw[4], wr[4], wd[4];
     __host__ __device__ __forceinline__ Relax(R om, double w0, double w1, double w2, double w3, R rho_,
                                               R drho_)
@@ -308,8 +298,7 @@ template <typename R, bool TWO_FMA = (sizeof(R) == 8)> struct Relax {
         }
     }
     __host__ __device__ __forceinline__ R operator()(int c, R h, R f) const {
-        if constexpr (TWO_FMA) return fma_r(wr[c], h, fma_r(keep, f, wd[c]));
-        else return fma_r(omw[c], fma_r(rho, h, drho), keep * f);
+        return fma_r(wr[c], h, fma_r(keep, f, wd[c]));
     }
 };
 
@@ -357,17 +346,263 @@ __host__ __device__ __forceinline__ void entropic_factors_one_division(
     }
 }
 
-// The fused collision of one cell, in place on shifted populations.  Returns the
+// ------------------------------------------------------------------ FP32 collisions
+//
+// The FP32 collision is written over a value type V: float (one cell) or f32x2 (two cells,
+// one in each half of a 64-bit register pair, advanced by the packed fma / mul / add.f32x2
+// instructions of sm_100 and later).  Both forms issue the same correctly rounded operations
+// in the same order, so the one-cell and the two-cell kernels store the same bits.  (The
+// scalar _rn intrinsics are never contracted; a packed product that only feeds packed sums
+// was seen to be, so such sums are written as fma.)
+struct f32x2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 a, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ f32x2 vadd(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 vmul(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 vfma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ f32x2 vsub(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+template <typename V> __device__ __forceinline__ V vset(float c);
+template <> __device__ __forceinline__ float vset<float>(float c) { return c; }
+template <> __device__ __forceinline__ f32x2 vset<f32x2>(float c) { return pack2(c, c); }
+
+// A product that keeps its own rounding when it feeds a sum (adding -0 changes nothing, and
+// an fma is never contracted further).
+template <typename V> __device__ __forceinline__ V vmul_alone(V a, V b) { return vfma(a, b, vset<V>(-0.0f)); }
+
+// Hardware reciprocal and reciprocal square root (a few ulp, far below the storage rounding
+// of the FP32 and binary16 formats).
+__device__ __forceinline__ float vrcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float vrsqrt(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ f32x2 vrcp(f32x2 a) {
+    float x, y;
+    unpack2(a, x, y);
+    return pack2(vrcp(x), vrcp(y));
+}
+__device__ __forceinline__ f32x2 vrsqrt(f32x2 a) {
+    float x, y;
+    unpack2(a, x, y);
+    return pack2(vrsqrt(x), vrsqrt(y));
+}
+__device__ __forceinline__ f32x2 vmax(f32x2 a, f32x2 b) {
+    float x, y, z, w;
+    unpack2(a, x, y);
+    unpack2(b, z, w);
+    return pack2(fmaxf(x, z), fmaxf(y, w));
+}
+
+template <typename V> struct Moments32 {
+    V rho, u[3];
+};
+
+// 2 beta of the FP32 collision from the largest per-axis key (see collision_rate).
+template <int EQ, bool BULK, typename V>
+__device__ __forceinline__ V rate32(V key_max, V omega0, V six_nu) {
+    if constexpr (!BULK) {
+        return omega0;
+    } else if constexpr (EQ == EQ_ENT) {
+        const V A2 = vsub(vset<V>(2.0f), key_max);
+        return vmul(vadd(A2, A2), vrcp(vfma(six_nu, vmul(key_max, key_max), A2)));
+    } else {
+        const V A = vfma(vset<V>(-4.5f), key_max, vset<V>(1.0f));
+        return vmul(vadd(A, A), vrcp(vadd(six_nu, A)));
+    }
+}
+
+// The relaxation f* = (1 - 2beta) f + 2beta w_i (drho + rho h_i) of one direction of weight
+// class c, in one of two forms: factored, 2beta w (rho h + drho) + (1 - 2beta) f, or for D2Q9
+// binary16 two FMAs with the per-class products 2beta w rho and 2beta w drho formed once.
+// (The results of the two differ in the last bit; each storage keeps its own.)
+template <int D, int P, typename V> struct Relax32 {
+    static constexpr bool kTwoFma = D == 2 && P == P_F16S;
+    V keep, rho, drho, omw[4], wr[4], wd[4];
+    __device__ __forceinline__ Relax32(V om, V rho_, V drho_) : keep(vsub(vset<V>(1.0f), om)), rho(rho_), drho(drho_) {
+#pragma unroll
+        for (int c = 0; c <= D; ++c) {
+            omw[c] = vmul(om, vset<V>((float)wclass_weight<D>(c)));
+            if constexpr (kTwoFma) {
+                wr[c] = vmul(omw[c], rho);
+                wd[c] = vmul(omw[c], drho);
+            }
+        }
+    }
+    __device__ __forceinline__ V operator()(int c, V h, V f) const {
+        if constexpr (kTwoFma) return vfma(wr[c], h, vfma(keep, f, wd[c]));
+        else return vfma(omw[c], vfma(rho, h, drho), vmul(keep, f));
+    }
+};
+
+// The fused FP32 collision, in place on shifted populations; returns the pre-collision
+// moments.
+template <int D, int P, int EQ, bool BULK, typename V>
+__device__ __forceinline__ Moments32<V> collide32(V (&f)[qof(D)], float rho0s, float omega0s, float six_nus) {
+    constexpr int Q = qof(D);
+    const V rho0 = vset<V>(rho0s), one = vset<V>(1.0f);
+    Moments32<V> m;
+    V j[3];
+    {
+        V a[9];
+        if constexpr (D == 2) {
+#pragma unroll
+            for (int p = 0; p < 9; ++p) a[p] = f[p];
+        } else {
+            V bz[9];
+#pragma unroll
+            for (int p = 0; p < 9; ++p) {
+                a[p] = vadd(vadd(f[p], f[p + 9]), f[p + 18]);
+                bz[p] = vsub(f[p + 18], f[p]);
+            }
+            j[2] = vadd(vadd(vadd(vadd(bz[0], bz[1]), vadd(bz[2], bz[3])), vadd(vadd(bz[4], bz[5]), vadd(bz[6], bz[7]))), bz[8]);
+        }
+        const V c0 = vadd(vadd(a[0], a[3]), a[6]);  // c_x = -1
+        const V c1 = vadd(vadd(a[1], a[4]), a[7]);  // c_x = 0
+        const V c2 = vadd(vadd(a[2], a[5]), a[8]);  // c_x = +1
+        m.rho = vadd(rho0, vadd(vadd(c0, c1), c2));
+        j[0] = vsub(c2, c0);
+        j[1] = vsub(vadd(vadd(a[6], a[7]), a[8]), vadd(vadd(a[0], a[1]), a[2]));
+    }
+    const V inv = vrcp(m.rho);
+    m.u[2] = vset<V>(0.0f);
+#pragma unroll
+    for (int a = 0; a < D; ++a) m.u[a] = vmul(j[a], inv);
+    const V drho = vsub(m.rho, rho0);
+    if constexpr (EQ == EQ_POLY2) {
+        V uu, k;
+        if constexpr (BULK) {
+            const V xx = vmul_alone(m.u[0], m.u[0]), yy = vmul_alone(m.u[1], m.u[1]);
+            uu = vadd(xx, yy);
+            k = vmax(xx, yy);
+            if constexpr (D == 3) k = vmax(k, vmul(m.u[2], m.u[2]));
+        } else {
+            uu = k = vfma(m.u[0], m.u[0], vmul(m.u[1], m.u[1]));
+        }
+        if constexpr (D == 3) uu = vfma(m.u[2], m.u[2], uu);
+        const Relax32<D, P, V> relax(rate32<EQ, BULK, V>(k, vset<V>(omega0s), vset<V>(six_nus)), m.rho, drho);
+        const V mh = vmul(vset<V>(-1.5f), uu);
+        const V upm = vadd(m.u[0], m.u[1]), umm = vsub(m.u[0], m.u[1]);
+        const V four5 = vset<V>(4.5f), three = vset<V>(3.0f), m1 = vset<V>(-1.0f);
+        f[Q / 2] = relax(0, mh, f[Q / 2]);
+#pragma unroll
+        for (int i = Q / 2 + 1; i < Q; ++i) {  // direction i and its opposite Q - 1 - i
+            const int cx = cxo(i), cy = cyo(i), cz = (D == 3) ? czo(i) : 0;
+            // c.u of i: the planar part (with its sign), then u_z
+            V cu;
+            bool neg = false;
+            if (cx == 0 && cy == 0) cu = m.u[2];
+            else if (cx == 0) { cu = m.u[1]; neg = cy < 0; }
+            else if (cy == 0) { cu = m.u[0]; neg = cx < 0; }
+            else if (cx == cy) { cu = upm; neg = cx < 0; }
+            else { cu = umm; neg = cx < 0; }
+            if (cz != 0 && (cx != 0 || cy != 0)) cu = neg ? vsub(m.u[2], cu) : vadd(cu, m.u[2]);
+            else if (neg) cu = vmul(cu, m1);
+            const V ncu = vmul(cu, m1);
+            const int c = wclass<D>(i);
+            f[i] = relax(c, vfma(cu, vfma(four5, cu, three), mh), f[i]);
+            f[Q - 1 - i] = relax(c, vfma(ncu, vfma(four5, ncu, three), mh), f[Q - 1 - i]);
+        }
+    } else {
+        V dm[3], d0[3], dp[3], key[3];  // d(-1), d(0), d(+1)
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const V u2 = vmul(m.u[a], m.u[a]), t3 = vmul(vset<V>(3.0f), u2);
+            if constexpr (EQ == EQ_ENT) {
+                const V s2 = vfma(vset<V>(3.0f), u2, one);
+                const V rs = vrsqrt(s2);  // S = s2 rs
+                key[a] = vmul(s2, rs);
+                const V sm1 = vmul(t3, vrcp(BULK ? vadd(one, key[a]) : vfma(s2, rs, one)));  // S - 1 without cancellation
+                d0[a] = vmul(sm1, vset<V>(-1.0f));
+                dp[a] = vfma(vset<V>(2.0f), sm1, vmul(vset<V>(3.0f), m.u[a]));
+                dm[a] = vfma(vset<V>(2.0f), sm1, vmul(vset<V>(-3.0f), m.u[a]));
+            } else {
+                d0[a] = vmul_alone(vset<V>(-1.5f), u2);
+                dp[a] = vfma(vset<V>(3.0f), m.u[a], t3);
+                dm[a] = vfma(vset<V>(-3.0f), m.u[a], t3);
+                key[a] = u2;
+            }
+        }
+        V kmax = key[0];
+        if constexpr (BULK) {
+            kmax = vmax(key[0], key[1]);
+            if constexpr (D == 3) kmax = vmax(kmax, key[2]);
+        }
+        const Relax32<D, P, V> relax(rate32<EQ, BULK, V>(kmax, vset<V>(omega0s), vset<V>(six_nus)), m.rho, drho);
+        const V dx[3] = {dm[0], d0[0], dp[0]}, dy[3] = {dm[1], d0[1], dp[1]};
+        const V tx[3] = {vadd(one, dm[0]), vadd(one, d0[0]), vadd(one, dp[0])};
+        if constexpr (D == 2) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                f[i] = relax(wclass<D>(i), vfma(dy[cyo(i) + 1], tx[cxo(i) + 1], dx[cxo(i) + 1]), f[i]);
+        } else {
+            const V ty[3] = {vadd(one, dm[1]), vadd(one, d0[1]), vadd(one, dp[1])};
+            const V dz[3] = {dm[2], d0[2], dp[2]};
+#pragma unroll
+            for (int p = 0; p < 9; ++p) {
+                const V exy = vfma(dy[cyo(p) + 1], tx[cxo(p) + 1], dx[cxo(p) + 1]);
+                const V txy = vmul(tx[cxo(p) + 1], ty[cyo(p) + 1]);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int i = p + 9 * q;
+                    f[i] = relax(wclass<D>(i), vfma(dz[q], txy, exy), f[i]);
+                }
+            }
+        }
+    }
+    return m;
+}
+
+// The fused FP64 collision of one cell, in place on shifted populations.  Returns the
 // pre-collision moments (the macroscopic state at the current time step).  The
 // equilibrium term h_i of each direction is formed inside the relaxation loop from the
 // per-axis factors, so only the Q populations and O(D^2) factors stay live.
-template <int D, int EQ, bool BULK, typename R, bool TWO_FMA = (sizeof(R) == 8)>
-__host__ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omega0, R six_nu) {
+template <int D, int P, int EQ, bool BULK, typename R>
+__device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omega0, R six_nu) {
     constexpr int Q = qof(D);
     // weights per number of nonzero velocity components, folded at compile time
     constexpr double kW0 = wclass_weight<D>(0), kW1 = wclass_weight<D>(1);
     constexpr double kW2 = wclass_weight<D>(2), kW3 = wclass_weight<D>(D >= 3 ? 3 : 0);
     CellMoments<R> m;
+    if constexpr (sizeof(R) == 4) {
+        const Moments32<float> v = collide32<D, P, EQ, BULK, float>(f, rho0, omega0, six_nu);
+        m.rho = v.rho;
+        for (int a = 0; a < 3; ++a) m.u[a] = v.u[a];
+        return m;
+    } else {
     R dm[3], d0[3], dp[3], key[3];  // per-axis factors (entropic and product forms)
     if constexpr (EQ == EQ_ENT && sizeof(R) == 8) {
         entropic_factors_one_division<D, R>(f, rho0, m, dm, d0, dp, key);
@@ -383,7 +618,7 @@ __host__ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho
         if constexpr (D == 3) k = fmax(k, m.u[2] * m.u[2]);
         const R om = collision_rate<EQ, BULK, R>(k, omega0, six_nu);
         const R mh = R(-1.5) * uu;
-        const Relax<R, TWO_FMA> relax(om, kW0, kW1, kW2, kW3, m.rho, drho);
+        const Relax<R> relax(om, kW0, kW1, kW2, kW3, m.rho, drho);
         const R upm = m.u[0] + m.u[1], umm = m.u[0] - m.u[1];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
@@ -403,7 +638,7 @@ __host__ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho
         R kmax = fmax(key[0], key[1]);
         if constexpr (D == 3) kmax = fmax(kmax, key[2]);
         const R om = collision_rate<EQ, BULK, R>(kmax, omega0, six_nu);
-        const Relax<R, TWO_FMA> relax(om, kW0, kW1, kW2, kW3, m.rho, drho);
+        const Relax<R> relax(om, kW0, kW1, kW2, kW3, m.rho, drho);
         const R dx[3] = {dm[0], d0[0], dp[0]};
         const R dy[3] = {dm[1], d0[1], dp[1]};
         const R tx[3] = {R(1) + dm[0], R(1) + d0[0], R(1) + dp[0]};
@@ -431,6 +666,7 @@ __host__ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho
         }
     }
     return m;
+    }
 }
 
 }  // namespace lbmd

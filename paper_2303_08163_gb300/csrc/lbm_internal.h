@@ -7,12 +7,15 @@
 
 namespace lbmh {
 
-// Layout of one lattice's populations: Q planes of `plane` elements (plane >= ncell,
-// padded so that every plane starts on a 256-byte boundary), x fastest within a plane.
+// Layout of one lattice's populations: Q planes of `plane` elements, x fastest within a
+// plane, rows `pitch` elements apart.  pitch == nx, or nx rounded up to whole 16-byte units
+// so that every row of a ragged lattice starts where a bulk copy may start (the cells
+// [nx, pitch) of a row are padding: copied with the row, never read by a real cell).
+// Planes start on 256-byte boundaries (plane >= pitch * ny * nz).
 struct Lattice {
     void *A;
     int64_t plane;
-    int nx, ny, nz;
+    int nx, ny, nz, pitch;
     int64_t ncell;
     int D, P;  // dimension (2 or 3), storage precision (lbmd::P_*)
 };
@@ -27,6 +30,7 @@ struct StepArgs {
     int diag;                     // 1 = reduce diagnostics into partials
     double *partials;             // [blocks][8] when diag
     int32_t *status;              // device status word (LBM_ETIMEOUT on a timed-out wait)
+    unsigned *sync;               // several steps a launch: ticket, exit and done counters (zero between launches)
     int64_t timeout_ns;           // limit of every bounded device wait
 };
 
@@ -42,6 +46,7 @@ struct TmaShape {
 };
 
 constexpr int kDiagWords = 8;  // mass, jx, jy, jz, kinetic, max|u|, nonfinite, unused
+constexpr int kSyncDone = 4;  // first done counter in StepArgs::sync (after the ticket and exit counters)
 constexpr int kTmaMaxStages = 8;  // deepest shared-memory pipeline of the TMA row kernel
 
 // api.cu: record the message of a failed call for lbm_last_error(); returns code.
@@ -68,11 +73,18 @@ int diag_blocks_generic(int64_t ncell);
 
 // k_tma_*.cu
 bool tma_supported(const Lattice &lat);
+// Row pitch (elements) of a lattice: nx, or nx rounded up for the TMA kernel.
+int padded_pitch(int D, int P, int64_t nx);
 int tma_smem_bytes(const Lattice &lat, const TmaShape &t);
 // Largest number of colliding threads per block of the TMA kernel for the lattice.
 int tma_thread_limit(const Lattice &lat);
 cudaError_t tma_prepare(const Lattice &lat, int eq, int bulk, int cap, int smem_bytes);
-cudaError_t step_tma(const StepArgs &a, const TmaShape &t, cudaStream_t s);
+// Done counters a lattice is given (a row group has at least one row).
+int64_t sync_units(const Lattice &lat);
+// Steps one launch may take: the limits on tickets and launch length.  1 when the lattice has
+// more units than counters.
+int64_t tma_max_steps(const Lattice &lat, const TmaShape &t);
+cudaError_t step_tma(const StepArgs &a, const TmaShape &t, int nsteps, cudaStream_t s);
 int tma_max_blocks_per_sm(const Lattice &lat, int eq, int bulk, const TmaShape &t);
 
 // k_batch.cu -- many independent lattices in one arena (FP64, shifted).  Instance k has

@@ -34,6 +34,32 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// Order this thread's accesses across the generic and async proxies (all state spaces).
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+__device__ __forceinline__ void red_release(unsigned *p, unsigned v) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Wait until the counter reaches `want` (it only grows), for at most timeout_ns nanoseconds
+// or until another block has reported an error.
+__device__ __forceinline__ bool wait_count_bounded(const unsigned *p, unsigned want, const int32_t *status,
+                                                   int64_t timeout_ns) {
+    if (ld_acquire(p) >= want) return true;
+    const uint64_t t0 = global_ns();
+    while (true) {
+        for (int k = 0; k < 64; ++k)
+            if (ld_acquire(p) >= want) return true;
+        if (*(const volatile int32_t *)status != 0) return false;
+        if ((int64_t)(global_ns() - t0) > timeout_ns) return false;
+    }
+}
+
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                  "r"(bytes)
