@@ -1102,16 +1102,17 @@ void lbm_destroy(lbm_ctx *c) {
 // ------------------------------------------------------------------- von Neumann analysis
 
 namespace {
-// Device buffers of one von Neumann call, freed on every return path.
-struct VnBufs {
-    void *p[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    ~VnBufs() {
-        for (void *q : p)
-            if (q) cudaFree(q);
+// Device buffer of one von Neumann call (one allocation: a call on a few thousand points takes
+// about as long as three cudaMalloc and cudaFree pairs), freed on every return path.
+struct VnBuf {
+    char *p = nullptr;
+    ~VnBuf() {
+        if (p) cudaFree(p);
     }
-    bool alloc(int i, size_t bytes) {
-        if (cudaMalloc(&p[i], bytes) != cudaSuccess) {
+    bool alloc(size_t bytes) {
+        if (cudaMalloc(&p, bytes) != cudaSuccess) {
             cudaGetLastError();
+            p = nullptr;
             return false;
         }
         return true;
@@ -1129,17 +1130,17 @@ int lbm_vn_eigenvalues(int eq_kind, int bulk_corr, int64_t count, const double *
         if (!(params[6 * p] > 0.5) || !(params[6 * p + 1] > 0))
             return fail(LBM_EINVAL, "point %lld: tau must be > 1/2 and rho > 0", (long long)p);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    VnBufs b;
-    if (!b.alloc(0, sizeof(double) * 6 * count) || !b.alloc(1, sizeof(double) * 18 * count) ||
-        !b.alloc(2, sizeof(int32_t)))
-        return fail(LBM_ENOMEM, "von Neumann buffers");
-    CK(cudaMemcpyAsync(b.p[0], params, sizeof(double) * 6 * count, cudaMemcpyHostToDevice, s), "params upload");
-    CK(cudaMemsetAsync(b.p[2], 0, sizeof(int32_t), s), "status clear");
-    CK(vn_eigs(eq_kind, bulk_corr, count, (const double *)b.p[0], (double *)b.p[1], (int32_t *)b.p[2], s),
-       "eigenvalue kernel");
+    VnBuf b;
+    const size_t in = sizeof(double) * 6 * count, res = sizeof(double) * 18 * count;
+    if (!b.alloc(in + res + sizeof(int32_t))) return fail(LBM_ENOMEM, "von Neumann buffers");
+    double *dp = (double *)b.p, *dout = (double *)(b.p + in);
+    int32_t *dst = (int32_t *)(b.p + in + res);
+    CK(cudaMemcpyAsync(dp, params, in, cudaMemcpyHostToDevice, s), "params upload");
+    CK(cudaMemsetAsync(dst, 0, sizeof(int32_t), s), "status clear");
+    CK(vn_eigs(eq_kind, bulk_corr, count, dp, dout, dst, s), "eigenvalue kernel");
     int32_t st = 0;
-    CK(cudaMemcpyAsync(out, b.p[1], sizeof(double) * 18 * count, cudaMemcpyDeviceToHost, s), "eigenvalue copy");
-    CK(cudaMemcpyAsync(&st, b.p[2], sizeof(int32_t), cudaMemcpyDeviceToHost, s), "status copy");
+    CK(cudaMemcpyAsync(out, dout, res, cudaMemcpyDeviceToHost, s), "eigenvalue copy");
+    CK(cudaMemcpyAsync(&st, dst, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "status copy");
     CK(cudaStreamSynchronize(s), "eigenvalue sync");
     if (st) return fail(LBM_ECUDA, "the QR iteration did not converge for some point");
     return LBM_OK;
@@ -1151,48 +1152,24 @@ int lbm_vn_stability_limit(int eq_kind, int64_t npairs, const double *nu, const 
         nk > 1024 || !(u_hi > 0) || u_hi >= 1.0 || iterations < 1 || iterations > 60 || !(tol >= 0))
         return fail(LBM_EINVAL, "bad stability-limit arguments");
     if (npairs == 0) return LBM_OK;
-    std::vector<double> tau(npairs), lo(npairs, 0.0), hi(npairs, u_hi), trial(npairs);
-    for (int64_t p = 0; p < npairs; ++p) {
+    for (int64_t p = 0; p < npairs; ++p)
         if (!(nu[p] > 0)) return fail(LBM_EINVAL, "nu must be positive");
-        tau[p] = 0.5 + 3.0 * nu[p];
-    }
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    VnBufs b;
-    if (!b.alloc(0, sizeof(double) * npairs) || !b.alloc(1, sizeof(double) * npairs) ||
-        !b.alloc(2, sizeof(double) * npairs) || !b.alloc(3, sizeof(unsigned long long) * npairs) ||
-        !b.alloc(4, sizeof(int32_t)))
-        return fail(LBM_ENOMEM, "stability buffers");
-    CK(cudaMemcpyAsync(b.p[0], tau.data(), sizeof(double) * npairs, cudaMemcpyHostToDevice, s), "tau upload");
-    CK(cudaMemcpyAsync(b.p[1], theta, sizeof(double) * npairs, cudaMemcpyHostToDevice, s), "theta upload");
-    CK(cudaMemsetAsync(b.p[4], 0, sizeof(int32_t), s), "status clear");
-    std::vector<unsigned long long> bits(npairs);
-    // first probe u_hi itself (a pair stable there reports u_hi), then bisect [0, u_hi]
-    for (int it = 0; it <= iterations; ++it) {
-        for (int64_t p = 0; p < npairs; ++p) trial[p] = it == 0 ? u_hi : 0.5 * (lo[p] + hi[p]);
-        CK(cudaMemcpyAsync(b.p[2], trial.data(), sizeof(double) * npairs, cudaMemcpyHostToDevice, s), "trial upload");
-        CK(cudaMemsetAsync(b.p[3], 0, sizeof(unsigned long long) * npairs, s), "radius clear");
-        CK(vn_radius(eq_kind, npairs, (const double *)b.p[0], (const double *)b.p[1], (const double *)b.p[2], nk,
-                     (unsigned long long *)b.p[3], (int32_t *)b.p[4], s),
-           "spectral radius kernel");
-        CK(cudaMemcpyAsync(bits.data(), b.p[3], sizeof(unsigned long long) * npairs, cudaMemcpyDeviceToHost, s),
-           "radius copy");
-        CK(cudaStreamSynchronize(s), "radius sync");
-        for (int64_t p = 0; p < npairs; ++p) {
-            double r;
-            memcpy(&r, &bits[p], sizeof r);
-            const bool stable = r <= 1.0 + tol;
-            if (it == 0) {
-                if (stable) lo[p] = hi[p] = u_hi;
-            } else if (lo[p] < hi[p]) {
-                if (stable) lo[p] = trial[p];
-                else hi[p] = trial[p];
-            }
-        }
-    }
+    const size_t bytes = vn_limit_bytes(npairs);
+    std::vector<char> host(bytes);
+    vn_limit_fill(host.data(), npairs, nu, theta, u_hi);
+    VnBuf b;
+    if (!b.alloc(bytes + sizeof(int32_t))) return fail(LBM_ENOMEM, "stability buffers");
+    int32_t *dst = (int32_t *)(b.p + bytes);
+    CK(cudaMemcpyAsync(b.p, host.data(), bytes, cudaMemcpyHostToDevice, s), "pair upload");
+    CK(cudaMemsetAsync(dst, 0, sizeof(int32_t), s), "status clear");
+    CK(vn_limit(eq_kind, npairs, b.p, nk, u_hi, iterations, tol, dst, s), "stability search");
     int32_t st = 0;
-    CK(cudaMemcpy(&st, b.p[4], sizeof(int32_t), cudaMemcpyDeviceToHost), "status copy");
+    CK(cudaMemcpyAsync(host.data(), b.p, bytes, cudaMemcpyDeviceToHost, s), "limit copy");
+    CK(cudaMemcpyAsync(&st, dst, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "status copy");
+    CK(cudaStreamSynchronize(s), "stability sync");
     if (st) return fail(LBM_ECUDA, "the QR iteration did not converge for some point");
-    for (int64_t p = 0; p < npairs; ++p) umax[p] = lo[p];
+    vn_limit_read(host.data(), npairs, umax);
     return LBM_OK;
 }
 

@@ -123,7 +123,12 @@ cudaError_t batch_populations(const double *arena, const int64_t *cell_start,
 // k_vn.cu
 cudaError_t vn_eigs(int eq, int bulk, int64_t count, const double *params, double *out, int32_t *status,
                     cudaStream_t s);
-cudaError_t vn_radius(int eq, int64_t npairs, const double *tau, const double *theta, const double *u_try, int nk,
-                      unsigned long long *radius_bits, int32_t *status, cudaStream_t s);
+// Stability-limit search: vn_limit_bytes of state per call, filled and read on the host, all
+// trials enqueued by vn_limit.
+size_t vn_limit_bytes(int64_t npairs);
+void vn_limit_fill(void *host, int64_t npairs, const double *nu, const double *theta, double u_hi);
+void vn_limit_read(const void *host, int64_t npairs, double *umax);
+cudaError_t vn_limit(int eq, int64_t npairs, void *pairs, int nk, double u_hi, int iterations, double tol,
+                     int32_t *status, cudaStream_t s);
 
 }  // namespace lbmh
