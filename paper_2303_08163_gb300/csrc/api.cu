@@ -88,6 +88,8 @@ struct lbm_ctx {
     int kernel_opt = 0;  // 0 auto, 1 generic, 2 tma
     int kernel = 1;
     int gen_threads = 256, gen_blocks = 1;
+    bool chosen = false;  // the caller named a kernel or a launch shape
+    int small_threads = 0, small_blocks = 0;  // several steps of a small lattice at once (0: too large)
     TmaShape tma{};
     bool use_graph = false;
     cudaGraphExec_t graph2 = nullptr;  // even + odd step
@@ -188,6 +190,17 @@ cudaError_t launch_one(lbm_ctx *c, int odd, int diag, cudaStream_t s) {
 // n steps without diagnostics from the layout `odd` describes: several to a launch with the
 // TMA kernel, one each with the one-cell kernel.
 cudaError_t launch_steps(lbm_ctx *c, int odd, int64_t n, cudaStream_t s) {
+    if (n > 1 && !c->chosen && c->small_threads > 0) {
+        // (launches of bounded length: FP64 steps of 5 us)
+        cudaError_t e = cudaSuccess;
+        while (n > 0 && e == cudaSuccess) {
+            const int64_t m = std::min<int64_t>(n, 10000);
+            e = steps_small(step_args(c, odd, 0), (int)m, c->small_blocks, c->small_threads, s);
+            odd ^= (int)(m & 1);
+            n -= m;
+        }
+        return e;
+    }
     int64_t most = 1;
     if (c->kernel == 2 && n > 1) most = tma_max_steps(c->lat, c->tma);
     cudaError_t e = cudaSuccess;
@@ -554,6 +567,7 @@ int autotune(lbm_ctx *c) {
     // memory, fewest stages and fewest threads: equally fast boxes then pick the same shape.
     const int reps = p->ncell * (int64_t)c->Q * es > ((int64_t)1 << 28) ? 4 : 10;
     std::vector<std::pair<float, size_t>> score;
+    p->chosen = true;  // time the candidates themselves
     for (size_t q = 0; q < cands.size(); ++q) {
         if (!apply_shape(p, cands[q])) continue;
         if (time_steps(p, p->step, 2) < 0 || !take_status_clean(p)) continue;
@@ -698,6 +712,7 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
     c->gen_threads = 256;
     c->gen_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((ncell + 255) / 256, (int64_t)sm_count() * 16));
     c->kernel = 1;
+    if (!small_shape(c->lat, c->eq, c->bulk, sm_count(), &c->small_threads, &c->small_blocks)) c->small_threads = 0;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         static bool loaded = false;
@@ -733,6 +748,7 @@ int lbm_set_option(lbm_ctx *c, int option, int64_t value) {
         if (value == 2 && !tma_selectable(c))
             return fail(LBM_EINVAL, "TMA row kernel needs Nx * sizeof(storage) to be a multiple of 16");
         c->kernel_opt = (int)value;
+        c->chosen = value != 0;
         if (value == 1) c->kernel = 1;
         if (value == 2 || value == 0) {
             if (tma_supported(c->lat)) {
@@ -1048,6 +1064,7 @@ int lbm_set_launch_shape(lbm_ctx *c, const int64_t shape[6]) {
         if (shape[1] < 32 || shape[1] > 256 || shape[1] % 32)
             return fail(LBM_EINVAL, "threads must be a multiple of 32 in [32, 256] for the one-cell kernel");
         c->kernel = 1;
+        c->chosen = true;
         c->gen_threads = (int)shape[1];
         c->gen_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((c->ncell + shape[1] - 1) / shape[1],
                                                                     (int64_t)sm_count() * 16));
@@ -1075,6 +1092,7 @@ int lbm_set_launch_shape(lbm_ctx *c, const int64_t shape[6]) {
     CK(tma_prepare(c->lat, c->eq, c->bulk, t.cap, t.smem_bytes), "shared memory attribute");
     c->tma = t;
     c->kernel = 2;
+    c->chosen = true;
     drop_graph(c);
     return LBM_OK;
 }

@@ -10,4 +10,13 @@ cudaError_t step_generic_d3(const StepArgs &a, int blocks, int threads, cudaStre
     default: return cudaErrorInvalidValue;
     }
 }
+
+const void *small_kernel_d3(int P, int eq, int bulk) {
+    switch (P) {
+    case lbmd::P_F64: return lbmd::small_kernel_dp<3, lbmd::P_F64>(eq, bulk);
+    case lbmd::P_F32: return lbmd::small_kernel_dp<3, lbmd::P_F32>(eq, bulk);
+    case lbmd::P_F16S: return lbmd::small_kernel_dp<3, lbmd::P_F16S>(eq, bulk);
+    default: return nullptr;
+    }
+}
 }  // namespace lbmh

@@ -13,6 +13,7 @@
 #pragma once
 
 #include "lbm_common.cuh"
+#include "ptx.cuh"
 
 namespace lbmd {
 
@@ -92,6 +93,114 @@ __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
         loc.flush(acc, a.rho0);
         diag_block_store(acc, a.partials + (int64_t)blockIdx.x * lbmh::kDiagWords);
     }
+}
+
+// ------------------------------------------------------------------ several steps at once
+//
+// A small lattice's steps are bound by latency: a launch, a pipeline's ramp, or in the TMA row
+// kernel's several-step form the way of a row through shared memory and its counters.  Here all
+// its cells are in registers at once, one (or a few) to a thread: a step is a load of the
+// populations from L2, the collision, the stores and one barrier of the whole grid (cooperative
+// launch: all blocks are resident).  The barrier's arrivals are spread over kBarCounters counters,
+// each on its own line; a block's first warp looks at all of them.  Per step against the TMA row
+// kernel: 64^2 FP64 8.0 -> 5.3 us (3.3 us of it one warp's 105 FP64 instructions at 64 clocks),
+// 64^2 FP32 3.9 -> 2.1, 32^3 binary16 6.1 -> 2.8, 48^3 6.8 -> 5.7 us.
+
+template <typename T> __device__ __forceinline__ T ld_l2(const T *p) { return __ldcg(p); }
+
+// Wait until every block has arrived `gen` times (counters never wrap: gen * blocks < 2^32).
+__device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned gen, const int32_t *status, int64_t timeout_ns) {
+    __shared__ int bad;
+    __syncthreads();  // every store of the block is issued
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) {
+            bad = 0;
+            __threadfence();
+            red_release(&sync[lbmh::kBarStride * (1 + blockIdx.x % lbmh::kBarCounters)], 1u);
+        }
+        bool ok = true;
+        if (threadIdx.x < lbmh::kBarCounters && threadIdx.x < gridDim.x) {
+            const unsigned arrive = (gridDim.x - threadIdx.x + lbmh::kBarCounters - 1) / lbmh::kBarCounters;
+            ok = wait_count_bounded(&sync[lbmh::kBarStride * (1 + threadIdx.x)], gen * arrive, status, timeout_ns);
+        }
+        if (__any_sync(0xffffffffu, !ok) && threadIdx.x == 0) bad = 1;
+    }
+    __syncthreads();
+    return bad == 0;
+}
+
+template <int D, int P, int EQ, bool BULK>
+__global__ void __launch_bounds__(256) k_steps_small(const lbmh::StepArgs a, int nsteps) {
+    using St = Storage<P>;
+    using T = typename St::T;
+    using R = typename St::R;
+    constexpr int Q = qof(D);
+    T *A = static_cast<T *>(a.lat.A);
+    const int nx = a.lat.nx, ny = a.lat.ny, nz = a.lat.nz, pitch = a.lat.pitch;
+    const int plane = (int)a.lat.plane, ncell = (int)a.lat.ncell;  // Q * plane < 2^31 (checked on the host)
+    const R rho0 = step_scalar<R>(a.rho0, a.rho0f), omega0 = step_scalar<R>(a.omega0, a.omega0f),
+            six_nu = step_scalar<R>(a.six_nu, a.six_nuf);
+    bool ok = true;
+    int here = -1, xs[3], rows[9];  // the thread's cell and its neighbours: columns, row starts by (dy + 1) + 3 (dz + 1)
+    for (int s = 0; s < nsteps && ok; ++s) {
+        const int odd = (a.odd + s) & 1;
+        for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < ncell; cell += gridDim.x * blockDim.x) {
+            if (cell != here) {  // once, where a thread has one cell
+                int x, y, z;
+                cell_coords(cell, ncell, nx, ny, x, y, z);
+                here = cell;
+                xs[0] = wrapi(x - 1, nx);
+                xs[1] = x;
+                xs[2] = wrapi(x + 1, nx);
+#pragma unroll
+                for (int q = 0; q < (D == 3 ? 9 : 3); ++q) {
+                    const int yy = wrapi(y + q % 3 - 1, ny), zz = D == 3 ? wrapi(z + q / 3 - 1, nz) : z;
+                    rows[q] = pitch * (yy + ny * zz);
+                }
+            }
+            const int self = rows[D == 3 ? 4 : 1] + xs[1];
+            if (!LBM_CHECK(self >= 0 && self < plane, a.status)) continue;
+            R f[Q];
+            if (!odd) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) f[i] = St::load(ld_l2(A + i * plane + self));
+            } else {
+#pragma unroll
+                for (int i = 0; i < Q; ++i)  // f_i(r) = A[opp(i)][r - c_i]
+                    f[i] = St::load(ld_l2(A + (Q - 1 - i) * plane + rows[(1 - cyo(i)) + (D == 3 ? 3 * (1 - czo(i)) : 0)] + xs[1 - cxo(i)]));
+            }
+            collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
+            if (!odd) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) A[(Q - 1 - i) * plane + self] = St::store(f[i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+                    A[i * plane + rows[(1 + cyo(i)) + (D == 3 ? 3 * (1 + czo(i)) : 0)] + xs[1 + cxo(i)]] = St::store(f[i]);
+            }
+        }
+        if (s + 1 < nsteps) ok = grid_barrier(a.sync, (unsigned)(s + 1), a.status, a.timeout_ns);
+    }
+    if (!ok && threadIdx.x == 0) report_status(a.status, -5); /* LBM_ETIMEOUT */
+    // the last block to finish clears the counters for the next launch
+    __syncthreads();
+    bool last = false;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&a.sync[1], 1u) == gridDim.x - 1;
+    }
+    if (__syncthreads_or(last))
+        for (int p = threadIdx.x; p < lbmh::kBarStride * (1 + lbmh::kBarCounters); p += blockDim.x) a.sync[p] = 0;
+}
+
+template <int D, int P> const void *small_kernel_dp(int eq, int bulk) {
+#define LBM_SMALL(EQv) \
+    if (eq == EQv) return bulk ? (const void *)k_steps_small<D, P, EQv, true> : (const void *)k_steps_small<D, P, EQv, false>;
+    LBM_SMALL(EQ_ENT)
+    LBM_SMALL(EQ_POLY2)
+    LBM_SMALL(EQ_PROD)
+#undef LBM_SMALL
+    return nullptr;
 }
 
 template <int D, int P>

@@ -46,6 +46,8 @@ struct TmaShape {
 };
 
 constexpr int kDiagWords = 8;  // mass, jx, jy, jz, kinetic, max|u|, nonfinite, unused
+constexpr int kBarCounters = 16;  // counters of a grid barrier in StepArgs::sync, the first at kBarStride,
+constexpr int kBarStride = 32;    // one to a 128-byte line
 constexpr int kSyncDone = 4;  // first done counter in StepArgs::sync (after the ticket and exit counters)
 constexpr int kTmaMaxStages = 8;  // deepest shared-memory pipeline of the TMA row kernel
 
@@ -54,6 +56,10 @@ int set_last_error(int code, const char *msg);
 
 // k_generic.cu
 cudaError_t step_generic(const StepArgs &a, int blocks, int threads, cudaStream_t s);
+// Several steps of a small lattice in one cooperative launch.  small_shape: threads and blocks of
+// the launch, false if the lattice is too large for it.
+bool small_shape(const Lattice &lat, int eq, int bulk, int sms, int *threads, int *blocks);
+cudaError_t steps_small(const StepArgs &a, int nsteps, int blocks, int threads, cudaStream_t s);
 cudaError_t init_fields(const Lattice &lat, int eq, double rho0, const void *rho, const void *u,
                         int dtype, cudaStream_t s);
 cudaError_t moments(const Lattice &lat, double rho0, int odd, void *rho, void *u, int dtype,

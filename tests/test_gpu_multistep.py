@@ -13,6 +13,8 @@ CASES = [
     (2, (64, 64, 1), 0, None), (2, (64, 1, 1), 0, None), (2, (64, 2, 1), 1, None), (2, (48, 3, 1), 2, None),
     (2, (256, 700, 1), 1, (2, 128, 2, 1, 64, 1024)), (2, (509, 381, 1), 1, None), (2, (40, 37, 1), 2, (2, 64, 3, 4, 40, 1024)),
     (3, (32, 32, 32), 2, None), (3, (16, 9, 1), 1, None), (3, (16, 5, 2), 2, None), (3, (16, 40, 3), 0, None),
+    # the largest lattice of the grid-barrier kernel on 152 SMs, and the next one
+    (2, (320, 380, 1), 1, None), (2, (320, 381, 1), 1, None), (3, (64, 50, 38), 2, None), (3, (61, 53, 37), 1, None),
     (3, (64, 30, 31), 1, None), (3, (67, 20, 11), 2, None), (3, (96, 64, 20), 2, (2, 128, 2, 1, 48, 1024)),
 ]
 
@@ -88,13 +90,37 @@ def test_states_larger_than_l2(D, dims, prec):
         lat.close()
 
 
-def test_lattices_on_two_streams():
+@pytest.mark.parametrize("D,dims,prec", [(2, (96, 70, 1), 0), (3, (40, 24, 20), 2), (3, (96, 80, 70), 2)])
+def test_steps_inside_a_stream_capture(D, dims, prec):
+    """lbm_step recorded in a caller's graph and replayed."""
+    import torch
+    from paper_2303_08163_gb300 import lbm
+    rho, u = inputs.random_state(D, dims, seed=31, u_max=0.05)
+    s = torch.cuda.Stream()
+    lats = [lbm.Lattice(D - 2, dims, 0.7, 0, 0, prec, stream=s) for _ in range(2)]
+    for lat in lats:
+        lat.init_fields(rho, u)
+        lat.step(6)
+        lat.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        lats[0].step(6)
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    lats[1].step(18)
+    assert np.array_equal(*(lat.get_populations("storage") for lat in lats))
+    for lat in lats:
+        lat.close()
+
+
+@pytest.mark.parametrize("dims", [(128, 128, 24), (32, 32, 32)])
+def test_lattices_on_two_streams(dims):
     """Two lattices stepping at once on their own streams: launches that wait for their own
     blocks' counters only."""
     import torch
     from paper_2303_08163_gb300 import lbm
     streams = [torch.cuda.Stream() for _ in range(2)]
-    dims = (128, 128, 24)
     rho, u = inputs.random_state(3, dims, seed=9, u_max=0.05)
     lats = [lbm.Lattice(1, dims, 0.6, 0, 0, 2, stream=s) for s in streams]
     for lat in lats:
