@@ -23,27 +23,54 @@ static inline int grid_for(int64_t n, int threads, int cap = 152 * 32) {
     return (int)g;
 }
 
+// The kernels between the caller's fields or populations and the stored ones are bound by HBM (FP64
+// storage by the FP64 pipe).  A thread has V neighbouring cells of a row: 2 for binary16 storage,
+// where a 2-byte access for each population leaves the memory pipe half used (512^3: initialisation
+// 2.43 -> 1.52 ms, moments 2.06 - 2.48 -> 1.45 - 1.85 ms, 1.39 ms of HBM time), otherwise 1.  Kernels that
+// write the stored populations run over the rows with their padding and write each plane where the
+// thread is, so that warps write whole aligned segments; shifts go into the reads (FP32
+// 245 x 196 x 172: initialisation 0.34 -> 0.21 ms; FP32 256^3 populations after an odd number of
+// steps 0.86 -> 0.60 ms.  FP64 populations, whose 8-byte accesses fill segments anyway, are
+// written where they belong: 0.14 against 0.19 ms on 128^3).
+
+// V stored values at p (V = 2: p even).
+template <int P, int V>
+__device__ __forceinline__ void store_v(typename Storage<P>::T *p, const typename Storage<P>::R (&v)[V]) {
+    if constexpr (V == 2) *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v[0], v[1]);
+    else *p = Storage<P>::store(v[0]);
+}
+
 // f = f^eq(rho, u), written in the even (canonical) layout, shifted by w_i rho0.
-template <int D, int P, int EQ, typename In>
+template <int D, int P, int EQ, int V, typename In>
 __global__ void k_init(lbmh::Lattice lat, double rho0d, const In *__restrict__ rho,
                        const In *__restrict__ u) {
-    using St = Storage<P>;
-    using R = typename St::R;
+    using R = typename Storage<P>::R;
     constexpr int Q = qof(D);
-    auto *A = static_cast<typename St::T *>(lat.A);
+    auto *A = static_cast<typename Storage<P>::T *>(lat.A);
     const R rho0 = R(rho0d);
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < lat.ncell;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const R r = R(rho[c]);
-        R uu[3] = {R(u[c]), R(u[lat.ncell + c]), D == 3 ? R(u[2 * lat.ncell + c]) : R(0)};
-        R h[Q];
-        equilibrium_h<D, EQ, R>(uu, h);
-        const R drho = r - rho0;
+    const int64_t padded = (int64_t)lat.pitch * lat.ny * lat.nz;
+    for (int64_t p = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); p < padded;
+         p += V * (int64_t)gridDim.x * blockDim.x) {
         int x, y, z;
-        cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
-        const int64_t cell = x + (int64_t)lat.pitch * (y + (int64_t)lat.ny * z);
+        cell_coords(p, padded, lat.pitch, lat.ny, x, y, z);
+        if (x >= lat.nx) continue;
+        const int64_t c = x + (int64_t)lat.nx * (y + (int64_t)lat.ny * z);
+        R r[V], drho[V], h[V][Q];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) A[(int64_t)i * lat.plane + cell] = St::store(R(wq<D>(i)) * fma_r(r, h[i], drho));
+        for (int v = 0; v < V; ++v) {
+            const int64_t cv = V == 1 || x + v < lat.nx ? c + v : c;  // (a row's last pair may end in its padding)
+            r[v] = R(rho[cv]);
+            R uu[3] = {R(u[cv]), R(u[lat.ncell + cv]), D == 3 ? R(u[2 * lat.ncell + cv]) : R(0)};
+            equilibrium_h<D, EQ, R>(uu, h[v]);
+            drho[v] = r[v] - rho0;
+        }
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            R f[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) f[v] = R(wq<D>(i)) * fma_r(r[v], h[v][i], drho[v]);
+            store_v<P, V>(A + (int64_t)i * lat.plane + p, f);
+        }
     }
 }
 
@@ -59,49 +86,131 @@ __device__ __forceinline__ void load_canonical(const lbmh::Lattice &lat, int odd
         f[i] = St::load(A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)]);
 }
 
-template <int D, int P, typename Out>
+// The same for V cells of a row from c (V = 2: nx and c even): both halves at once where the layout
+// has them side by side.
+template <int D, int P, int V>
+__device__ __forceinline__ void load_canonical_v(const lbmh::Lattice &lat, int odd, int64_t c,
+                                                 typename Storage<P>::R (&f)[V][qof(D)]) {
+    int x, y, z;
+    if constexpr (V == 1) {
+        load_canonical<D, P>(lat, odd, c, f[0], x, y, z);
+    } else {
+        cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
+        const auto *A = static_cast<const __half *>(lat.A);
+#pragma unroll
+        for (int i = 0; i < qof(D); ++i) {
+            const int64_t a = aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd);
+            if (!odd || cxo(i) == 0) {
+                const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(A + a));
+                f[0][i] = v.x;
+                f[1][i] = v.y;
+            } else {
+                f[0][i] = __half2float(A[a]);
+                f[1][i] = __half2float(A[aa_index<D>(i, x + 1, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)]);
+            }
+        }
+    }
+}
+
+template <int D, int P, int V, typename Out>
 __global__ void k_moments(lbmh::Lattice lat, double rho0d, int odd, Out *__restrict__ rho,
                           Out *__restrict__ u) {
     using R = typename Storage<P>::R;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < lat.ncell;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        R f[qof(D)];
-        int x, y, z;
-        load_canonical<D, P>(lat, odd, c, f, x, y, z);
-        const CellMoments<R> m = moments_shifted<D, R>(f, R(rho0d));
-        rho[c] = Out(m.rho);
-        u[c] = Out(m.u[0]);
-        u[lat.ncell + c] = Out(m.u[1]);
-        if (D == 3) u[2 * lat.ncell + c] = Out(m.u[2]);
+    for (int64_t c = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); c < lat.ncell;
+         c += V * (int64_t)gridDim.x * blockDim.x) {
+        R f[V][qof(D)];
+        load_canonical_v<D, P, V>(lat, odd, c, f);
+        CellMoments<R> m[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) m[v] = moments_shifted<D, R>(f[v], R(rho0d));
+#pragma unroll
+        for (int v = 0; v < V; ++v) rho[c + v] = Out(m[v].rho);
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+#pragma unroll
+            for (int v = 0; v < V; ++v) u[a * lat.ncell + c + v] = Out(m[v].u[a]);
     }
 }
 
-template <int D, int P, typename Out>
-__global__ void k_get_pop(lbmh::Lattice lat, double rho0, int odd, Out *__restrict__ f) {
+// w_i rho0 of one weight class: the double, and split into two floats for FP32 callers.
+struct ClassShift {
+    double w[4];
+    float hi[4], lo[4];
+};
+
+// g + w rho0 and f - w rho0 in the caller's type.  For FP32 storage and callers the sum is formed in
+// FP32 with its rounding error carried (two-sum), so that it is the FP64 sum rounded to FP32 but
+// for the last of 48 bits: conversions to and from FP64 and an FP64 addition for each population
+// took 19.6 ms on a 512^3 binary16 lattice (3.2 ms of HBM time) on the FP64 pipe.
+__device__ __forceinline__ float two_sum(float a, float b, float c) {  // a + b + c, |c| << |a + b|
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return __fadd_rn(s, __fadd_rn(e, c));
+}
+template <typename R, typename Out>
+__device__ __forceinline__ Out unshift(R g, const ClassShift &k, int c) {
+    if constexpr (sizeof(R) == 4 && sizeof(Out) == 4) return two_sum(g, k.hi[c], k.lo[c]);
+    else return Out((double)g + k.w[c]);
+}
+template <typename R, typename In>
+__device__ __forceinline__ R shift(In f, const ClassShift &k, int c) {
+    if constexpr (sizeof(R) == 4 && sizeof(In) == 4) return two_sum(f, -k.hi[c], -k.lo[c]);
+    else return R((double)f - k.w[c]);
+}
+
+template <int D, int P, int V, typename Out>
+__global__ void k_get_pop(lbmh::Lattice lat, ClassShift k, int odd, Out *__restrict__ f) {
     using R = typename Storage<P>::R;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < lat.ncell;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        R g[qof(D)];
-        int x, y, z;
-        load_canonical<D, P>(lat, odd, c, g, x, y, z);
+    for (int64_t c = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); c < lat.ncell;
+         c += V * (int64_t)gridDim.x * blockDim.x) {
+        R g[V][qof(D)];
+        load_canonical_v<D, P, V>(lat, odd, c, g);
 #pragma unroll
-        for (int i = 0; i < qof(D); ++i) f[(int64_t)i * lat.ncell + c] = Out((double)g[i] + wq<D>(i) * rho0);
+        for (int i = 0; i < qof(D); ++i)
+#pragma unroll
+            for (int v = 0; v < V; ++v) f[(int64_t)i * lat.ncell + c + v] = unshift<R, Out>(g[v][i], k, wclass<D>(i));
     }
 }
 
-template <int D, int P, typename In>
-__global__ void k_set_pop(lbmh::Lattice lat, double rho0, int odd, const In *__restrict__ f) {
-    using St = Storage<P>;
-    using R = typename St::R;
-    auto *A = static_cast<typename St::T *>(lat.A);
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < lat.ncell;
-         c += (int64_t)gridDim.x * blockDim.x) {
+template <int D, int P, int V, typename In>
+__global__ void k_set_pop(lbmh::Lattice lat, ClassShift k, int odd, const In *__restrict__ f) {
+    using R = typename Storage<P>::R;
+    constexpr int Q = qof(D);
+    auto *A = static_cast<typename Storage<P>::T *>(lat.A);
+    const int64_t padded = (int64_t)lat.pitch * lat.ny * lat.nz;
+    for (int64_t p = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); p < padded;
+         p += V * (int64_t)gridDim.x * blockDim.x) {
         int x, y, z;
-        cell_coords(c, lat.ncell, lat.nx, lat.ny, x, y, z);
+        cell_coords(p, padded, lat.pitch, lat.ny, x, y, z);
+        if (x >= lat.nx) continue;
+        if constexpr (P == P_F64) {
+            const int64_t c = x + (int64_t)lat.nx * (y + (int64_t)lat.ny * z);
 #pragma unroll
-        for (int i = 0; i < qof(D); ++i) {
-            const double v = (double)f[(int64_t)i * lat.ncell + c] - wq<D>(i) * rho0;
-            A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)] = St::store(R(v));
+            for (int i = 0; i < Q; ++i)
+                A[aa_index<D>(i, x, y, z, lat.nx, lat.ny, lat.nz, lat.pitch, lat.plane, odd)] =
+                    shift<R, In>(f[(int64_t)i * lat.ncell + c], k, wclass<D>(i));
+            continue;
+        }
+        In v[Q][V];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            // slot opp(i) of this cell holds f_i of the cell c_i further after an odd number of
+            // steps, slot i holds its own f_i after an even one
+            const int yy = odd ? wrapi(y + cyo(i), lat.ny) : y;
+            const int zz = D == 3 && odd ? wrapi(z + czo(i), lat.nz) : z;
+            const In *row = f + (int64_t)i * lat.ncell + (int64_t)lat.nx * (yy + (int64_t)lat.ny * zz);
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                const int xv = x + q < lat.nx ? x + q : x;
+                v[i][q] = row[odd ? wrapi(xv + cxo(i), lat.nx) : xv];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            R r[V];
+#pragma unroll
+            for (int q = 0; q < V; ++q) r[q] = shift<R, In>(v[i][q], k, wclass<D>(i));
+            store_v<P, V>(A + (int64_t)(odd ? Q - 1 - i : i) * lat.plane + p, r);
         }
     }
 }
@@ -256,16 +365,31 @@ cudaError_t steps_small(const StepArgs &a, int nsteps, int blocks, int threads, 
         else return cudaErrorInvalidValue;                                                 \
     } while (0)
 
+// Pairs of binary16 cells: rows (with their padding where the kernel writes them) of even length.
+static bool pairs_ok(const Lattice &lat, bool writes) { return ((writes ? lat.pitch : lat.nx) & 1) == 0; }
+
+#define LBM_DISPATCH_DPV(D_, P_, PAIRS_, CALL)                                                              \
+    do {                                                                                                    \
+        if ((P_) == P_F16S && (PAIRS_)) {                                                                   \
+            if ((D_) == 2) { constexpr int DD = 2, PP = P_F16S, VV = 2; CALL; }                             \
+            else { constexpr int DD = 3, PP = P_F16S, VV = 2; CALL; }                                       \
+        } else {                                                                                            \
+            constexpr int VV = 1;                                                                           \
+            LBM_DISPATCH_DP(D_, P_, CALL);                                                                  \
+        }                                                                                                   \
+    } while (0)
+
 cudaError_t init_fields(const Lattice &lat, int eq, double rho0, const void *rho, const void *u,
                         int dtype, cudaStream_t s) {
-    const int g = grid_for(lat.ncell, 256);
+    const bool two = pairs_ok(lat, true);
+    const int g = grid_for((int64_t)lat.pitch * lat.ny * lat.nz / (two && lat.P == P_F16S ? 2 : 1), 256);
 #define LBM_INIT_EQ(EQv)                                                                         \
     if (eq == EQv) {                                                                             \
         if (dtype == 0)                                                                          \
-            LBM_DISPATCH_DP(lat.D, lat.P, (k_init<DD, PP, EQv, double><<<g, 256, 0, s>>>(        \
+            LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_init<DD, PP, EQv, VV, double><<<g, 256, 0, s>>>(        \
                                                 lat, rho0, (const double *)rho, (const double *)u))); \
         else                                                                                     \
-            LBM_DISPATCH_DP(lat.D, lat.P, (k_init<DD, PP, EQv, float><<<g, 256, 0, s>>>(         \
+            LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_init<DD, PP, EQv, VV, float><<<g, 256, 0, s>>>(         \
                                                 lat, rho0, (const float *)rho, (const float *)u))); \
         return cudaGetLastError();                                                               \
     }
@@ -278,35 +402,51 @@ cudaError_t init_fields(const Lattice &lat, int eq, double rho0, const void *rho
 
 cudaError_t moments(const Lattice &lat, double rho0, int odd, void *rho, void *u, int dtype,
                     cudaStream_t s) {
-    const int g = grid_for(lat.ncell, 256);
+    const bool two = pairs_ok(lat, false);
+    const int g = grid_for(lat.ncell / (two && lat.P == P_F16S ? 2 : 1), 256);
     if (dtype == 0)
-        LBM_DISPATCH_DP(lat.D, lat.P, (k_moments<DD, PP, double><<<g, 256, 0, s>>>(lat, rho0, odd, (double *)rho, (double *)u)));
+        LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_moments<DD, PP, VV, double><<<g, 256, 0, s>>>(lat, rho0, odd, (double *)rho, (double *)u)));
     else
-        LBM_DISPATCH_DP(lat.D, lat.P, (k_moments<DD, PP, float><<<g, 256, 0, s>>>(lat, rho0, odd, (float *)rho, (float *)u)));
+        LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_moments<DD, PP, VV, float><<<g, 256, 0, s>>>(lat, rho0, odd, (float *)rho, (float *)u)));
     return cudaGetLastError();
+}
+
+static ClassShift class_shift(int D, double rho0) {
+    ClassShift k;
+    for (int c = 0; c < 4; ++c) {
+        k.w[c] = (D == 2 ? (c <= 2 ? wclass_weight<2>(c) : 0.0) : wclass_weight<3>(c)) * rho0;
+        k.hi[c] = (float)k.w[c];
+        k.lo[c] = (float)(k.w[c] - (double)k.hi[c]);
+    }
+    return k;
 }
 
 cudaError_t get_populations(const Lattice &lat, double rho0, int odd, void *f, int dtype,
                             cudaStream_t s) {
-    const int g = grid_for(lat.ncell, 256);
+    const bool two = pairs_ok(lat, false);
+    const int g = grid_for(lat.ncell / (two && lat.P == P_F16S && dtype != 2 ? 2 : 1), 256);
+    const ClassShift k = class_shift(lat.D, rho0);
     if (dtype == 2)
         LBM_DISPATCH_DP(lat.D, lat.P, (k_get_pop_raw<DD, PP><<<g, 256, 0, s>>>(lat, odd, (typename Storage<PP>::T *)f)));
     else if (dtype == 0)
-        LBM_DISPATCH_DP(lat.D, lat.P, (k_get_pop<DD, PP, double><<<g, 256, 0, s>>>(lat, rho0, odd, (double *)f)));
+        LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_get_pop<DD, PP, VV, double><<<g, 256, 0, s>>>(lat, k, odd, (double *)f)));
     else
-        LBM_DISPATCH_DP(lat.D, lat.P, (k_get_pop<DD, PP, float><<<g, 256, 0, s>>>(lat, rho0, odd, (float *)f)));
+        LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_get_pop<DD, PP, VV, float><<<g, 256, 0, s>>>(lat, k, odd, (float *)f)));
     return cudaGetLastError();
 }
 
 cudaError_t set_populations(const Lattice &lat, double rho0, int odd, const void *f, int dtype,
                             cudaStream_t s) {
-    const int g = grid_for(lat.ncell, 256);
+    const bool two = pairs_ok(lat, true);
+    const int64_t cells = dtype == 2 ? lat.ncell : (int64_t)lat.pitch * lat.ny * lat.nz;
+    const int g = grid_for(cells / (two && lat.P == P_F16S && dtype != 2 ? 2 : 1), 256);
+    const ClassShift k = class_shift(lat.D, rho0);
     if (dtype == 2)
         LBM_DISPATCH_DP(lat.D, lat.P, (k_set_pop_raw<DD, PP><<<g, 256, 0, s>>>(lat, odd, (const typename Storage<PP>::T *)f)));
     else if (dtype == 0)
-        LBM_DISPATCH_DP(lat.D, lat.P, (k_set_pop<DD, PP, double><<<g, 256, 0, s>>>(lat, rho0, odd, (const double *)f)));
+        LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_set_pop<DD, PP, VV, double><<<g, 256, 0, s>>>(lat, k, odd, (const double *)f)));
     else
-        LBM_DISPATCH_DP(lat.D, lat.P, (k_set_pop<DD, PP, float><<<g, 256, 0, s>>>(lat, rho0, odd, (const float *)f)));
+        LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_set_pop<DD, PP, VV, float><<<g, 256, 0, s>>>(lat, k, odd, (const float *)f)));
     return cudaGetLastError();
 }
 
