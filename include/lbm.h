@@ -281,7 +281,8 @@ int lbm_batch_get_populations(lbm_batch *b, void *f, int dtype, int on_device);
 /* Number of cells of all instances together, and the current step counter. */
 int lbm_batch_info(lbm_batch *b, int64_t *total_cells, int64_t *step);
 
-/* Launch shape of the batched kernel: out[0] = threads per block, out[1] = blocks,
+/* Launch shape of the batched kernel: out[0] = threads per block, out[1] = blocks (where the
+ * library gives instances teams of blocks, the number of teams: one per instance),
  * out[2] = largest per-block cell load, out[3] = mean per-block cell load. */
 int lbm_batch_launch_info(lbm_batch *b, int64_t out[4]);
 
@@ -290,14 +291,16 @@ int lbm_batch_launch_info(lbm_batch *b, int64_t out[4]);
  * [32, 256]) and `blocks` (1 .. min(count, 32 x the SM count)).  Instances are
  * re-assigned to the blocks longest-first (each to the least-loaded block so far); a
  * block owns whole instances, so blocks never wait for one another and more blocks than
- * fit on the GPU at once simply run in waves.  Returns LBM_EINVAL for other values.
+ * fit on the GPU at once simply run in waves.  Returns LBM_EINVAL for other values.  (Without
+ * this call a batch of few or uneven instances, whose largest would keep one SM busy longer than
+ * its share, gives each instance a team of blocks in proportion to its cells.)
  */
 int lbm_batch_set_launch_shape(lbm_batch *b, int threads, int64_t blocks);
 
 /*
  * Launch-shape autotuner of the batched kernel: times `steps` steps (1 .. 100000) of the
  * current state under each candidate shape (64, 128 or 256 threads; 1, 2, 3, 4, 6, 8, 12
- * or 16 blocks per SM), twice, and keeps the fastest (among shapes within 0.5 % of it, the
+ * or 16 blocks per SM, and the teams of blocks where the batch has them), twice, and keeps the fastest (among shapes within 0.5 % of it, the
  * one with the fewest blocks, then threads).  The state, the step counter and the status
  * are restored afterwards, so the call changes only the launch shape; the probes of the
  * timed steps are written to samples that the next lbm_batch_step rewrites.  Needs one

@@ -117,6 +117,14 @@ struct lbm_batch {
     int64_t step = 0;
     int blocks = 0, threads = 256;
     int block_cap = 0;  // capacity of d_block_start (blocks + 1 entries at most)
+    // teams of blocks (k_step_teams) instead of whole instances per block
+    bool teams = false;
+    int team_blocks = 0;
+    int64_t team_max = 0;             // largest number of cells of a block
+    char *d_team = nullptr;           // one allocation for the team's tables, sums, counters and status
+    int32_t *team_instance = nullptr, *team_part = nullptr, *team_size = nullptr, *team_status = nullptr;
+    double *team_partials = nullptr;
+    unsigned *team_sync = nullptr;
     int64_t max_load = 0, mean_load = 0;
     std::vector<int32_t> dims;
     std::vector<int64_t> cell_start;
@@ -1268,6 +1276,87 @@ static cudaError_t batch_assign(lbm_batch *b, int nb) {
     return cudaSuccess;
 }
 
+// Plans teams of blocks where the largest instance alone would keep an SM busy longer than its
+// share of all cells.  Sets team_blocks (0: no teams) and uploads the tables.  The smallest number
+// of cells a block for which all blocks are resident: 608 blocks of 128 threads for D2Q9, so every
+// SM's FP64 pipe has several warps.  30 lattices of
+// 16^2 .. 96^2: 185 -> 17 us a step, 60 of 16^2 .. 256^2: 1225 -> 100 us.
+static cudaError_t batch_plan_teams(lbm_batch *b) {
+    b->team_blocks = 0;
+    b->team_max = 0;
+    const std::vector<int64_t> &cs = b->cell_start;
+    int64_t largest = 0;
+    for (int64_t k = 0; k < b->count; ++k) largest = std::max(largest, cs[k + 1] - cs[k]);
+    const int sms = sm_count();
+    if (largest * sms * 10 <= b->total * 11 || largest * b->Q >= ((int64_t)1 << 31)) return cudaSuccess;
+    const int cap = team_block_capacity(b->D, b->eq, b->bulk, sms);
+    if (b->count > cap) return cudaSuccess;
+    auto blocks_for = [&](int64_t per) {
+        int64_t n = 0;
+        for (int64_t k = 0; k < b->count; ++k) n += (cs[k + 1] - cs[k] + per - 1) / per;
+        return n;
+    };
+    int64_t lo = 1, hi = (largest + kTeamThreads - 1) / kTeamThreads;  // cells a block / threads
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) / 2;
+        if (blocks_for(mid * kTeamThreads) <= cap) hi = mid;
+        else lo = mid + 1;
+    }
+    const int64_t per = lo * kTeamThreads;
+    std::vector<int32_t> inst, part, size(b->count);
+    for (int64_t k = 0; k < b->count; ++k) {
+        const int64_t n = cs[k + 1] - cs[k];
+        size[k] = (int32_t)((n + per - 1) / per);
+        for (int32_t q = 0; q < size[k]; ++q) {
+            inst.push_back((int32_t)k);
+            part.push_back(q);
+        }
+        b->team_max = std::max(b->team_max, (n + size[k] - 1) / size[k]);
+    }
+    // the busiest SM with teams (its blocks at most) against the busiest one without (the largest
+    // instance): 600 lattices of 16^2 .. 160^2 have a block each and little to share out
+    const int64_t nbl = (int64_t)inst.size();
+    if ((nbl + sms - 1) / sms * b->team_max * 10 > std::max(largest, b->total / sms) * 11) return cudaSuccess;
+    const size_t nb = inst.size();
+    auto pad = [](size_t n) { return (n + 255) / 256 * 256; };
+    const size_t sync = pad(sizeof(unsigned) * kBarStride * (b->count + 1)), sums = pad(sizeof(double) * 16 * nb);
+    const size_t table = pad(sizeof(int32_t) * nb), sizes = pad(sizeof(int32_t) * b->count);
+    if (cudaMalloc(&b->d_team, 256 + sync + sums + 2 * table + sizes) != cudaSuccess) {
+        cudaGetLastError();
+        return cudaSuccess;  // no room: whole instances per block
+    }
+    char *p = b->d_team;
+    b->team_status = (int32_t *)p;
+    b->team_sync = (unsigned *)(p += 256);
+    b->team_partials = (double *)(p += sync);
+    b->team_instance = (int32_t *)(p += sums);
+    b->team_part = (int32_t *)(p += table);
+    b->team_size = (int32_t *)(p += table);
+    cudaError_t e = cudaMemset(b->d_team, 0, 256 + sync);
+    if (e == cudaSuccess) e = cudaMemcpy(b->team_instance, inst.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b->team_part, part.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b->team_size, size.data(), sizeof(int32_t) * b->count, cudaMemcpyHostToDevice);
+    b->team_blocks = (int)nb;
+    return e;
+}
+
+static void batch_use_teams(lbm_batch *b) {
+    b->teams = true;
+    b->threads = kTeamThreads;
+    b->blocks = b->team_blocks;
+    b->max_load = b->team_max;
+    b->mean_load = b->total / b->team_blocks;
+}
+
+// LBM_ETIMEOUT if a team's bounded wait ran out (the stream is idle).
+static int batch_team_status(lbm_batch *b) {
+    if (!b->teams) return LBM_OK;
+    int32_t st = 0;
+    CK(cudaMemcpy(&st, b->team_status, sizeof st, cudaMemcpyDeviceToHost), "status read");
+    if (st != 0) return batch_sticky(b, fail(LBM_ETIMEOUT, "a bounded device wait ran out (status %d)", st));
+    return LBM_OK;
+}
+
 int lbm_batch_create(lbm_batch **out, int lattice, int64_t count, const int32_t *dims,
                      const double *tau, int eq_kind, int bulk_corr, int precision, double rho0,
                      void *cuda_stream) {
@@ -1330,7 +1419,11 @@ int lbm_batch_create(lbm_batch **out, int lattice, int64_t count, const int32_t 
     up(b->d_dims, dims, sizeof(int32_t) * 3 * count);
     up(b->d_omega, om.data(), sizeof(double) * count);
     up(b->d_sixnu, sn.data(), sizeof(double) * count);
-    if (e == cudaSuccess) e = batch_assign(b, (int)std::min<int64_t>(count, (int64_t)sm_count() * 2));
+    if (e == cudaSuccess) e = batch_plan_teams(b);
+    if (e == cudaSuccess) {
+        if (b->team_blocks > 0) batch_use_teams(b);
+        else e = batch_assign(b, (int)std::min<int64_t>(count, (int64_t)sm_count() * 2));
+    }
     if (e == cudaSuccess) e = cudaMemset(b->arena, 0, arena_bytes);
     if (e == cudaSuccess) e = cudaMemset(b->d_status, 0, sizeof(int32_t) * count);
     if (e != cudaSuccess) {
@@ -1439,7 +1532,18 @@ static BatchArgs batch_args(lbm_batch *b, int64_t n) {
     a.step0 = b->step;
     a.nsteps = n;
     a.every_k = b->d_tw ? b->every_k : 0;
+    a.team_instance = b->team_instance;
+    a.team_part = b->team_part;
+    a.team_size = b->team_size;
+    a.team_partials = b->team_partials;
+    a.team_sync = b->team_sync;
+    a.team_status = b->team_status;
+    a.timeout_ns = wait_timeout_ns();
     return a;
+}
+
+static cudaError_t batch_launch(lbm_batch *b, const BatchArgs &a, cudaStream_t s) {
+    return b->teams ? step_teams(a, b->blocks, s) : step_batch(a, b->blocks, b->threads, s);
 }
 
 int lbm_batch_step(lbm_batch *b, int64_t n) {
@@ -1460,7 +1564,7 @@ int lbm_batch_step(lbm_batch *b, int64_t n) {
     cudaGraphExec_t ge = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t el = step_batch(a, b->blocks, b->threads, cap);
+        cudaError_t el = batch_launch(b, a, cap);
         e = cudaStreamEndCapture(cap, &g);
         if (e == cudaSuccess && el != cudaSuccess) e = el;
     }
@@ -1483,6 +1587,7 @@ int lbm_batch_probe_series(lbm_batch *b, double *out, int64_t max_samples, int64
     if (!out || have == 0) return LBM_OK;
     const int64_t take = std::min(have, max_samples);
     CK(cudaStreamSynchronize(b->stream), "series sync");
+    if ((rc = batch_team_status(b))) return rc;
     CK(cudaMemcpy2D(out, sizeof(double) * 8 * max_samples, b->d_series, sizeof(double) * 8 * b->max_samples,
                     sizeof(double) * 8 * take, b->count, cudaMemcpyDeviceToHost),
        "series copy");
@@ -1495,7 +1600,7 @@ int lbm_batch_status(lbm_batch *b, int32_t *status) {
     if (!status) return fail(LBM_EINVAL, "null output");
     CK(cudaMemcpyAsync(status, b->d_status, sizeof(int32_t) * b->count, cudaMemcpyDeviceToHost, b->stream), "status copy");
     CK(cudaStreamSynchronize(b->stream), "status sync");
-    return LBM_OK;
+    return batch_team_status(b);
 }
 
 int lbm_batch_moments(lbm_batch *b, void *rho, void *u, int dtype, int on_device) {
@@ -1528,6 +1633,7 @@ int lbm_batch_moments(lbm_batch *b, void *rho, void *u, int dtype, int on_device
             CK(cudaMemcpyAsync(u, du, es * b->total * b->D, cudaMemcpyDeviceToHost, b->stream), "moments copy");
         }
         CK(cudaStreamSynchronize(b->stream), "moments sync");
+        return batch_team_status(b);
     }
     return LBM_OK;
 }
@@ -1553,6 +1659,7 @@ int lbm_batch_get_populations(lbm_batch *b, void *f, int dtype, int on_device) {
     if (!on_device) {
         CK(cudaMemcpyAsync(f, d, bytes, cudaMemcpyDeviceToHost, b->stream), "population copy");
         CK(cudaStreamSynchronize(b->stream), "population sync");
+        return batch_team_status(b);
     }
     return LBM_OK;
 }
@@ -1567,7 +1674,7 @@ int lbm_batch_info(lbm_batch *b, int64_t *total_cells, int64_t *step) {
 int lbm_batch_launch_info(lbm_batch *b, int64_t out[4]) {
     if (!b || !out) return fail(LBM_EINVAL, "null argument");
     out[0] = b->threads;
-    out[1] = b->blocks;
+    out[1] = b->teams ? b->count : b->blocks;  // a team counts once
     out[2] = b->max_load;
     out[3] = b->mean_load;
     return LBM_OK;
@@ -1581,6 +1688,7 @@ int lbm_batch_set_launch_shape(lbm_batch *b, int threads, int64_t blocks) {
         return fail(LBM_EINVAL, "blocks must be in [1, %d] (32 per SM, at most one per instance)", b->block_cap);
     cudaError_t e = batch_assign(b, (int)blocks);
     if (e != cudaSuccess) return batch_sticky(b, cuda_fail("batch assignment", e));
+    b->teams = false;
     b->threads = threads;
     return LBM_OK;
 }
@@ -1614,11 +1722,23 @@ int lbm_batch_autotune(lbm_batch *b, int64_t steps) {
     CK(cudaMemcpyAsync(keep.status, b->d_status, sizeof(int32_t) * b->count, cudaMemcpyDeviceToDevice, b->stream),
        "tuning backup");
     const int saved_threads = b->threads, saved_blocks = b->blocks;
+    const bool saved_teams = b->teams;
     struct Cand {
-        int threads, blocks;
+        int threads, blocks;  // blocks 0: teams
         float ms;
     };
     std::vector<Cand> cands;
+    if (b->team_blocks > 0) cands.push_back({kTeamThreads, 0, -1.f});
+    auto use = [&](int threads, int blocks) -> cudaError_t {
+        if (blocks == 0) {
+            batch_use_teams(b);
+            return cudaSuccess;
+        }
+        const cudaError_t ea = batch_assign(b, blocks);
+        b->teams = false;
+        b->threads = threads;
+        return ea;
+    };
     for (int th : {64, 128, 256})
         for (int r : {1, 2, 3, 4, 6, 8, 12, 16}) {
             const int nb = (int)std::min<int64_t>((int64_t)sm_count() * r, b->block_cap);
@@ -1635,11 +1755,11 @@ int lbm_batch_autotune(lbm_batch *b, int64_t steps) {
     }
     for (int round = 0; round < 2 && e == cudaSuccess; ++round)
         for (Cand &q : cands) {
-            e = batch_assign(b, q.blocks);
+            e = use(q.threads, q.blocks);
             if (e != cudaSuccess) break;
             const BatchArgs a = batch_args(b, steps);
             e = cudaEventRecord(e0, b->stream);
-            if (e == cudaSuccess) e = step_batch(a, q.blocks, q.threads, b->stream);
+            if (e == cudaSuccess) e = batch_launch(b, a, b->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float ms = -1;
@@ -1661,8 +1781,7 @@ int lbm_batch_autotune(lbm_batch *b, int64_t steps) {
     for (const Cand &q : cands)
         if (q.ms > 0 && (!best || q.ms < best->ms)) best = &q;
     if (!best) {
-        e = batch_assign(b, saved_blocks);
-        b->threads = saved_threads;
+        e = use(saved_threads, saved_teams ? 0 : saved_blocks);
         if (e != cudaSuccess) return batch_sticky(b, cuda_fail("batch assignment", e));
         return fail(LBM_ECUDA, "batch tuning found no runnable launch shape");
     }
@@ -1672,9 +1791,8 @@ int lbm_batch_autotune(lbm_batch *b, int64_t steps) {
         if (q.ms > 0 && q.ms <= limit &&
             (q.blocks < pick->blocks || (q.blocks == pick->blocks && q.threads < pick->threads)))
             pick = &q;
-    e = batch_assign(b, pick->blocks);
+    e = use(pick->threads, pick->blocks);
     if (e != cudaSuccess) return batch_sticky(b, cuda_fail("batch assignment", e));
-    b->threads = pick->threads;
     return LBM_OK;
 }
 
@@ -1682,7 +1800,7 @@ int lbm_batch_sync(lbm_batch *b) {
     int rc = batch_check(b);
     if (rc) return rc;
     CK(cudaStreamSynchronize(b->stream), "batch sync");
-    return LBM_OK;
+    return batch_team_status(b);
 }
 
 void lbm_batch_destroy(lbm_batch *b) {
@@ -1699,6 +1817,7 @@ void lbm_batch_destroy(lbm_batch *b) {
     cudaFree(b->d_tw_off);
     cudaFree(b->d_series);
     cudaFree(b->d_status);
+    cudaFree(b->d_team);
     cudaGetLastError();
     delete b;
 }

@@ -17,9 +17,16 @@
 
 namespace lbmd {
 
+// A population, from L2 where other SMs write it during the launch.
+template <bool L2, typename T> __device__ __forceinline__ T ld_pop(const T *p) {
+    if constexpr (L2) return __ldcg(p);
+    else return *p;
+}
+
 // One AA-pattern update of cell (x, y, z) of a lattice stored as Q planes of `plane`
-// elements at A; returns the cell's pre-collision moments.
-template <int D, int P, int EQ, bool BULK>
+// elements at A; returns the cell's pre-collision moments.  L2: the populations are read past
+// the SM's own cache (several steps in one launch, blocks that exchange populations).
+template <int D, int P, int EQ, bool BULK, bool L2 = false>
 __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
     typename Storage<P>::T *__restrict__ A, int64_t plane, int nx, int ny, int nz, int pitch, int x, int y,
     int z, int odd, typename Storage<P>::R rho0, typename Storage<P>::R omega0,
@@ -41,14 +48,14 @@ __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
     R f[Q];
     if (!odd) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) f[i] = St::load(A[(int64_t)i * plane + cell]);
+        for (int i = 0; i < Q; ++i) f[i] = St::load(ld_pop<L2>(A + (int64_t)i * plane + cell));
     } else {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             // f_i(r) = A[opp(i)][r - c_i]
             const int64_t src = xs[1 - cxo(i)] +
                                 (int64_t)pitch * (ys[1 - cyo(i)] + (int64_t)ny * zs[1 - (D == 3 ? czo(i) : 0)]);
-            f[i] = St::load(A[(int64_t)(Q - 1 - i) * plane + src]);
+            f[i] = St::load(ld_pop<L2>(A + (int64_t)(Q - 1 - i) * plane + src));
         }
     }
     const CellMoments<R> m = collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
@@ -106,8 +113,6 @@ __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
 // kernel: 64^2 FP64 8.0 -> 5.3 us (3.3 us of it one warp's 105 FP64 instructions at 64 clocks),
 // 64^2 FP32 3.9 -> 2.1, 32^3 binary16 6.1 -> 2.8, 48^3 6.8 -> 5.7 us.
 
-template <typename T> __device__ __forceinline__ T ld_l2(const T *p) { return __ldcg(p); }
-
 // Wait until every block has arrived `gen` times (counters never wrap: gen * blocks < 2^32).
 __device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned gen, const int32_t *status, int64_t timeout_ns) {
     __shared__ int bad;
@@ -124,6 +129,19 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned gen, const
             ok = wait_count_bounded(&sync[lbmh::kBarStride * (1 + threadIdx.x)], gen * arrive, status, timeout_ns);
         }
         if (__any_sync(0xffffffffu, !ok) && threadIdx.x == 0) bad = 1;
+    }
+    __syncthreads();
+    return bad == 0;
+}
+
+// The same for the blocks of one counter (it grows by the number of blocks a step).
+__device__ __forceinline__ bool team_barrier(unsigned *counter, unsigned want, const int32_t *status, int64_t timeout_ns) {
+    __shared__ int bad;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        red_release(counter, 1u);
+        bad = !wait_count_bounded(counter, want, status, timeout_ns);
     }
     __syncthreads();
     return bad == 0;
@@ -163,11 +181,11 @@ __global__ void __launch_bounds__(256) k_steps_small(const lbmh::StepArgs a, int
             R f[Q];
             if (!odd) {
 #pragma unroll
-                for (int i = 0; i < Q; ++i) f[i] = St::load(ld_l2(A + i * plane + self));
+                for (int i = 0; i < Q; ++i) f[i] = St::load(ld_pop<true>(A + i * plane + self));
             } else {
 #pragma unroll
                 for (int i = 0; i < Q; ++i)  // f_i(r) = A[opp(i)][r - c_i]
-                    f[i] = St::load(ld_l2(A + (Q - 1 - i) * plane + rows[(1 - cyo(i)) + (D == 3 ? 3 * (1 - czo(i)) : 0)] + xs[1 - cxo(i)]));
+                    f[i] = St::load(ld_pop<true>(A + (Q - 1 - i) * plane + rows[(1 - cyo(i)) + (D == 3 ? 3 * (1 - czo(i)) : 0)] + xs[1 - cxo(i)]));
             }
             collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
             if (!odd) {

@@ -113,7 +113,18 @@ struct BatchArgs {
     int D, eq, bulk;
     double rho0;
     int64_t step0, nsteps, every_k;  // first step, steps in this launch, probe period (0 = off)
+    // teams of blocks (k_step_teams): instance and part of each block, blocks of each instance,
+    // probe sums [2][blocks][8], counters (exits, then one per instance, kBarStride apart)
+    const int32_t *team_instance, *team_part, *team_size;
+    double *team_partials;
+    unsigned *team_sync;
+    int32_t *team_status;
+    int64_t timeout_ns;
 };
+constexpr int kTeamThreads = 128;  // threads of a team's block
+// Blocks of the team kernel that are resident at once.
+int team_block_capacity(int D, int eq, int bulk, int sms);
+cudaError_t step_teams(const BatchArgs &a, int blocks, cudaStream_t s);
 cudaError_t step_batch(const BatchArgs &a, int blocks, int threads, cudaStream_t s);
 const void *batch_kernel(int D, int eq, int bulk);
 cudaError_t batch_init(double *arena, const int64_t *cell_start, const int32_t *dims,
