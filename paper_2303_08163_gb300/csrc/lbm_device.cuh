@@ -73,9 +73,9 @@ template <> struct Storage<P_F16S> {
     static __host__ __device__ __forceinline__ T store(R v) { return __float2half_rn(v); }
 };
 
-// Arithmetic helpers: FP64 keeps IEEE sqrt and division (parity path); FP32 uses the
-// hardware reciprocal square root and fast division (a few ulp, far below the
-// storage rounding of the FP32 and binary16 formats).
+// Arithmetic helpers of the field transfers: FP64 takes IEEE square root and division (the
+// collisions have rcp_ulp and sqrt_ulp below); FP32 the hardware reciprocal square root and fast
+// division (a few ulp, far below the storage rounding of the FP32 and binary16 formats).
 __host__ __device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
 __host__ __device__ __forceinline__ float sqrt_r(float x) {
 #ifdef __CUDA_ARCH__
@@ -259,10 +259,11 @@ __host__ __device__ __forceinline__ R equilibrium_h(const R (&u)[3], R (&h)[qof(
     }
 }
 
-// Density and momentum of one cell from shifted populations.  The partial sums follow the
-// tensor structure of the lattice (first over c_z, then c_y, then c_x).
+// Density (its difference from rho0 is returned) and momentum of one cell from shifted
+// populations.  The partial sums follow the tensor structure of the lattice (first over c_z, then
+// c_y, then c_x).
 template <int D, typename R>
-__host__ __device__ __forceinline__ void moment_sums(const R (&f)[qof(D)], R rho0, R &rho, R (&j)[3]) {
+__host__ __device__ __forceinline__ R moment_sums(const R (&f)[qof(D)], R rho0, R &rho, R (&j)[3]) {
     R a[9], bz[9];
     if constexpr (D == 2) {
 #pragma unroll
@@ -285,6 +286,7 @@ __host__ __device__ __forceinline__ void moment_sums(const R (&f)[qof(D)], R rho
         j[2] = ((bz[0] + bz[1]) + (bz[2] + bz[3])) + ((bz[4] + bz[5]) + (bz[6] + bz[7])) + bz[8];
     }
     rho = rho0 + rt;
+    return rt;
 }
 
 // Moments of one cell from shifted populations: rho and u = j / rho.
@@ -301,71 +303,73 @@ __host__ __device__ __forceinline__ CellMoments<R> moments_shifted(const R (&f)[
     return m;
 }
 
-// The FP64 relaxation f* = (1 - 2beta) f + 2beta w_i (drho + rho h_i) of one direction of
-// weight class c: two FMAs per direction, with the per-class products 2beta w rho and
-// 2beta w drho formed once per cell (fewest instructions on the FP64 pipe, the bound).
-template <typename R> struct Relax {
-    R keep, rho, drho, omw[4], wr[4], wd[4];
-    __host__ __device__ __forceinline__ Relax(R om, double w0, double w1, double w2, double w3, R rho_,
-                                              R drho_)
-        : keep(R(1) - om), rho(rho_), drho(drho_) {
-        const double w[4] = {w0, w1, w2, w3};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            omw[c] = om * R(w[c]);
-            wr[c] = omw[c] * rho;
-            wd[c] = omw[c] * drho;
-        }
-    }
-    __host__ __device__ __forceinline__ R operator()(int c, R h, R f) const {
-        return fma_r(wr[c], h, fma_r(keep, f, wd[c]));
-    }
+// The terms of the FP64 tensor-product equilibria (entropic, product).  With t_a(c) = 1 + d_a(c)
+// the factor of axis a, d = prod t_a - 1 and X_a(c) = rho d_a(c), the deviation of a direction's
+// equilibrium over its weight is
+//   g = drho + rho d = (drho + X_x) + t_x X_y (+ t_x t_y X_z),
+// one FMA per direction and axis beyond the first; the relaxation f* = (1 - 2beta) f + 2beta w g is
+// two more.  (FP64 collisions are bound by their instruction count.  Forming rho d from d instead
+// took the products 2beta w rho and 2beta w drho per weight and d itself: 4 instructions more in
+// 2-D, 10 in 3-D, and no X without a product with 1/rho.)
+//
+// Entropic form: with j3 = 3 j, T_a = rho S_a = sqrt(rho^2 + j3_a j_a) and q_a = rho + T_a, the term
+// rho (S_a - 1) is j3_a j_a / q_a (no cancellation: an ulp of T stays an ulp), and one reciprocal of
+// rho prod q_a gives 1/rho and every 1/q_a.  Errors against 64-bit references are those of the
+// direct forms with IEEE division and square root (2-D and 3-D, all options).
+// 4096-lattice sweep: 5.20 -> 4.79 ms a step with the own reciprocal and square root, 4.53 with
+// these terms; D3Q27 128^3 882 -> 842 -> 820 us.
+template <typename R> struct TensorTerms {
+    R drho, irho, X[3][3], key[3];  // X by axis and c + 1; key: what the bulk coefficient depends on
 };
 
-// FP64 entropic collisions: the moments and the per-axis factors with one IEEE division.
-// With T_a = rho S_a = sqrt(rho^2 + 3 j_a^2) and q_a = rho + T_a = rho (1 + S_a), the
-// identities 1/rho = (prod_a q_a) / (rho prod_a q_a) and S_a - 1 = 3 u_a^2 / (1 + S_a) =
-// 3 j_a^2 / (rho q_a) let one reciprocal of rho prod_a q_a serve 1/rho and every axis
-// (exact rewrites, a few ulp apart from the separate divisions).  S - 1 is formed without
-// cancellation, so an ulp of T stays an ulp: the errors against 64-bit references are those of
-// the IEEE operations (2-D and 3-D, all options).  4096-lattice sweep: 5.20 -> 4.79 ms a step.
-template <int D, typename R>
-__device__ __forceinline__ void entropic_factors_one_division(
-    const R (&f)[qof(D)], R rho0, CellMoments<R> &m, R (&dm)[3], R (&d0)[3], R (&dp)[3], R (&key)[3]) {
-    R j[3];
-    moment_sums<D, R>(f, rho0, m.rho, j);
-    const R rho = m.rho, rho2 = rho * rho;
-    R j3[3], T[3], q[3], cof[3];
+template <int D, int EQ, typename R>
+__device__ __forceinline__ void tensor_terms(const R (&f)[qof(D)], R rho0, CellMoments<R> &m, TensorTerms<R> &t) {
+    R j[3], j3[3];
+    t.drho = moment_sums<D, R>(f, rho0, m.rho, j);
+    const R rho = m.rho;
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        j3[a] = R(3) * j[a];
-        T[a] = sqrt_ulp(fma_r(j3[a], j[a], rho2));
-        q[a] = rho + T[a];
-    }
-    R qprod;
-    if constexpr (D == 2) {
-        cof[0] = q[1];
-        cof[1] = q[0];
-        qprod = q[0] * q[1];
+    for (int a = 0; a < D; ++a) j3[a] = R(3) * j[a];
+    if constexpr (EQ == EQ_ENT) {
+        const R rho2 = rho * rho;
+        R jj[3], T[3], q[3], others[3], all;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            jj[a] = j3[a] * j[a];
+            T[a] = sqrt_ulp(rho2 + jj[a]);
+            q[a] = rho + T[a];
+        }
+        if constexpr (D == 2) {
+            others[0] = q[1];
+            others[1] = q[0];
+        } else {
+            others[0] = q[1] * q[2];
+            others[1] = q[0] * q[2];
+            others[2] = q[0] * q[1];
+        }
+        all = q[0] * others[0];
+        const R r = rcp_ulp(rho * all), v = r * rho;  // v = 1 / prod q
+        t.irho = r * all;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const R e = jj[a] * (v * others[a]);  // rho (S - 1)
+            t.X[a][0] = fma_r(R(2), e, -j3[a]);
+            t.X[a][1] = -e;
+            t.X[a][2] = fma_r(R(2), e, j3[a]);
+            t.key[a] = T[a] * t.irho;
+        }
     } else {
-        cof[0] = q[1] * q[2];
-        cof[1] = q[0] * q[2];
-        cof[2] = q[0] * q[1];
-        qprod = q[0] * cof[0];
-    }
-    const R r = rcp_ulp(rho * qprod);
-    const R irho = r * qprod;
-    m.u[2] = R(0);
+        t.irho = rcp_ulp(rho);
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        m.u[a] = j[a] * irho;
-        const R sm1 = (j3[a] * j[a]) * (r * cof[a]);  // S - 1 without cancellation
-        const R u3 = j3[a] * irho;
-        d0[a] = -sm1;
-        dp[a] = fma_r(R(2), sm1, u3);
-        dm[a] = fma_r(R(2), sm1, -u3);
-        key[a] = T[a] * irho;
+        for (int a = 0; a < D; ++a) {
+            const R u = j[a] * t.irho;
+            t.X[a][0] = fma_r(j3[a], u, -j3[a]);
+            t.X[a][1] = R(-0.5) * (j3[a] * u);
+            t.X[a][2] = fma_r(j3[a], u, j3[a]);
+            t.key[a] = u * u;
+        }
     }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m.u[a] = a < D ? j[a] * t.irho : R(0);
 }
 
 // ------------------------------------------------------------------ FP32 collisions
@@ -625,25 +629,27 @@ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omeg
         for (int a = 0; a < 3; ++a) m.u[a] = v.u[a];
         return m;
     } else {
-    R dm[3], d0[3], dp[3], key[3];  // per-axis factors (entropic and product forms)
-    if constexpr (EQ == EQ_ENT && sizeof(R) == 8) {
-        entropic_factors_one_division<D, R>(f, rho0, m, dm, d0, dp, key);
-    } else {
+    // 2beta w by weight class and 1 - 2beta
+    const auto relaxation = [&](R om, R (&omw)[4]) {
+        const double w[4] = {kW0, kW1, kW2, kW3};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) omw[c] = om * R(w[c]);
+        return R(1) - om;
+    };
+    R omw[4];
+    if constexpr (EQ == EQ_POLY2) {
         R j[3];
-        moment_sums<D, R>(f, rho0, m.rho, j);
+        const R drho = moment_sums<D, R>(f, rho0, m.rho, j);
         const R inv = rcp_ulp(m.rho);
         for (int a = 0; a < 3; ++a) m.u[a] = j[a] * inv;
-        if constexpr (EQ != EQ_POLY2) all_axis_factors<D, EQ>(m.u, dm, d0, dp, key);
-    }
-    const R drho = m.rho - rho0;
-    if constexpr (EQ == EQ_POLY2) {
         R uu = m.u[0] * m.u[0] + m.u[1] * m.u[1];
         if constexpr (D == 3) uu = fma_r(m.u[2], m.u[2], uu);
         R k = fmax(m.u[0] * m.u[0], m.u[1] * m.u[1]);
         if constexpr (D == 3) k = fmax(k, m.u[2] * m.u[2]);
         const R om = collision_rate<EQ, BULK, R>(k, omega0, six_nu);
-        const R mh = R(-1.5) * uu;
-        const Relax<R> relax(om, kW0, kW1, kW2, kW3, m.rho, drho);
+        const R keep = relaxation(om, omw);
+        // drho + rho h with h = 3 u.c + 9/2 (u.c)^2 - 3/2 u^2
+        const R base = fma_r(R(-1.5) * m.rho, uu, drho), r3 = R(3) * m.rho, r45 = R(4.5) * m.rho;
         const R upm = m.u[0] + m.u[1], umm = m.u[0] - m.u[1];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
@@ -656,37 +662,34 @@ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omeg
             else cu = cx > 0 ? umm : -umm;
             if (cz == 1) cu = cu + m.u[2];
             if (cz == -1) cu = cu - m.u[2];
-            const R h = fma_r(cu, fma_r(R(4.5), cu, R(3)), mh);
-            f[i] = relax(wclass<D>(i), h, f[i]);
+            const R g = i == Q / 2 ? base : fma_r(cu, fma_r(r45, cu, r3), base);
+            f[i] = fma_r(omw[wclass<D>(i)], g, keep * f[i]);
         }
     } else {
-        R kmax = fmax(key[0], key[1]);
-        if constexpr (D == 3) kmax = fmax(kmax, key[2]);
+        TensorTerms<R> t;
+        tensor_terms<D, EQ, R>(f, rho0, m, t);
+        R kmax = fmax(t.key[0], t.key[1]);
+        if constexpr (D == 3) kmax = fmax(kmax, t.key[2]);
         const R om = collision_rate<EQ, BULK, R>(kmax, omega0, six_nu);
-        const Relax<R> relax(om, kW0, kW1, kW2, kW3, m.rho, drho);
-        const R dx[3] = {dm[0], d0[0], dp[0]};
-        const R dy[3] = {dm[1], d0[1], dp[1]};
-        const R tx[3] = {R(1) + dm[0], R(1) + d0[0], R(1) + dp[0]};
-        if constexpr (D == 2) {
+        const R keep = relaxation(om, omw);
+        R ex[3], tx[3], ty[3];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const R h = fma_r(dy[cyo(i) + 1], tx[cxo(i) + 1], dx[cxo(i) + 1]);
-                f[i] = relax(wclass<D>(i), h, f[i]);
-            }
-        } else {
-            const R ty[3] = {R(1) + dm[1], R(1) + d0[1], R(1) + dp[1]};
-            const R dz[3] = {dm[2], d0[2], dp[2]};
+        for (int c = 0; c < 3; ++c) {
+            ex[c] = t.drho + t.X[0][c];
+            tx[c] = fma_r(t.X[0][c], t.irho, R(1));
+            if constexpr (D == 3) ty[c] = fma_r(t.X[1][c], t.irho, R(1));
+        }
 #pragma unroll
-            for (int p = 0; p < 9; ++p) {
-                // h = prod (1 + d) - 1 over x, y, z = e_xy + d_z (1 + e_xy)
-                const R exy = fma_r(dy[cyo(p) + 1], tx[cxo(p) + 1], dx[cxo(p) + 1]);
-                const R txy = tx[cxo(p) + 1] * ty[cyo(p) + 1];
+        for (int p = 0; p < 9; ++p) {
+            const int x = cxo(p) + 1, y = cyo(p) + 1;
+            const R exy = fma_r(tx[x], t.X[1][y], ex[x]);
+            if constexpr (D == 2) {
+                f[p] = fma_r(omw[wclass<D>(p)], exy, keep * f[p]);
+            } else {
+                const R txy = tx[x] * ty[y];
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    const int i = p + 9 * q;
-                    const R h = fma_r(dz[q], txy, exy);
-                    f[i] = relax(wclass<D>(i), h, f[i]);
-                }
+                for (int q = 0; q < 3; ++q)
+                    f[p + 9 * q] = fma_r(omw[wclass<D>(p + 9 * q)], fma_r(txy, t.X[2][q], exy), keep * f[p + 9 * q]);
             }
         }
     }
