@@ -89,7 +89,7 @@ struct lbm_ctx {
     int kernel = 1;
     int gen_threads = 256, gen_blocks = 1;
     bool chosen = false;  // the caller named a kernel or a launch shape
-    int small_threads = 0, small_blocks = 0;  // several steps of a small lattice at once (0: too large)
+    SmallShape small;  // several steps of a small lattice at once (0 threads: too large)
     TmaShape tma{};
     bool use_graph = false;
     cudaGraphExec_t graph2 = nullptr;  // even + odd step
@@ -198,12 +198,12 @@ cudaError_t launch_one(lbm_ctx *c, int odd, int diag, cudaStream_t s) {
 // n steps without diagnostics from the layout `odd` describes: several to a launch with the
 // TMA kernel, one each with the one-cell kernel.
 cudaError_t launch_steps(lbm_ctx *c, int odd, int64_t n, cudaStream_t s) {
-    if (n > 1 && !c->chosen && c->small_threads > 0) {
+    if (n > 1 && !c->chosen && c->small.threads > 0) {
         // (launches of bounded length: FP64 steps of 5 us)
         cudaError_t e = cudaSuccess;
         while (n > 0 && e == cudaSuccess) {
             const int64_t m = std::min<int64_t>(n, 10000);
-            e = steps_small(step_args(c, odd, 0), (int)m, c->small_blocks, c->small_threads, s);
+            e = steps_small(step_args(c, odd, 0), (int)m, c->small, s);
             odd ^= (int)(m & 1);
             n -= m;
         }
@@ -720,7 +720,7 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
     c->gen_threads = 256;
     c->gen_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((ncell + 255) / 256, (int64_t)sm_count() * 16));
     c->kernel = 1;
-    if (!small_shape(c->lat, c->eq, c->bulk, sm_count(), &c->small_threads, &c->small_blocks)) c->small_threads = 0;
+    if (!small_shape(c->lat, c->eq, c->bulk, sm_count(), c->small)) c->small.threads = 0;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         static bool loaded = false;

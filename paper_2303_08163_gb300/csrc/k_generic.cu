@@ -10,8 +10,8 @@
 namespace lbmh {
 cudaError_t step_generic_d2(const StepArgs &a, int blocks, int threads, cudaStream_t s);
 cudaError_t step_generic_d3(const StepArgs &a, int blocks, int threads, cudaStream_t s);
-const void *small_kernel_d2(int P, int eq, int bulk);
-const void *small_kernel_d3(int P, int eq, int bulk);
+const void *small_kernel_d2(int P, int eq, int bulk, bool lanes);
+const void *small_kernel_d3(int P, int eq, int bulk, bool lanes);
 }  // namespace lbmh
 
 namespace lbmd {
@@ -328,30 +328,39 @@ cudaError_t step_generic(const StepArgs &a, int blocks, int threads, cudaStream_
     return a.lat.D == 2 ? step_generic_d2(a, blocks, threads, s) : step_generic_d3(a, blocks, threads, s);
 }
 
+static const void *small_kernel(const Lattice &lat, int eq, int bulk, bool lanes) {
+    return lat.D == 2 ? small_kernel_d2(lat.P, eq, bulk, lanes) : small_kernel_d3(lat.P, eq, bulk, lanes);
+}
+
 // Up to 800 cells an SM (48^3: 727) the grid-barrier kernel is the faster one; with more a thread
 // has several cells, whose loads follow one another, and the TMA row kernel's copies overlap
 // (509 x 381 FP32, 1276 cells an SM: 6.8 us a step against 5.3; 64^3 binary16 9.1 against 7.7).
-bool small_shape(const Lattice &lat, int eq, int bulk, int sms, int *threads, int *blocks) {
+// FP64 lattices of at most 40 cells an SM have a cell on three lanes: a warp on each quarter is all
+// there is either way, and a warp instruction costs the same for 7 cells as for 10 of three lanes
+// (with 41 to 80 an SM quarter would have two such warps, as long as one of 32 cells).
+bool small_shape(const Lattice &lat, int eq, int bulk, int sms, SmallShape &t) {
     if (lat.ncell > (int64_t)800 * sms || lat.plane * qof(lat.D) >= ((int64_t)1 << 31)) return false;
-    const void *fn = lat.D == 2 ? small_kernel_d2(lat.P, eq, bulk) : small_kernel_d3(lat.P, eq, bulk);
     const int64_t per = (lat.ncell + sms - 1) / sms;  // cells an SM
-    const int t = (int)std::min<int64_t>(256, (per + 31) / 32 * 32);
+    t.lanes = lat.P == P_F64 && per <= 40;
+    const int warp = t.lanes ? 10 : 32;  // cells a warp
+    const int64_t warps = std::min<int64_t>(8, (per + warp - 1) / warp);
+    t.threads = (int)(32 * warps);
+    const void *fn = small_kernel(lat, eq, bulk, t.lanes);
     int nb = 0;
-    if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, t, 0) != cudaSuccess || nb < 1) {
+    if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, t.threads, 0) != cudaSuccess || nb < 1) {
         cudaGetLastError();
         return false;
     }
-    *threads = t;
-    *blocks = (int)std::min<int64_t>((lat.ncell + t - 1) / t, (int64_t)nb * sms);
+    t.blocks = (int)std::min<int64_t>((lat.ncell + warps * warp - 1) / (warps * warp), (int64_t)nb * sms);
     return true;
 }
 
-cudaError_t steps_small(const StepArgs &a, int nsteps, int blocks, int threads, cudaStream_t s) {
-    const void *fn = a.lat.D == 2 ? small_kernel_d2(a.lat.P, a.eq, a.bulk) : small_kernel_d3(a.lat.P, a.eq, a.bulk);
+cudaError_t steps_small(const StepArgs &a, int nsteps, const SmallShape &t, cudaStream_t s) {
+    const void *fn = small_kernel(a.lat, a.eq, a.bulk, t.lanes);
     if (!fn) return cudaErrorInvalidValue;
     StepArgs aa = a;
     void *args[] = {(void *)&aa, (void *)&nsteps};
-    return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(threads), args, 0, s);
+    return cudaLaunchCooperativeKernel(fn, dim3(t.blocks), dim3(t.threads), args, 0, s);
 }
 
 #define LBM_DISPATCH_DP(D_, P_, CALL)                                                      \

@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
 // populations from L2, the collision, the stores and one barrier of the whole grid (cooperative
 // launch: all blocks are resident).  The barrier's arrivals are spread over kBarCounters counters,
 // each on its own line; a block's first warp looks at all of them.  Per step against the TMA row
-// kernel: 64^2 FP64 8.0 -> 5.3 us (3.3 us of it one warp's 105 FP64 instructions at 64 clocks),
+// kernel: 90^2 FP64 8.2 -> 4.6 us (2.6 us of it one warp's 82 FP64 instructions at 64 clocks),
 // 64^2 FP32 3.9 -> 2.1, 32^3 binary16 6.1 -> 2.8, 48^3 6.8 -> 5.7 us.
 
 // Wait until every block has arrived `gen` times (counters never wrap: gen * blocks < 2^32).
@@ -145,6 +145,20 @@ __device__ __forceinline__ bool team_barrier(unsigned *counter, unsigned want, c
     }
     __syncthreads();
     return bad == 0;
+}
+
+// The end of a several-step launch: reports a wait that ran out; the last block to finish clears
+// the counters for the next launch.
+__device__ __forceinline__ void steps_finish(const lbmh::StepArgs &a, bool ok) {
+    if (!ok && threadIdx.x == 0) report_status(a.status, -5); /* LBM_ETIMEOUT */
+    __syncthreads();
+    bool last = false;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&a.sync[1], 1u) == gridDim.x - 1;
+    }
+    if (__syncthreads_or(last))
+        for (int p = threadIdx.x; p < lbmh::kBarStride * (1 + lbmh::kBarCounters); p += blockDim.x) a.sync[p] = 0;
 }
 
 template <int D, int P, int EQ, bool BULK>
@@ -199,16 +213,81 @@ __global__ void __launch_bounds__(256) k_steps_small(const lbmh::StepArgs a, int
         }
         if (s + 1 < nsteps) ok = grid_barrier(a.sync, (unsigned)(s + 1), a.status, a.timeout_ns);
     }
-    if (!ok && threadIdx.x == 0) report_status(a.status, -5); /* LBM_ETIMEOUT */
-    // the last block to finish clears the counters for the next launch
-    __syncthreads();
-    bool last = false;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(&a.sync[1], 1u) == gridDim.x - 1;
+    steps_finish(a, ok);
+}
+
+// A cell on three lanes of a warp (collide_lanes), ten cells to a warp: the lane's share of the
+// loads and stores.  Lane c of a group has the directions i = p + F c.
+template <int D> struct LaneCell {
+    static constexpr int Q = qof(D), F = lane_pops(D), N = D == 3 ? 3 : 1;
+    int c, base, x, y, z, plane, self, xs[3];
+    int ahead[N], behind[N];  // rows of r + c e_last + dy and of their mirror images, by dy + 1 (3-D)
+    bool run;                 // the group has a cell of its own
+    // first: the first cell of the block (cells first .. ncell are the block's and its successors')
+    __device__ __forceinline__ LaneCell(int first, int ncell, int nx, int ny, int nz, int pitch, int plane_, int32_t *status)
+        : plane(plane_) {
+        const int lane = threadIdx.x & 31, cell = first + (int)(threadIdx.x >> 5) * 10 + lane / 3;
+        c = lane % 3;
+        base = lane < 30 ? lane - c : 27;  // (lanes 30 and 31 only take part in the shuffles)
+        run = lane < 30 && cell < ncell;
+        cell_coords(run ? cell : 0, ncell, nx, ny, x, y, z);
+        self = x + pitch * (y + ny * z);
+        xs[0] = wrapi(x - 1, nx);
+        xs[1] = x;
+        xs[2] = wrapi(x + 1, nx);
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            const int dy = D == 3 ? q - 1 : c - 1, dz = D == 3 ? c - 1 : 0;
+            ahead[q] = pitch * (wrapi(y + dy, ny) + (D == 3 ? ny * wrapi(z + dz, nz) : 0));
+            behind[q] = pitch * (wrapi(y - dy, ny) + (D == 3 ? ny * wrapi(z - dz, nz) : 0));
+        }
+        run = run && LBM_CHECK(self >= 0 && self < plane, status);
     }
-    if (__syncthreads_or(last))
-        for (int p = threadIdx.x; p < lbmh::kBarStride * (1 + lbmh::kBarCounters); p += blockDim.x) a.sync[p] = 0;
+    __device__ __forceinline__ void load(const double *A, int odd, double (&f)[F]) const {
+#pragma unroll
+        for (int p = 0; p < F; ++p) {
+            f[p] = 0.0;  // f_i(r) = A[opp(i)][r - c_i] on odd steps
+            if (run && odd) f[p] = ld_pop<true>(A + (Q - 1 - p - F * c) * plane + behind[D == 3 ? p / 3 : 0] + xs[1 - cxo(p)]);
+            if (run && !odd) f[p] = ld_pop<true>(A + (p + F * c) * plane + self);
+        }
+    }
+    __device__ __forceinline__ void store(double *A, int odd, const double (&f)[F]) const {
+#pragma unroll
+        for (int p = 0; p < F; ++p) {
+            if (run && odd) A[(p + F * c) * plane + ahead[D == 3 ? p / 3 : 0] + xs[1 + cxo(p)]] = f[p];
+            if (run && !odd) A[(Q - 1 - p - F * c) * plane + self] = f[p];
+        }
+    }
+};
+
+// Several steps of an FP64 lattice of at most 40 cells an SM: a warp of ten cells to each quarter,
+// one cell to a group of lanes.  Entropic with bulk correction, a cell per thread against three
+// lanes: 64^2 5.1 -> 4.0 us a step, 80 x 76 5.1 -> 4.2, 16^3 9.4 -> 6.0, 20 x 16 x 19 9.5 -> 6.4.
+template <int D, int EQ, bool BULK>
+__global__ void __launch_bounds__(128) k_steps_lanes(const lbmh::StepArgs a, int nsteps) {
+    double *A = static_cast<double *>(a.lat.A);
+    const LaneCell<D> cell((int)(blockIdx.x * (blockDim.x / 32) * 10), (int)a.lat.ncell, a.lat.nx, a.lat.ny, a.lat.nz,
+                           a.lat.pitch, (int)a.lat.plane, a.status);  // Q * plane < 2^31 (checked on the host)
+    bool ok = true;
+    for (int s = 0; s < nsteps && ok; ++s) {
+        const int odd = (a.odd + s) & 1;
+        double f[LaneCell<D>::F];
+        cell.load(A, odd, f);
+        collide_lanes<D, EQ, BULK>(f, cell.c, cell.base, a.rho0, a.omega0, a.six_nu);
+        cell.store(A, odd, f);
+        if (s + 1 < nsteps) ok = grid_barrier(a.sync, (unsigned)(s + 1), a.status, a.timeout_ns);
+    }
+    steps_finish(a, ok);
+}
+
+template <int D> const void *lanes_kernel_d(int eq, int bulk) {
+#define LBM_LANES(EQv) \
+    if (eq == EQv) return bulk ? (const void *)k_steps_lanes<D, EQv, true> : (const void *)k_steps_lanes<D, EQv, false>;
+    LBM_LANES(EQ_ENT)
+    LBM_LANES(EQ_POLY2)
+    LBM_LANES(EQ_PROD)
+#undef LBM_LANES
+    return nullptr;
 }
 
 template <int D, int P> const void *small_kernel_dp(int eq, int bulk) {

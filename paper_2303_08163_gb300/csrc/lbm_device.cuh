@@ -697,4 +697,131 @@ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omeg
     }
 }
 
+// ------------------------------------------------------------------ one FP64 cell on three lanes
+//
+// An FP64 warp instruction takes an SM quarter 64 clocks however many lanes it has: where there
+// are fewer cells than lanes, the lanes of a warp that are left over cost nothing.  Here a cell is
+// spread over three neighbouring lanes, lane c of the group holding the populations with
+// c_last = c - 1 (c_y in 2-D, c_z in 3-D), f[p] = f_{p + F c}, F = 3 or 9.  A lane sums its own
+// populations, forms the terms of one axis and relaxes its own populations; partial sums and terms
+// go between the lanes by shuffles.  Every lane adds the partial sums in the same order, so the
+// three hold the same bits of rho, u and 2beta.  About 45 FP64 instructions in place of 82 in 2-D,
+// 100 of 195 in 3-D (entropic).  All 32 lanes call it; `base` is the first lane of the caller's group.
+__host__ __device__ constexpr int lane_pops(int D) { return D == 2 ? 3 : 9; }
+
+template <typename R> __device__ __forceinline__ R from_lane(R v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+
+template <int D, int EQ, bool BULK>
+__device__ __forceinline__ CellMoments<double> collide_lanes(double (&f)[lane_pops(D)], int c, int base, double rho0,
+                                                             double omega0, double six_nu) {
+    using R = double;
+    constexpr int F = lane_pops(D);
+    CellMoments<R> m;
+    R j[3] = {0, 0, 0}, sum, part[2] = {0, 0};  // sums over the lane's populations: all, c_x f, c_y f (3-D)
+    if constexpr (D == 2) {
+        sum = (f[0] + f[1]) + f[2];
+        part[0] = f[2] - f[0];
+    } else {
+        const R c0 = (f[0] + f[3]) + f[6], c1 = (f[1] + f[4]) + f[7], c2 = (f[2] + f[5]) + f[8];
+        sum = (c0 + c1) + c2;
+        part[0] = c2 - c0;
+        part[1] = ((f[6] + f[7]) + f[8]) - ((f[0] + f[1]) + f[2]);
+    }
+    const R s0 = from_lane(sum, base), s1 = from_lane(sum, base + 1), s2 = from_lane(sum, base + 2);
+    const R drho = (s0 + s1) + s2;
+    m.rho = rho0 + drho;
+    j[D - 1] = s2 - s0;
+#pragma unroll
+    for (int a = 0; a < D - 1; ++a) j[a] = (from_lane(part[a], base) + from_lane(part[a], base + 1)) + from_lane(part[a], base + 2);
+    const R rho = m.rho;
+    R om, base_g = 0, irho = 0, ex[3], tx[3], Y[3], Z = 0, r3 = 0, r45 = 0;
+    if constexpr (EQ == EQ_POLY2) {
+        irho = rcp_ulp(rho);
+        for (int a = 0; a < 3; ++a) m.u[a] = j[a] * irho;
+        R uu = m.u[0] * m.u[0] + m.u[1] * m.u[1], k = fmax(m.u[0] * m.u[0], m.u[1] * m.u[1]);
+        if constexpr (D == 3) {
+            uu = fma(m.u[2], m.u[2], uu);
+            k = fmax(k, m.u[2] * m.u[2]);
+        }
+        om = collision_rate<EQ, BULK, R>(k, omega0, six_nu);
+        base_g = fma(-1.5 * rho, uu, drho);
+        r3 = 3.0 * rho;
+        r45 = 4.5 * rho;
+    } else {
+        // the terms of one axis per lane: lane c forms axis min(c, D - 1)
+        const R ja = c == 0 ? j[0] : (D == 2 || c == 1 ? j[1] : j[2]);
+        const R j3 = 3.0 * ja;
+        R X[3], key;
+        if constexpr (EQ == EQ_ENT) {
+            const R jj = j3 * ja, T = sqrt_ulp(fma(rho, rho, jj)), q = rho + T;
+            const R q0 = from_lane(q, base), q1 = from_lane(q, base + 1);
+            R others, all;
+            if constexpr (D == 2) {
+                others = c == 0 ? q1 : q0;
+                all = q0 * q1;
+            } else {
+                const R q2 = from_lane(q, base + 2);
+                others = (c == 0 ? q1 : q0) * (c == 2 ? q1 : q2);
+                all = q0 * (q1 * q2);
+            }
+            const R r = rcp_ulp(rho * all), v = r * rho;
+            irho = r * all;
+            const R e = jj * (v * others);  // rho (S - 1)
+            X[0] = fma(2.0, e, -j3);
+            X[1] = -e;
+            X[2] = fma(2.0, e, j3);
+            key = T * irho;
+        } else {
+            irho = rcp_ulp(rho);
+            const R u = ja * irho;
+            X[0] = fma(j3, u, -j3);
+            X[1] = -0.5 * (j3 * u);
+            X[2] = fma(j3, u, j3);
+            key = u * u;
+        }
+        for (int a = 0; a < 3; ++a) m.u[a] = a < D ? j[a] * irho : 0.0;
+        R kmax = 0;
+        if constexpr (BULK) {
+            kmax = fmax(from_lane(key, base), from_lane(key, base + 1));
+            if constexpr (D == 3) kmax = fmax(kmax, from_lane(key, base + 2));
+        }
+        om = collision_rate<EQ, BULK, R>(kmax, omega0, six_nu);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const R Xx = from_lane(X[i], base);
+            Y[i] = from_lane(X[i], base + 1);
+            ex[i] = drho + Xx;
+            tx[i] = fma(Xx, irho, 1.0);
+        }
+        if constexpr (D == 3) {
+            const R z0 = from_lane(X[0], base + 2), z1 = from_lane(X[1], base + 2), z2 = from_lane(X[2], base + 2);
+            Z = c == 0 ? z0 : (c == 1 ? z1 : z2);
+        }
+    }
+    // 2beta w by the number of nonzero components but the last
+    const R keep = 1.0 - om;
+    R omw[D];
+#pragma unroll
+    for (int n = 0; n < D; ++n) omw[n] = om * (c == 1 ? wclass_weight<D>(n) : wclass_weight<D>(n + 1));
+#pragma unroll
+    for (int p = 0; p < F; ++p) {
+        const int cx = cxo(p), cy = D == 3 ? cyo(p) : 0;  // the direction's components but the last
+        R g;
+        if constexpr (EQ == EQ_POLY2) {
+            R cu = cx == 0 ? 0.0 : (cx > 0 ? m.u[0] : -m.u[0]);
+            if (D == 3 && cy != 0) cu = cy > 0 ? cu + m.u[1] : cu - m.u[1];
+            cu = c == 1 ? cu : (c == 2 ? cu + m.u[D - 1] : cu - m.u[D - 1]);
+            g = fma(cu, fma(r45, cu, r3), base_g);
+        } else if constexpr (D == 2) {
+            const R Yc = c == 0 ? Y[0] : (c == 1 ? Y[1] : Y[2]);
+            g = fma(tx[cx + 1], Yc, ex[cx + 1]);
+        } else {
+            const R exy = fma(tx[cx + 1], Y[cy + 1], ex[cx + 1]), txy = tx[cx + 1] * fma(Y[cy + 1], irho, 1.0);
+            g = fma(txy, Z, exy);
+        }
+        f[p] = fma(omw[(cx != 0) + (cy != 0)], g, keep * f[p]);
+    }
+    return m;
+}
+
 }  // namespace lbmd

@@ -56,10 +56,14 @@ int set_last_error(int code, const char *msg);
 
 // k_generic.cu
 cudaError_t step_generic(const StepArgs &a, int blocks, int threads, cudaStream_t s);
-// Several steps of a small lattice in one cooperative launch.  small_shape: threads and blocks of
-// the launch, false if the lattice is too large for it.
-bool small_shape(const Lattice &lat, int eq, int bulk, int sms, int *threads, int *blocks);
-cudaError_t steps_small(const StepArgs &a, int nsteps, int blocks, int threads, cudaStream_t s);
+// Several steps of a small lattice in one cooperative launch.  small_shape: the launch, false if
+// the lattice is too large for it.
+struct SmallShape {
+    int threads = 0, blocks = 0;
+    bool lanes = false;  // an FP64 cell on three lanes (k_steps_lanes)
+};
+bool small_shape(const Lattice &lat, int eq, int bulk, int sms, SmallShape &t);
+cudaError_t steps_small(const StepArgs &a, int nsteps, const SmallShape &t, cudaStream_t s);
 cudaError_t init_fields(const Lattice &lat, int eq, double rho0, const void *rho, const void *u,
                         int dtype, cudaStream_t s);
 cudaError_t moments(const Lattice &lat, double rho0, int odd, void *rho, void *u, int dtype,
