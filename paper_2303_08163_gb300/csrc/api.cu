@@ -119,6 +119,7 @@ struct lbm_batch {
     int block_cap = 0;  // capacity of d_block_start (blocks + 1 entries at most)
     // teams of blocks (k_step_teams) instead of whole instances per block
     bool teams = false;
+    int team_cluster = 0;             // blocks of a cluster (k_step_clusters), 0: teams over L2
     int team_blocks = 0;
     int64_t team_max = 0;             // largest number of cells of a block
     char *d_team = nullptr;           // one allocation for the team's tables, sums, counters and status
@@ -1281,6 +1282,10 @@ static cudaError_t batch_assign(lbm_batch *b, int nb) {
 // of cells a block for which all blocks are resident: 608 blocks of 128 threads for D2Q9, so every
 // SM's FP64 pipe has several warps.  30 lattices of
 // 16^2 .. 96^2: 185 -> 17 us a step, 60 of 16^2 .. 256^2: 1225 -> 100 us.
+// Small instances that have an SM to every block take clusters of three-lane cells, whatever the
+// shares: 36 lines of 128 cells 4.1 -> 2.4 us a step, 76 of 64 3.7 -> 2.5.  With more blocks than
+// SMs nothing is left of it: 38 lines of 128 cells, whose clusters no longer all find a place of
+// their own, 4.1 -> 3.8 us.
 static cudaError_t batch_plan_teams(lbm_batch *b) {
     b->team_blocks = 0;
     b->team_max = 0;
@@ -1288,6 +1293,14 @@ static cudaError_t batch_plan_teams(lbm_batch *b) {
     int64_t largest = 0;
     for (int64_t k = 0; k < b->count; ++k) largest = std::max(largest, cs[k + 1] - cs[k]);
     const int sms = sm_count();
+    const int64_t cluster = (largest + kClusterCells - 1) / kClusterCells;
+    if (cluster <= kClusterBlocks && b->count * cluster <= sms &&
+        batch_cluster_capacity(b->D, b->eq, b->bulk, (int)cluster) >= b->count) {
+        b->team_cluster = (int)cluster;
+        b->team_blocks = (int)(b->count * cluster);
+        b->team_max = std::min<int64_t>(largest, kClusterCells);
+        return cudaSuccess;
+    }
     if (largest * sms * 10 <= b->total * 11 || largest * b->Q >= ((int64_t)1 << 31)) return cudaSuccess;
     const int cap = team_block_capacity(b->D, b->eq, b->bulk, sms);
     if (b->count > cap) return cudaSuccess;
@@ -1350,7 +1363,7 @@ static void batch_use_teams(lbm_batch *b) {
 
 // LBM_ETIMEOUT if a team's bounded wait ran out (the stream is idle).
 static int batch_team_status(lbm_batch *b) {
-    if (!b->teams) return LBM_OK;
+    if (!b->teams || b->team_cluster > 0) return LBM_OK;  // (a cluster's barrier is the hardware's)
     int32_t st = 0;
     CK(cudaMemcpy(&st, b->team_status, sizeof st, cudaMemcpyDeviceToHost), "status read");
     if (st != 0) return batch_sticky(b, fail(LBM_ETIMEOUT, "a bounded device wait ran out (status %d)", st));
@@ -1538,6 +1551,7 @@ static BatchArgs batch_args(lbm_batch *b, int64_t n) {
     a.team_partials = b->team_partials;
     a.team_sync = b->team_sync;
     a.team_status = b->team_status;
+    a.team_cluster = b->team_cluster;
     a.timeout_ns = wait_timeout_ns();
     return a;
 }

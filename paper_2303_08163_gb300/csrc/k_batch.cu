@@ -11,7 +11,8 @@
 // sample per instance; a non-finite mass marks the instance's status with t + 1.
 //
 // A batch whose largest instance alone would keep one SM busy longer than its share (few
-// instances, or uneven ones) is advanced by teams of blocks instead, see k_step_teams.
+// instances, or uneven ones) is advanced by teams of blocks instead, see k_step_teams, and one of a
+// few short instances by clusters, see k_step_clusters.
 #include <algorithm>
 
 #include "k_generic_step.cuh"
@@ -199,6 +200,146 @@ __global__ void __launch_bounds__(lbmh::kTeamThreads) k_step_teams(const lbmh::B
         for (int64_t p = threadIdx.x; p <= a.count; p += blockDim.x) a.team_sync[lbmh::kBarStride * p] = 0;
 }
 
+// Sums over the ten groups of three lanes of a warp: lanes 0 to 2 return the sums of the values of
+// the lanes with their c.  (Four additions; lanes 30 and 31 hold zero.)
+__device__ __forceinline__ double group_sums(double v) {
+    v += __shfl_down_sync(0xffffffffu, v, 15);            // groups 0 .. 4
+    const double v4 = __shfl_down_sync(0xffffffffu, v, 12);
+    v += __shfl_down_sync(0xffffffffu, v, 6);             // 0 + 2, 1 + 3
+    v += __shfl_down_sync(0xffffffffu, v, 3);
+    return v + v4;
+}
+
+// Clusters: an instance of at most eight blocks of kClusterCells cells is a thread-block cluster
+// that keeps the populations in its blocks' shared memory for the whole launch.  A cell is on three
+// lanes (collide_lanes), a warp of ten cells to each SM quarter; neighbours in another block are read
+// and written through distributed shared memory, and a step ends with the cluster's hardware barrier.
+// A location is read and then written by the lanes of one cell within a step, and every store of a
+// warp depends on all its loads (the collision's shuffles), so one barrier a step is enough.
+// Short lattices are bound by the FP64 chain and the step's synchronisation: 28 lines of 128 cells
+// (entropic, bulk correction) probed every 10 steps, a block each 4.6 us a step, teams of 4 blocks
+// with three-lane cells through L2 4.9, clusters 3.0; probed on every step 6.4 -> 3.8.  A probe's
+// projections are split over a cell's lanes as well (all on one lane: 4.8 us).
+template <int D, int EQ, bool BULK>
+__global__ void __launch_bounds__(lbmh::kTeamThreads) k_step_clusters(const lbmh::BatchArgs a) {
+    constexpr int N = kProbe<D>, Q = qof(D), F = lane_pops(D), C = lbmh::kClusterCells;
+    constexpr int kWarps = lbmh::kTeamThreads / 32;
+    __shared__ double pop[Q * C];  // plane i of the block's cells at i C
+    __shared__ double red[kWarps][8], sums[2][8];
+    const int csize = a.team_cluster, k = blockIdx.x / csize, part = blockIdx.x % csize;
+    const int nx = a.dims[3 * k], ny = a.dims[3 * k + 1], nz = a.dims[3 * k + 2];
+    const int64_t c0 = a.cell_start[k];
+    const int ncell = (int)(a.cell_start[k + 1] - c0), parts = (ncell + C - 1) / C;
+    double *A = a.arena + (int64_t)Q * c0 + part * C;
+    const int mine = min(C, ncell - part * C);  // cells of the block (none: it only takes part in the barriers)
+    const double om = a.omega0[k], sn = a.six_nu[k];
+    const double2 *tw = a.twiddle + a.tw_offset[k];
+    for (int p = threadIdx.x; p < Q * C; p += lbmh::kTeamThreads)
+        if (p % C < mine) pop[p] = A[(int64_t)(p / C) * ncell + p % C];
+    // the lane's cell and the addresses of its odd-step reads f_i(r) = A[opp(i)][r - c_i] and writes
+    // A[i][r + c_i], directions i = p + F c
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane % 3, base = lane < 30 ? lane - c : 27;
+    const int here = warp * 10 + lane / 3;
+    const bool run = lane < 30 && here < mine;
+    int x, y, z;
+    cell_coords(run ? part * C + here : 0, ncell, nx, ny, x, y, z);
+    uint32_t src[F], dst[F];
+    const uint32_t pop0 = smem_u32(pop);
+#pragma unroll
+    for (int p = 0; p < F; ++p) {
+        const int i = p + F * c, dx = cxo(p), dy = D == 3 ? cyo(p) : c - 1, dz = D == 3 ? c - 1 : 0;
+        const int from = wrapi(x - dx, nx) + nx * (wrapi(y - dy, ny) + ny * wrapi(z - dz, nz));
+        const int to = wrapi(x + dx, nx) + nx * (wrapi(y + dy, ny) + ny * wrapi(z + dz, nz));
+        const bool ok = LBM_CHECK(from >= 0 && from < ncell && to >= 0 && to < ncell, nullptr);
+        src[p] = cluster_addr(pop0 + 8 * ((Q - 1 - i) * C + (ok ? from % C : 0)), ok ? from / C : part);
+        dst[p] = cluster_addr(pop0 + 8 * (i * C + (ok ? to % C : 0)), ok ? to / C : part);
+    }
+    // exp(-i k.r) of the cell; lane c projects rho, j_x or j_y, in 3-D lane 0 also j_z
+    double pr = 0.0, pi = 0.0;
+    if (a.every_k > 0 && run) {
+        const double2 tx = tw[x], ty = tw[nx + y];
+        pr = tx.x * ty.x - tx.y * ty.y;
+        pi = tx.x * ty.y + tx.y * ty.x;
+        if (D == 3) {
+            const double2 tz = tw[nx + ny + z];
+            const double qr = pr * tz.x - pi * tz.y;
+            pi = pr * tz.y + pi * tz.x;
+            pr = qr;
+        }
+    }
+    const bool busy = warp * 10 < mine;
+    if (lane < 8) red[warp][lane] = 0.0;  // (2-D: no j_z)
+    cluster_barrier();
+    int64_t until = a.every_k > 0 ? (a.every_k - a.step0 % a.every_k) % a.every_k : a.nsteps;  // steps to the next probe
+    unsigned probes = 0;
+    for (int64_t s = 0; s < a.nsteps; ++s) {
+        const int64_t t = a.step0 + s;
+        const int odd = (int)(t & 1);
+        const bool probe = until == 0;
+        until = probe ? a.every_k - 1 : until - 1;
+        if (busy) {
+            double f[F];
+#pragma unroll
+            for (int p = 0; p < F; ++p) {
+                f[p] = 0.0;
+                if (run) f[p] = odd ? cluster_ld(src[p]) : pop[(p + F * c) * C + here];
+            }
+            const CellMoments<double> m = collide_lanes<D, EQ, BULK>(f, c, base, a.rho0, om, sn);
+            if (run) {
+#pragma unroll
+                for (int p = 0; p < F; ++p) {
+                    if (odd) cluster_st(dst[p], f[p]);
+                    else pop[(Q - 1 - p - F * c) * C + here] = f[p];
+                }
+            }
+            if (probe) {
+                const double q = c == 0 ? m.rho : m.rho * (c == 1 ? m.u[0] : m.u[1]);
+                const double re = group_sums(run ? q * pr : 0.0), im = group_sums(run ? q * pi : 0.0);
+                if (lane < 3) {
+                    red[warp][2 * c] = re;
+                    red[warp][2 * c + 1] = im;
+                }
+                if constexpr (D == 3) {
+                    const double jz = m.rho * m.u[2];
+                    const double re3 = group_sums(run ? jz * pr : 0.0), im3 = group_sums(run ? jz * pi : 0.0);
+                    if (lane == 0) {
+                        red[warp][6] = re3;
+                        red[warp][7] = im3;
+                    }
+                }
+            }
+        }
+        if (probe) {  // sums of the block, in pairs as in the teams
+            __syncthreads();
+            if (threadIdx.x < 8) {
+                double sum = 0.0;
+                for (int w = 0; w * 10 < mine; ++w) sum += red[w][threadIdx.x];
+                sums[probes & 1][threadIdx.x] = sum;
+            }
+        }
+        cluster_barrier();
+        if (probe) {
+            // lane j adds up the parts' sums j: the last warp of the last block with cells, which
+            // often has none of its own
+            if (part == parts - 1 && warp == kWarps - 1) {
+                double sum = 0.0;
+                const uint32_t at = smem_u32(&sums[probes & 1][lane & 7]);
+                for (int q = 0; q < parts; ++q) sum += cluster_ld(cluster_addr(at, q));
+                const bool fin = __all_sync(0xffffffffu, (lane & 7) >= N || isfinite(sum));
+                const double mass = from_lane(sum, 0);
+                if (lane >= N) sum = fin ? 0.0 : mass - mass;  // as probe_record
+                const int64_t sample = t / a.every_k;
+                if (lane < 8 && sample < a.max_samples) a.series[((int64_t)k * a.max_samples + sample) * 8 + lane] = sum;
+                if (lane == 0 && !fin && a.status[k] == 0) a.status[k] = (int32_t)(t + 1);
+            }
+            ++probes;
+        }
+    }
+    for (int p = threadIdx.x; p < Q * C; p += lbmh::kTeamThreads)
+        if (p % C < mine) A[(int64_t)(p / C) * ncell + p % C] = pop[p];
+    cluster_barrier();  // no block leaves while its sums may be read
+}
+
 // Instance of a packed global cell index (binary search over cell_start).
 __device__ __forceinline__ int find_instance(const int64_t *cell_start, int64_t count, int64_t g) {
     int64_t lo = 0, hi = count - 1;
@@ -308,11 +449,56 @@ int team_block_capacity(int D, int eq, int bulk, int sms) {
     return nb * sms;
 }
 
+static const void *cluster_kernel(int D, int eq, int bulk) {
+#define LBM_BC(Dv, EQv)                                                                                  \
+    if (D == Dv && eq == EQv)                                                                            \
+        return bulk ? (const void *)k_step_clusters<Dv, EQv, true> : (const void *)k_step_clusters<Dv, EQv, false>;
+    LBM_BC(2, EQ_ENT)
+    LBM_BC(2, EQ_POLY2)
+    LBM_BC(2, EQ_PROD)
+    LBM_BC(3, EQ_ENT)
+    LBM_BC(3, EQ_POLY2)
+    LBM_BC(3, EQ_PROD)
+#undef LBM_BC
+    return nullptr;
+}
+
+static void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, int blocks, int cluster, cudaStream_t s) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kTeamThreads);
+    cfg.stream = s;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+}
+
+int batch_cluster_capacity(int D, int eq, int bulk, int cluster) {
+    const void *fn = cluster_kernel(D, eq, bulk);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    cluster_config(cfg, at, cluster, cluster, nullptr);
+    int n = 0;
+    if (!fn || cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
 cudaError_t step_teams(const BatchArgs &a, int blocks, cudaStream_t s) {
-    const void *fn = team_kernel(a.D, a.eq, a.bulk);
-    if (!fn) return cudaErrorInvalidValue;
     BatchArgs aa = a;
     void *args[] = {(void *)&aa};
+    const void *fn = a.team_cluster > 0 ? cluster_kernel(a.D, a.eq, a.bulk) : team_kernel(a.D, a.eq, a.bulk);
+    if (!fn) return cudaErrorInvalidValue;
+    if (a.team_cluster > 0) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        cluster_config(cfg, at, blocks, a.team_cluster, s);
+        return cudaLaunchKernelExC(&cfg, fn, args);
+    }
     return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kTeamThreads), args, 0, s);
 }
 

@@ -123,9 +123,14 @@ struct BatchArgs {
     double *team_partials;
     unsigned *team_sync;
     int32_t *team_status;
+    int team_cluster;  // blocks of an instance's thread-block cluster (k_step_clusters), 0: teams
     int64_t timeout_ns;
 };
 constexpr int kTeamThreads = 128;  // threads of a team's block
+constexpr int kClusterCells = kTeamThreads / 32 * 10;  // cells of a cluster's block, three lanes each
+constexpr int kClusterBlocks = 8;                      // largest portable cluster
+// Clusters of that many blocks that are resident at once.
+int batch_cluster_capacity(int D, int eq, int bulk, int cluster);
 // Blocks of the team kernel that are resident at once.
 int team_block_capacity(int D, int eq, int bulk, int sms);
 cudaError_t step_teams(const BatchArgs &a, int blocks, cudaStream_t s);

@@ -1,4 +1,4 @@
-"""FP64 cells on three lanes of a warp (small lattices) against one cell per thread."""
+"""FP64 cells on three lanes of a warp (small lattices and batches) against one cell per thread."""
 import numpy as np
 import pytest
 
@@ -33,3 +33,39 @@ def test_lanes_match_one_cell_per_thread(D, dims, eq, bulk):
     for lat in lats:
         lat.sync()
         lat.close()
+
+
+# full and partial blocks, a block an SM at most (152 blocks), one more
+BATCHES = [(2, [(128, 1, 1)] * 28), (2, [(40, 1, 1), (1, 1, 1), (41, 1, 1), (9, 11, 1)]), (2, [(5, 8, 1)] * 152), (2, [(5, 8, 1)] * 153),
+           (3, [(16, 9, 1), (1, 1, 1), (4, 5, 6)])]
+
+
+@pytest.mark.parametrize("eq,bulk", [(0, 1), (1, 0), (2, 1)])
+@pytest.mark.parametrize("D,dims", BATCHES)
+def test_lanes_of_a_batch(D, dims, eq, bulk):
+    from paper_2303_08163_gb300 import lbm
+    dims = np.array(dims, dtype=np.int32)
+    n = len(dims)
+    rng = np.random.default_rng(n)
+    tau = 0.5 + rng.uniform(0.05, 0.5, n)
+    kvec = rng.integers(0, 3, (n, 3)).astype(np.int32)
+    kvec[:, 2] *= D == 3
+    fields = [inputs.random_state(D, tuple(int(v) for v in d), seed=20 + i, u_max=0.1) for i, d in enumerate(dims)]
+    rho = np.concatenate([f[0] for f in fields])
+    u = np.concatenate([f[1].reshape(-1) for f in fields])
+    out = []
+    for whole in (False, True):
+        b = lbm.Batch(lbm.D2Q9 if D == 2 else lbm.D3Q27, dims, tau, eq, bulk)
+        if whole:
+            b.set_launch_shape(64, min(n, 3))
+        b.init_fields(rho, u)
+        b.set_probe(kvec, 2)
+        for steps in STEPS:
+            b.step(steps)
+        out.append((b.get_populations(), b.probe_series(), b.status()))
+        b.close()
+    (f0, s0, st0), (f1, s1, st1) = out
+    assert np.array_equal(st0, st1) and not st0.any()
+    assert np.max(np.abs(f0 - f1)) <= TOL
+    cells = dims.prod(axis=1)[:, None, None]
+    assert s0.shape == s1.shape and np.all(np.abs(s0 - s1) <= 9 * TOL * cells)
