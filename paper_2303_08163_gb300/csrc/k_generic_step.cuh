@@ -120,7 +120,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned gen, const
     if (threadIdx.x < 32) {
         if (threadIdx.x == 0) {
             bad = 0;
-            __threadfence();
             red_release(&sync[lbmh::kBarStride * (1 + blockIdx.x % lbmh::kBarCounters)], 1u);
         }
         bool ok = true;
@@ -139,7 +138,6 @@ __device__ __forceinline__ bool team_barrier(unsigned *counter, unsigned want, c
     __shared__ int bad;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         red_release(counter, 1u);
         bad = !wait_count_bounded(counter, want, status, timeout_ns);
     }
