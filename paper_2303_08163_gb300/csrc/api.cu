@@ -78,8 +78,9 @@ struct lbm_ctx {
     int sticky = 0;
     // diagnostics
     int64_t diag_every = 0;
-    int32_t *status = nullptr;   // start of one allocation that holds these five
+    int32_t *status = nullptr;   // start of one allocation that holds these six
     unsigned *sync = nullptr;    // counters of several-step launches
+    void *msg = nullptr;         // words of a small lattice's several-step launches
     double *partials = nullptr;  // [kPartialsCap][8]
     double *hist = nullptr;      // [kHistCap][8]
     double *scratch = nullptr;   // one record
@@ -184,6 +185,7 @@ StepArgs step_args(lbm_ctx *c, int odd, int diag) {
     a.partials = c->partials;
     a.status = c->status;
     a.sync = c->sync;
+    a.msg = c->msg;
     a.timeout_ns = wait_timeout_ns();
     return a;
 }
@@ -200,10 +202,10 @@ cudaError_t launch_one(lbm_ctx *c, int odd, int diag, cudaStream_t s) {
 // TMA kernel, one each with the one-cell kernel.
 cudaError_t launch_steps(lbm_ctx *c, int odd, int64_t n, cudaStream_t s) {
     if (n > 1 && !c->chosen && c->small.threads > 0) {
-        // (launches of bounded length: FP64 steps of 5 us)
+        // (launches of bounded length: at most 90 ms with FP64 steps of 45 us)
         cudaError_t e = cudaSuccess;
         while (n > 0 && e == cudaSuccess) {
-            const int64_t m = std::min<int64_t>(n, 10000);
+            const int64_t m = std::min<int64_t>(n, 2000);
             e = steps_small(step_args(c, odd, 0), (int)m, c->small, s);
             odd ^= (int)(m & 1);
             n -= m;
@@ -703,25 +705,33 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
     const size_t zeroed = 256 + (sizeof(unsigned) * (kSyncDone + sync_units(c->lat)) + 255) / 256 * 256;
     const size_t recs = sizeof(double) * kDiagWords * (kPartialsCap + kHistCap + 4);
     char *aux = nullptr;
-    if (cudaMalloc(&aux, zeroed + recs) != cudaSuccess) {
+    size_t msg = small_shape(c->lat, c->eq, c->bulk, sm_count(), c->small) ? (small_msg_bytes(c->lat) + 255) / 256 * 256 : 0;
+    cudaError_t ea = cudaMalloc(&aux, zeroed + msg + recs);
+    if (ea != cudaSuccess && msg > 0) {  // no room for the words: as a larger lattice
+        cudaGetLastError();
+        msg = 0;
+        ea = cudaMalloc(&aux, zeroed + recs);
+    }
+    if (msg == 0) c->small.threads = 0;
+    if (ea != cudaSuccess) {
         cudaGetLastError();
         lbm_destroy(c);
         return fail(LBM_ENOMEM, "diagnostics buffers");
     }
     c->status = reinterpret_cast<int32_t *>(aux);
     c->sync = reinterpret_cast<unsigned *>(aux + 256);
-    c->partials = reinterpret_cast<double *>(aux + zeroed);
+    c->msg = aux + zeroed;
+    c->partials = reinterpret_cast<double *>(aux + zeroed + msg);
     c->hist = c->partials + kDiagWords * kPartialsCap;
     c->scratch = c->hist + 8 * kHistCap;
     if (cudaMemsetAsync(c->lat.A, 0, bytes, c->stream) != cudaSuccess ||
-        cudaMemsetAsync(aux, 0, zeroed, c->stream) != cudaSuccess) {
+        cudaMemsetAsync(aux, 0, zeroed + msg, c->stream) != cudaSuccess) {
         lbm_destroy(c);
         return cuda_fail("initial memset", cudaGetLastError());
     }
     c->gen_threads = 256;
     c->gen_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((ncell + 255) / 256, (int64_t)sm_count() * 16));
     c->kernel = 1;
-    if (!small_shape(c->lat, c->eq, c->bulk, sm_count(), c->small)) c->small.threads = 0;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         static bool loaded = false;

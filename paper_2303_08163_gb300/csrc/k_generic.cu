@@ -10,8 +10,8 @@
 namespace lbmh {
 cudaError_t step_generic_d2(const StepArgs &a, int blocks, int threads, cudaStream_t s);
 cudaError_t step_generic_d3(const StepArgs &a, int blocks, int threads, cudaStream_t s);
-const void *small_kernel_d2(int P, int eq, int bulk, bool lanes);
-const void *small_kernel_d3(int P, int eq, int bulk, bool lanes);
+const void *small_kernel_d2(int P, int eq, int bulk, bool lanes, bool many);
+const void *small_kernel_d3(int P, int eq, int bulk, bool lanes, bool many);
 }  // namespace lbmh
 
 namespace lbmd {
@@ -328,35 +328,53 @@ cudaError_t step_generic(const StepArgs &a, int blocks, int threads, cudaStream_
     return a.lat.D == 2 ? step_generic_d2(a, blocks, threads, s) : step_generic_d3(a, blocks, threads, s);
 }
 
-static const void *small_kernel(const Lattice &lat, int eq, int bulk, bool lanes) {
-    return lat.D == 2 ? small_kernel_d2(lat.P, eq, bulk, lanes) : small_kernel_d3(lat.P, eq, bulk, lanes);
+static const void *small_kernel(const Lattice &lat, int eq, int bulk, const SmallShape &t) {
+    return lat.D == 2 ? small_kernel_d2(lat.P, eq, bulk, t.lanes, t.many) : small_kernel_d3(lat.P, eq, bulk, t.lanes, t.many);
 }
 
-// Up to 800 cells an SM (48^3: 727) the grid-barrier kernel is the faster one; with more a thread
-// has several cells, whose loads follow one another, and the TMA row kernel's copies overlap
-// (509 x 381 FP32, 1276 cells an SM: 6.8 us a step against 5.3; 64^3 binary16 9.1 against 7.7).
-// FP64 lattices of at most 40 cells an SM have a cell on three lanes: a warp on each quarter is all
-// there is either way, and a warp instruction costs the same for 7 cells as for 10 of three lanes
-// (with 41 to 80 an SM quarter would have two such warps, as long as one of 32 cells).
+// The largest lattice of the several-step kernel, in cells an SM: what the threads of its resident
+// blocks hold, one cell each, and twice that where two rounds are still faster than the TMA row kernel
+// (512^2 FP32 3.9 us a step against 5.1; 512^2 binary16 4.6 - 5.9 against 4.9, so not there;
+// 56^3 binary16 8.3 against 7.4, but 60^3, whose short ragged rows that kernel does not take, 8.3
+// against 17).  FP64 in 3-D takes three rounds (48^3 45 us).
+static int64_t small_limit(const Lattice &lat) {
+    if (lat.D == 2) return lat.P == P_F16S ? 1280 : lat.P == P_F32 ? 2048 : 1024;
+    return lat.P == P_F16S && !tma_supported(lat) ? 1536 : 768;
+}
+
+// An SM's cells are spread over as few blocks as hold them, all with equally many warps.  FP64
+// lattices of at most 40 cells an SM have a cell on three lanes: a warp on each quarter is all there
+// is either way, and a warp instruction costs the same for 7 cells as for 10 of three lanes (with 41
+// to 80 cells an SM quarter would have two such warps, as long as one of 32 cells).
 bool small_shape(const Lattice &lat, int eq, int bulk, int sms, SmallShape &t) {
-    if (lat.ncell > (int64_t)800 * sms || lat.plane * qof(lat.D) >= ((int64_t)1 << 31)) return false;
+    if (lat.ncell > small_limit(lat) * sms || lat.plane * qof(lat.D) >= ((int64_t)1 << 31)) return false;
     const int64_t per = (lat.ncell + sms - 1) / sms;  // cells an SM
     t.lanes = lat.P == P_F64 && per <= 40;
     const int warp = t.lanes ? 10 : 32;  // cells a warp
-    const int64_t warps = std::min<int64_t>(8, (per + warp - 1) / warp);
-    t.threads = (int)(32 * warps);
-    const void *fn = small_kernel(lat, eq, bulk, t.lanes);
+    const int64_t warps = (per + warp - 1) / warp;
+    int64_t n = std::min<int64_t>((warps + 7) / 8, small_blocks(lat.D, lat.P));
+    // several rounds of the 3-D FP64 kernel: one block with all the registers (44^3 45 us, 61 in two)
+    if (lat.D == 3 && lat.P == P_F64 && warps > 16) n = 1;
+    t.many = n > 1;
+    t.threads = (int)(32 * std::min<int64_t>(8, (warps + n - 1) / n));
+    const int64_t cells = t.threads / 32 * warp;
+    const void *fn = small_kernel(lat, eq, bulk, t);
     int nb = 0;
     if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, t.threads, 0) != cudaSuccess || nb < 1) {
         cudaGetLastError();
         return false;
     }
-    t.blocks = (int)std::min<int64_t>((lat.ncell + warps * warp - 1) / (warps * warp), (int64_t)nb * sms);
+    t.blocks = (int)std::min<int64_t>((lat.ncell + cells - 1) / cells, (int64_t)nb * sms);
     return true;
 }
 
+size_t small_msg_bytes(const Lattice &lat) {
+    const size_t word = lat.P == P_F64 ? 16 : lat.P == P_F32 ? 8 : 4;  // a population and a step number
+    return kMsgHead + word * qof(lat.D) * lat.plane;
+}
+
 cudaError_t steps_small(const StepArgs &a, int nsteps, const SmallShape &t, cudaStream_t s) {
-    const void *fn = small_kernel(a.lat, a.eq, a.bulk, t.lanes);
+    const void *fn = small_kernel(a.lat, a.eq, a.bulk, t);
     if (!fn) return cudaErrorInvalidValue;
     StepArgs aa = a;
     void *args[] = {(void *)&aa, (void *)&nsteps};

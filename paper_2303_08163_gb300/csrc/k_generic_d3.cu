@@ -11,12 +11,12 @@ cudaError_t step_generic_d3(const StepArgs &a, int blocks, int threads, cudaStre
     }
 }
 
-const void *small_kernel_d3(int P, int eq, int bulk, bool lanes) {
+const void *small_kernel_d3(int P, int eq, int bulk, bool lanes, bool many) {
     if (lanes) return lbmd::lanes_kernel_d<3>(eq, bulk);
     switch (P) {
-    case lbmd::P_F64: return lbmd::small_kernel_dp<3, lbmd::P_F64>(eq, bulk);
-    case lbmd::P_F32: return lbmd::small_kernel_dp<3, lbmd::P_F32>(eq, bulk);
-    case lbmd::P_F16S: return lbmd::small_kernel_dp<3, lbmd::P_F16S>(eq, bulk);
+    case lbmd::P_F64: return lbmd::small_kernel_dp<3, lbmd::P_F64>(eq, bulk, many);
+    case lbmd::P_F32: return lbmd::small_kernel_dp<3, lbmd::P_F32>(eq, bulk, many);
+    case lbmd::P_F16S: return lbmd::small_kernel_dp<3, lbmd::P_F16S>(eq, bulk, many);
     default: return nullptr;
     }
 }

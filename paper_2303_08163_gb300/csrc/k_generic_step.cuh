@@ -106,34 +106,103 @@ __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
 //
 // A small lattice's steps are bound by latency: a launch, a pipeline's ramp, or in the TMA row
 // kernel's several-step form the way of a row through shared memory and its counters.  Here all
-// its cells are in registers at once, one (or a few) to a thread: a step is a load of the
-// populations from L2, the collision, the stores and one barrier of the whole grid (cooperative
-// launch: all blocks are resident).  The barrier's arrivals are spread over kBarCounters counters,
-// each on its own line; a block's first warp looks at all of them.  Per step against the TMA row
-// kernel: 90^2 FP64 8.2 -> 4.6 us (2.6 us of it one warp's 82 FP64 instructions at 64 clocks),
-// 64^2 FP32 3.9 -> 2.1, 32^3 binary16 6.1 -> 2.8, 48^3 6.8 -> 5.7 us.
+// its cells are in registers at once, one (or a few) to a thread, in one cooperative launch (all
+// blocks are resident), and no barrier separates the steps: within the launch a population travels
+// in one word with the number of the step that wrote it, through a buffer with the layout of the
+// lattice (rows unpadded: a warp's cells are contiguous across the end of a row, 300^2 binary16
+// 1.8 us a step, 2.7 with the lattice's own padding).  A cell reads a location until it finds its own step's number there.  A location is read
+// and then rewritten by one cell a step (the AA pattern), so nothing can be overwritten before it
+// was read, and a word is written and read whole, so neither fences nor counters are needed: a step
+// is a store, a load and the collision.  The first step reads and the last one writes the lattice's
+// own array.  The numbers go on from launch to launch (the buffer's head, advanced by the last block),
+// so the words of an earlier launch, all one behind the next launch's first, never match.
+// Per step with the TMA row kernel, with a barrier of the whole grid in place of the numbers (release
+// fence, counter, acquire: 1 us), and so: 64^2 FP32 3.9, 1.86, 0.91 us; 64^2 FP64 8.0, 3.45, 2.65;
+// 32^3 binary16 6.1, 2.49, 1.57; 340^2 FP32 4.6, 3.16, 1.95; 48^3 binary16 6.8, 4.5, 4.1.
+struct MsgHead {
+    unsigned step, exits;
+};
 
-// Wait until every block has arrived `gen` times (counters never wrap: gen * blocks < 2^32).
-__device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned gen, const int32_t *status, int64_t timeout_ns) {
-    __shared__ int bad;
-    __syncthreads();  // every store of the block is issued
-    if (threadIdx.x < 32) {
-        if (threadIdx.x == 0) {
-            bad = 0;
-            red_release(&sync[lbmh::kBarStride * (1 + blockIdx.x % lbmh::kBarCounters)], 1u);
-        }
-        bool ok = true;
-        if (threadIdx.x < lbmh::kBarCounters && threadIdx.x < gridDim.x) {
-            const unsigned arrive = (gridDim.x - threadIdx.x + lbmh::kBarCounters - 1) / lbmh::kBarCounters;
-            ok = wait_count_bounded(&sync[lbmh::kBarStride * (1 + threadIdx.x)], gen * arrive, status, timeout_ns);
-        }
-        if (__any_sync(0xffffffffu, !ok) && threadIdx.x == 0) bad = 1;
+template <int P> struct Msg;
+template <> struct Msg<P_F16S> {  // population, step modulo 2^16
+    using W = uint32_t;
+    static __device__ __forceinline__ bool take(const W *p, unsigned want, float &v) {
+        W w;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(p) : "memory");
+        v = __half2float(__ushort_as_half((unsigned short)w));
+        return w >> 16 == (want & 0xffffu);
     }
-    __syncthreads();
-    return bad == 0;
+    static __device__ __forceinline__ void give(W *p, unsigned step, float v) {
+        const W w = step << 16 | __half_as_ushort(Storage<P_F16S>::store(v));
+        asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(w) : "memory");
+    }
+};
+template <> struct Msg<P_F32> {
+    using W = uint64_t;
+    static __device__ __forceinline__ bool take(const W *p, unsigned want, float &v) {
+        W w;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+        v = __uint_as_float((unsigned)w);
+        return (unsigned)(w >> 32) == want;
+    }
+    static __device__ __forceinline__ void give(W *p, unsigned step, float v) {
+        const W w = (W)step << 32 | __float_as_uint(v);
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+    }
+};
+template <> struct Msg<P_F64> {  // two words, a half of the population and the step in each
+    using W = ulonglong2;
+    static __device__ __forceinline__ bool take(const W *p, unsigned want, double &v) {
+        unsigned long long x, y;
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(p) : "memory");
+        v = __hiloint2double((int)(unsigned)y, (int)(unsigned)x);
+        return (unsigned)(x >> 32) == want && (unsigned)(y >> 32) == want;
+    }
+    static __device__ __forceinline__ void give(W *p, unsigned step, double v) {
+        const unsigned long long t = (unsigned long long)step << 32;
+        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | (unsigned)__double2loint(v)),
+                     "l"(t | (unsigned)__double2hiint(v))
+                     : "memory");
+    }
+};
+
+// Reads the populations f[p] = M[at(p)] of the lanes that `run` until all of the warp's carry the
+// number `want` (the lanes go on together: a collision in two halves of a warp takes twice as long,
+// 90^2 FP64 6.8 against 3.6 us a step); false when the wait runs out or another thread has reported
+// an error.  All 32 lanes call it.
+template <int P, int N, typename R, typename At>
+__device__ __forceinline__ bool msg_take(const typename Msg<P>::W *M, unsigned want, R (&f)[N], const At &at, bool run,
+                                         const int32_t *status, int64_t timeout_ns) {
+    uint64_t t0 = 0;
+    for (int tries = 1;; ++tries) {
+        bool all = true;
+        if (run) {
+#pragma unroll
+            for (int p = 0; p < N; ++p) all &= Msg<P>::take(M + at(p), want, f[p]);
+        }
+        if (__all_sync(0xffffffffu, all)) return true;
+        if (tries % 64 == 0) {
+            if (t0 == 0) t0 = global_ns();
+            const bool stop = *(const volatile int32_t *)status != 0 || (int64_t)(global_ns() - t0) > timeout_ns;
+            if (__any_sync(0xffffffffu, stop)) return false;
+        }
+    }
 }
 
-// The same for the blocks of one counter (it grows by the number of blocks a step).
+// The end of a several-step launch: reports a wait that ran out; the last block to finish moves the
+// step number on.
+__device__ __forceinline__ void steps_finish(const lbmh::StepArgs &a, int nsteps, bool ok) {
+    if (!ok) report_status(a.status, -5); /* LBM_ETIMEOUT */
+    MsgHead *head = static_cast<MsgHead *>(a.msg);
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&head->exits, 1u) == gridDim.x - 1) {
+        head->exits = 0;
+        head->step += (unsigned)nsteps;
+    }
+}
+
+// Barrier of the blocks of one counter, which grows by their number a step.  (The release orders the
+// stores of the whole block: they precede it through the block's own barrier.)
 __device__ __forceinline__ bool team_barrier(unsigned *counter, unsigned want, const int32_t *status, int64_t timeout_ns) {
     __shared__ int bad;
     __syncthreads();
@@ -145,36 +214,26 @@ __device__ __forceinline__ bool team_barrier(unsigned *counter, unsigned want, c
     return bad == 0;
 }
 
-// The end of a several-step launch: reports a wait that ran out; the last block to finish clears
-// the counters for the next launch.
-__device__ __forceinline__ void steps_finish(const lbmh::StepArgs &a, bool ok) {
-    if (!ok && threadIdx.x == 0) report_status(a.status, -5); /* LBM_ETIMEOUT */
-    __syncthreads();
-    bool last = false;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(&a.sync[1], 1u) == gridDim.x - 1;
-    }
-    if (__syncthreads_or(last))
-        for (int p = threadIdx.x; p < lbmh::kBarStride * (1 + lbmh::kBarCounters); p += blockDim.x) a.sync[p] = 0;
-}
-
-template <int D, int P, int EQ, bool BULK>
-__global__ void __launch_bounds__(256) k_steps_small(const lbmh::StepArgs a, int nsteps) {
+template <int D, int P, int EQ, bool BULK, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_steps_small(const lbmh::StepArgs a, int nsteps) {
     using St = Storage<P>;
     using T = typename St::T;
     using R = typename St::R;
+    using W = typename Msg<P>::W;
     constexpr int Q = qof(D);
     T *A = static_cast<T *>(a.lat.A);
+    W *M = reinterpret_cast<W *>(static_cast<char *>(a.msg) + lbmh::kMsgHead);
+    const unsigned step0 = __ldcg(&static_cast<const MsgHead *>(a.msg)->step);
     const int nx = a.lat.nx, ny = a.lat.ny, nz = a.lat.nz, pitch = a.lat.pitch;
     const int plane = (int)a.lat.plane, ncell = (int)a.lat.ncell;  // Q * plane < 2^31 (checked on the host)
     const R rho0 = step_scalar<R>(a.rho0, a.rho0f), omega0 = step_scalar<R>(a.omega0, a.omega0f),
             six_nu = step_scalar<R>(a.six_nu, a.six_nuf);
     bool ok = true;
-    int here = -1, xs[3], rows[9];  // the thread's cell and its neighbours: columns, row starts by (dy + 1) + 3 (dz + 1)
+    int here = -1, xs[3], rows[9];  // the thread's cell and its neighbours: columns, rows by (dy + 1) + 3 (dz + 1)
     for (int s = 0; s < nsteps && ok; ++s) {
         const int odd = (a.odd + s) & 1;
-        for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < ncell; cell += gridDim.x * blockDim.x) {
+        for (int first = blockIdx.x * blockDim.x + (threadIdx.x & ~31); first < ncell && ok; first += gridDim.x * blockDim.x) {
+            const int cell = min(first + (int)(threadIdx.x & 31), ncell - 1);
             if (cell != here) {  // once, where a thread has one cell
                 int x, y, z;
                 cell_coords(cell, ncell, nx, ny, x, y, z);
@@ -185,40 +244,64 @@ __global__ void __launch_bounds__(256) k_steps_small(const lbmh::StepArgs a, int
 #pragma unroll
                 for (int q = 0; q < (D == 3 ? 9 : 3); ++q) {
                     const int yy = wrapi(y + q % 3 - 1, ny), zz = D == 3 ? wrapi(z + q / 3 - 1, nz) : z;
-                    rows[q] = pitch * (yy + ny * zz);
+                    rows[q] = yy + ny * zz;
                 }
             }
-            const int self = rows[D == 3 ? 4 : 1] + xs[1];
-            if (!LBM_CHECK(self >= 0 && self < plane, a.status)) continue;
-            R f[Q];
-            if (!odd) {
+            const bool run = first + (int)(threadIdx.x & 31) < ncell &&
+                             LBM_CHECK(here >= 0 && rows[D == 3 ? 4 : 1] * pitch + xs[1] < plane, a.status);
+            R f[Q] = {};
+            // where direction i is read and written: A[i][r] and A[opp(i)][r], odd steps
+            // A[opp(i)][r - c_i] and A[i][r + c_i]
+            const auto at = [&](int i, int c, int slot, int pit) {
+                const int row = rows[(1 + c * cyo(i)) + (D == 3 ? 3 * (1 + c * czo(i)) : 0)];
+                return slot * plane + row * pit + xs[1 + c * cxo(i)];
+            };
+            const auto in = [&](int i, int o, int pit) { return o ? at(i, -1, Q - 1 - i, pit) : at(i, 0, i, pit); };
+            const auto out = [&](int i, int o, int pit) { return o ? at(i, 1, i, pit) : at(i, 0, Q - 1 - i, pit); };
+            const auto take = [&](int o) {
+                return msg_take<P>(M, step0 + s, f, [&](int i) { return in(i, o, nx); }, run, a.status, a.timeout_ns);
+            };
+            const auto give = [&](int o) {
 #pragma unroll
-                for (int i = 0; i < Q; ++i) f[i] = St::load(ld_pop<true>(A + i * plane + self));
-            } else {
-#pragma unroll
-                for (int i = 0; i < Q; ++i)  // f_i(r) = A[opp(i)][r - c_i]
-                    f[i] = St::load(ld_pop<true>(A + (Q - 1 - i) * plane + rows[(1 - cyo(i)) + (D == 3 ? 3 * (1 - czo(i)) : 0)] + xs[1 - cxo(i)]));
-            }
-            collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
-            if (!odd) {
-#pragma unroll
-                for (int i = 0; i < Q; ++i) A[(Q - 1 - i) * plane + self] = St::store(f[i]);
-            } else {
+                for (int i = 0; i < Q; ++i) Msg<P>::give(M + out(i, o, nx), step0 + s + 1, f[i]);
+            };
+            // Even and odd code of its own where registers are scarce (48^3 binary16 4.1 against 5.4 us
+            // a step, 512^2 4.1 against 4.5); one code with the parity's addresses chosen where they
+            // are not: the compiler then keeps fewer of them (32^3 1.6 against 1.8).
+            if (s == 0) {
 #pragma unroll
                 for (int i = 0; i < Q; ++i)
-                    A[i * plane + rows[(1 + cyo(i)) + (D == 3 ? 3 * (1 + czo(i)) : 0)] + xs[1 + cxo(i)]] = St::store(f[i]);
+                    if (run) f[i] = St::load(A[in(i, odd, pitch)]);
+            } else if (MINB == 1) {
+                ok = take(odd);
+            } else if (odd) {
+                ok = take(1);
+            } else {
+                ok = take(0);
+            }
+            if (!ok) break;
+            collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
+            if (!run) continue;
+            if (s + 1 == nsteps) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) A[out(i, odd, pitch)] = St::store(f[i]);
+            } else if (MINB == 1) {
+                give(odd);
+            } else if (odd) {
+                give(1);
+            } else {
+                give(0);
             }
         }
-        if (s + 1 < nsteps) ok = grid_barrier(a.sync, (unsigned)(s + 1), a.status, a.timeout_ns);
     }
-    steps_finish(a, ok);
+    steps_finish(a, nsteps, ok);
 }
 
 // A cell on three lanes of a warp (collide_lanes), ten cells to a warp: the lane's share of the
 // loads and stores.  Lane c of a group has the directions i = p + F c.
 template <int D> struct LaneCell {
     static constexpr int Q = qof(D), F = lane_pops(D), N = D == 3 ? 3 : 1;
-    int c, base, x, y, z, plane, self, xs[3];
+    int c, base, plane, self, xs[3];
     int ahead[N], behind[N];  // rows of r + c e_last + dy and of their mirror images, by dy + 1 (3-D)
     bool run;                 // the group has a cell of its own
     // first: the first cell of the block (cells first .. ncell are the block's and its successors')
@@ -228,6 +311,7 @@ template <int D> struct LaneCell {
         c = lane % 3;
         base = lane < 30 ? lane - c : 27;  // (lanes 30 and 31 only take part in the shuffles)
         run = lane < 30 && cell < ncell;
+        int x, y, z;
         cell_coords(run ? cell : 0, ncell, nx, ny, x, y, z);
         self = x + pitch * (y + ny * z);
         xs[0] = wrapi(x - 1, nx);
@@ -241,41 +325,49 @@ template <int D> struct LaneCell {
         }
         run = run && LBM_CHECK(self >= 0 && self < plane, status);
     }
-    __device__ __forceinline__ void load(const double *A, int odd, double (&f)[F]) const {
-#pragma unroll
-        for (int p = 0; p < F; ++p) {
-            f[p] = 0.0;  // f_i(r) = A[opp(i)][r - c_i] on odd steps
-            if (run && odd) f[p] = ld_pop<true>(A + (Q - 1 - p - F * c) * plane + behind[D == 3 ? p / 3 : 0] + xs[1 - cxo(p)]);
-            if (run && !odd) f[p] = ld_pop<true>(A + (p + F * c) * plane + self);
-        }
+    // where direction p + F c is read and written
+    __device__ __forceinline__ int in(int p, int odd) const {
+        return odd ? (Q - 1 - p - F * c) * plane + behind[D == 3 ? p / 3 : 0] + xs[1 - cxo(p)] : (p + F * c) * plane + self;
     }
-    __device__ __forceinline__ void store(double *A, int odd, const double (&f)[F]) const {
-#pragma unroll
-        for (int p = 0; p < F; ++p) {
-            if (run && odd) A[(p + F * c) * plane + ahead[D == 3 ? p / 3 : 0] + xs[1 + cxo(p)]] = f[p];
-            if (run && !odd) A[(Q - 1 - p - F * c) * plane + self] = f[p];
-        }
+    __device__ __forceinline__ int out(int p, int odd) const {
+        return odd ? (p + F * c) * plane + ahead[D == 3 ? p / 3 : 0] + xs[1 + cxo(p)] : (Q - 1 - p - F * c) * plane + self;
     }
 };
 
 // Several steps of an FP64 lattice of at most 40 cells an SM: a warp of ten cells to each quarter,
 // one cell to a group of lanes.  Entropic with bulk correction, a cell per thread against three
-// lanes: 64^2 5.1 -> 4.0 us a step, 80 x 76 5.1 -> 4.2, 16^3 9.4 -> 6.0, 20 x 16 x 19 9.5 -> 6.4.
+// lanes (with the grid's barrier in both): 64^2 5.1 -> 4.0 us a step, 80 x 76 5.1 -> 4.2,
+// 16^3 9.4 -> 6.0, 20 x 16 x 19 9.5 -> 6.4.
 template <int D, int EQ, bool BULK>
 __global__ void __launch_bounds__(128) k_steps_lanes(const lbmh::StepArgs a, int nsteps) {
+    using W = Msg<P_F64>::W;
+    constexpr int F = lane_pops(D);
     double *A = static_cast<double *>(a.lat.A);
+    W *M = reinterpret_cast<W *>(static_cast<char *>(a.msg) + lbmh::kMsgHead);
+    const unsigned step0 = __ldcg(&static_cast<const MsgHead *>(a.msg)->step);
     const LaneCell<D> cell((int)(blockIdx.x * (blockDim.x / 32) * 10), (int)a.lat.ncell, a.lat.nx, a.lat.ny, a.lat.nz,
                            a.lat.pitch, (int)a.lat.plane, a.status);  // Q * plane < 2^31 (checked on the host)
     bool ok = true;
-    for (int s = 0; s < nsteps && ok; ++s) {
+    for (int s = 0; s < nsteps; ++s) {
         const int odd = (a.odd + s) & 1;
-        double f[LaneCell<D>::F];
-        cell.load(A, odd, f);
+        double f[F] = {};
+        if (s == 0) {
+#pragma unroll
+            for (int p = 0; p < F; ++p) if (cell.run) f[p] = A[cell.in(p, odd)];
+        } else {
+            ok = msg_take<P_F64>(M, step0 + s, f, [&](int p) { return cell.in(p, odd); }, cell.run, a.status, a.timeout_ns);
+            if (!ok) break;
+        }
         collide_lanes<D, EQ, BULK>(f, cell.c, cell.base, a.rho0, a.omega0, a.six_nu);
-        cell.store(A, odd, f);
-        if (s + 1 < nsteps) ok = grid_barrier(a.sync, (unsigned)(s + 1), a.status, a.timeout_ns);
+        if (cell.run) {
+#pragma unroll
+            for (int p = 0; p < F; ++p) {
+                if (s + 1 == nsteps) A[cell.out(p, odd)] = f[p];
+                else Msg<P_F64>::give(M + cell.out(p, odd), step0 + s + 1, f[p]);
+            }
+        }
     }
-    steps_finish(a, ok);
+    steps_finish(a, nsteps, ok);
 }
 
 template <int D> const void *lanes_kernel_d(int eq, int bulk) {
@@ -288,9 +380,13 @@ template <int D> const void *lanes_kernel_d(int eq, int bulk) {
     return nullptr;
 }
 
-template <int D, int P> const void *small_kernel_dp(int eq, int bulk) {
-#define LBM_SMALL(EQv) \
-    if (eq == EQv) return bulk ? (const void *)k_steps_small<D, P, EQv, true> : (const void *)k_steps_small<D, P, EQv, false>;
+template <int D, int P> const void *small_kernel_dp(int eq, int bulk, bool many) {
+    constexpr int B = lbmh::small_blocks(D, P);
+#define LBM_SMALL(EQv)                                                                          \
+    if (eq == EQv && !many)                                                                     \
+        return bulk ? (const void *)k_steps_small<D, P, EQv, true, 1> : (const void *)k_steps_small<D, P, EQv, false, 1>; \
+    if (eq == EQv)                                                                              \
+        return bulk ? (const void *)k_steps_small<D, P, EQv, true, B> : (const void *)k_steps_small<D, P, EQv, false, B>;
     LBM_SMALL(EQ_ENT)
     LBM_SMALL(EQ_POLY2)
     LBM_SMALL(EQ_PROD)

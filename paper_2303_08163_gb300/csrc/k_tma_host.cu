@@ -117,7 +117,7 @@ static bool chain_geom(const Lattice &lat, const TmaShape &t, int nsteps, lbmd::
 
 // (a grid barrier's counters share the space of the done counters)
 int64_t sync_units(const Lattice &lat) {
-    return std::max<int64_t>(kBarStride * (1 + kBarCounters), std::min<int64_t>((int64_t)lat.ny * lat.nz, (int64_t)1 << 22));
+    return std::min<int64_t>((int64_t)lat.ny * lat.nz, (int64_t)1 << 22);
 }
 
 int64_t tma_max_steps(const Lattice &lat, const TmaShape &t) {

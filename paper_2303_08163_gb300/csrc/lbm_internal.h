@@ -31,6 +31,7 @@ struct StepArgs {
     double *partials;             // [blocks][8] when diag
     int32_t *status;              // device status word (LBM_ETIMEOUT on a timed-out wait)
     unsigned *sync;               // several steps a launch: ticket, exit and done counters (zero between launches)
+    void *msg;                    // steps of a small lattice: step number and words (zero at first)
     int64_t timeout_ns;           // limit of every bounded device wait
 };
 
@@ -46,8 +47,7 @@ struct TmaShape {
 };
 
 constexpr int kDiagWords = 8;  // mass, jx, jy, jz, kinetic, max|u|, nonfinite, unused
-constexpr int kBarCounters = 16;  // counters of a grid barrier in StepArgs::sync, the first at kBarStride,
-constexpr int kBarStride = 32;    // one to a 128-byte line
+constexpr int kBarStride = 32;  // counters of team barriers, one to a 128-byte line
 constexpr int kSyncDone = 4;  // first done counter in StepArgs::sync (after the ticket and exit counters)
 constexpr int kTmaMaxStages = 8;  // deepest shared-memory pipeline of the TMA row kernel
 
@@ -61,7 +61,13 @@ cudaError_t step_generic(const StepArgs &a, int blocks, int threads, cudaStream_
 struct SmallShape {
     int threads = 0, blocks = 0;
     bool lanes = false;  // an FP64 cell on three lanes (k_steps_lanes)
+    bool many = false;   // several blocks to an SM: the kernel with fewer registers
 };
+// Blocks of 256 threads an SM that kernel's registers allow (P: 0 FP64, 1 FP32, 2 binary16).
+constexpr int small_blocks(int D, int P) { return D == 2 ? (P == 2 ? 5 : 4) : P == 0 ? 2 : 3; }
+// Bytes of StepArgs::msg, its words after the first kMsgHead.
+constexpr int kMsgHead = 256;
+size_t small_msg_bytes(const Lattice &lat);
 bool small_shape(const Lattice &lat, int eq, int bulk, int sms, SmallShape &t);
 cudaError_t steps_small(const StepArgs &a, int nsteps, const SmallShape &t, cudaStream_t s);
 cudaError_t init_fields(const Lattice &lat, int eq, double rho0, const void *rho, const void *u,
