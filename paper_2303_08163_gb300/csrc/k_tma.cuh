@@ -46,6 +46,17 @@ constexpr int kTmaMaxThreads = 256;  // consumer threads of the D3Q27 kernels; o
 // D2Q9 binary16 kernels (under 100 registers) may run up to 512 consumers
 __host__ __device__ constexpr int tma_max_threads(int D, int P) { return D == 2 && P == 2 ? 512 : kTmaMaxThreads; }
 
+// Division by a number fixed for the launch (dividends below 2^31): see the loader.
+struct FastDiv {
+    unsigned d, m, s;
+};
+__host__ inline FastDiv fast_div(unsigned d) {
+    unsigned s = 0;
+    while (s < 31 && (1u << s) < d) ++s;
+    return {d, (unsigned)((((uint64_t)1 << (31 + s)) + d - 1) / d), 31 + s};  // m d - 2^(31+s) < d <= 2^s
+}
+__device__ __forceinline__ unsigned div_by(unsigned n, const FastDiv &f) { return (unsigned)(((uint64_t)n * f.m) >> f.s); }
+
 // bufstride (elements between direction buffers) equals the compile-time buffer
 // capacity CAPB / sizeof(storage) of the kernel instantiation.  rowstride is the distance
 // between the rows of a job in shared memory: the row pitch for whole rows (the copies
@@ -55,6 +66,7 @@ struct TmaGeom {
     int64_t njobs;
     // several steps in one launch (nsteps > 1), see decode_chain
     int nsteps, npos, ncross, strips, stripw, pjobs, depth, lag;
+    FastDiv by_nseg, by_ygroups, by_npos, by_strips, by_pjobs, by_depth;
 };
 
 constexpr int kTmaCaps[4] = {1024, 2048, 4096, 8192};  // bytes per direction buffer
@@ -77,8 +89,8 @@ __device__ __forceinline__ JobPos job_at(const lbmh::StepArgs &a, const TmaGeom 
 
 // One step (nsteps == 1): job number -> rows and segment.
 __device__ __forceinline__ JobPos decode_job(const lbmh::StepArgs &a, const TmaGeom &g, unsigned job) {
-    const unsigned rest = job / (unsigned)g.nseg;
-    const unsigned zq = rest / (unsigned)g.ygroups;
+    const unsigned rest = div_by(job, g.by_nseg);
+    const unsigned zq = div_by(rest, g.by_ygroups);
     return job_at(a, g, (int)zq, (int)(rest - zq * (unsigned)g.ygroups), (int)(job - rest * (unsigned)g.nseg), a.odd);
 }
 
@@ -120,26 +132,27 @@ __host__ __device__ __forceinline__ void chain_strip(const TmaGeom &g, int k, in
 
 __device__ __forceinline__ ChainJob decode_chain(const lbmh::StepArgs &a, const TmaGeom &g, unsigned ticket) {
     ChainJob r;
-    const unsigned slot = ticket / (unsigned)g.pjobs;
+    const unsigned slot = div_by(ticket, g.by_pjobs);
     const unsigned jj = ticket - slot * (unsigned)g.pjobs;
-    const unsigned phase = slot / (unsigned)g.depth;
+    const unsigned phase = div_by(slot, g.by_depth);
     const int t = (int)(slot - phase * (unsigned)g.depth);
     const int x = (int)phase - g.lag * t;
     r.step = -1;
     r.p = r.c = 0;
     r.j = JobPos{0, 0, 0, 0, 0, 0};
     if (x < 0) return r;
-    const int qk = x / g.npos, i = x - qk * g.npos, q = qk / g.strips, k = qk - q * g.strips;
+    const int qk = (int)div_by((unsigned)x, g.by_npos), i = x - qk * g.npos;
+    const int q = (int)div_by((unsigned)qk, g.by_strips), k = qk - q * g.strips;
     const int s = q * g.depth + t;
     if (s >= g.nsteps) return r;
     int lo, hi;
     chain_strip(g, k, t, lo, hi);
-    const unsigned row = jj / (unsigned)g.nseg;
+    const unsigned row = div_by(jj, g.by_nseg);
     int c = lo + (int)row;
     if (c >= hi) return r;
     if (c >= g.ncross) c -= g.ncross;
     r.step = s;
-    r.p = (int)(((unsigned)s + (unsigned)i) % (unsigned)g.npos);
+    r.p = s + i - (int)div_by((unsigned)(s + i), g.by_npos) * g.npos;
     r.c = c;
     const bool flat = a.lat.D == 2;
     r.j = job_at(a, g, flat ? 0 : r.p, flat ? r.p : c, (int)(jj - row * (unsigned)g.nseg), (a.odd + s) & 1);
@@ -195,65 +208,77 @@ __device__ __forceinline__ bool bulk_ok(const lbmh::StepArgs &a, const TmaGeom &
 #endif
 }
 
-// Loads of buffer b of a job into its stage (issued by producer lane b).
+// What lane b of the loader and the storer knows of buffer b for the whole launch: its velocity and
+// the planes it is filled from on even and odd steps.
+template <typename T> struct LaneBuf {
+    int b, cx, cy, cz;
+    T *even, *odd;
+};
+template <int D, typename T>
+__device__ __forceinline__ LaneBuf<T> lane_buf(const lbmh::StepArgs &a, int lane) {
+    constexpr int Q = qof(D);
+    const int b = lane < Q ? lane : 0;
+    T *A = static_cast<T *>(a.lat.A);
+    return {b, cxo(b), cyo(b), D == 3 ? czo(b) : 0, A + (int64_t)b * a.lat.plane, A + (int64_t)(Q - 1 - b) * a.lat.plane};
+}
+
+// The rows of a job's buffer in global memory: `first` of them from `at`, the others (past the
+// periodic edge) from `rest`.
+template <typename T> struct JobRows {
+    T *at, *rest;
+    int first;
+};
+template <int D, typename T>
+__device__ __forceinline__ JobRows<T> job_rows(const lbmh::StepArgs &a, const JobPos &j, const LaneBuf<T> &l) {
+    const int ny = a.lat.ny;
+    const int z = D == 3 && j.odd ? wrapi(j.z - l.cz, a.lat.nz) : j.z, y = j.odd ? wrapi(j.y0 - l.cy, ny) : j.y0;
+    T *plane = (j.odd ? l.odd : l.even) + ((int64_t)z * ny) * a.lat.pitch + j.X0;
+    return {plane + (int64_t)y * a.lat.pitch, plane, min(j.nrows, ny - y)};
+}
+
+// Loads of a lane's buffer of a job into its stage.
 template <int D, typename T>
 __device__ __forceinline__ void tma_issue_loads(const lbmh::StepArgs &a, const TmaGeom &g,
-                                                const JobPos &j, int b, T *st, uint64_t *bar) {
+                                                const JobPos &j, const LaneBuf<T> &l, T *st, uint64_t *bar) {
     constexpr int U = 16 / (int)sizeof(T);
-    const int nx = a.lat.nx, ny = a.lat.ny;
-    T *sbuf = st + (int64_t)b * g.bufstride;
-    int r = 0;
-    while (r < j.nrows) {
-        const int ysrc = j.odd ? wrapi(j.y0 + r - cyo(b), ny) : j.y0 + r;
-        const int run = min(j.nrows - r, ny - ysrc);
-        const T *src = buffer_row<D, T>(a, j.odd, b, j.z, j.y0 + r) + j.X0;
-        T *dst = sbuf + r * g.rowstride + g.halo;
-        const uint32_t bytes = (uint32_t)(run * copy_len(g, j) * (int)sizeof(T));
-        if (bulk_ok<D, T>(a, g, st, dst, src, bytes)) bulk_g2s(dst, src, bytes, bar);
-        r += run;
+    const int nx = a.lat.nx, n = copy_len(g, j) * (int)sizeof(T);
+    const JobRows<T> rows = job_rows<D, T>(a, j, l);
+    T *sbuf = st + l.b * g.bufstride;
+    T *dst = sbuf + g.halo;
+    if (bulk_ok<D, T>(a, g, st, dst, rows.at, rows.first * n)) bulk_g2s(dst, rows.at, rows.first * n, bar);
+    if (rows.first < j.nrows) {
+        T *d2 = dst + rows.first * g.rowstride;
+        const uint32_t bytes = (j.nrows - rows.first) * n;
+        if (bulk_ok<D, T>(a, g, st, d2, rows.rest, bytes)) bulk_g2s(d2, rows.rest, bytes, bar);
     }
-    if (j.odd && g.nseg > 1) {
-        const T *grow = buffer_row<D, T>(a, j.odd, b, j.z, j.y0);
-        if (cxo(b) == 1) {
-            const int xs = j.X0 == 0 ? nx - U : j.X0 - U;
-            if (bulk_ok<D, T>(a, g, st, sbuf, grow + xs, U * sizeof(T))) bulk_g2s(sbuf, grow + xs, U * sizeof(T), bar);
-        } else if (cxo(b) == -1) {
-            const int xs = (j.X0 + j.len == nx) ? 0 : j.X0 + j.len;
-            T *dst = sbuf + g.halo + j.len;
-            if (bulk_ok<D, T>(a, g, st, dst, grow + xs, U * sizeof(T))) bulk_g2s(dst, grow + xs, U * sizeof(T), bar);
-        }
+    if (j.odd && g.nseg > 1 && l.cx != 0) {  // the halo (one row)
+        const int x = l.cx == 1 ? (j.X0 == 0 ? nx - U : j.X0 - U) : (j.X0 + j.len == nx ? 0 : j.X0 + j.len);
+        const T *src = rows.at + (x - j.X0);
+        T *d2 = l.cx == 1 ? sbuf : dst + j.len;
+        if (bulk_ok<D, T>(a, g, st, d2, src, U * sizeof(T))) bulk_g2s(d2, src, U * sizeof(T), bar);
     }
 }
 
-// Stores of buffer b of a job back to global memory (issued by producer lane b).
+// Stores of a lane's buffer of a job back to global memory.
 template <int D, typename T>
 __device__ __forceinline__ void tma_issue_stores(const lbmh::StepArgs &a, const TmaGeom &g,
-                                                 const JobPos &j, int b, T *st) {
+                                                 const JobPos &j, const LaneBuf<T> &l, T *st) {
     constexpr int U = 16 / (int)sizeof(T);
-    const int ny = a.lat.ny;
-    T *sbuf = st + (int64_t)b * g.bufstride;
+    const JobRows<T> rows = job_rows<D, T>(a, j, l);
+    const T *src = st + l.b * g.bufstride + g.halo;
     if (!(j.odd && g.nseg > 1)) {
-        int r = 0;
-        while (r < j.nrows) {
-            const int ysrc = j.odd ? wrapi(j.y0 + r - cyo(b), ny) : j.y0 + r;
-            const int run = min(j.nrows - r, ny - ysrc);
-            T *dst = buffer_row<D, T>(a, j.odd, b, j.z, j.y0 + r) + j.X0;
-            const T *src = sbuf + r * g.rowstride + g.halo;
-            const uint32_t bytes = (uint32_t)(run * copy_len(g, j) * (int)sizeof(T));
-            if (bulk_ok<D, T>(a, g, st, src, dst, bytes)) bulk_s2g(dst, src, bytes);
-            r += run;
+        const int n = copy_len(g, j) * (int)sizeof(T);
+        if (bulk_ok<D, T>(a, g, st, src, rows.at, rows.first * n)) bulk_s2g(rows.at, src, rows.first * n);
+        if (rows.first < j.nrows) {
+            const T *s2 = src + rows.first * g.rowstride;
+            const uint32_t bytes = (j.nrows - rows.first) * n;
+            if (bulk_ok<D, T>(a, g, st, s2, rows.rest, bytes)) bulk_s2g(rows.rest, s2, bytes);
         }
-    } else {
-        T *grow = buffer_row<D, T>(a, j.odd, b, j.z, j.y0);
-        if (cxo(b) == 0) {
-            const uint32_t bytes = (uint32_t)(j.len * (int)sizeof(T));
-            if (bulk_ok<D, T>(a, g, st, sbuf + g.halo, grow + j.X0, bytes)) bulk_s2g(grow + j.X0, sbuf + g.halo, bytes);
-        } else if (j.len > U) {
-            const int off = cxo(b) == 1 ? 0 : U;  // skip the ragged end the plain stores take
-            const uint32_t bytes = (uint32_t)((j.len - U) * (int)sizeof(T));
-            if (bulk_ok<D, T>(a, g, st, sbuf + g.halo + off, grow + j.X0 + off, bytes))
-                bulk_s2g(grow + j.X0 + off, sbuf + g.halo + off, bytes);
-        }
+    } else if (l.cx == 0 || j.len > U) {
+        // (one row) without the ragged end the plain stores take
+        const int off = l.cx == -1 ? U : 0;
+        const uint32_t bytes = (uint32_t)((l.cx == 0 ? j.len : j.len - U) * (int)sizeof(T));
+        if (bulk_ok<D, T>(a, g, st, src + off, rows.at + off, bytes)) bulk_s2g(rows.at + off, src + off, bytes);
     }
 }
 
@@ -351,7 +376,7 @@ __device__ __forceinline__ void tma_compute(const lbmh::StepArgs &a, const TmaGe
             six_nu = step_scalar<R>(a.six_nu, a.six_nuf);
     const int ncells = j.nrows * j.len;
     DiagLocal<R> loc;
-    int r = tid / j.len;
+    int r = tid < j.len ? 0 : tid / j.len;  // (mostly 0)
     int xl = tid - r * j.len;
     for (int c = tid; c < ncells; c += nthr) {
         const CellPos p = cell_pos(g, r, xl, j.len);
@@ -416,7 +441,7 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
     const int hl = j.len >> 1;  // len is even here
     const int npairs = j.nrows * hl;
     DiagLocal<float> loc;
-    int r = tid / hl;
+    int r = tid < hl ? 0 : tid / hl;  // (mostly 0)
     int xh = tid - r * hl;
     for (int c = tid; c < npairs; c += nthr) {
         T *row = st + r * g.rowstride + g.halo;
@@ -532,7 +557,15 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
     DiagAcc acc;
     bool failed = false;
     if (role == 1) {
-        // loader: takes the jobs, waits for the steps they need, refills the stages
+        // loader: takes the jobs, waits for the steps they need, refills the stages.  Its work for a
+        // job, like the storer's, is one serial chain, and a block gets no more jobs than they can
+        // handle: measured in clocks a job (4096^2 FP32, 6400 in all), decoding 1950 (eleven divisions,
+        // hence FastDiv), the counters and the full proxy fence 2200, issuing the copies 1750, and in
+        // the storer issue 1300, wait 1900, another proxy fence and the release 2100.  Without the
+        // divisions, with the fence on global memory only and none in the storer: 5600.  Several steps
+        // a launch: 4096^2 FP32 118 -> 142 GLUPS, 4096^2 binary16 184 -> 205, 256^3 FP32 41.4 -> 46.0,
+        // 512^3 binary16 73 -> 78.  (Two tickets at a time, decoded by half a warp each: 4 - 8 % slower.)
+        const LaneBuf<T> buf = lane_buf<D, T>(a, lane);
         const unsigned total = chain ? (unsigned)chain_tickets(g) : (unsigned)g.njobs;
         unsigned next = blockIdx.x;
         if (chain && lane == 0) next = atomicAdd(&a.sync[0], 1u);
@@ -578,7 +611,7 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
                     end = true;
                 }
                 // what other SMs' copy engines and threads wrote, before this SM's copy engine reads
-                fence_proxy_async();
+                fence_proxy_async_global();
             }
             if (lane == 0) {
                 if (end) jp.nrows = 0;
@@ -587,7 +620,7 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
                 mbar_arrive_expect_tx(&full[s], end ? 0u : tma_job_bytes<D, T>(a, g, jp));
             }
             if (end) break;
-            if (lane < Q) tma_issue_loads<D, T>(a, g, jp, lane, sm + s * stage_elems, &full[s]);
+            if (lane < Q) tma_issue_loads<D, T>(a, g, jp, buf, sm + s * stage_elems, &full[s]);
             if (++s == S) {
                 s = 0;
                 phase ^= 1u;
@@ -596,6 +629,7 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
         }
     } else if (role == 2) {
         // storer: writes collided stages back, frees them, and reports finished jobs
+        const LaneBuf<T> buf = lane_buf<D, T>(a, lane);
         int s = 0;
         uint32_t phase = 0;
         for (;;) {
@@ -609,14 +643,15 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
             if (jq.nrows == 0) break;
             T *st = sm + s * stage_elems;
             if (jq.odd && g.nseg > 1) tma_plain_stores<D, T>(a, g, jq, st, lane, 32);
-            if (lane < Q) tma_issue_stores<D, T>(a, g, jq, lane, st);
+            if (lane < Q) tma_issue_stores<D, T>(a, g, jq, buf, st);
             bulk_commit();
             bulk_wait_read<0>();
             __syncwarp();
             if (lane == 0) mbar_arrive_cta(&freed[s]);
             if (chain) {
+                // (a completed group's writes are visible to its thread; another proxy fence here
+                // held the storer for some 800 clocks a job)
                 bulk_wait_all();
-                fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) red_release(&a.sync[lbmh::kSyncDone + unit], 1u);
             }
