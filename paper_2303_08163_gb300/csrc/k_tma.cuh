@@ -429,7 +429,10 @@ __device__ __forceinline__ void st_pair(float *b, int p, f32x2 v) {
 
 // MODE 0: even step; 1: odd step, whole rows; 2: odd step, segments; -1: chosen at run
 // time from the step parity and the job layout (one loop body for all three).
-template <int D, int P, int EQ, bool BULK, int CAPB, int MODE>
+// LONE: rows of odd length, in pairs as well (cell by cell before: 2047 x 2000 FP32 77 -> 102 GLUPS,
+// binary16 161 -> 206; 301 x 200 x 200 binary16 56 -> 61; FP32 in 3-D is bound elsewhere).  Another copy
+// of the body: with both in one, 512^3 binary16 72 against 79 GLUPS.
+template <int D, int P, int EQ, bool BULK, int CAPB, int MODE, bool LONE>
 __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const TmaGeom &g,
                                                   const JobPos &j, typename Storage<P>::T *st, DiagAcc &acc,
                                                   int tid, int nthr) {
@@ -437,8 +440,11 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
     using T = typename St::T;
     constexpr int Q = qof(D);
     constexpr int bs = CAPB / (int)sizeof(T);  // elements between direction buffers
-    const int mode = MODE >= 0 ? MODE : (!j.odd ? 0 : (g.nseg == 1 ? 1 : 2));
-    const int hl = j.len >> 1;  // len is even here
+    const int mode = MODE >= 0 ? MODE : (!j.odd ? 0 : (LONE || g.nseg == 1 ? 1 : 2));
+    // Rows of odd length are padded whole rows: their last pair of the even step is a cell and an element
+    // of the padding; in the odd step the first pair is cell 0 twice, and the others follow.
+    constexpr int lone = LONE ? 1 : 0;
+    const int hl = (j.len + lone) >> 1;
     const int npairs = j.nrows * hl;
     DiagLocal<float> loc;
     int r = tid < hl ? 0 : tid / hl;  // (mostly 0)
@@ -448,19 +454,30 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
         // cells xa and xb = xa + 1 (the odd pairing of whole rows wraps its last pair to
         // cell 0); pm = xa - 1 and pp = xb + 1 are the outer neighbours, inside the row for
         // whole rows (xa >= 1 in the odd pairing) and in the halos for segments
-        const int xa = 2 * xh + (mode == 1 ? 1 : 0);
-        const int xb = (mode == 1 && xa + 1 == j.len) ? 0 : xa + 1;
+        const bool twice = LONE && mode == 1 && xh == 0;
+        const int xa = twice ? 0 : 2 * xh + (mode == 1 ? 1 - 2 * lone : 0);
+        const int xb = twice || (mode == 1 && xa + 1 == j.len) ? 0 : xa + 1;
+        // its neighbours are not at consecutive positions
+        const bool apart = LONE && mode == 1 && (twice || xb + 1 == j.len);
         const int pm = xa - 1;
         const int pp = xb + 1;
         // checked builds: every position the pair touches lies inside its direction buffer
         const int row_off = r * g.rowstride + g.halo;
-        const int lo = mode == 0 ? xa : min(min(pm, xa), xb);
-        const int hi = mode == 0 ? xa + 1 : max(max(xb + 1, pp), xa);
+        const int lo = mode == 0 ? xa : twice ? 0 : min(min(pm, xa), xb);
+        const int hi = mode == 0 ? xa + 1 : twice ? j.len - 1 : max(max(xb + 1, pp), xa);
         if (LBM_CHECK(row_off + lo >= 0 && row_off + hi < bs, a.status)) {
             f32x2 f[Q];
             if (mode == 0) {
     #pragma unroll
                 for (int i = 0; i < Q; ++i) f[i] = ld_pair(row + i * bs, xa);
+            } else if (apart) {
+                const int ma = twice ? j.len - 1 : pm, mb = twice ? ma : xa, qa = twice ? 1 : xb, qb = twice ? 1 : 0;
+    #pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const T *b = row + i * bs;
+                    f[i] = cxo(i) == 0 ? pack2(St::load(b[xa]), St::load(b[xb]))
+                                       : cxo(i) == 1 ? pack2(St::load(b[ma]), St::load(b[mb])) : pack2(St::load(b[qa]), St::load(b[qb]));
+                }
             } else if (mode == 1) {
     #pragma unroll
                 for (int i = 0; i < Q; ++i) {
@@ -491,6 +508,9 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
                         if (cxo(i) == 0) {
                             b[xa] = St::store(va);
                             b[xb] = St::store(vb);
+                        } else if (apart) {
+                            b[cxo(i) == 1 ? (twice ? 1 : xb) : (twice ? j.len - 1 : pm)] = St::store(va);
+                            b[cxo(i) == 1 ? (twice ? 1 : 0) : (twice ? j.len - 1 : xa)] = St::store(vb);
                         } else {
                             st_pair(b, cxo(i) == 1 ? xb : pm, f[i]);
                         }
@@ -513,7 +533,7 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
     #pragma unroll
                 for (int q = 0; q < 3; ++q) unpack2(m.u[q], ua[q], ub[q]);
                 loc.add(ra, ua, a.rho0f);
-                loc.add(rb, ub, a.rho0f);
+                if (!LONE || (!twice && xb < j.len)) loc.add(rb, ub, a.rho0f);
             }
         }
         xh += nthr;
@@ -677,19 +697,23 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
             const JobPos jp = jobq[s];
             if (jp.nrows > 0) {
                 T *st = sm + s * stage_elems;
-                if (P == P_F64 || (jp.len & 1)) {
+                if constexpr (P == P_F64) {
                     tma_compute<D, P, EQ, BULK, CAPB>(a, g, jp, st, acc, threadIdx.x, ncons);
-                } else if constexpr (P != P_F64 && D == 3) {
+                } else if (jp.len & 1) {
+                    if (D == 3) tma_compute_pairs<D, P, EQ, BULK, CAPB, -1, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else if (jp.odd) tma_compute_pairs<D, P, EQ, BULK, CAPB, D == 3 ? -1 : 1, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else tma_compute_pairs<D, P, EQ, BULK, CAPB, D == 3 ? -1 : 0, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                } else if constexpr (D == 3) {
                     // the D3Q27 pair body is long: one copy serves the three pairings (three
                     // specialised copies measured slower)
-                    tma_compute_pairs<D, P, EQ, BULK, CAPB, -1>(a, g, jp, st, acc, threadIdx.x, ncons);
-                } else if constexpr (P != P_F64) {
+                    tma_compute_pairs<D, P, EQ, BULK, CAPB, -1, false>(a, g, jp, st, acc, threadIdx.x, ncons);
+                } else {
                     if (!jp.odd)
-                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 0>(a, g, jp, st, acc, threadIdx.x, ncons);
+                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 0, false>(a, g, jp, st, acc, threadIdx.x, ncons);
                     else if (g.nseg == 1)
-                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 1>(a, g, jp, st, acc, threadIdx.x, ncons);
+                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 1, false>(a, g, jp, st, acc, threadIdx.x, ncons);
                     else
-                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 2>(a, g, jp, st, acc, threadIdx.x, ncons);
+                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 2, false>(a, g, jp, st, acc, threadIdx.x, ncons);
                 }
                 fence_proxy_async_smem();
                 __syncwarp();
