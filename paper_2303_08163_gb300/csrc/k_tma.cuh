@@ -697,7 +697,11 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
             const JobPos jp = jobq[s];
             if (jp.nrows > 0) {
                 T *st = sm + s * stage_elems;
+                // One step a launch of D3Q27 is bound by HBM (0.97 of the copy peak), and two cells a
+                // thread only bunch its accesses: 512^3 binary16 60.1 GLUPS against 56.8.
                 if constexpr (P == P_F64) {
+                    tma_compute<D, P, EQ, BULK, CAPB>(a, g, jp, st, acc, threadIdx.x, ncons);
+                } else if (D == 3 && !chain && !(jp.len & 1)) {
                     tma_compute<D, P, EQ, BULK, CAPB>(a, g, jp, st, acc, threadIdx.x, ncons);
                 } else if (jp.len & 1) {
                     if (D == 3) tma_compute_pairs<D, P, EQ, BULK, CAPB, -1, true>(a, g, jp, st, acc, threadIdx.x, ncons);

@@ -43,3 +43,31 @@ def test_fp32_populations_round_like_fp64_sums(D, dims, prec):
         f = back.astype(np.float64)
         assert np.allclose(r, rho0 + f.sum(0), rtol=0, atol=1e-12 if prec == 0 else 64 * 2 ** -24)
     lat.close()
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("D,dims", [(3, (66, 5, 3)), (2, (64, 3, 1))])
+def test_outputs_that_start_between_pairs(D, dims, dtype):
+    """Device outputs aligned to one value only, against aligned ones: the same bits."""
+    import torch
+    from paper_2303_08163_gb300 import lbm
+    rho, u = inputs.random_state(D, dims, seed=8, u_max=0.1)
+    lat = lbm.Lattice(D - 2, dims, 0.6, 0, 0, 2)
+    lat.init_fields(rho, u)
+    td = torch.float32 if dtype == np.float32 else torch.float64
+    n = lat.ncell
+
+    def take(off):
+        r = torch.zeros(n + 4, dtype=td, device="cuda")[off:off + n]
+        v = torch.zeros(D * n + 4, dtype=td, device="cuda")[off:off + D * n].view(D, n)
+        f = torch.zeros(lat.Q * n + 4, dtype=td, device="cuda")[off:off + lat.Q * n].view(lat.Q, n)
+        lat.moments(dtype, out=(r, v))
+        lat.get_populations(dtype, out=f)
+        torch.cuda.synchronize()
+        return r, v, f
+
+    for steps in (0, 1):
+        lat.step(steps)
+        for a, b in zip(take(0), take(1)):
+            assert torch.equal(a, b)
+    lat.close()
