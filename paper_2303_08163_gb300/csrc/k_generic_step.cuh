@@ -73,7 +73,8 @@ __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
     return m;
 }
 
-template <int D, int P, int EQ, bool BULK>
+// DIAG: with the diagnostics' sums (see tma_compute on why not a run-time condition).
+template <int D, int P, int EQ, bool BULK, bool DIAG>
 __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
     using St = Storage<P>;
     using T = typename St::T;
@@ -91,12 +92,12 @@ __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
         cell_coords(cell, a.lat.ncell, nx, ny, x, y, z);
         const CellMoments<R> m = aa_cell_step<D, P, EQ, BULK>(A, a.lat.plane, nx, ny, nz, a.lat.pitch, x, y, z,
                                                               a.odd, rho0, omega0, six_nu, a.status);
-        if (a.diag) {
+        if (DIAG) {
             loc.add(m.rho, m.u, rho0);
             if (loc.count == 16) loc.flush(acc, a.rho0);
         }
     }
-    if (a.diag) {
+    if (DIAG) {
         loc.flush(acc, a.rho0);
         diag_block_store(acc, a.partials + (int64_t)blockIdx.x * lbmh::kDiagWords);
     }
@@ -107,18 +108,19 @@ __global__ void __launch_bounds__(256) k_step_generic(const lbmh::StepArgs a) {
 // A small lattice's steps are bound by latency: a launch, a pipeline's ramp, or in the TMA row
 // kernel's several-step form the way of a row through shared memory and its counters.  Here all
 // its cells are in registers at once, one (or a few) to a thread, in one cooperative launch (all
-// blocks are resident), and no barrier separates the steps: within the launch a population travels
-// in one word with the number of the step that wrote it, through a buffer with the layout of the
-// lattice (rows unpadded: a warp's cells are contiguous across the end of a row, 300^2 binary16
-// 1.8 us a step, 2.7 with the lattice's own padding).  A cell reads a location until it finds its own step's number there.  A location is read
-// and then rewritten by one cell a step (the AA pattern), so nothing can be overwritten before it
-// was read, and a word is written and read whole, so neither fences nor counters are needed: a step
-// is a store, a load and the collision.  The first step reads and the last one writes the lattice's
-// own array.  The numbers go on from launch to launch (the buffer's head, advanced by the last block),
-// so the words of an earlier launch, all one behind the next launch's first, never match.
-// Per step with the TMA row kernel, with a barrier of the whole grid in place of the numbers (release
-// fence, counter, acquire: 1 us), and so: 64^2 FP32 3.9, 1.86, 0.91 us; 64^2 FP64 8.0, 3.45, 2.65;
-// 32^3 binary16 6.1, 2.49, 1.57; 340^2 FP32 4.6, 3.16, 1.95; 48^3 binary16 6.8, 4.5, 4.1.
+// blocks are resident), and no barrier separates the steps: within the launch a population
+// travels in one word with the number of the step that wrote it, through a buffer with the layout
+// of the lattice (rows unpadded: a warp's cells are contiguous across the end of a row, 300^2
+// binary16 1.8 us a step, 2.7 with the lattice's own padding).  A cell reads a location until it
+// finds its own step's number there.  A location is read and then rewritten by one cell a step
+// (the AA pattern), so nothing can be overwritten before it was read, and a word is written and
+// read whole, so neither fences nor counters are needed: a step is a store, a load and the
+// collision.  The first step reads and the last one writes the lattice's own array.  The numbers
+// go on from launch to launch (the buffer's head, advanced by the last block), so the words of an
+// earlier launch, all one behind the next launch's first, never match. Per step with the TMA row
+// kernel, with a barrier of the whole grid in place of the numbers (release fence, counter,
+// acquire: 1 us), and so: 64^2 FP32 3.9, 1.86, 0.91 us; 64^2 FP64 8.0, 3.45, 2.65; 32^3 binary16
+// 6.1, 2.49, 1.57; 340^2 FP32 4.6, 3.16, 1.95; 48^3 binary16 6.8, 4.5, 4.1.
 struct MsgHead {
     unsigned step, exits;
 };
@@ -398,7 +400,8 @@ template <int D, int P>
 cudaError_t launch_generic_dp(const lbmh::StepArgs &a, int blocks, int threads, cudaStream_t s) {
 #define LBM_GEN(EQv, Bv)                                                                   \
     if (a.eq == EQv && a.bulk == Bv) {                                                     \
-        k_step_generic<D, P, EQv, Bv><<<blocks, threads, 0, s>>>(a);                        \
+        if (a.diag) k_step_generic<D, P, EQv, Bv, true><<<blocks, threads, 0, s>>>(a);      \
+        else k_step_generic<D, P, EQv, Bv, false><<<blocks, threads, 0, s>>>(a);            \
         return cudaGetLastError();                                                          \
     }
     LBM_GEN(EQ_ENT, false)

@@ -36,13 +36,15 @@
 // so neighbouring segments never write the same location.
 #pragma once
 
+#include <type_traits>
+
 #include "lbm_common.cuh"
 #include "ptx.cuh"
 
 namespace lbmd {
 
 using lbmh::kTmaMaxStages;
-constexpr int kTmaMaxThreads = 256;  // consumer threads of the D3Q27 kernels; one producer warp more
+constexpr int kTmaMaxThreads = 256;  // consumer threads of the D3Q27 kernels; two service warps more
 // D2Q9 binary16 kernels (under 100 registers) may run up to 512 consumers
 __host__ __device__ constexpr int tma_max_threads(int D, int P) { return D == 2 && P == 2 ? 512 : kTmaMaxThreads; }
 
@@ -364,8 +366,11 @@ __device__ __forceinline__ void tma_store_cell(typename Storage<P>::T *st, const
     }
 }
 
-// Collide every cell of a job in place in its stage, one cell per thread per iteration.
-template <int D, int P, int EQ, bool BULK, int CAPB>
+// Collide every cell of a job in place in its stage, one cell per thread per iteration.  DIAG: with
+// the diagnostics' sums, which only launches of one step have (as a run-time condition their FP64
+// additions took their slots on the FP64 pipe all the same: 512^3 binary16 78.8 -> 80.8 GLUPS, 4096^2
+// binary16 203 -> 221 without).
+template <int D, int P, int EQ, bool BULK, int CAPB, bool DIAG>
 __device__ __forceinline__ void tma_compute(const lbmh::StepArgs &a, const TmaGeom &g,
                                             const JobPos &j, typename Storage<P>::T *st,
                                             DiagAcc &acc, int tid, int nthr) {
@@ -386,7 +391,7 @@ __device__ __forceinline__ void tma_compute(const lbmh::StepArgs &a, const TmaGe
             tma_load_cell<D, P, CAPB>(st, p, j.odd, f);
             const CellMoments<R> m = collide<D, P, EQ, BULK, R>(f, rho0, omega0, six_nu);
             tma_store_cell<D, P, CAPB>(st, p, j.odd, f);
-            if (a.diag) loc.add(m.rho, m.u, rho0);
+            if (DIAG && a.diag) loc.add(m.rho, m.u, rho0);
         }
         xl += nthr;
         while (xl >= j.len) {
@@ -394,7 +399,7 @@ __device__ __forceinline__ void tma_compute(const lbmh::StepArgs &a, const TmaGe
             ++r;
         }
     }
-    if (a.diag) loc.flush(acc, a.rho0);
+    if (DIAG && a.diag) loc.flush(acc, a.rho0);
 }
 
 // FP32 and binary16 storage: two neighbouring cells per thread per iteration, one in each
@@ -432,7 +437,8 @@ __device__ __forceinline__ void st_pair(float *b, int p, f32x2 v) {
 // LONE: rows of odd length, in pairs as well (cell by cell before: 2047 x 2000 FP32 77 -> 102 GLUPS,
 // binary16 161 -> 206; 301 x 200 x 200 binary16 56 -> 61; FP32 in 3-D is bound elsewhere).  Another copy
 // of the body: with both in one, 512^3 binary16 72 against 79 GLUPS.
-template <int D, int P, int EQ, bool BULK, int CAPB, int MODE, bool LONE>
+// DIAG: as in tma_compute.
+template <int D, int P, int EQ, bool BULK, int CAPB, int MODE, bool LONE, bool DIAG>
 __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const TmaGeom &g,
                                                   const JobPos &j, typename Storage<P>::T *st, DiagAcc &acc,
                                                   int tid, int nthr) {
@@ -527,7 +533,7 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
                     }
                 }
             }
-            if (a.diag) {
+            if (DIAG && a.diag) {
                 float ra, rb, ua[3], ub[3];
                 unpack2(m.rho, ra, rb);
     #pragma unroll
@@ -542,7 +548,7 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
             ++r;
         }
     }
-    if (a.diag) loc.flush(acc, a.rho0);
+    if (DIAG && a.diag) loc.flush(acc, a.rho0);
 }
 
 // The warps after the consumers: the loader and the storer.
@@ -697,27 +703,36 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
             const JobPos jp = jobq[s];
             if (jp.nrows > 0) {
                 T *st = sm + s * stage_elems;
-                // One step a launch of D3Q27 is bound by HBM (0.97 of the copy peak), and two cells a
-                // thread only bunch its accesses: 512^3 binary16 60.1 GLUPS against 56.8.
+                const auto pairs = [&](auto mode, auto lone, auto diag) {
+                    tma_compute_pairs<D, P, EQ, BULK, CAPB, mode.value, lone.value, diag.value>(a, g, jp, st, acc, threadIdx.x, ncons);
+                };
+                using std::integral_constant;
+                constexpr std::true_type yes;
+                constexpr std::false_type no;
+                constexpr integral_constant<int, -1> any;
                 if constexpr (P == P_F64) {
-                    tma_compute<D, P, EQ, BULK, CAPB>(a, g, jp, st, acc, threadIdx.x, ncons);
-                } else if (D == 3 && !chain && !(jp.len & 1)) {
-                    tma_compute<D, P, EQ, BULK, CAPB>(a, g, jp, st, acc, threadIdx.x, ncons);
-                } else if (jp.len & 1) {
-                    if (D == 3) tma_compute_pairs<D, P, EQ, BULK, CAPB, -1, true>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else if (jp.odd) tma_compute_pairs<D, P, EQ, BULK, CAPB, D == 3 ? -1 : 1, true>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else tma_compute_pairs<D, P, EQ, BULK, CAPB, D == 3 ? -1 : 0, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    if (chain) tma_compute<D, P, EQ, BULK, CAPB, false>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
                 } else if constexpr (D == 3) {
-                    // the D3Q27 pair body is long: one copy serves the three pairings (three
-                    // specialised copies measured slower)
-                    tma_compute_pairs<D, P, EQ, BULK, CAPB, -1, false>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    // The D3Q27 pair body is long: one copy serves the three pairings (three
+                    // specialised copies measured slower).  One step a launch is bound by HBM (0.97 of the
+                    // copy peak), and two cells a thread only bunch its accesses: 512^3 binary16 60.1
+                    // GLUPS against 56.8.
+                    if (!chain) tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else if (jp.len & 1) pairs(any, yes, no);
+                    else pairs(any, no, no);
                 } else {
-                    if (!jp.odd)
-                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 0, false>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else if (g.nseg == 1)
-                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 1, false>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else
-                        tma_compute_pairs<D, P, EQ, BULK, CAPB, 2, false>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    constexpr integral_constant<int, 0> even;
+                    constexpr integral_constant<int, 1> rows;
+                    constexpr integral_constant<int, 2> segments;
+                    if (!chain && (jp.len & 1)) pairs(any, yes, yes);
+                    else if (!chain) pairs(any, no, yes);
+                    else if (jp.len & 1) {
+                        if (jp.odd) pairs(rows, yes, no);
+                        else pairs(even, yes, no);
+                    } else if (!jp.odd) pairs(even, no, no);
+                    else if (g.nseg == 1) pairs(rows, no, no);
+                    else pairs(segments, no, no);
                 }
                 fence_proxy_async_smem();
                 __syncwarp();

@@ -37,7 +37,7 @@ struct StepArgs {
 
 // Launch shape of the TMA row-staged kernel.
 struct TmaShape {
-    int threads;    // consumer threads per block (one producer warp is added)
+    int threads;    // consumer threads per block (the loader and the storer warp are added)
     int blocks;     // grid size (persistent blocks)
     int stages;     // shared-memory pipeline depth (>= 2)
     int rows;       // rows per job (>= 1; 1 when the row is split into segments)
