@@ -846,6 +846,8 @@ def compare_precisions(torch, lbm, dev, w, args, rho, u, sm_mhz=None):
             gb = 2 * Q * ESIZE[prec] * ncell / (ms * 1e-3) / 1e9
             glups = ncell / (ms * 1e-3) / 1e9
             out[key] = {"GLUPS": glups, "ms_per_step": ms, "GB_s": gb,
+                        # algorithmic bytes of a step: the timed lbm_step(n) passes HBM once for
+                        # several steps, so the fraction may exceed 1
                         "hbm_frac": gb / (measured_peaks().get("hbm_gbs") or 6800.0),
                         "launch": lat.launch_info()}
             if prec == 0:
