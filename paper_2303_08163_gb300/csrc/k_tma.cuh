@@ -711,22 +711,23 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
                 constexpr std::false_type no;
                 constexpr integral_constant<int, -1> any;
                 if constexpr (P == P_F64) {
-                    if (chain) tma_compute<D, P, EQ, BULK, CAPB, false>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    if (a.diag) tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else tma_compute<D, P, EQ, BULK, CAPB, false>(a, g, jp, st, acc, threadIdx.x, ncons);
                 } else if constexpr (D == 3) {
                     // The D3Q27 pair body is long: one copy serves the three pairings (three
                     // specialised copies measured slower).  One step a launch is bound by HBM (0.97 of the
                     // copy peak), and two cells a thread only bunch its accesses: 512^3 binary16 60.1
                     // GLUPS against 56.8.
-                    if (!chain) tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    if (a.diag) tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+                    else if (!chain) tma_compute<D, P, EQ, BULK, CAPB, false>(a, g, jp, st, acc, threadIdx.x, ncons);
                     else if (jp.len & 1) pairs(any, yes, no);
                     else pairs(any, no, no);
                 } else {
                     constexpr integral_constant<int, 0> even;
                     constexpr integral_constant<int, 1> rows;
                     constexpr integral_constant<int, 2> segments;
-                    if (!chain && (jp.len & 1)) pairs(any, yes, yes);
-                    else if (!chain) pairs(any, no, yes);
+                    if (a.diag && (jp.len & 1)) pairs(any, yes, yes);
+                    else if (a.diag) pairs(any, no, yes);
                     else if (jp.len & 1) {
                         if (jp.odd) pairs(rows, yes, no);
                         else pairs(even, yes, no);
