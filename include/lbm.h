@@ -257,8 +257,8 @@ int lbm_batch_init_fields(lbm_batch *b, const void *rho, const void *u, int dtyp
  */
 int lbm_batch_set_probe(lbm_batch *b, const int32_t *kvec, int64_t every_k);
 
-/* Advance every instance by n steps in one persistent kernel launch, replayed from a
- * captured CUDA graph. */
+/* Advance every instance by n steps in one persistent kernel launch (teams of blocks: one per
+ * 2000 steps), replayed from a captured CUDA graph. */
 int lbm_batch_step(lbm_batch *b, int64_t n);
 
 /*

@@ -1581,25 +1581,30 @@ int lbm_batch_step(lbm_batch *b, int64_t n) {
         const int64_t last = b->step + n - 1;
         if ((rc = batch_reserve_series(b, last / b->every_k + 1))) return batch_sticky(b, rc);
     }
-    const BatchArgs a = batch_args(b, n);
-    // one persistent launch, captured into a graph and replayed on the object's stream
-    cudaStream_t cap;
-    CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "batch capture stream");
-    cudaGraph_t g = nullptr;
-    cudaGraphExec_t ge = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        cudaError_t el = batch_launch(b, a, cap);
-        e = cudaStreamEndCapture(cap, &g);
-        if (e == cudaSuccess && el != cudaSuccess) e = el;
+    for (int64_t left = n; left > 0;) {
+        // one persistent launch (of teams: of a bounded number of steps), captured into a graph and
+        // replayed on the object's stream
+        const int64_t m = b->teams && b->team_cluster == 0 ? team_launch_steps(left) : left;
+        const BatchArgs a = batch_args(b, m);
+        cudaStream_t cap;
+        CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "batch capture stream");
+        cudaGraph_t g = nullptr;
+        cudaGraphExec_t ge = nullptr;
+        cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            cudaError_t el = batch_launch(b, a, cap);
+            e = cudaStreamEndCapture(cap, &g);
+            if (e == cudaSuccess && el != cudaSuccess) e = el;
+        }
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
+        if (e == cudaSuccess) e = cudaGraphLaunch(ge, b->stream);
+        if (ge) cudaGraphExecDestroy(ge);
+        if (g) cudaGraphDestroy(g);
+        cudaStreamDestroy(cap);
+        if (e != cudaSuccess) return batch_sticky(b, cuda_fail("batch launch", e));
+        b->step += m;
+        left -= m;
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
-    if (e == cudaSuccess) e = cudaGraphLaunch(ge, b->stream);
-    if (ge) cudaGraphExecDestroy(ge);
-    if (g) cudaGraphDestroy(g);
-    cudaStreamDestroy(cap);
-    if (e != cudaSuccess) return batch_sticky(b, cuda_fail("batch launch", e));
-    b->step += n;
     return LBM_OK;
 }
 

@@ -133,6 +133,9 @@ struct BatchArgs {
     int64_t timeout_ns;
 };
 constexpr int kTeamThreads = 128;  // threads of a team's block
+// Of n steps, those of the next launch of teams.  A team's counter grows by its blocks a step and is
+// compared as a 32-bit number: without a limit 608 blocks of one instance passed 2^32 after 7 million steps.
+constexpr int64_t team_launch_steps(int64_t n) { return n < 2000 ? n : 2000; }
 constexpr int kClusterCells = kTeamThreads / 32 * 10;  // cells of a cluster's block, three lanes each
 constexpr int kClusterBlocks = 8;                      // largest portable cluster
 // Clusters of that many blocks that are resident at once.
