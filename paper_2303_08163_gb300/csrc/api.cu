@@ -438,7 +438,7 @@ bool apply_shape(lbm_ctx *c, const std::vector<int> &v) {
     TmaShape t{};
     if (!shape_from_record(c, v, &kernel, &t, &gt, &gb)) return false;
     if (kernel == 2) {
-        if (tma_prepare(c->lat, c->eq, c->bulk, t.cap, t.smem_bytes) != cudaSuccess) {
+        if (tma_prepare(c->lat, c->eq, c->bulk, t.cap) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
@@ -747,7 +747,7 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
         }
     }
     if (tma_supported(c->lat) && default_tma_shape(c, c->tma)) {
-        tma_prepare(c->lat, c->eq, c->bulk, c->tma.cap, c->tma.smem_bytes);
+        tma_prepare(c->lat, c->eq, c->bulk, c->tma.cap);
         c->kernel = 2;
     }
     cudaGetLastError();
@@ -774,7 +774,7 @@ int lbm_set_option(lbm_ctx *c, int option, int64_t value) {
             if (tma_supported(c->lat)) {
                 if (c->tma.smem_bytes <= 0 && !default_tma_shape(c, c->tma))
                     return fail(LBM_ECUDA, "no TMA launch shape fits this lattice");
-                tma_prepare(c->lat, c->eq, c->bulk, c->tma.cap, c->tma.smem_bytes);
+                tma_prepare(c->lat, c->eq, c->bulk, c->tma.cap);
                 c->kernel = 2;
             } else {
                 c->kernel = 1;
@@ -1109,7 +1109,7 @@ int lbm_set_launch_shape(lbm_ctx *c, const int64_t shape[6]) {
     const int nb = tma_max_blocks_per_sm(c->lat, c->eq, c->bulk, t);
     if (nb < 1) return fail(LBM_EINVAL, "launch shape does not fit on the device");
     t.blocks = sm_count() * nb;
-    CK(tma_prepare(c->lat, c->eq, c->bulk, t.cap, t.smem_bytes), "shared memory attribute");
+    CK(tma_prepare(c->lat, c->eq, c->bulk, t.cap), "shared memory attribute");
     c->tma = t;
     c->kernel = 2;
     c->chosen = true;

@@ -17,6 +17,8 @@ LBM_DECL_CAP(3, 4096)
 LBM_DECL_CAP(3, 8192)
 #undef LBM_DECL_CAP
 
+constexpr int kTmaMaxSmem = 227 * 1024;  // shared memory of a block, static and dynamic
+
 static const void *tma_kernel(const Lattice &lat, int eq, int bulk, int cap) {
     if (lat.D == 2) {
         switch (cap) {
@@ -153,20 +155,28 @@ int tma_smem_bytes(const Lattice &lat, const TmaShape &t) {
     if (g.njobs >= ((int64_t)1 << 31)) return -1;
     if (t.threads < 32 || t.threads > lbmd::tma_max_threads(lat.D, lat.P) || t.threads % 32) return -1;
     const int64_t bytes = (int64_t)t.stages * lbmd::qof(lat.D) * t.cap;
-    return bytes > 227 * 1024 ? -1 : (int)bytes;
+    return bytes > kTmaMaxSmem ? -1 : (int)bytes;
 }
 
-cudaError_t tma_prepare(const Lattice &lat, int eq, int bulk, int cap, int smem_bytes) {
+// The dynamic shared memory limit belongs to the kernel function, which every lattice of the same
+// kind shares, whatever its launch shape: it is set to the most a block can have and never lowered.
+// (With the size of the shape at hand, creating a lattice of 2 stages made the launches of one of 3
+// stages fail.)
+cudaError_t tma_prepare(const Lattice &lat, int eq, int bulk, int cap) {
     const void *fn = tma_kernel(lat, eq, bulk, cap);
     if (!fn) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, fn);
+    const int most = kTmaMaxSmem - (int)at.sharedSizeBytes;
+    if (e == cudaSuccess && at.maxDynamicSharedSizeBytes < most)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e;
 }
 
 int tma_max_blocks_per_sm(const Lattice &lat, int eq, int bulk, const TmaShape &t) {
     const void *fn = tma_kernel(lat, eq, bulk, t.cap);
     int n = 0;
-    if (!fn) return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem_bytes) != cudaSuccess) {
+    if (tma_prepare(lat, eq, bulk, t.cap) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

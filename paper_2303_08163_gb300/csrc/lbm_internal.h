@@ -94,7 +94,8 @@ int padded_pitch(int D, int P, int64_t nx);
 int tma_smem_bytes(const Lattice &lat, const TmaShape &t);
 // Largest number of colliding threads per block of the TMA kernel for the lattice.
 int tma_thread_limit(const Lattice &lat);
-cudaError_t tma_prepare(const Lattice &lat, int eq, int bulk, int cap, int smem_bytes);
+// Raises the kernel's dynamic shared memory limit to the most a block can have.
+cudaError_t tma_prepare(const Lattice &lat, int eq, int bulk, int cap);
 // Done counters a lattice is given (a row group has at least one row).
 int64_t sync_units(const Lattice &lat);
 // Steps one launch may take: the limits on tickets and launch length.  1 when the lattice has
