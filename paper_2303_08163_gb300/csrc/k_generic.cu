@@ -151,7 +151,7 @@ struct ClassShift {
 __device__ __forceinline__ float two_sum(float a, float b, float c) {  // a + b + c, |c| << |a + b|
     const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
     const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return __fadd_rn(s, __fadd_rn(e, c));
+    return isfinite(s) ? __fadd_rn(s, __fadd_rn(e, c)) : s;  // (the error of an infinite sum is no number)
 }
 template <typename R, typename Out>
 __device__ __forceinline__ Out unshift(R g, const ClassShift &k, int c) {
