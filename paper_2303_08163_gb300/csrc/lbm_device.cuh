@@ -95,6 +95,11 @@ __host__ __device__ __forceinline__ float div_r(float a, float b) {
 __host__ __device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
 __host__ __device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
 
+// Products of the FP64 collisions that feed a sum.  Whether the compiler fuses such a product into the
+// sum depends on the code around it; the collisions of all kernels (a cell on a thread, a cell on
+// three lanes, steps with diagnostics) store the same bits because no operation is left to it.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // FP64 reciprocal and square root of the collisions: the hardware approximation of PTX
 // rcp / rsqrt.approx.ftz.f64 (better than 2^-20) and one step of a third-order Householder
 // iteration, whose error e^3 lies far below the last bit; what is left is the rounding of the last
@@ -191,10 +196,10 @@ __device__ __forceinline__ R collision_rate(R key_max, R omega0, R six_nu) {
     } else if constexpr (EQ == EQ_ENT) {
         const R S = key_max;
         const R A2 = R(2) - S;                      // A S^2
-        return R(2) * A2 * rcp_ulp(fma_r(six_nu, S * S, A2));
+        return mul_rn(R(2) * A2, rcp_ulp(fma_r(six_nu, S * S, A2)));
     } else {
         const R A = fma_r(R(-4.5), key_max, R(1));  // 1 - 3/2 u^2 / vs^2
-        return R(2) * A * rcp_ulp(six_nu + A);
+        return mul_rn(R(2) * A, rcp_ulp(six_nu + A));
     }
 }
 
@@ -322,20 +327,48 @@ template <typename R> struct TensorTerms {
     R drho, irho, X[3][3], key[3];  // X by axis and c + 1; key: what the bulk coefficient depends on
 };
 
+// The moment sums of the FP64 collision: first over the populations of each last velocity component
+// (what one of the three lanes of collide_lanes holds), then over those.
+template <int D> __device__ __forceinline__ void last_axis_sums(const double *f, double &sum, double (&part)[2]) {
+    if constexpr (D == 2) {
+        sum = (f[0] + f[1]) + f[2];
+        part[0] = f[2] - f[0];
+        part[1] = 0.0;
+    } else {
+        const double c0 = (f[0] + f[3]) + f[6], c1 = (f[1] + f[4]) + f[7], c2 = (f[2] + f[5]) + f[8];
+        sum = (c0 + c1) + c2;
+        part[0] = c2 - c0;
+        part[1] = ((f[6] + f[7]) + f[8]) - ((f[0] + f[1]) + f[2]);
+    }
+}
+template <int D>
+__device__ __forceinline__ double collision_sums(const double (&f)[qof(D)], double rho0, double &rho, double (&j)[3]) {
+    constexpr int F = D == 2 ? 3 : 9;
+    double s[3], p[3][2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) last_axis_sums<D>(f + F * c, s[c], p[c]);
+    const double drho = (s[0] + s[1]) + s[2];
+    rho = rho0 + drho;
+    j[2] = 0.0;
+#pragma unroll
+    for (int a = 0; a < D - 1; ++a) j[a] = (p[0][a] + p[1][a]) + p[2][a];
+    j[D - 1] = s[2] - s[0];
+    return drho;
+}
+
 template <int D, int EQ, typename R>
 __device__ __forceinline__ void tensor_terms(const R (&f)[qof(D)], R rho0, CellMoments<R> &m, TensorTerms<R> &t) {
     R j[3], j3[3];
-    t.drho = moment_sums<D, R>(f, rho0, m.rho, j);
+    t.drho = collision_sums<D>(f, rho0, m.rho, j);
     const R rho = m.rho;
 #pragma unroll
     for (int a = 0; a < D; ++a) j3[a] = R(3) * j[a];
     if constexpr (EQ == EQ_ENT) {
-        const R rho2 = rho * rho;
         R jj[3], T[3], q[3], others[3], all;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
             jj[a] = j3[a] * j[a];
-            T[a] = sqrt_ulp(rho2 + jj[a]);
+            T[a] = sqrt_ulp(fma_r(rho, rho, jj[a]));
             q[a] = rho + T[a];
         }
         if constexpr (D == 2) {
@@ -351,11 +384,11 @@ __device__ __forceinline__ void tensor_terms(const R (&f)[qof(D)], R rho0, CellM
         t.irho = r * all;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            const R e = jj[a] * (v * others[a]);  // rho (S - 1)
+            const R e = mul_rn(jj[a], v * others[a]);  // rho (S - 1)
             t.X[a][0] = fma_r(R(2), e, -j3[a]);
             t.X[a][1] = -e;
             t.X[a][2] = fma_r(R(2), e, j3[a]);
-            t.key[a] = T[a] * t.irho;
+            t.key[a] = mul_rn(T[a], t.irho);
         }
     } else {
         t.irho = rcp_ulp(rho);
@@ -363,13 +396,13 @@ __device__ __forceinline__ void tensor_terms(const R (&f)[qof(D)], R rho0, CellM
         for (int a = 0; a < D; ++a) {
             const R u = j[a] * t.irho;
             t.X[a][0] = fma_r(j3[a], u, -j3[a]);
-            t.X[a][1] = R(-0.5) * (j3[a] * u);
+            t.X[a][1] = mul_rn(R(-0.5), j3[a] * u);
             t.X[a][2] = fma_r(j3[a], u, j3[a]);
             t.key[a] = u * u;
         }
     }
 #pragma unroll
-    for (int a = 0; a < 3; ++a) m.u[a] = a < D ? j[a] * t.irho : R(0);
+    for (int a = 0; a < 3; ++a) m.u[a] = a < D ? mul_rn(j[a], t.irho) : R(0);
 }
 
 // ------------------------------------------------------------------ FP32 collisions
@@ -639,10 +672,10 @@ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omeg
     R omw[4];
     if constexpr (EQ == EQ_POLY2) {
         R j[3];
-        const R drho = moment_sums<D, R>(f, rho0, m.rho, j);
+        const R drho = collision_sums<D>(f, rho0, m.rho, j);
         const R inv = rcp_ulp(m.rho);
-        for (int a = 0; a < 3; ++a) m.u[a] = j[a] * inv;
-        R uu = m.u[0] * m.u[0] + m.u[1] * m.u[1];
+        for (int a = 0; a < 3; ++a) m.u[a] = mul_rn(j[a], inv);
+        R uu = fma_r(m.u[0], m.u[0], m.u[1] * m.u[1]);
         if constexpr (D == 3) uu = fma_r(m.u[2], m.u[2], uu);
         R k = fmax(m.u[0] * m.u[0], m.u[1] * m.u[1]);
         if constexpr (D == 3) k = fmax(k, m.u[2] * m.u[2]);
@@ -705,7 +738,8 @@ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omeg
 // c_last = c - 1 (c_y in 2-D, c_z in 3-D), f[p] = f_{p + F c}, F = 3 or 9.  A lane sums its own
 // populations, forms the terms of one axis and relaxes its own populations; partial sums and terms
 // go between the lanes by shuffles.  Every lane adds the partial sums in the same order, so the
-// three hold the same bits of rho, u and 2beta.  About 45 FP64 instructions in place of 82 in 2-D,
+// three hold the same bits of rho, u and 2beta, and the operations are those of collide, so the
+// populations get the same bits from both.  About 45 FP64 instructions in place of 82 in 2-D,
 // 100 of 195 in 3-D (entropic).  All 32 lanes call it; `base` is the first lane of the caller's group.
 __host__ __device__ constexpr int lane_pops(int D) { return D == 2 ? 3 : 9; }
 
@@ -717,16 +751,8 @@ __device__ __forceinline__ CellMoments<double> collide_lanes(double (&f)[lane_po
     using R = double;
     constexpr int F = lane_pops(D);
     CellMoments<R> m;
-    R j[3] = {0, 0, 0}, sum, part[2] = {0, 0};  // sums over the lane's populations: all, c_x f, c_y f (3-D)
-    if constexpr (D == 2) {
-        sum = (f[0] + f[1]) + f[2];
-        part[0] = f[2] - f[0];
-    } else {
-        const R c0 = (f[0] + f[3]) + f[6], c1 = (f[1] + f[4]) + f[7], c2 = (f[2] + f[5]) + f[8];
-        sum = (c0 + c1) + c2;
-        part[0] = c2 - c0;
-        part[1] = ((f[6] + f[7]) + f[8]) - ((f[0] + f[1]) + f[2]);
-    }
+    R j[3] = {0, 0, 0}, sum, part[2];  // sums over the lane's populations: all, c_x f, c_y f (3-D)
+    last_axis_sums<D>(f, sum, part);
     const R s0 = from_lane(sum, base), s1 = from_lane(sum, base + 1), s2 = from_lane(sum, base + 2);
     const R drho = (s0 + s1) + s2;
     m.rho = rho0 + drho;
@@ -737,8 +763,8 @@ __device__ __forceinline__ CellMoments<double> collide_lanes(double (&f)[lane_po
     R om, base_g = 0, irho = 0, ex[3], tx[3], Y[3], Z = 0, r3 = 0, r45 = 0;
     if constexpr (EQ == EQ_POLY2) {
         irho = rcp_ulp(rho);
-        for (int a = 0; a < 3; ++a) m.u[a] = j[a] * irho;
-        R uu = m.u[0] * m.u[0] + m.u[1] * m.u[1], k = fmax(m.u[0] * m.u[0], m.u[1] * m.u[1]);
+        for (int a = 0; a < 3; ++a) m.u[a] = mul_rn(j[a], irho);
+        R uu = fma(m.u[0], m.u[0], m.u[1] * m.u[1]), k = fmax(m.u[0] * m.u[0], m.u[1] * m.u[1]);
         if constexpr (D == 3) {
             uu = fma(m.u[2], m.u[2], uu);
             k = fmax(k, m.u[2] * m.u[2]);
@@ -766,20 +792,20 @@ __device__ __forceinline__ CellMoments<double> collide_lanes(double (&f)[lane_po
             }
             const R r = rcp_ulp(rho * all), v = r * rho;
             irho = r * all;
-            const R e = jj * (v * others);  // rho (S - 1)
+            const R e = mul_rn(jj, v * others);  // rho (S - 1)
             X[0] = fma(2.0, e, -j3);
             X[1] = -e;
             X[2] = fma(2.0, e, j3);
-            key = T * irho;
+            key = mul_rn(T, irho);
         } else {
             irho = rcp_ulp(rho);
             const R u = ja * irho;
             X[0] = fma(j3, u, -j3);
-            X[1] = -0.5 * (j3 * u);
+            X[1] = mul_rn(-0.5, j3 * u);
             X[2] = fma(j3, u, j3);
             key = u * u;
         }
-        for (int a = 0; a < 3; ++a) m.u[a] = a < D ? j[a] * irho : 0.0;
+        for (int a = 0; a < 3; ++a) m.u[a] = a < D ? mul_rn(j[a], irho) : 0.0;
         R kmax = 0;
         if constexpr (BULK) {
             kmax = fmax(from_lane(key, base), from_lane(key, base + 1));
