@@ -53,6 +53,10 @@ int sm_count() {
     return n;
 }
 
+// 6 nu of the corrected rate 2 A / (6 nu + A), of a size whose square is a number (the rate is 0 to
+// all digits long before).
+double six_nu_of(double tau) { return std::min(6.0 * (tau - 0.5) / 3.0, 1e150); }
+
 int64_t wait_timeout_ns() {
     const char *e = getenv("LBM_WAIT_TIMEOUT_NS");
     if (e && *e) {
@@ -674,7 +678,7 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
     c->tau = tau;
     c->rho0 = rho0;
     c->omega0 = 1.0 / tau;
-    c->six_nu = 6.0 * (tau - 0.5) / 3.0;
+    c->six_nu = six_nu_of(tau);
     c->stream = static_cast<cudaStream_t>(cuda_stream);
     const int es = esize_of(precision);
     const int64_t align = 256 / es;
@@ -1416,7 +1420,7 @@ int lbm_batch_create(lbm_batch **out, int lattice, int64_t count, const int32_t 
     std::vector<double> om(count), sn(count);
     for (int64_t k = 0; k < count; ++k) {
         om[k] = 1.0 / tau[k];
-        sn[k] = 6.0 * (tau[k] - 0.5) / 3.0;
+        sn[k] = six_nu_of(tau[k]);
     }
     b->block_cap = batch_block_cap(count);
     b->threads = 256;

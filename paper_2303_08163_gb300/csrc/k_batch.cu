@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256) k_step_batch(const lbmh::BatchArgs a) {
 // beyond the block's own.  A probe's partial sums go through a buffer per block, in pairs so that
 // the next probe does not overwrite sums the team's first block is still adding up.
 template <int D, int EQ, bool BULK>
-__global__ void __launch_bounds__(lbmh::kTeamThreads) k_step_teams(const lbmh::BatchArgs a) {
+__global__ void __launch_bounds__(lbmh::kTeamThreads, D == 2 ? 5 : 3) k_step_teams(const lbmh::BatchArgs a) {
     constexpr int N = kProbe<D>, Q = qof(D);
     constexpr int kWarps = lbmh::kTeamThreads / 32;
     __shared__ double red[kWarps][8];

@@ -24,6 +24,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace lbmd {
 
 enum { P_F64 = 0, P_F32 = 1, P_F16S = 2 };
@@ -107,6 +109,8 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 // take 3 and 5 instructions; the IEEE division measured 5.5, the square root 9.8.
 //   1/x     = y (1 + e + e^2),             e = 1 - x y
 //   sqrt(x) = t (1 + e (1/2 + 3/8 e)),     t = x y, e = 1 - t y
+// The approximations flush what is no normal number to zero (then 0 x infinity: no number), so x
+// and 1/x have to be normal.
 __device__ __forceinline__ double rcp_ulp(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -118,6 +122,20 @@ __device__ __forceinline__ double sqrt_ulp(double x) {
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double t = x * y, e = fma(-t, y, 1.0);
     return fma(t * e, fma(e, 0.375, 0.5), t);
+}
+
+// Exponents by integer arithmetic, which costs the FP64 pipe nothing: x / 2^n (exact; what falls below
+// the normal numbers becomes some number below them, what rises above them becomes infinite or no
+// number), and 1/x within an ulp for every x for which both are normal.
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20 & 0x7ff) - 1023; }
+__device__ __forceinline__ double scale_down(double x, int n) {
+    const int hi = __double2hiint(x), e = hi >> 20 & 0x7ff;
+    const int t = min(max(e - n, 0), 0x7ff);
+    return e == 0 ? x : __hiloint2double((hi & (int)0x800fffff) | t << 20, __double2loint(x));
+}
+__device__ __forceinline__ double rcp_any(double x) {
+    const int n = exponent_of(x);
+    return scale_down(rcp_ulp(scale_down(x, n)), n);
 }
 
 template <typename R> struct CellMoments {
@@ -319,10 +337,55 @@ __host__ __device__ __forceinline__ CellMoments<R> moments_shifted(const R (&f)[
 //
 // Entropic form: with j3 = 3 j, T_a = rho S_a = sqrt(rho^2 + j3_a j_a) and q_a = rho + T_a, the term
 // rho (S_a - 1) is j3_a j_a / q_a (no cancellation: an ulp of T stays an ulp), and one reciprocal of
-// rho prod q_a gives 1/rho and every 1/q_a.  Errors against 64-bit references are those of the
-// direct forms with IEEE division and square root (2-D and 3-D, all options).
+// the product rho prod q_a gives 1/rho and every 1/q_a.  Errors against 64-bit references are those
+// of the direct forms with IEEE division and square root (2-D and 3-D, all options).
 // 4096-lattice sweep: 5.20 -> 4.79 ms a step with the own reciprocal and square root, 4.53 with
 // these terms; D3Q27 128^3 882 -> 842 -> 820 us.
+// Where rho is negative T is the other root, and the product, of the order rho^(D+1), leaves FP64's
+// range long before rho does (rho0 = 1e80).  The product itself tells both (terms_ok): it is negative,
+// or too small or large.  Such a cell forms its terms with the sign of rho, and without rho's power of
+// two, which changes nothing but the exponents.  (All cells in that way: sweep 4.79 -> 4.92 ms a step;
+// only those that need it: 4.79, 64^2 2.67 -> 2.74, 48^3 48 -> 49.5 us a step.)
+__device__ __forceinline__ bool terms_ok(double product) { return ((unsigned)__double2hiint(product) >> 20) - 64u < 1920u; }
+
+// e_a = rho (S_a - 1), key_a = S_a and 1/rho; returns the product.  SIGNED: for rho of any sign.
+template <int D, bool SIGNED>
+__device__ __forceinline__ double entropic_terms(double rho, const double (&j)[3], double (&e)[D], double (&key)[D], double &irho) {
+    double jj[D], T[D], q[D], others[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        jj[a] = 3.0 * j[a] * j[a];
+        T[a] = sqrt_ulp(fma(rho, rho, jj[a]));
+        if constexpr (SIGNED) T[a] = copysign(T[a], rho);
+        q[a] = rho + T[a];
+    }
+    if constexpr (D == 2) {
+        others[0] = q[1];
+        others[1] = q[0];
+    } else {
+        others[0] = q[1] * q[2];
+        others[1] = q[0] * q[2];
+        others[2] = q[0] * q[1];
+    }
+    const double all = q[0] * others[0], product = rho * all, r = rcp_ulp(product), v = r * rho;  // v = 1 / prod q
+    irho = r * all;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        e[a] = mul_rn(jj[a], v * others[a]);
+        key[a] = mul_rn(T[a], irho);
+    }
+    return product;
+}
+template <int D>
+__device__ __forceinline__ void entropic_terms_any(double rho, const double (&j)[3], double (&e)[D], double (&key)[D], double &irho) {
+    const int n = exponent_of(rho);
+    const double j1[3] = {scale_down(j[0], n), scale_down(j[1], n), scale_down(j[2], n)};
+    entropic_terms<D, true>(scale_down(rho, n), j1, e, key, irho);
+    irho = scale_down(irho, n);
+#pragma unroll
+    for (int a = 0; a < D; ++a) e[a] = scale_down(e[a], -n);
+}
+
 template <typename R> struct TensorTerms {
     R drho, irho, X[3][3], key[3];  // X by axis and c + 1; key: what the bulk coefficient depends on
 };
@@ -364,34 +427,17 @@ __device__ __forceinline__ void tensor_terms(const R (&f)[qof(D)], R rho0, CellM
 #pragma unroll
     for (int a = 0; a < D; ++a) j3[a] = R(3) * j[a];
     if constexpr (EQ == EQ_ENT) {
-        R jj[3], T[3], q[3], others[3], all;
+        R e[D], key[D];
+        if (!terms_ok(entropic_terms<D, false>(rho, j, e, key, t.irho))) entropic_terms_any<D>(rho, j, e, key, t.irho);
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            jj[a] = j3[a] * j[a];
-            T[a] = sqrt_ulp(fma_r(rho, rho, jj[a]));
-            q[a] = rho + T[a];
-        }
-        if constexpr (D == 2) {
-            others[0] = q[1];
-            others[1] = q[0];
-        } else {
-            others[0] = q[1] * q[2];
-            others[1] = q[0] * q[2];
-            others[2] = q[0] * q[1];
-        }
-        all = q[0] * others[0];
-        const R r = rcp_ulp(rho * all), v = r * rho;  // v = 1 / prod q
-        t.irho = r * all;
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            const R e = mul_rn(jj[a], v * others[a]);  // rho (S - 1)
-            t.X[a][0] = fma_r(R(2), e, -j3[a]);
-            t.X[a][1] = -e;
-            t.X[a][2] = fma_r(R(2), e, j3[a]);
-            t.key[a] = mul_rn(T[a], t.irho);
+            t.X[a][0] = fma_r(R(2), e[a], -j3[a]);
+            t.X[a][1] = -e[a];
+            t.X[a][2] = fma_r(R(2), e[a], j3[a]);
+            t.key[a] = key[a];
         }
     } else {
-        t.irho = rcp_ulp(rho);
+        t.irho = rcp_any(rho);
 #pragma unroll
         for (int a = 0; a < D; ++a) {
             const R u = j[a] * t.irho;
@@ -673,7 +719,7 @@ __device__ __forceinline__ CellMoments<R> collide(R (&f)[qof(D)], R rho0, R omeg
     if constexpr (EQ == EQ_POLY2) {
         R j[3];
         const R drho = collision_sums<D>(f, rho0, m.rho, j);
-        const R inv = rcp_ulp(m.rho);
+        const R inv = rcp_any(m.rho);
         for (int a = 0; a < 3; ++a) m.u[a] = mul_rn(j[a], inv);
         R uu = fma_r(m.u[0], m.u[0], m.u[1] * m.u[1]);
         if constexpr (D == 3) uu = fma_r(m.u[2], m.u[2], uu);
@@ -762,7 +808,7 @@ __device__ __forceinline__ CellMoments<double> collide_lanes(double (&f)[lane_po
     const R rho = m.rho;
     R om, base_g = 0, irho = 0, ex[3], tx[3], Y[3], Z = 0, r3 = 0, r45 = 0;
     if constexpr (EQ == EQ_POLY2) {
-        irho = rcp_ulp(rho);
+        irho = rcp_any(rho);
         for (int a = 0; a < 3; ++a) m.u[a] = mul_rn(j[a], irho);
         R uu = fma(m.u[0], m.u[0], m.u[1] * m.u[1]), k = fmax(m.u[0] * m.u[0], m.u[1] * m.u[1]);
         if constexpr (D == 3) {
@@ -779,26 +825,40 @@ __device__ __forceinline__ CellMoments<double> collide_lanes(double (&f)[lane_po
         const R j3 = 3.0 * ja;
         R X[3], key;
         if constexpr (EQ == EQ_ENT) {
-            const R jj = j3 * ja, T = sqrt_ulp(fma(rho, rho, jj)), q = rho + T;
-            const R q0 = from_lane(q, base), q1 = from_lane(q, base + 1);
-            R others, all;
-            if constexpr (D == 2) {
-                others = c == 0 ? q1 : q0;
-                all = q0 * q1;
-            } else {
-                const R q2 = from_lane(q, base + 2);
-                others = (c == 0 ? q1 : q0) * (c == 2 ? q1 : q2);
-                all = q0 * (q1 * q2);
+            // entropic_terms with an axis to a lane; all lanes again where some cell of the warp needs it
+            R e;
+            const auto terms = [&](R r, R v, auto is_signed) {
+                R jj = 3.0 * v * v, T = sqrt_ulp(fma(r, r, jj));
+                if constexpr (decltype(is_signed)::value) T = copysign(T, r);
+                const R q = r + T;
+                const R q0 = from_lane(q, base), q1 = from_lane(q, base + 1);
+                R others, all;
+                if constexpr (D == 2) {
+                    others = c == 0 ? q1 : q0;
+                    all = q0 * q1;
+                } else {
+                    const R q2 = from_lane(q, base + 2);
+                    others = (c == 0 ? q1 : q0) * (c == 2 ? q1 : q2);
+                    all = q0 * (q1 * q2);
+                }
+                const R product = r * all, w = rcp_ulp(product), z = w * r;
+                irho = w * all;
+                e = mul_rn(jj, z * others);
+                key = mul_rn(T, irho);
+                return product;
+            };
+            const bool ok = terms_ok(terms(rho, ja, std::false_type()));
+            if (!__all_sync(0xffffffffu, ok)) {
+                const int n = ok ? 0 : exponent_of(rho);
+                terms(scale_down(rho, n), scale_down(ja, n), std::true_type());
+                irho = scale_down(irho, n);
+                e = scale_down(e, -n);
             }
-            const R r = rcp_ulp(rho * all), v = r * rho;
-            irho = r * all;
-            const R e = mul_rn(jj, v * others);  // rho (S - 1)
             X[0] = fma(2.0, e, -j3);
             X[1] = -e;
             X[2] = fma(2.0, e, j3);
-            key = mul_rn(T, irho);
         } else {
-            irho = rcp_ulp(rho);
+            irho = rcp_any(rho);
             const R u = ja * irho;
             X[0] = fma(j3, u, -j3);
             X[1] = mul_rn(-0.5, j3 * u);
