@@ -269,7 +269,8 @@ int lbm_batch_step(lbm_batch *b, int64_t n);
 int lbm_batch_probe_series(lbm_batch *b, double *out, int64_t max_samples, int64_t *nsamples);
 
 /* Per-instance status, host int32 [count]: 0 = finite so far, s + 1 = the first probed
- * step s at which the instance's mass or momentum was not finite (synchronises). */
+ * step s at which the instance's mass or momentum was not finite, LBM_ECHECK = a check failed
+ * (checked builds); synchronises. */
 int lbm_batch_status(lbm_batch *b, int32_t *status);
 
 /* rho and u of every instance (packed as in lbm_batch_init_fields). */

@@ -87,11 +87,11 @@ __device__ __forceinline__ void probe_record(const lbmh::BatchArgs &a, int k, in
 template <int D, int EQ, bool BULK, bool L2, bool PROBE>
 __device__ __forceinline__ void batch_cells(double *A, int64_t ncell, int nx, int ny, int nz, int64_t first, int64_t stride,
                                             int odd, double rho0, double om, double sn, const double2 *tw,
-                                            double (&acc)[kProbe<D>]) {
+                                            double (&acc)[kProbe<D>], int32_t *status) {
     for (int64_t c = first; c < ncell; c += stride) {
         int x, y, z;
         cell_coords(c, ncell, nx, ny, x, y, z);
-        const CellMoments<double> m = aa_cell_step<D, P_F64, EQ, BULK, L2>(A, ncell, nx, ny, nz, nx, x, y, z, odd, rho0, om, sn);
+        const CellMoments<double> m = aa_cell_step<D, P_F64, EQ, BULK, L2>(A, ncell, nx, ny, nz, nx, x, y, z, odd, rho0, om, sn, status);
         if constexpr (PROBE) probe_add<D>(acc, m, tw, nx, ny, x, y, z);
     }
 }
@@ -114,8 +114,8 @@ __global__ void __launch_bounds__(256) k_step_batch(const lbmh::BatchArgs a) {
             const double om = a.omega0[k], sn = a.six_nu[k];
             const double2 *tw = a.twiddle + a.tw_offset[k];
             double acc[N] = {};
-            if (probe) batch_cells<D, EQ, BULK, false, true>(A, ncell, nx, ny, nz, threadIdx.x, blockDim.x, odd, a.rho0, om, sn, tw, acc);
-            else batch_cells<D, EQ, BULK, false, false>(A, ncell, nx, ny, nz, threadIdx.x, blockDim.x, odd, a.rho0, om, sn, tw, acc);
+            if (probe) batch_cells<D, EQ, BULK, false, true>(A, ncell, nx, ny, nz, threadIdx.x, blockDim.x, odd, a.rho0, om, sn, tw, acc, a.status + k);
+            else batch_cells<D, EQ, BULK, false, false>(A, ncell, nx, ny, nz, threadIdx.x, blockDim.x, odd, a.rho0, om, sn, tw, acc, a.status + k);
             if (probe) {
                 // fixed-order block reduction: within the warps, then the warps in order
                 const double v = warp_sums(acc);
@@ -163,8 +163,8 @@ __global__ void __launch_bounds__(lbmh::kTeamThreads, D == 2 ? 5 : 3) k_step_tea
         const int odd = (int)(t & 1);
         const bool probe = a.every_k > 0 && (t % a.every_k) == 0;
         double acc[N] = {};
-        if (probe) batch_cells<D, EQ, BULK, true, true>(A, ncell, nx, ny, nz, first, stride, odd, a.rho0, om, sn, tw, acc);
-        else batch_cells<D, EQ, BULK, true, false>(A, ncell, nx, ny, nz, first, stride, odd, a.rho0, om, sn, tw, acc);
+        if (probe) batch_cells<D, EQ, BULK, true, true>(A, ncell, nx, ny, nz, first, stride, odd, a.rho0, om, sn, tw, acc, a.status + k);
+        else batch_cells<D, EQ, BULK, true, false>(A, ncell, nx, ny, nz, first, stride, odd, a.rho0, om, sn, tw, acc, a.status + k);
         double *buf = a.team_partials + ((int64_t)(probes & 1) * gridDim.x + blockIdx.x) * 8;
         if (probe) {
             const double v = warp_sums(acc);
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(lbmh::kTeamThreads) k_step_clusters(const lbmh
         const int i = p + F * c, dx = cxo(p), dy = D == 3 ? cyo(p) : c - 1, dz = D == 3 ? c - 1 : 0;
         const int from = wrapi(x - dx, nx) + nx * (wrapi(y - dy, ny) + ny * wrapi(z - dz, nz));
         const int to = wrapi(x + dx, nx) + nx * (wrapi(y + dy, ny) + ny * wrapi(z + dz, nz));
-        const bool ok = LBM_CHECK(from >= 0 && from < ncell && to >= 0 && to < ncell, nullptr);
+        const bool ok = LBM_CHECK(from >= 0 && from < ncell && to >= 0 && to < ncell, a.status + k);
         src[p] = cluster_addr(pop0 + 8 * ((Q - 1 - i) * C + (ok ? from % C : 0)), ok ? from / C : part);
         dst[p] = cluster_addr(pop0 + 8 * (i * C + (ok ? to % C : 0)), ok ? to / C : part);
     }

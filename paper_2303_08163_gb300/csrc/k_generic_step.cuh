@@ -30,7 +30,7 @@ template <int D, int P, int EQ, bool BULK, bool L2 = false>
 __device__ __forceinline__ CellMoments<typename Storage<P>::R> aa_cell_step(
     typename Storage<P>::T *__restrict__ A, int64_t plane, int nx, int ny, int nz, int pitch, int x, int y,
     int z, int odd, typename Storage<P>::R rho0, typename Storage<P>::R omega0,
-    typename Storage<P>::R six_nu, int32_t *status = nullptr) {
+    typename Storage<P>::R six_nu, int32_t *status) {
     using St = Storage<P>;
     using R = typename St::R;
     constexpr int Q = qof(D);

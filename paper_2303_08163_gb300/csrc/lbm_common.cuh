@@ -18,7 +18,7 @@ __device__ __forceinline__ void report_status(int32_t *status, int32_t code) { a
 // every check is the constant true and compiles away.
 #ifdef LBM_CHECKED
 __device__ __forceinline__ bool lbm_check(bool ok, int32_t *status) {
-    if (!ok && status) report_status(status, -7);
+    if (!ok) report_status(status, -7);
     return ok;
 }
 #define LBM_CHECK(ok, status) ::lbmd::lbm_check((ok), (status))
