@@ -95,7 +95,8 @@ struct lbm_ctx {
     int gen_threads = 256, gen_blocks = 1;
     bool chosen = false;  // the caller named a kernel or a launch shape
     SmallShape small;  // several steps of a small lattice at once (0 threads: too large)
-    TmaShape tma{};
+    TmaShape tma{};      // of several steps a launch
+    TmaShape tma_one{};  // of one
     bool use_graph = false;
     cudaGraphExec_t graph2 = nullptr;  // even + odd step
     // grow-only device staging for calls with host buffers
@@ -194,11 +195,11 @@ StepArgs step_args(lbm_ctx *c, int odd, int diag) {
     return a;
 }
 
-int launch_blocks(lbm_ctx *c) { return c->kernel == 2 ? c->tma.blocks : c->gen_blocks; }
+int launch_blocks(lbm_ctx *c) { return c->kernel == 2 ? c->tma_one.one_blocks : c->gen_blocks; }
 
 cudaError_t launch_one(lbm_ctx *c, int odd, int diag, cudaStream_t s) {
     const StepArgs a = step_args(c, odd, diag);
-    if (c->kernel == 2) return step_tma(a, c->tma, 1, s);
+    if (c->kernel == 2) return step_tma(a, c->tma_one, 1, s);
     return step_generic(a, c->gen_blocks, c->gen_threads, s);
 }
 
@@ -256,9 +257,7 @@ bool default_tma_shape(lbm_ctx *c, TmaShape &t) {
     t.stages = 2;
     t.smem_bytes = tma_smem_bytes(c->lat, t);
     if (t.smem_bytes < 0) return false;
-    const int nb = tma_max_blocks_per_sm(c->lat, c->eq, c->bulk, t);
-    if (nb < 1) return false;
-    t.blocks = sm_count() * nb;
+    if (!tma_set_blocks(c->lat, c->eq, c->bulk, sm_count(), t)) return false;
     // A lattice of few rows is spread over all blocks, one job each: jobs of full buffers would
     // leave most SMs without work (64^2 FP64: 8 jobs, 20.5 us a step; 64 jobs, 7.9 us).
     const int64_t groups = std::max<int64_t>(1, t.blocks / c->lat.nz);  // row groups of a plane
@@ -270,6 +269,22 @@ bool default_tma_shape(lbm_ctx *c, TmaShape &t) {
            2 * ((c->lat.ny + t.rows - 1) / t.rows) * (int64_t)c->lat.nz < 3 * (int64_t)t.blocks)
         t.rows = (t.rows + 1) / 2;
     return true;
+}
+
+// The default shape of single steps: that of several, but for FP32 rows of 2-D lattices that pass HBM
+// each step.  Those go in segments of up to 516 cells and 3 stages: steps launched one by one of 4096^2
+// 200 -> 193 us, 3000^2 109 -> 105, 2048 x 4096 102 -> 98, 5000^2 294 -> 285 (with diagnostics 223 -> 216,
+// 136 -> 133, 125 -> 123, 322 -> 317); in L2 (1024^2, 1400^2) 3 stages are slower.
+TmaShape default_one_shape(lbm_ctx *c, const TmaShape &t) {
+    TmaShape o = t;
+    const int64_t state = (int64_t)c->Q * c->lat.plane * 4;
+    if (c->D != 2 || c->prec != LBM_F32 || c->lat.pitch != c->lat.nx || c->lat.nx <= 516 || state <= kTmaResident) return o;
+    const int64_t n = (c->lat.nx + 515) / 516;
+    o.seg = (int)(((c->lat.nx + n - 1) / n + 3) / 4 * 4);
+    o.rows = 1;
+    o.stages = 3;
+    o.smem_bytes = tma_smem_bytes(c->lat, o);
+    return o.smem_bytes > 0 && tma_set_blocks(c->lat, c->eq, c->bulk, sm_count(), o) ? o : t;
 }
 
 // Callers may ask for the TMA kernel on unpadded rows only; padded ones use it by the
@@ -427,9 +442,7 @@ bool shape_from_record(lbm_ctx *c, const std::vector<int> &v, int *kernel, TmaSh
     if (s.rows < 1 || s.seg < 16 / esize_of(c->prec)) return false;
     s.smem_bytes = tma_smem_bytes(c->lat, s);
     if (s.smem_bytes < 0 || s.smem_bytes != v[7]) return false;
-    const int nb = tma_max_blocks_per_sm(c->lat, c->eq, c->bulk, s);
-    if (nb < 1) return false;
-    s.blocks = sm_count() * nb;
+    if (!tma_set_blocks(c->lat, c->eq, c->bulk, sm_count(), s)) return false;
     *kernel = 2;
     *t = s;
     return true;
@@ -446,7 +459,7 @@ bool apply_shape(lbm_ctx *c, const std::vector<int> &v) {
             cudaGetLastError();
             return false;
         }
-        c->tma = t;
+        c->tma = c->tma_one = t;
     } else {
         c->gen_threads = gt;
         c->gen_blocks = gb;
@@ -568,11 +581,9 @@ int autotune(lbm_ctx *c) {
                         t.cap = cap;
                         t.smem_bytes = tma_smem_bytes(c->lat, t);
                         if (t.smem_bytes < 0) continue;
-                        const int nb = tma_max_blocks_per_sm(c->lat, c->eq, c->bulk, t);
-                        if (nb < 1) continue;
+                        if (!tma_set_blocks(c->lat, c->eq, c->bulk, sm_count(), t)) continue;
                         // keep 2..4 stages per block only when several blocks share an SM
-                        if (nb * st > 16) continue;
-                        t.blocks = sm_count() * nb;
+                        if (t.blocks / sm_count() * st > 16) continue;
                         cands.push_back({2, t.threads, t.blocks, t.stages, t.rows, t.seg, t.cap, t.smem_bytes});
                     }
         }
@@ -751,7 +762,7 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
         }
     }
     if (tma_supported(c->lat) && default_tma_shape(c, c->tma)) {
-        tma_prepare(c->lat, c->eq, c->bulk, c->tma.cap);
+        c->tma_one = default_one_shape(c, c->tma);
         c->kernel = 2;
     }
     cudaGetLastError();
@@ -776,9 +787,10 @@ int lbm_set_option(lbm_ctx *c, int option, int64_t value) {
         if (value == 1) c->kernel = 1;
         if (value == 2 || value == 0) {
             if (tma_supported(c->lat)) {
-                if (c->tma.smem_bytes <= 0 && !default_tma_shape(c, c->tma))
-                    return fail(LBM_ECUDA, "no TMA launch shape fits this lattice");
-                tma_prepare(c->lat, c->eq, c->bulk, c->tma.cap);
+                if (c->tma.smem_bytes <= 0) {
+                    if (!default_tma_shape(c, c->tma)) return fail(LBM_ECUDA, "no TMA launch shape fits this lattice");
+                    c->tma_one = default_one_shape(c, c->tma);
+                }
                 c->kernel = 2;
             } else {
                 c->kernel = 1;
@@ -1110,11 +1122,8 @@ int lbm_set_launch_shape(lbm_ctx *c, const int64_t shape[6]) {
     t.cap = (int)shape[5];
     t.smem_bytes = tma_smem_bytes(c->lat, t);
     if (t.smem_bytes < 0) return fail(LBM_EINVAL, "launch shape does not fit (segment, rows, cap or stages)");
-    const int nb = tma_max_blocks_per_sm(c->lat, c->eq, c->bulk, t);
-    if (nb < 1) return fail(LBM_EINVAL, "launch shape does not fit on the device");
-    t.blocks = sm_count() * nb;
-    CK(tma_prepare(c->lat, c->eq, c->bulk, t.cap), "shared memory attribute");
-    c->tma = t;
+    if (!tma_set_blocks(c->lat, c->eq, c->bulk, sm_count(), t)) return fail(LBM_EINVAL, "launch shape does not fit on the device");
+    c->tma = c->tma_one = t;
     c->kernel = 2;
     c->chosen = true;
     drop_graph(c);

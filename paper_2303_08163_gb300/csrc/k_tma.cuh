@@ -13,21 +13,22 @@
 // memory and buffer b is stored back to exactly the global location it was loaded from.
 // Different jobs touch disjoint global locations, so jobs need no ordering.
 //
-// Data movement (warp specialised): after the colliding (consumer) warps come a loader and a
-// storer warp.  Lane b of the loader issues the cp.async.bulk copies of buffer b (global ->
-// shared, completion counted in transaction bytes on the stage's `full` mbarrier).  Consumer
-// warps wait on `full`, collide the job in place, fence their shared-memory writes for the
-// async proxy and arrive on the stage's `empty` mbarrier.  Lane b of the storer then issues
-// the cp.async.bulk stores of buffer b, and once they have read the stage it arrives on
-// `freed` and the loader refills it.  Two warps, because a loader that waits for another
-// block's step (below) must not hold up the stores that other blocks wait for.  Rows must
-// start on 16-byte boundaries: the row pitch is a multiple of 16 bytes (a ragged row is
-// padded to it, and whole rows are copied with their padding; the cells of the padding are
-// never read by a real cell).
+// Data movement (warp specialised): after the colliding (consumer) warps come one or two service
+// warps.  Lane b of a loading warp issues the cp.async.bulk copies of buffer b (global -> shared,
+// completion counted in transaction bytes on the stage's `full` mbarrier).  Consumer warps wait on
+// `full`, collide the job in place, fence their shared-memory writes for the async proxy and arrive
+// on the stage's `empty` mbarrier.  Lane b of a storing warp then issues the cp.async.bulk stores of
+// buffer b, and once they have read the stage it can be refilled.  Rows must start on 16-byte
+// boundaries: the row pitch is a multiple of 16 bytes (a ragged row is padded to it, and whole rows
+// are copied with their padding; the cells of the padding are never read by a real cell).
 //
-// One launch advances one step (jobs strided over the blocks, no waits; the diagnostics are
-// reduced here) or several (jobs by ticket, with counters of finished jobs; see
-// decode_chain).
+// Two kernels.  k_step_tma advances one step (jobs strided over the blocks, no waits between them; the
+// diagnostics are reduced here): one service warp stores and refills.  k_steps_tma advances several
+// (jobs by ticket, with counters of finished jobs; see decode_chain): a loader and a storer, because a
+// loader that waits for another block's step must not hold up the stores that other blocks wait for.
+// With both in one kernel (a loader and a storer for single steps too, registers for the longer
+// body) single steps lost 2 % of 512^3 binary16 (2.19 -> 2.23 ms; now 2.18) and 3 % of 128^3, and
+// several steps gained 1 % by the parting (512^3 1.67 -> 1.64 ms a step).
 //
 // Segmented rows (seg < Nx) carry a halo of U = 16 / sizeof(storage) cells on each side.
 // In the odd step the cells of a segment touch positions [X0 - 1, X0 + len - 1) of the
@@ -71,8 +72,6 @@ struct TmaGeom {
     FastDiv by_nseg, by_ygroups, by_npos, by_strips, by_pjobs, by_depth;
 };
 
-constexpr int kTmaCaps[4] = {1024, 2048, 4096, 8192};  // bytes per direction buffer
-
 struct JobPos {
     int z, y0, nrows, X0, len;
     int odd;  // AA parity of the job's step
@@ -89,7 +88,7 @@ __device__ __forceinline__ JobPos job_at(const lbmh::StepArgs &a, const TmaGeom 
     return j;
 }
 
-// One step (nsteps == 1): job number -> rows and segment.
+// Single steps: job number -> rows and segment.
 __device__ __forceinline__ JobPos decode_job(const lbmh::StepArgs &a, const TmaGeom &g, unsigned job) {
     const unsigned rest = div_by(job, g.by_nseg);
     const unsigned zq = div_by(rest, g.by_ygroups);
@@ -411,8 +410,7 @@ __device__ __forceinline__ void tma_compute(const lbmh::StepArgs &a, const TmaGe
 // Odd step, segments (no wrap inside the job): cells (x, x + 1), x even, own the pair at x in
 // the c_x = 0 buffers and go one half at a time elsewhere.  The operations and conversions
 // round exactly as the one-cell path does, so the stored state is the same bit for bit.  Rows
-// of odd length (padded rows) go one cell at a time: a pairing that wraps has no aligned
-// pairs there.
+// of odd length (padded rows) have a body of their own, LONE below.
 __device__ __forceinline__ f32x2 ld_pair(const __half *b, int p) {
     const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(b + p));
     return pack2(v.x, v.y);
@@ -551,11 +549,174 @@ __device__ __forceinline__ void tma_compute_pairs(const lbmh::StepArgs &a, const
     if (DIAG && a.diag) loc.flush(acc, a.rho0);
 }
 
-// The warps after the consumers: the loader and the storer.
+// A job's collisions, by the bodies that suit the storage.  CHAIN: several steps a launch; DIAG: with
+// the diagnostics' sums (single steps only).
+template <int D, int P, int EQ, bool BULK, int CAPB, bool CHAIN, bool DIAG>
+__device__ __forceinline__ void tma_collide(const lbmh::StepArgs &a, const TmaGeom &g, const JobPos &jp,
+                                            typename Storage<P>::T *st, DiagAcc &acc, int tid, int nthr) {
+    const auto pairs = [&](auto mode, auto lone) {
+        tma_compute_pairs<D, P, EQ, BULK, CAPB, mode.value, lone.value, DIAG>(a, g, jp, st, acc, tid, nthr);
+    };
+    using std::integral_constant;
+    constexpr std::true_type yes;
+    constexpr std::false_type no;
+    constexpr integral_constant<int, -1> any;
+    // One D3Q27 step a launch is bound by HBM (0.97 of the copy peak), and two cells a thread only bunch
+    // its accesses: 512^3 binary16 2.19 against 2.33 ms a step (128^3, in L2, 47 against 42.5 us).  With
+    // diagnostics the longer body is what counts: two cells a thread 2.38 against 2.42 ms, 256^3 317
+    // against 343 us.  2-D FP32 rows of odd length: 54 us in pairs, 59 cell by cell (2047 x 2000).
+    if constexpr (P == P_F64 || (D == 3 && !CHAIN && !(DIAG && P == P_F16S))) {
+        tma_compute<D, P, EQ, BULK, CAPB, DIAG>(a, g, jp, st, acc, tid, nthr);
+    } else if constexpr (D == 3 || DIAG) {
+        // The D3Q27 pair body is long: one copy serves the three pairings (three
+        // specialised copies measured slower).
+        if (jp.len & 1) pairs(any, yes);
+        else pairs(any, no);
+    } else {
+        constexpr integral_constant<int, 0> even;
+        constexpr integral_constant<int, 1> rows;
+        constexpr integral_constant<int, 2> segments;
+        if (jp.len & 1) {
+            if (jp.odd) pairs(rows, yes);
+            else pairs(even, yes);
+        } else if (!jp.odd) pairs(even, no);
+        else if (g.nseg == 1) pairs(rows, no);
+        else pairs(segments, no);
+    }
+}
+
+// One step a launch: jobs strided over the blocks.  One service warp: lane b stores the buffer b of a
+// collided stage, waits until that store has read it, and refills the same buffer with the next job's;
+// the lanes do not wait for one another.
+template <int D, int P, int EQ, bool BULK, int CAPB>
+__global__ void __launch_bounds__(tma_max_threads(D, P) + 32) k_step_tma(const lbmh::StepArgs a, const TmaGeom g) {
+    using T = typename Storage<P>::T;
+    constexpr int Q = qof(D);
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t full[kTmaMaxStages];
+    __shared__ __align__(8) uint64_t empty[kTmaMaxStages];
+    T *sm = reinterpret_cast<T *>(smem_raw);
+    const int64_t stage_elems = (int64_t)Q * (CAPB / (int)sizeof(T));
+    const int S = g.stages;
+    const int ncons = (int)blockDim.x - 32;
+    const int lane = threadIdx.x & 31;
+    const unsigned total = (unsigned)g.njobs, G = gridDim.x;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], ncons / 32);
+        }
+        fence_barrier_init();
+    }
+    __syncthreads();
+    DiagAcc acc;
+    bool failed = false;
+    if ((int)threadIdx.x >= ncons) {
+        const LaneBuf<T> buf = lane_buf<D, T>(a, lane);
+        // stage s, and the parity of the phase in which its job before was collided; `held` jobs are in
+        // the stages, the oldest of them `old`
+        int s = 0, held = 0;
+        uint32_t phase = 1;
+        unsigned old = blockIdx.x, job = blockIdx.x;
+        for (; job < total; job += G) {
+            const JobPos jp = decode_job(a, g, job);
+            T *st = sm + s * stage_elems;
+            if (held == S) {
+                const bool ok = mbar_wait_bounded(&empty[s], phase, a.timeout_ns);
+                if (__any_sync(0xffffffffu, !ok)) {
+                    failed = true;
+                    break;
+                }
+                const JobPos jq = decode_job(a, g, old);
+                old += G;
+                if (a.odd && g.nseg > 1) {
+                    tma_plain_stores<D, T>(a, g, jq, st, lane, 32);
+                    __syncwarp();  // every lane's plain stores read the stage before any refill
+                }
+                if (lane == 0) mbar_arrive_expect_tx(&full[s], tma_job_bytes<D, T>(a, g, jp));
+                if (lane < Q) {
+                    tma_issue_stores<D, T>(a, g, jq, buf, st);
+                    bulk_commit();
+                    bulk_wait_read<0>();
+                    tma_issue_loads<D, T>(a, g, jp, buf, st, &full[s]);
+                }
+            } else {
+                ++held;
+                if (lane == 0) mbar_arrive_expect_tx(&full[s], tma_job_bytes<D, T>(a, g, jp));
+                if (lane < Q) tma_issue_loads<D, T>(a, g, jp, buf, st, &full[s]);
+            }
+            if (++s == S) {
+                s = 0;
+                phase ^= 1u;
+            }
+        }
+        // store back the jobs that are left, the oldest first
+        if (held < S) {
+            s = 0;
+            phase = 0;
+        }
+        for (; held > 0 && !failed; --held) {
+            const bool ok = mbar_wait_bounded(&empty[s], phase, a.timeout_ns);
+            if (__any_sync(0xffffffffu, !ok)) {
+                failed = true;
+                break;
+            }
+            const JobPos jq = decode_job(a, g, old);
+            old += G;
+            T *st = sm + s * stage_elems;
+            if (a.odd && g.nseg > 1) tma_plain_stores<D, T>(a, g, jq, st, lane, 32);
+            if (lane < Q) {
+                tma_issue_stores<D, T>(a, g, jq, buf, st);
+                bulk_commit();
+            }
+            if (++s == S) {
+                s = 0;
+                phase ^= 1u;
+            }
+        }
+        bulk_wait_all();
+        if (failed) {
+            // let loads still in flight land before the block's shared memory is released: of the stages
+            // that hold jobs, s has the one that was not collided in time, the others have later ones
+            for (; held > 0; --held) {
+                (void)mbar_wait_bounded(&full[s], phase, a.timeout_ns);
+                if (++s == S) {
+                    s = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+    } else {
+        int s = 0;
+        uint32_t phase = 0;
+        for (unsigned job = blockIdx.x; job < total; job += G) {
+            const bool ok = mbar_wait_bounded(&full[s], phase, a.timeout_ns);
+            if (__any_sync(0xffffffffu, !ok)) {
+                failed = true;
+                break;
+            }
+            T *st = sm + s * stage_elems;
+            const JobPos jp = decode_job(a, g, job);
+            if (a.diag) tma_collide<D, P, EQ, BULK, CAPB, false, true>(a, g, jp, st, acc, threadIdx.x, ncons);
+            else tma_collide<D, P, EQ, BULK, CAPB, false, false>(a, g, jp, st, acc, threadIdx.x, ncons);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cta(&empty[s]);
+            if (++s == S) {
+                s = 0;
+                phase ^= 1u;
+            }
+        }
+    }
+    if (failed && lane == 0) report_status(a.status, -5); /* LBM_ETIMEOUT */
+    if (a.diag) diag_block_store(acc, a.partials + (int64_t)blockIdx.x * lbmh::kDiagWords);
+}
+
+// Several steps a launch (see decode_chain).  The warps after the consumers are the loader and the storer.
 constexpr int kTmaServiceThreads = 64;
 
 template <int D, int P, int EQ, bool BULK, int CAPB>
-__global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_step_tma(const lbmh::StepArgs a, const TmaGeom g) {
+__global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_steps_tma(const lbmh::StepArgs a, const TmaGeom g) {
     using T = typename Storage<P>::T;
     constexpr int Q = qof(D);
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -570,7 +731,6 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
     const int ncons = (int)blockDim.x - kTmaServiceThreads;
     const int lane = threadIdx.x & 31;
     const int role = (int)threadIdx.x < ncons ? 0 : ((int)threadIdx.x < ncons + 32 ? 1 : 2);
-    const bool chain = g.nsteps > 1;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -580,7 +740,7 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
         fence_barrier_init();
     }
     __syncthreads();
-    DiagAcc acc;
+    DiagAcc acc;  // (no diagnostics here)
     bool failed = false;
     if (role == 1) {
         // loader: takes the jobs, waits for the steps they need, refills the stages.  Its work for a
@@ -592,30 +752,25 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
         // a launch: 4096^2 FP32 118 -> 142 GLUPS, 4096^2 binary16 184 -> 205, 256^3 FP32 41.4 -> 46.0,
         // 512^3 binary16 73 -> 78.  (Two tickets at a time, decoded by half a warp each: 4 - 8 % slower.)
         const LaneBuf<T> buf = lane_buf<D, T>(a, lane);
-        const unsigned total = chain ? (unsigned)chain_tickets(g) : (unsigned)g.njobs;
-        unsigned next = blockIdx.x;
-        if (chain && lane == 0) next = atomicAdd(&a.sync[0], 1u);
+        const unsigned total = (unsigned)chain_tickets(g);
+        unsigned next = 0;
+        if (lane == 0) next = atomicAdd(&a.sync[0], 1u);
         int s = 0;
         uint32_t phase = 0;
         bool wrapped = false;
         for (;;) {
             JobPos jp{0, 0, 0, 0, 0, 0};
-            unsigned job = chain ? __shfl_sync(0xffffffffu, next, 0) : next;
+            const unsigned job = __shfl_sync(0xffffffffu, next, 0);
             bool end = job >= total;
             int step = 0, up = 0, uc = 0;
             if (!end) {
-                if (chain) {
-                    const ChainJob c = decode_chain(a, g, job);
-                    if (lane == 0) next = atomicAdd(&a.sync[0], 1u);  // in flight while this job is set up
-                    if (c.step < 0) continue;
-                    jp = c.j;
-                    step = c.step;
-                    up = c.p;
-                    uc = c.c;
-                } else {
-                    next = job + gridDim.x;
-                    jp = decode_job(a, g, job);
-                }
+                const ChainJob c = decode_chain(a, g, job);
+                if (lane == 0) next = atomicAdd(&a.sync[0], 1u);  // in flight while this job is set up
+                if (c.step < 0) continue;
+                jp = c.j;
+                step = c.step;
+                up = c.p;
+                uc = c.c;
             }
             if (wrapped) {  // the stage's last job has been stored
                 const bool ok = mbar_wait_bounded(&freed[s], phase ^ 1u, a.timeout_ns);
@@ -674,13 +829,11 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
             bulk_wait_read<0>();
             __syncwarp();
             if (lane == 0) mbar_arrive_cta(&freed[s]);
-            if (chain) {
-                // (a completed group's writes are visible to its thread; another proxy fence here
-                // held the storer for some 800 clocks a job)
-                bulk_wait_all();
-                __syncwarp();
-                if (lane == 0) red_release(&a.sync[lbmh::kSyncDone + unit], 1u);
-            }
+            // (a completed group's writes are visible to its thread; another proxy fence here
+            // held the storer for some 800 clocks a job)
+            bulk_wait_all();
+            __syncwarp();
+            if (lane == 0) red_release(&a.sync[lbmh::kSyncDone + unit], 1u);
             if (++s == S) {
                 s = 0;
                 phase ^= 1u;
@@ -703,38 +856,7 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
             const JobPos jp = jobq[s];
             if (jp.nrows > 0) {
                 T *st = sm + s * stage_elems;
-                const auto pairs = [&](auto mode, auto lone, auto diag) {
-                    tma_compute_pairs<D, P, EQ, BULK, CAPB, mode.value, lone.value, diag.value>(a, g, jp, st, acc, threadIdx.x, ncons);
-                };
-                using std::integral_constant;
-                constexpr std::true_type yes;
-                constexpr std::false_type no;
-                constexpr integral_constant<int, -1> any;
-                if constexpr (P == P_F64) {
-                    if (a.diag) tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else tma_compute<D, P, EQ, BULK, CAPB, false>(a, g, jp, st, acc, threadIdx.x, ncons);
-                } else if constexpr (D == 3) {
-                    // The D3Q27 pair body is long: one copy serves the three pairings (three
-                    // specialised copies measured slower).  One step a launch is bound by HBM (0.97 of the
-                    // copy peak), and two cells a thread only bunch its accesses: 512^3 binary16 60.1
-                    // GLUPS against 56.8.
-                    if (a.diag) tma_compute<D, P, EQ, BULK, CAPB, true>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else if (!chain) tma_compute<D, P, EQ, BULK, CAPB, false>(a, g, jp, st, acc, threadIdx.x, ncons);
-                    else if (jp.len & 1) pairs(any, yes, no);
-                    else pairs(any, no, no);
-                } else {
-                    constexpr integral_constant<int, 0> even;
-                    constexpr integral_constant<int, 1> rows;
-                    constexpr integral_constant<int, 2> segments;
-                    if (a.diag && (jp.len & 1)) pairs(any, yes, yes);
-                    else if (a.diag) pairs(any, no, yes);
-                    else if (jp.len & 1) {
-                        if (jp.odd) pairs(rows, yes, no);
-                        else pairs(even, yes, no);
-                    } else if (!jp.odd) pairs(even, no, no);
-                    else if (g.nseg == 1) pairs(rows, no, no);
-                    else pairs(segments, no, no);
-                }
+                tma_collide<D, P, EQ, BULK, CAPB, true, false>(a, g, jp, st, acc, threadIdx.x, ncons);
                 fence_proxy_async_smem();
                 __syncwarp();
             }
@@ -747,37 +869,41 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_
         }
     }
     if (failed && lane == 0) report_status(a.status, -5); /* LBM_ETIMEOUT */
-    if (chain) {
-        // the last block to finish clears the counters for the next launch
-        __syncthreads();
-        bool last = false;
-        if (threadIdx.x == 0) {
-            __threadfence();
-            last = atomicAdd(&a.sync[1], 1u) == gridDim.x - 1;
-        }
-        if (__syncthreads_or(last)) {
-            uint4 *w = reinterpret_cast<uint4 *>(a.sync);
-            for (int p = threadIdx.x; p < (lbmh::kSyncDone + g.npos * g.ncross + 3) / 4; p += blockDim.x)
-                w[p] = make_uint4(0, 0, 0, 0);
-        }
+    // the last block to finish clears the counters for the next launch
+    __syncthreads();
+    bool last = false;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&a.sync[1], 1u) == gridDim.x - 1;
     }
-    if (a.diag) diag_block_store(acc, a.partials + (int64_t)blockIdx.x * lbmh::kDiagWords);
+    if (__syncthreads_or(last)) {
+        uint4 *w = reinterpret_cast<uint4 *>(a.sync);
+        for (int p = threadIdx.x; p < (lbmh::kSyncDone + g.npos * g.ncross + 3) / 4; p += blockDim.x)
+            w[p] = make_uint4(0, 0, 0, 0);
+    }
 }
 
 template <int D, int P, int CAPB>
-const void *tma_kernel_dpc(int eq, int bulk) {
-    if (eq == EQ_ENT) return bulk ? (const void *)k_step_tma<D, P, EQ_ENT, true, CAPB> : (const void *)k_step_tma<D, P, EQ_ENT, false, CAPB>;
-    if (eq == EQ_POLY2) return bulk ? (const void *)k_step_tma<D, P, EQ_POLY2, true, CAPB> : (const void *)k_step_tma<D, P, EQ_POLY2, false, CAPB>;
-    if (eq == EQ_PROD) return bulk ? (const void *)k_step_tma<D, P, EQ_PROD, true, CAPB> : (const void *)k_step_tma<D, P, EQ_PROD, false, CAPB>;
+const void *tma_kernel_dpc(int eq, int bulk, bool several) {
+#define LBM_TMA(EQv, Bv)                                                                                       \
+    if (eq == EQv && (bulk != 0) == Bv)                                                                        \
+        return several ? (const void *)k_steps_tma<D, P, EQv, Bv, CAPB> : (const void *)k_step_tma<D, P, EQv, Bv, CAPB>;
+    LBM_TMA(EQ_ENT, false)
+    LBM_TMA(EQ_ENT, true)
+    LBM_TMA(EQ_POLY2, false)
+    LBM_TMA(EQ_POLY2, true)
+    LBM_TMA(EQ_PROD, false)
+    LBM_TMA(EQ_PROD, true)
+#undef LBM_TMA
     return nullptr;
 }
 
 template <int D, int CAPB>
-const void *tma_kernel_dc(int P, int eq, int bulk) {
+const void *tma_kernel_dc(int P, int eq, int bulk, bool several) {
     switch (P) {
-    case P_F64: return tma_kernel_dpc<D, P_F64, CAPB>(eq, bulk);
-    case P_F32: return tma_kernel_dpc<D, P_F32, CAPB>(eq, bulk);
-    case P_F16S: return tma_kernel_dpc<D, P_F16S, CAPB>(eq, bulk);
+    case P_F64: return tma_kernel_dpc<D, P_F64, CAPB>(eq, bulk, several);
+    case P_F32: return tma_kernel_dpc<D, P_F32, CAPB>(eq, bulk, several);
+    case P_F16S: return tma_kernel_dpc<D, P_F16S, CAPB>(eq, bulk, several);
     default: return nullptr;
     }
 }

@@ -2,5 +2,5 @@
 #include "k_tma.cuh"
 
 namespace lbmh {
-const void *tma_kernel_d3_c8192(int P, int eq, int bulk) { return lbmd::tma_kernel_dc<3, 8192>(P, eq, bulk); }
+const void *tma_kernel_d3_c8192(int P, int eq, int bulk, bool several) { return lbmd::tma_kernel_dc<3, 8192>(P, eq, bulk, several); }
 }  // namespace lbmh

@@ -6,7 +6,7 @@
 
 namespace lbmh {
 
-#define LBM_DECL_CAP(d, c) const void *tma_kernel_d##d##_c##c(int P, int eq, int bulk);
+#define LBM_DECL_CAP(d, c) const void *tma_kernel_d##d##_c##c(int P, int eq, int bulk, bool several);
 LBM_DECL_CAP(2, 1024)
 LBM_DECL_CAP(2, 2048)
 LBM_DECL_CAP(2, 4096)
@@ -19,20 +19,20 @@ LBM_DECL_CAP(3, 8192)
 
 constexpr int kTmaMaxSmem = 227 * 1024;  // shared memory of a block, static and dynamic
 
-static const void *tma_kernel(const Lattice &lat, int eq, int bulk, int cap) {
+static const void *tma_kernel(const Lattice &lat, int eq, int bulk, int cap, bool several) {
     if (lat.D == 2) {
         switch (cap) {
-        case 1024: return tma_kernel_d2_c1024(lat.P, eq, bulk);
-        case 2048: return tma_kernel_d2_c2048(lat.P, eq, bulk);
-        case 4096: return tma_kernel_d2_c4096(lat.P, eq, bulk);
-        case 8192: return tma_kernel_d2_c8192(lat.P, eq, bulk);
+        case 1024: return tma_kernel_d2_c1024(lat.P, eq, bulk, several);
+        case 2048: return tma_kernel_d2_c2048(lat.P, eq, bulk, several);
+        case 4096: return tma_kernel_d2_c4096(lat.P, eq, bulk, several);
+        case 8192: return tma_kernel_d2_c8192(lat.P, eq, bulk, several);
         }
     } else {
         switch (cap) {
-        case 1024: return tma_kernel_d3_c1024(lat.P, eq, bulk);
-        case 2048: return tma_kernel_d3_c2048(lat.P, eq, bulk);
-        case 4096: return tma_kernel_d3_c4096(lat.P, eq, bulk);
-        case 8192: return tma_kernel_d3_c8192(lat.P, eq, bulk);
+        case 1024: return tma_kernel_d3_c1024(lat.P, eq, bulk, several);
+        case 2048: return tma_kernel_d3_c2048(lat.P, eq, bulk, several);
+        case 4096: return tma_kernel_d3_c4096(lat.P, eq, bulk, several);
+        case 8192: return tma_kernel_d3_c8192(lat.P, eq, bulk, several);
         }
     }
     return nullptr;
@@ -84,8 +84,7 @@ static lbmd::TmaGeom geom(const Lattice &lat, const TmaShape &t) {
 // the first and the last of them fits in L2: the jobs in flight (every stage of every block and
 // a ticket or two more) spread over depth x pjobs jobs a phase, and two positions for the neighbours.
 static bool chain_geom(const Lattice &lat, const TmaShape &t, int nsteps, lbmd::TmaGeom &g) {
-    constexpr int64_t kResident = (int64_t)75 << 20;  // state that stays in the 129 MB L2 between steps
-    constexpr int64_t kWindow = (int64_t)60 << 20;    // and the travelling window of a larger one
+    constexpr int64_t kWindow = (int64_t)60 << 20;  // the travelling window of a state that does not stay in L2
     g.nsteps = nsteps;
     g.npos = lat.D == 3 ? lat.nz : g.ygroups;
     g.ncross = lat.D == 3 ? g.ygroups : 1;
@@ -97,7 +96,7 @@ static bool chain_geom(const Lattice &lat, const TmaShape &t, int nsteps, lbmd::
     g.lag = 0;
     const int64_t state = (int64_t)lbmd::qof(lat.D) * lat.plane * esize(lat.P);
     // (112^3 binary16, 72 MiB: 74.9 GLUPS against 73.6 swept; 1600^2 FP32, 88 MiB: 121 against 143 swept)
-    if (state <= kResident || lat.P == lbmd::P_F64) return true;
+    if (state <= kTmaResident || lat.P == lbmd::P_F64) return true;
     const int64_t unit = state / ((int64_t)g.npos * g.ncross);
     // (measured in GLUPS, 3-D / 2-D: with a job more in the lag 256^3 FP32 44.7 against 46.0 and 128^3
     // FP32 44.8 against 47.8, but 4096^2 binary16 205 against 200 and 2048^2 FP32 132 against 128;
@@ -163,41 +162,50 @@ int tma_smem_bytes(const Lattice &lat, const TmaShape &t) {
 // (With the size of the shape at hand, creating a lattice of 2 stages made the launches of one of 3
 // stages fail.)
 cudaError_t tma_prepare(const Lattice &lat, int eq, int bulk, int cap) {
-    const void *fn = tma_kernel(lat, eq, bulk, cap);
-    if (!fn) return cudaErrorInvalidValue;
-    cudaFuncAttributes at;
-    cudaError_t e = cudaFuncGetAttributes(&at, fn);
-    const int most = kTmaMaxSmem - (int)at.sharedSizeBytes;
-    if (e == cudaSuccess && at.maxDynamicSharedSizeBytes < most)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    return e;
+    for (const bool several : {false, true}) {
+        const void *fn = tma_kernel(lat, eq, bulk, cap, several);
+        if (!fn) return cudaErrorInvalidValue;
+        cudaFuncAttributes at;
+        cudaError_t e = cudaFuncGetAttributes(&at, fn);
+        const int most = kTmaMaxSmem - (int)at.sharedSizeBytes;
+        if (e == cudaSuccess && at.maxDynamicSharedSizeBytes < most)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
-int tma_max_blocks_per_sm(const Lattice &lat, int eq, int bulk, const TmaShape &t) {
-    const void *fn = tma_kernel(lat, eq, bulk, t.cap);
-    int n = 0;
+bool tma_set_blocks(const Lattice &lat, int eq, int bulk, int sms, TmaShape &t) {
     if (tma_prepare(lat, eq, bulk, t.cap) != cudaSuccess) {
         cudaGetLastError();
-        return 0;
+        return false;
     }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, t.threads + lbmd::kTmaServiceThreads, t.smem_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
+    for (const bool several : {false, true}) {
+        const void *fn = tma_kernel(lat, eq, bulk, t.cap, several);
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, t.threads + (several ? lbmd::kTmaServiceThreads : 32), t.smem_bytes) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (n < 1) return false;
+        (several ? t.blocks : t.one_blocks) = sms * n;
     }
-    return n;
+    return true;
 }
 
 cudaError_t step_tma(const StepArgs &a, const TmaShape &t, int nsteps, cudaStream_t s) {
-    const void *fn = tma_kernel(a.lat, a.eq, a.bulk, t.cap);
+    const bool several = nsteps > 1;
+    const void *fn = tma_kernel(a.lat, a.eq, a.bulk, t.cap, several);
     if (!fn) return cudaErrorInvalidValue;
     lbmd::TmaGeom g = geom(a.lat, t);
     StepArgs aa = a;
     void *args[] = {(void *)&aa, (void *)&g};
-    int blocks = t.blocks;
-    if (nsteps > 1) {
+    int blocks = t.one_blocks;
+    if (several) {
         if (!chain_geom(a.lat, t, nsteps, g)) return cudaErrorInvalidValue;
         // more blocks than jobs of one step would only wait for one another
-        blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, g.njobs));
+        blocks = (int)std::min<int64_t>(t.blocks, std::max<int64_t>(1, g.njobs));
     }
     g.by_nseg = lbmd::fast_div(g.nseg);
     g.by_ygroups = lbmd::fast_div(g.ygroups);
@@ -205,8 +213,8 @@ cudaError_t step_tma(const StepArgs &a, const TmaShape &t, int nsteps, cudaStrea
     g.by_strips = lbmd::fast_div(std::max(1, g.strips));
     g.by_pjobs = lbmd::fast_div(std::max(1, g.pjobs));
     g.by_depth = lbmd::fast_div(std::max(1, g.depth));
-    // t.threads consumer threads plus the loader and the storer warp
-    return cudaLaunchKernel(fn, dim3(blocks), dim3(t.threads + lbmd::kTmaServiceThreads), args, (size_t)t.smem_bytes, s);
+    // t.threads consumer threads plus the service warp, or the loader and the storer
+    return cudaLaunchKernel(fn, dim3(blocks), dim3(t.threads + (several ? lbmd::kTmaServiceThreads : 32)), args, (size_t)t.smem_bytes, s);
 }
 
 }  // namespace lbmh

@@ -37,8 +37,9 @@ struct StepArgs {
 
 // Launch shape of the TMA row-staged kernel.
 struct TmaShape {
-    int threads;    // consumer threads per block (the loader and the storer warp are added)
-    int blocks;     // grid size (persistent blocks)
+    int threads;    // consumer threads per block (the service warps are added)
+    int blocks;     // grid size (persistent blocks) of several steps a launch
+    int one_blocks; // and of one
     int stages;     // shared-memory pipeline depth (>= 2)
     int rows;       // rows per job (>= 1; 1 when the row is split into segments)
     int seg;        // cells per row segment (== nx for whole rows)
@@ -49,6 +50,7 @@ struct TmaShape {
 constexpr int kDiagWords = 8;  // mass, jx, jy, jz, kinetic, max|u|, nonfinite, unused
 constexpr int kBarStride = 32;  // counters of team barriers, one to a 128-byte line
 constexpr int kSyncDone = 4;  // first done counter in StepArgs::sync (after the ticket and exit counters)
+constexpr int64_t kTmaResident = (int64_t)75 << 20;  // populations that stay in the 129 MB L2 between steps
 constexpr int kTmaMaxStages = 8;  // deepest shared-memory pipeline of the TMA row kernel
 
 // api.cu: record the message of a failed call for lbm_last_error(); returns code.
@@ -94,7 +96,7 @@ int padded_pitch(int D, int P, int64_t nx);
 int tma_smem_bytes(const Lattice &lat, const TmaShape &t);
 // Largest number of colliding threads per block of the TMA kernel for the lattice.
 int tma_thread_limit(const Lattice &lat);
-// Raises the kernel's dynamic shared memory limit to the most a block can have.
+// Raises the kernels' dynamic shared memory limits to the most a block can have.
 cudaError_t tma_prepare(const Lattice &lat, int eq, int bulk, int cap);
 // Done counters a lattice is given (a row group has at least one row).
 int64_t sync_units(const Lattice &lat);
@@ -102,7 +104,8 @@ int64_t sync_units(const Lattice &lat);
 // more units than counters.
 int64_t tma_max_steps(const Lattice &lat, const TmaShape &t);
 cudaError_t step_tma(const StepArgs &a, const TmaShape &t, int nsteps, cudaStream_t s);
-int tma_max_blocks_per_sm(const Lattice &lat, int eq, int bulk, const TmaShape &t);
+// Sets the grid sizes of a shape: as many blocks as fit on the device.  False if none does.
+bool tma_set_blocks(const Lattice &lat, int eq, int bulk, int sms, TmaShape &t);
 
 // k_batch.cu -- many independent lattices in one arena (FP64, shifted).  Instance k has
 // ncell_k = cell_start[k + 1] - cell_start[k] cells; its populations are Q planes of
