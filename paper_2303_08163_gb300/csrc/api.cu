@@ -217,8 +217,9 @@ cudaError_t launch_steps(lbm_ctx *c, int odd, int64_t n, cudaStream_t s) {
         }
         return e;
     }
+    // (a few FP64 steps in 2-D are as well launched one by one: 512^2, two steps 66 us each, one by one 52)
     int64_t most = 1;
-    if (c->kernel == 2 && n > 1) most = tma_max_steps(c->lat, c->tma);
+    if (c->kernel == 2 && n > (c->D == 2 && c->prec == LBM_F64 ? 4 : 1)) most = tma_max_steps(c->lat, c->tma);
     cudaError_t e = cudaSuccess;
     while (n > 0 && e == cudaSuccess) {
         const int64_t m = std::min(n, most);

@@ -46,3 +46,20 @@ def test_single_steps(D, dims, prec, shape, eq, bulk):
     for lat in lats:
         lat.sync()
         lat.close()
+
+
+@pytest.mark.parametrize("dims", [(300, 500, 1), (512, 400, 1), (640, 260, 1)])
+def test_few_fp64_steps(dims):
+    """Numbers of FP64 steps on both sides of the rule, at both parities."""
+    from paper_2303_08163_gb300 import lbm
+    rho, u = inputs.random_state(2, dims, seed=3, u_max=0.1)
+    lats = [lbm.Lattice(lbm.D2Q9, dims, 0.6, 0, 1, lbm.F64) for _ in range(2)]
+    lats[1].set_launch_shape(lbm.KERNEL_GENERIC, 128)
+    for lat in lats:
+        lat.init_fields(rho, u)
+    for n in (2, 3, 4, 5, 6, 1, 4, 5):
+        for lat in lats:
+            lat.step(n)
+        assert np.array_equal(*(lat.get_populations("storage") for lat in lats)), n
+    for lat in lats:
+        lat.close()
