@@ -356,11 +356,11 @@ __global__ void __launch_bounds__(kVnThreads) k_vn_eigs(int64_t count, const dou
 }
 
 // The bisection state of one (nu, theta) pair.  A round sweeps all wave vectors at the pair's
-// next trial speed.  Beside it the round looks ahead: at the trial speeds that may follow (a
-// binary tree below the swept one, node n with children 2 n after an unstable and 2 n + 1 after
-// a stable trial) it tries the one wave vector that made the last unstable trial unstable.
+// next trial speed.  Beside it the round looks ahead: it tries the one wave vector that made the last
+// unstable trial unstable at the trial speeds that follow as long as trials are unstable, after an
+// unstable swept trial and after a stable one (vn_look_node; in the tree of trials below the swept
+// one, node 1, node n has children 2 n after an unstable and 2 n + 1 after a stable trial).
 // Where that is unstable again the trial is decided, and needs no sweep.
-constexpr int kLook = 64;  // nodes of the tree (node 1 is the swept trial)
 struct VnPair {
     double tau, theta, lo, hi, trial;
     double A[81];              // delta + J at the trial speed
@@ -370,7 +370,7 @@ struct VnPair {
     int level;                 // trials decided (the first is u_hi itself)
     int done;                  // the limit is known
     unsigned long long look;   // `cand` as the round began
-    int unstable[kLook];       // what the look-ahead found
+    int unstable[lbmh::kVnLooks];  // what the look-ahead found
 };
 
 // The bisection interval of tree node n below [lo, hi] (whose midpoint is node 1).
@@ -384,10 +384,10 @@ __device__ __forceinline__ double vn_node(double &lo, double &hi, int n) {
 }
 
 // One round (54 pairs x 25 x 25 wave vectors, 14 trials: a search took 15 sweeps of 4.1 ms and now
-// 42 - 44 ms in all, 4.1 ms for the equilibrium that is stable at u_hi).  Blocks of the look-ahead (32 / G nodes of one pair each), then of the sweep (32 / G
-// wave vectors of one pair each).  A pair whose limit is known, or that some wave vector has
-// already shown to be unstable, is skipped: one is enough.  The largest radius is kept per pair by
-// an integer atomicMax on its bits (order-preserving for values >= 0).
+// 42 ms in all, 4.1 ms for the equilibrium that is stable at u_hi).  Blocks of the look-ahead (32 / G
+// trial speeds of one pair each), then of the sweep (32 / G wave vectors of one pair each).  A pair whose limit is known, or that some wave vector has already shown to be unstable,
+// is skipped: one is enough.  The largest radius is kept per pair by an integer atomicMax on its bits
+// (order-preserving for values >= 0).  A look-ahead that does not converge decides nothing.
 template <int G, int EQ>
 __global__ void __launch_bounds__(kVnThreads) k_vn_round(int64_t npairs, VnPair *pairs, int nk, double tol,
                                                          int32_t *status) {
@@ -396,19 +396,19 @@ __global__ void __launch_bounds__(kVnThreads) k_vn_round(int64_t npairs, VnPair 
     const Mat<G> M(sm);
     const int m = (threadIdx.x & 31) / G;
     const int nkk = nk * nk;
-    const int64_t looks = npairs * (kLook / per), work = looks + npairs * ((nkk + per - 1) / per);
+    const int64_t looks = npairs * ((lbmh::kVnLooks + per - 1) / per), work = looks + npairs * ((nkk + per - 1) / per);
     for (int64_t w = blockIdx.x; w < work; w += gridDim.x) {
         const bool look = w < looks;
         const int64_t v = look ? w : w - looks, chunk = v / npairs, pr = v - chunk * npairs;
         VnPair *P = pairs + pr;
-        const int q = (int)chunk * per + m;  // tree node or wave vector
+        const int q = (int)chunk * per + m;  // number of the trial looked at, or wave vector
         const int kk = look ? (int)(unsigned)P->look - 1 : q;
         // (one lane reads what other blocks write, so that the group takes one branch)
         unsigned long long seen = 0;
         if (M.g == 0 && !look) seen = *(volatile unsigned long long *)&P->worst;
         seen = __shfl_sync(0xffffffffu, seen, threadIdx.x & 31 & ~(G - 1));
         const bool todo = !P->done && kk >= 0 && kk < nkk &&
-                          (look ? q >= 2 && P->level > 0 : !(__longlong_as_double((long long)seen) > 1.0 + tol));
+                          (look ? q < lbmh::kVnLooks && P->level > 0 : !(__longlong_as_double((long long)seen) > 1.0 + tol));
         if (todo) {
             const int ix = kk % nk, iy = kk / nk;
             const double pi = 3.14159265358979323846;
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kVnThreads) k_vn_round(int64_t npairs, VnPair 
             double ux = 0.0, uy = 0.0;
             if (look) {
                 double lo = P->lo, hi = P->hi, st, ct;
-                const double u = vn_node(lo, hi, q);
+                const double u = vn_node(lo, hi, lbmh::vn_look_node(q));
                 sincos(P->theta, &st, &ct);
                 ux = u * ct;
                 uy = u * st;
@@ -431,14 +431,15 @@ __global__ void __launch_bounds__(kVnThreads) k_vn_round(int64_t npairs, VnPair 
                 }
                 M.set_row(i, row, kx, ky);
             }
-            if (!eig_hessenberg_qr(M) && M.g == 0) atomicExch(status, 1);
+            const bool converged = eig_hessenberg_qr(M);
+            if (!converged && !look && M.g == 0) atomicExch(status, 1);
             if (M.g == 0) {
                 double r = 0.0;
                 for (int a = 0; a < kN; ++a) r = fmax(r, cabsd(M.get(a, a)));
                 if (!(r >= 0.0)) r = 1e300;  // NaN: treat as unstable
                 const bool unstable = r > 1.0 + tol;
                 if (look) {
-                    P->unstable[q] = unstable;
+                    P->unstable[q] = converged && unstable;
                 } else {
                     atomicMax(&P->worst, (unsigned long long)__double_as_longlong(r));
                     if (unstable)
@@ -463,32 +464,33 @@ __global__ void __launch_bounds__(32) k_vn_bisect(int64_t npairs, VnPair *pairs,
         int done = P->done, level = P->level;
         if (!start && !done) {
             const bool stable = __longlong_as_double((long long)P->worst) <= 1.0 + tol;
-            int node = 1;
+            int next = 0, last = 0;  // the look-ahead's trials that follow
             if (level == 0) {  // the trial was u_hi itself: a pair stable there reports u_hi
                 if (stable) {
                     lo = hi = u_hi;
                     done = 1;
                 }
-                node = kLook;  // nothing was looked up yet
+                next = last = 0;  // nothing was looked up yet
             } else {
                 if (lo < hi) {
                     if (stable) lo = trial;
                     else hi = trial;
                 }
-                node = stable ? 3 : 2;
+                next = stable ? lbmh::kVnLooks / 2 : 0;
+                last = next + lbmh::kVnLooks / 2;
             }
             ++level;
             trial = 0.5 * (lo + hi);
-            while (level <= iterations && node < kLook && P->unstable[node]) {
+            while (level <= iterations && next < last && P->unstable[next]) {
                 if (lo < hi) hi = trial;
-                node = 2 * node;
+                ++next;
                 ++level;
                 trial = 0.5 * (lo + hi);
             }
             if (level > iterations) done = 1;
         }
         __syncwarp();
-        for (int q = threadIdx.x; q < kLook; q += 32) P->unstable[q] = 0;
+        if (threadIdx.x < lbmh::kVnLooks) P->unstable[threadIdx.x] = 0;
         if (threadIdx.x == 0) {
             P->lo = lo;
             P->hi = hi;
@@ -573,7 +575,7 @@ static cudaError_t vn_limit_g(int64_t npairs, VnPair *P, int nk, double u_hi, in
                                int32_t *status, cudaStream_t s) {
     constexpr int per = kVnThreads / G;
     const int gb = grid_n(npairs);
-    const int gr = grid_n(npairs * (kLook / per + ((int64_t)nk * nk + per - 1) / per));
+    const int gr = grid_n(npairs * ((kVnLooks + per - 1) / per + ((int64_t)nk * nk + per - 1) / per));
     k_vn_bisect<EQ><<<gb, 32, 0, s>>>(npairs, P, 1, iterations, u_hi, tol);
     for (int it = 0; it <= iterations; ++it) {  // every round decides at least one trial of a pair
         k_vn_round<G, EQ><<<gr, kVnThreads, 0, s>>>(npairs, P, nk, tol, status);

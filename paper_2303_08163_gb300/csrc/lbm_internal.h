@@ -162,6 +162,11 @@ cudaError_t batch_populations(const double *arena, const int64_t *cell_start,
 // k_vn.cu
 cudaError_t vn_eigs(int eq, int bulk, int64_t count, const double *params, double *out, int32_t *status,
                     cudaStream_t s);
+// Trial speeds that a round of the stability search looks ahead at, as nodes of the tree of trials below
+// the swept one (node 1; node n is followed by 2 n if unstable, 2 n + 1 if stable): those that unstable
+// trials lead to after an unstable swept one (2, 4, .. 32), and after a stable one (3, 6, .. 48).
+constexpr int kVnLooks = 10;
+constexpr int vn_look_node(int q) { return q < kVnLooks / 2 ? 2 << q : 3 << (q - kVnLooks / 2); }
 // Stability-limit search: vn_limit_bytes of state per call, filled and read on the host, all
 // trials enqueued by vn_limit.
 size_t vn_limit_bytes(int64_t npairs);
