@@ -385,23 +385,36 @@ __device__ __forceinline__ double vn_node(double &lo, double &hi, int n) {
 
 // One round (54 pairs x 25 x 25 wave vectors, 14 trials: a search took 15 sweeps of 4.1 ms and now
 // 42 ms in all, 4.1 ms for the equilibrium that is stable at u_hi).  Blocks of the look-ahead (32 / G
-// trial speeds of one pair each), then of the sweep (32 / G wave vectors of one pair each).  A pair whose limit is known, or that some wave vector has already shown to be unstable,
+// trial speeds of one pair each), then of the sweep (32 / G wave vectors of one pair each); without the
+// look-ahead 32 / G wave vectors of whichever pairs they belong to.  A pair whose limit is known, or that some wave vector has already shown to be unstable,
 // is skipped: one is enough.  The largest radius is kept per pair by an integer atomicMax on its bits
 // (order-preserving for values >= 0).  A look-ahead that does not converge decides nothing.
 template <int G, int EQ>
 __global__ void __launch_bounds__(kVnThreads) k_vn_round(int64_t npairs, VnPair *pairs, int nk, double tol,
-                                                         int32_t *status) {
+                                                         bool ahead, int32_t *status) {
     constexpr int per = kVnThreads / G;
     __shared__ double2 sm[kN * kN * per];
     const Mat<G> M(sm);
     const int m = (threadIdx.x & 31) / G;
     const int nkk = nk * nk;
-    const int64_t looks = npairs * ((lbmh::kVnLooks + per - 1) / per), work = looks + npairs * ((nkk + per - 1) / per);
+    const int64_t looks = ahead ? npairs * ((lbmh::kVnLooks + per - 1) / per) : 0;
+    const int64_t work = ahead ? looks + npairs * ((nkk + per - 1) / per) : (npairs * nkk + per - 1) / per;
     for (int64_t w = blockIdx.x; w < work; w += gridDim.x) {
         const bool look = w < looks;
-        const int64_t v = look ? w : w - looks, chunk = v / npairs, pr = v - chunk * npairs;
+        // the pair, and the number of the trial looked at or of the wave vector
+        int64_t pr;
+        int q;
+        if (ahead) {
+            const int64_t v = look ? w : w - looks, chunk = v / npairs;
+            pr = v - chunk * npairs;
+            q = (int)chunk * per + m;
+        } else {
+            const int64_t v = w * per + m;
+            pr = v / nkk;
+            q = pr < npairs ? (int)(v - pr * nkk) : nkk;
+            pr = pr < npairs ? pr : 0;
+        }
         VnPair *P = pairs + pr;
-        const int q = (int)chunk * per + m;  // number of the trial looked at, or wave vector
         const int kk = look ? (int)(unsigned)P->look - 1 : q;
         // (one lane reads what other blocks write, so that the group takes one branch)
         unsigned long long seen = 0;
@@ -575,10 +588,16 @@ static cudaError_t vn_limit_g(int64_t npairs, VnPair *P, int nk, double u_hi, in
                                int32_t *status, cudaStream_t s) {
     constexpr int per = kVnThreads / G;
     const int gb = grid_n(npairs);
-    const int gr = grid_n(npairs * ((kVnLooks + per - 1) / per + ((int64_t)nk * nk + per - 1) / per));
+    // The look-ahead where it costs little: at most an eighth of a sweep, or no more than there are SM
+    // quarters to run it beside the sweep.  Otherwise the wave vectors of the pairs lie densely on the lanes
+    // (2000 pairs, 3 x 3 wave vectors: look-ahead and a block for each pair 132 ms, no look-ahead 83, densely 28; one
+    // matrix a thread and all sweeps took 34).
+    const int64_t looks = (kVnLooks + per - 1) / per, sweep = ((int64_t)nk * nk + per - 1) / per;
+    const bool ahead = 8 * looks <= sweep || npairs * (looks + sweep) <= 608;
+    const int gr = grid_n(ahead ? npairs * (sweep + looks) : (npairs * nk * nk + per - 1) / per);
     k_vn_bisect<EQ><<<gb, 32, 0, s>>>(npairs, P, 1, iterations, u_hi, tol);
     for (int it = 0; it <= iterations; ++it) {  // every round decides at least one trial of a pair
-        k_vn_round<G, EQ><<<gr, kVnThreads, 0, s>>>(npairs, P, nk, tol, status);
+        k_vn_round<G, EQ><<<gr, kVnThreads, 0, s>>>(npairs, P, nk, tol, ahead, status);
         k_vn_bisect<EQ><<<gb, 32, 0, s>>>(npairs, P, 0, iterations, u_hi, tol);
     }
     return cudaGetLastError();
