@@ -28,10 +28,21 @@ static inline int grid_for(int64_t n, int threads, int cap = 152 * 32) {
 // where a 2-byte access for each population leaves the memory pipe half used (512^3: initialisation
 // 2.43 -> 1.52 ms, moments 2.06 - 2.48 -> 1.45 - 1.85 ms, 1.39 ms of HBM time), otherwise 1.  Kernels that
 // write the stored populations run over the rows with their padding and write each plane where the
-// thread is, so that warps write whole aligned segments; shifts go into the reads (FP32
-// 245 x 196 x 172: initialisation 0.34 -> 0.21 ms; FP32 256^3 populations after an odd number of
-// steps 0.86 -> 0.60 ms.  FP64 populations, whose 8-byte accesses fill segments anyway, are
-// written where they belong: 0.14 against 0.19 ms on 128^3).
+// thread is, so that warps write whole aligned segments, the padding (with the row's last value) included;
+// shifts go into the reads (FP32 245 x 196 x 172: initialisation 0.34 -> 0.21 ms; FP32 256^3
+// populations after an odd number of steps 0.86 -> 0.60 ms.  FP64 populations, whose 8-byte accesses
+// fill segments anyway, are written where they belong: 0.14 against 0.19 ms on 128^3).
+
+// Cell of an element of the padded rows (in the padding: the row's last cell), for V = 2 the first of two.
+__device__ __forceinline__ int64_t padded_cell(const lbmh::Lattice &lat, int64_t p, int64_t padded, int &x) {
+    x = 0;
+    if (lat.pitch == lat.nx) return p;
+    int64_t row;
+    if (padded < ((int64_t)1 << 31)) row = (unsigned)p / (unsigned)lat.pitch;
+    else row = p / lat.pitch;
+    x = min((int)(p - row * lat.pitch), lat.nx - 1);
+    return row * lat.nx + x;
+}
 
 // V stored values at p (V = 2: p even).
 template <int P, int V>
@@ -60,14 +71,12 @@ __global__ void k_init(lbmh::Lattice lat, double rho0d, const In *__restrict__ r
     const int64_t padded = (int64_t)lat.pitch * lat.ny * lat.nz;
     for (int64_t p = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); p < padded;
          p += V * (int64_t)gridDim.x * blockDim.x) {
-        int x, y, z;
-        cell_coords(p, padded, lat.pitch, lat.ny, x, y, z);
-        if (x >= lat.nx) continue;
-        const int64_t c = x + (int64_t)lat.nx * (y + (int64_t)lat.ny * z);
+        int x;
+        const int64_t c = padded_cell(lat, p, padded, x);
         R r[V], drho[V], h[V][Q];
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            const int64_t cv = V == 1 || x + v < lat.nx ? c + v : c;  // (a row's last pair may end in its padding)
+            const int64_t cv = V == 1 || lat.pitch == lat.nx || x + v < lat.nx ? c + v : c;  // (a row's last pair may end in its padding)
             r[v] = R(rho[cv]);
             R uu[3] = {R(u[cv]), R(u[lat.ncell + cv]), D == 3 ? R(u[2 * lat.ncell + cv]) : R(0)};
             equilibrium_h<D, EQ, R>(uu, h[v]);
@@ -188,8 +197,8 @@ __global__ void k_set_pop(lbmh::Lattice lat, ClassShift k, int odd, const In *__
          p += V * (int64_t)gridDim.x * blockDim.x) {
         int x, y, z;
         cell_coords(p, padded, lat.pitch, lat.ny, x, y, z);
-        if (x >= lat.nx) continue;
         if constexpr (P == P_F64) {
+            if (x >= lat.nx) continue;
             const int64_t c = x + (int64_t)lat.nx * (y + (int64_t)lat.ny * z);
 #pragma unroll
             for (int i = 0; i < Q; ++i)
@@ -207,7 +216,7 @@ __global__ void k_set_pop(lbmh::Lattice lat, ClassShift k, int odd, const In *__
             const In *row = f + (int64_t)i * lat.ncell + (int64_t)lat.nx * (yy + (int64_t)lat.ny * zz);
 #pragma unroll
             for (int q = 0; q < V; ++q) {
-                const int xv = x + q < lat.nx ? x + q : x;
+                const int xv = min(x + q, lat.nx - 1);
                 v[i][q] = row[odd ? wrapi(xv + cxo(i), lat.nx) : xv];
             }
         }
