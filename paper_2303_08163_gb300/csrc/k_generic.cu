@@ -30,8 +30,9 @@ static inline int grid_for(int64_t n, int threads, int cap = 152 * 32) {
 // write the stored populations run over the rows with their padding and write each plane where the
 // thread is, so that warps write whole aligned segments, the padding (with the row's last value) included;
 // shifts go into the reads (FP32 245 x 196 x 172: initialisation 0.34 -> 0.21 ms; FP32 256^3
-// populations after an odd number of steps 0.86 -> 0.60 ms.  FP64 populations, whose 8-byte accesses
-// fill segments anyway, are written where they belong: 0.14 against 0.19 ms on 128^3).
+// populations after an odd number of steps 0.86 -> 0.60 ms).  Populations from FP64 arrays into FP64 or
+// FP32 storage are written where they belong: their reads are the wider ones (128^3 FP64 0.14 against
+// 0.19 ms, FP32 0.21 against 0.26).
 
 // Cell of an element of the padded rows (in the padding: the row's last cell), for V = 2 the first of two.
 __device__ __forceinline__ int64_t padded_cell(const lbmh::Lattice &lat, int64_t p, int64_t padded, int &x) {
@@ -197,7 +198,7 @@ __global__ void k_set_pop(lbmh::Lattice lat, ClassShift k, int odd, const In *__
          p += V * (int64_t)gridDim.x * blockDim.x) {
         int x, y, z;
         cell_coords(p, padded, lat.pitch, lat.ny, x, y, z);
-        if constexpr (P == P_F64) {
+        if constexpr (P == P_F64 || (P == P_F32 && sizeof(In) == 8)) {
             if (x >= lat.nx) continue;
             const int64_t c = x + (int64_t)lat.nx * (y + (int64_t)lat.ny * z);
 #pragma unroll
