@@ -408,8 +408,13 @@ cudaError_t steps_small(const StepArgs &a, int nsteps, const SmallShape &t, cuda
         else return cudaErrorInvalidValue;                                                 \
     } while (0)
 
-// Pairs of binary16 cells: rows (with their padding where the kernel writes them) of even length.
-static bool pairs_ok(const Lattice &lat, bool writes) { return ((writes ? lat.pitch : lat.nx) & 1) == 0; }
+// Pairs of binary16 cells: rows (with their padding where the kernel writes them) of even length, and
+// more threads than the latency needs: half as many are slower on 32^3 (moments 4.5 against 3.9 us), for
+// FP64 populations, each a conversion on the FP64 pipe, up to 64^3 or 1024^2 (35 against 31 us, 40.7
+// against 39.6; 2047 x 2000 134 us in pairs, 140 without).
+static bool pairs_ok(const Lattice &lat, bool writes, bool fp64_pops) {
+    return ((writes ? lat.pitch : lat.nx) & 1) == 0 && lat.ncell >= (int64_t)1 << (fp64_pops ? 21 : 17);
+}
 // The caller's array p (dtype 0 FP64, 1 FP32) may be written two values at a time.
 static bool pairs_fit(const void *p, int dtype) { return (uintptr_t)p % (dtype == 0 ? 16 : 8) == 0; }
 
@@ -426,7 +431,7 @@ static bool pairs_fit(const void *p, int dtype) { return (uintptr_t)p % (dtype =
 
 cudaError_t init_fields(const Lattice &lat, int eq, double rho0, const void *rho, const void *u,
                         int dtype, cudaStream_t s) {
-    const bool two = pairs_ok(lat, true);
+    const bool two = pairs_ok(lat, true, false);
     const int g = grid_for((int64_t)lat.pitch * lat.ny * lat.nz / (two && lat.P == P_F16S ? 2 : 1), 256);
 #define LBM_INIT_EQ(EQv)                                                                         \
     if (eq == EQv) {                                                                             \
@@ -447,7 +452,7 @@ cudaError_t init_fields(const Lattice &lat, int eq, double rho0, const void *rho
 
 cudaError_t moments(const Lattice &lat, double rho0, int odd, void *rho, void *u, int dtype,
                     cudaStream_t s) {
-    const bool two = pairs_ok(lat, false) && pairs_fit(rho, dtype) && pairs_fit(u, dtype);
+    const bool two = pairs_ok(lat, false, false) && pairs_fit(rho, dtype) && pairs_fit(u, dtype);
     const int g = grid_for(lat.ncell / (two && lat.P == P_F16S ? 2 : 1), 256);
     if (dtype == 0)
         LBM_DISPATCH_DPV(lat.D, lat.P, two, (k_moments<DD, PP, VV, double><<<g, 256, 0, s>>>(lat, rho0, odd, (double *)rho, (double *)u)));
@@ -468,7 +473,7 @@ static ClassShift class_shift(int D, double rho0) {
 
 cudaError_t get_populations(const Lattice &lat, double rho0, int odd, void *f, int dtype,
                             cudaStream_t s) {
-    const bool two = pairs_ok(lat, false) && pairs_fit(f, dtype);
+    const bool two = pairs_ok(lat, false, dtype == 0) && pairs_fit(f, dtype);
     const int g = grid_for(lat.ncell / (two && lat.P == P_F16S && dtype != 2 ? 2 : 1), 256);
     const ClassShift k = class_shift(lat.D, rho0);
     if (dtype == 2)
@@ -482,7 +487,7 @@ cudaError_t get_populations(const Lattice &lat, double rho0, int odd, void *f, i
 
 cudaError_t set_populations(const Lattice &lat, double rho0, int odd, const void *f, int dtype,
                             cudaStream_t s) {
-    const bool two = pairs_ok(lat, true);
+    const bool two = pairs_ok(lat, true, dtype == 0);
     const int64_t cells = dtype == 2 ? lat.ncell : (int64_t)lat.pitch * lat.ny * lat.nz;
     const int g = grid_for(cells / (two && lat.P == P_F16S && dtype != 2 ? 2 : 1), 256);
     const ClassShift k = class_shift(lat.D, rho0);
