@@ -1386,9 +1386,10 @@ static void batch_use_teams(lbm_batch *b) {
     b->mean_load = b->total / b->team_blocks;
 }
 
-// LBM_ETIMEOUT if a team's bounded wait ran out (the stream is idle).
+// LBM_ETIMEOUT if a team's bounded wait ran out (the stream is idle), whatever launch shape the batch has
+// been given since.
 static int batch_team_status(lbm_batch *b) {
-    if (!b->teams || b->team_cluster > 0) return LBM_OK;  // (a cluster's barrier is the hardware's)
+    if (!b->team_status) return LBM_OK;  // (no teams, or clusters, whose barrier is the hardware's)
     int32_t st = 0;
     CK(cudaMemcpy(&st, b->team_status, sizeof st, cudaMemcpyDeviceToHost), "status read");
     if (st != 0) return batch_sticky(b, fail(LBM_ETIMEOUT, "a bounded device wait ran out (status %d)", st));
