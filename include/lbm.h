@@ -216,7 +216,7 @@ int lbm_launch_info(lbm_ctx *ctx, int64_t out[8]);
  * 512 for D2Q9 with binary16 storage; two copy-issuing warps are added), `stages`
  * shared-memory stages (2..8), `rows` rows per job when whole rows fit, `seg` cells per
  * row segment (seg >= Nx for whole rows; otherwise a multiple of 16 / sizeof(storage), and
- * never below it) and `cap` bytes per direction buffer (1024, 2048, 4096 or 8192).  The
+ * never below it; ragged rows, which are stored padded, go whole) and `cap` bytes per direction buffer (1024, 2048, 4096 or 8192).  The
  * one-cell kernel takes at most 256 threads.  The block count is the largest that fits on
  * the device.  Returns LBM_EINVAL for a negative entry, an entry above INT32_MAX, or a
  * shape the lattice or the device cannot run.

@@ -288,8 +288,8 @@ TmaShape default_one_shape(lbm_ctx *c, const TmaShape &t) {
     return o.smem_bytes > 0 && tma_set_blocks(c->lat, c->eq, c->bulk, sm_count(), o) ? o : t;
 }
 
-// Callers may ask for the TMA kernel on unpadded rows only; padded ones use it by the
-// library's own choice (LBM_OPT_KERNEL 0) or the tuner's.
+// LBM_OPT_KERNEL 2 asks for the TMA kernel on unpadded rows only; padded ones use it by the library's own
+// choice (LBM_OPT_KERNEL 0), the tuner's or a launch shape.
 bool tma_selectable(lbm_ctx *c) { return tma_supported(c->lat) && c->lat.pitch == c->lat.nx; }
 
 void drop_graph(lbm_ctx *c) {
@@ -1109,7 +1109,8 @@ int lbm_set_launch_shape(lbm_ctx *c, const int64_t shape[6]) {
         return LBM_OK;
     }
     if (shape[0] != 2) return fail(LBM_EINVAL, "kernel must be 1 or 2");
-    if (!tma_selectable(c)) return fail(LBM_EINVAL, "TMA row kernel needs Nx * sizeof(storage) %% 16 == 0");
+    // (padded rows too, whole: a shape that lbm_launch_info reports can be set on a lattice of its size)
+    if (!tma_supported(c->lat)) return fail(LBM_EINVAL, "TMA row kernel needs Nx * sizeof(storage) %% 16 == 0, or padded rows");
     const int tmax = tma_thread_limit(c->lat);
     if (shape[1] < 32 || shape[1] > tmax || shape[1] % 32)
         return fail(LBM_EINVAL, "threads must be a multiple of 32 in [32, %d] for this lattice and storage", tmax);
