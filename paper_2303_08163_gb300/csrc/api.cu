@@ -138,6 +138,11 @@ struct lbm_batch {
     int sticky = 0;
 };
 
+extern "C" {
+static int create_lattice(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, int eq_kind,
+                          int bulk_corr, int precision, double rho0, void *cuda_stream, bool pad);
+}
+
 namespace {
 
 int cuda_fail(const char *what, cudaError_t e) {
@@ -534,7 +539,8 @@ int autotune(lbm_ctx *c) {
     if (c->D == 2 && keep < c->dims[1]) keep = std::max<int64_t>(64, keep / 64 * 64);
     pd[cut] = std::min<int64_t>(c->dims[cut], keep);
     ProxyCtx px;
-    int rc = lbm_create(&px.p, c->lattice, pd, c->tau, c->eq, c->bulk, c->prec, c->rho0, c->stream);
+    // (its planes are copied byte for byte, so its rows have to be padded as the lattice's are)
+    int rc = create_lattice(&px.p, c->lattice, pd, c->tau, c->eq, c->bulk, c->prec, c->rho0, c->stream, c->lat.pitch != c->lat.nx);
     if (rc) return rc;
     lbm_ctx *p = px.p;
     p->step = c->step;  // the same AA parity: the copied planes are a consistent layout
@@ -663,8 +669,9 @@ const char *lbm_last_error(void) { return g_err.c_str(); }
 
 int lbm_version(void) { return 10100; }
 
-int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, int eq_kind,
-               int bulk_corr, int precision, double rho0, void *cuda_stream) {
+// pad: ragged rows may be padded for the TMA kernel.
+static int create_lattice(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, int eq_kind,
+                          int bulk_corr, int precision, double rho0, void *cuda_stream, bool pad) {
     if (!out || !dims) return fail(LBM_EINVAL, "null argument");
     *out = nullptr;
     if (lattice != LBM_D2Q9 && lattice != LBM_D3Q27) return fail(LBM_EINVAL, "bad lattice %d", lattice);
@@ -694,26 +701,17 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
     c->stream = static_cast<cudaStream_t>(cuda_stream);
     const int es = esize_of(precision);
     const int64_t align = 256 / es;
-    c->lat.pitch = padded_pitch(c->D, precision, dims[0]);
-    int64_t plane = (c->lat.pitch * dims[1] * dims[2] + align - 1) / align * align;
+    c->lat.pitch = pad ? padded_pitch(c->D, precision, dims[0]) : (int)dims[0];
+    const int64_t plane = (c->lat.pitch * dims[1] * dims[2] + align - 1) / align * align;
     c->lat.nx = (int)dims[0];
     c->lat.ny = (int)dims[1];
     c->lat.nz = (int)dims[2];
     c->lat.ncell = ncell;
     c->lat.D = c->D;
     c->lat.P = precision;
-    size_t bytes = (size_t)c->Q * plane * es;
-    cudaError_t em = cudaMalloc(&c->lat.A, bytes);
-    if (em != cudaSuccess && c->lat.pitch != c->lat.nx) {
-        // no room for the padding: unpadded rows (and the one-cell kernel)
-        cudaGetLastError();
-        c->lat.pitch = c->lat.nx;
-        plane = (ncell + align - 1) / align * align;
-        bytes = (size_t)c->Q * plane * es;
-        em = cudaMalloc(&c->lat.A, bytes);
-    }
+    const size_t bytes = (size_t)c->Q * plane * es;
     c->lat.plane = plane;
-    if (em != cudaSuccess) {
+    if (cudaMalloc(&c->lat.A, bytes) != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return fail(LBM_ENOMEM, "population storage of %zu bytes", bytes);
@@ -769,6 +767,15 @@ int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, in
     cudaGetLastError();
     *out = c;
     return LBM_OK;
+}
+
+int lbm_create(lbm_ctx **out, int lattice, const int64_t dims[3], double tau, int eq_kind,
+               int bulk_corr, int precision, double rho0, void *cuda_stream) {
+    int rc = create_lattice(out, lattice, dims, tau, eq_kind, bulk_corr, precision, rho0, cuda_stream, true);
+    // no room for the padding: unpadded rows (and the one-cell kernel)
+    if (rc == LBM_ENOMEM && padded_pitch(lattice == LBM_D2Q9 ? 2 : 3, precision, dims[0]) != dims[0])
+        rc = create_lattice(out, lattice, dims, tau, eq_kind, bulk_corr, precision, rho0, cuda_stream, false);
+    return rc;
 }
 
 int lbm_set_option(lbm_ctx *c, int option, int64_t value) {
