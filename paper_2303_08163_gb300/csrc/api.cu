@@ -90,7 +90,6 @@ struct lbm_ctx {
     double *scratch = nullptr;   // one record
     int64_t hist_count = 0;
     // launch
-    int kernel_opt = 0;  // 0 auto, 1 generic, 2 tma
     int kernel = 1;
     int gen_threads = 256, gen_blocks = 1;
     bool chosen = false;  // the caller named a kernel or a launch shape
@@ -790,7 +789,6 @@ int lbm_set_option(lbm_ctx *c, int option, int64_t value) {
         if (value < 0 || value > 2) return fail(LBM_EINVAL, "kernel must be 0, 1 or 2");
         if (value == 2 && !tma_selectable(c))
             return fail(LBM_EINVAL, "TMA row kernel needs Nx * sizeof(storage) to be a multiple of 16");
-        c->kernel_opt = (int)value;
         c->chosen = value != 0;
         if (value == 1) c->kernel = 1;
         if (value == 2 || value == 0) {
