@@ -102,7 +102,8 @@ enum lbm_option {
     LBM_OPT_KERNEL = 1,     /* 0 = auto, 1 = generic one-cell-per-thread kernel,
                                2 = TMA row-staged kernel (needs Nx * sizeof % 16 == 0; auto also
                                takes it for longer ragged rows, which it stores padded) */
-    LBM_OPT_USE_GRAPH = 2,  /* 1 = replay steps from a captured CUDA graph (default 0) */
+    LBM_OPT_USE_GRAPH = 2,  /* 1 = replay single steps, two at a time, from a captured CUDA graph
+                               (default 0; without it many steps share a launch, which is faster) */
     LBM_OPT_TUNE = 3        /* 1 = time the candidate launch shapes now and keep the best */
 };
 
@@ -155,9 +156,12 @@ int lbm_set_option(lbm_ctx *ctx, int option, int64_t value);
 int lbm_init_fields(lbm_ctx *ctx, const void *rho, const void *u, int dtype, int on_device);
 
 /*
- * Advance n >= 0 time steps of Eq. (1) with the fused stream-collide kernel (AA pattern, in
- * place): one launch for many steps with the TMA row-staged kernel, one launch per step with
- * the one-cell kernel and for steps with diagnostics.  When LBM_OPT_DIAG_EVERY = K > 0 the
+ * Advance n >= 0 time steps of Eq. (1) with the fused stream-collide kernels (AA pattern, in
+ * place): one launch for many steps with the TMA row-staged kernel and, for lattices small
+ * enough to be on the SMs at once, with kernels of their own; one launch per step with the
+ * one-cell kernel, for n = 1 and for steps with diagnostics.  The stored values are the same
+ * bits whichever kernels run, however the steps are divided into calls, with diagnostics or
+ * without.  When LBM_OPT_DIAG_EVERY = K > 0 the
  * step kernels of steps t with t % K == 0 also reduce the diagnostics of state t; the
  * call then synchronises and returns LBM_ENONFINITE if any of them saw a non-finite
  * cell (the state is kept for inspection).
@@ -202,8 +206,9 @@ int lbm_sample_populations(lbm_ctx *ctx, const int64_t *cells, int64_t count, do
 int lbm_step_count(lbm_ctx *ctx, int64_t *out);
 
 /*
- * Launch shape of the step kernel chosen for this context: out[0] = kernel (1 generic,
- * 2 TMA row-staged), out[1] = threads per block, out[2] = blocks, out[3] = pipeline
+ * Launch shape of the step kernel chosen for this context (several steps of a small lattice
+ * take other kernels until a kernel or a shape is named; single steps of long FP32 rows in 2-D
+ * have a default shape of their own): out[0] = kernel (1 generic, 2 TMA row-staged), out[1] = threads per block, out[2] = blocks, out[3] = pipeline
  * stages, out[4] = rows per job, out[5] = cells per row segment, out[6] = dynamic
  * shared memory bytes, out[7] = population storage bytes (with the padding of ragged rows).
  */
@@ -213,7 +218,7 @@ int lbm_launch_info(lbm_ctx *ctx, int64_t out[8]);
  * Choose the step kernel's launch shape explicitly.  shape = {kernel, threads, stages,
  * rows, seg, cap}: kernel 1 = generic (threads per block, the rest ignored), 2 = TMA
  * row-staged with `threads` colliding threads per block (a multiple of 32, at most 256,
- * 512 for D2Q9 with binary16 storage; two copy-issuing warps are added), `stages`
+ * 512 for D2Q9 with binary16 storage; one or two copy-issuing warps are added), `stages`
  * shared-memory stages (2..8), `rows` rows per job when whole rows fit, `seg` cells per
  * row segment (seg >= Nx for whole rows; otherwise a multiple of 16 / sizeof(storage), and
  * never below it; ragged rows, which are stored padded, go whole) and `cap` bytes per direction buffer (1024, 2048, 4096 or 8192).  The
@@ -283,7 +288,7 @@ int lbm_batch_get_populations(lbm_batch *b, void *f, int dtype, int on_device);
 int lbm_batch_info(lbm_batch *b, int64_t *total_cells, int64_t *step);
 
 /* Launch shape of the batched kernel: out[0] = threads per block, out[1] = blocks (where the
- * library gives instances teams of blocks, the number of teams: one per instance),
+ * library gives instances teams or clusters of blocks, their number: one per instance),
  * out[2] = largest per-block cell load, out[3] = mean per-block cell load. */
 int lbm_batch_launch_info(lbm_batch *b, int64_t out[4]);
 
@@ -294,14 +299,15 @@ int lbm_batch_launch_info(lbm_batch *b, int64_t out[4]);
  * block owns whole instances, so blocks never wait for one another and more blocks than
  * fit on the GPU at once simply run in waves.  Returns LBM_EINVAL for other values.  (Without
  * this call a batch of few or uneven instances, whose largest would keep one SM busy longer than
- * its share, gives each instance a team of blocks in proportion to its cells.)
+ * its share, gives each instance a team of blocks in proportion to its cells, and one of few short
+ * instances a thread-block cluster each.)
  */
 int lbm_batch_set_launch_shape(lbm_batch *b, int threads, int64_t blocks);
 
 /*
  * Launch-shape autotuner of the batched kernel: times `steps` steps (1 .. 100000) of the
  * current state under each candidate shape (64, 128 or 256 threads; 1, 2, 3, 4, 6, 8, 12
- * or 16 blocks per SM, and the teams of blocks where the batch has them), twice, and keeps the fastest (among shapes within 0.5 % of it, the
+ * or 16 blocks per SM, and the teams or clusters of blocks where the batch has them), twice, and keeps the fastest (among shapes within 0.5 % of it, the
  * one with the fewest blocks, then threads).  The state, the step counter and the status
  * are restored afterwards, so the call changes only the launch shape; the probes of the
  * timed steps are written to samples that the next lbm_batch_step rewrites.  Needs one
@@ -319,7 +325,7 @@ void lbm_batch_destroy(lbm_batch *b);
 
 /*
  * Eigenvalues of the amplification matrix M = E (delta + J) of Eq. (eq:VN_eigen) for count
- * parameter points, computed on the GPU in FP64 (one point per thread).  J = 2 beta
+ * parameter points, computed on the GPU in FP64 (one to four lanes of a warp a point).  J = 2 beta
  * (d f^eq / d f - I) is the Jacobian of the collision operator at f = f^eq(rho, u), with
  * the exact derivatives of the eq_kind equilibrium; E_ij = exp(-i c_i . k) delta_ij.
  * With bulk_corr = 1, 2 beta is the corrected rate of Eq. (eq:redefined_relaxation rate)

@@ -238,9 +238,8 @@ cudaError_t launch_steps(lbm_ctx *c, int odd, int64_t n, cudaStream_t s) {
 // Default TMA shape, used until the tuner runs.  128 colliding threads and 2 stages: two
 // blocks per SM for D3Q27 with direction buffers of 2048 bytes (4096 when a row is longer, up
 // to 4096 bytes), three for D2Q9 with 4096 bytes (4096^2 FP32, 200 steps with diagnostics
-// every 10: 27.2 ms, against 30.4 with 3 stages and two blocks; steps launched one by one 0.203
-// against 0.205 ms).  Whole rows filling the buffer when a row
-// fits, otherwise equal aligned segments; as many blocks as fit on the device.
+// every 10: 27.2 ms, against 30.4 with 3 stages and two blocks).  Whole rows filling the buffer
+// when a row fits, otherwise equal aligned segments; as many blocks as fit on the device.
 bool default_tma_shape(lbm_ctx *c, TmaShape &t) {
     const int es = esize_of(c->prec);
     const int64_t rowb = c->lat.pitch * (int64_t)es;
