@@ -9,7 +9,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <queue>
 #include <string>
 #include <tuple>
@@ -1212,21 +1214,24 @@ int lbm_vn_stability_limit(int eq_kind, int64_t npairs, const double *nu, const 
     for (int64_t p = 0; p < npairs; ++p)
         if (!(nu[p] > 0)) return fail(LBM_EINVAL, "nu must be positive");
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const size_t bytes = vn_limit_bytes(npairs);
-    std::vector<char> host(bytes);
-    vn_limit_fill(host.data(), npairs, nu, theta, u_hi);
+    const size_t state = vn_limit_bytes(npairs), col = sizeof(double) * (size_t)npairs;
+    std::unique_ptr<double[]> host(new (std::nothrow) double[2 * (size_t)npairs]);
     VnBuf b;
-    if (!b.alloc(bytes + sizeof(int32_t))) return fail(LBM_ENOMEM, "stability buffers");
-    int32_t *dst = (int32_t *)(b.p + bytes);
-    CK(cudaMemcpyAsync(b.p, host.data(), bytes, cudaMemcpyHostToDevice, s), "pair upload");
+    if (!host || !b.alloc(state + 3 * col + sizeof(int32_t))) return fail(LBM_ENOMEM, "stability buffers");
+    for (int64_t p = 0; p < npairs; ++p) {
+        host[2 * p] = 0.5 + 3.0 * nu[p];
+        host[2 * p + 1] = theta[p];
+    }
+    double *din = (double *)(b.p + state), *dlim = (double *)(b.p + state + 2 * col);
+    int32_t *dst = (int32_t *)(b.p + state + 3 * col);
+    CK(cudaMemcpyAsync(din, host.get(), 2 * col, cudaMemcpyHostToDevice, s), "pair upload");
     CK(cudaMemsetAsync(dst, 0, sizeof(int32_t), s), "status clear");
-    CK(vn_limit(eq_kind, npairs, b.p, nk, u_hi, iterations, tol, dst, s), "stability search");
+    CK(vn_limit(eq_kind, npairs, b.p, din, dlim, nk, u_hi, iterations, tol, dst, s), "stability search");
     int32_t st = 0;
-    CK(cudaMemcpyAsync(host.data(), b.p, bytes, cudaMemcpyDeviceToHost, s), "limit copy");
     CK(cudaMemcpyAsync(&st, dst, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "status copy");
     CK(cudaStreamSynchronize(s), "stability sync");
     if (st) return fail(LBM_ECUDA, "the QR iteration did not converge for some point");
-    vn_limit_read(host.data(), npairs, umax);
+    CK(cudaMemcpy(umax, dlim, col, cudaMemcpyDeviceToHost), "limit copy");
     return LBM_OK;
 }
 

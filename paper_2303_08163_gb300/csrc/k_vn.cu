@@ -466,15 +466,24 @@ __global__ void __launch_bounds__(kVnThreads) k_vn_round(int64_t npairs, VnPair 
     }
 }
 
-// After a round (or before the first): narrow each pair's interval by the swept trial and by what
-// the look-ahead decided, set its next trial speed and form delta + J there, one pair to a block.
+// After a round: narrow each pair's interval by the swept trial and by what the look-ahead decided, set
+// its next trial speed and form delta + J there, one pair to a block; before the first (`start`): the
+// pair's state from in[2 p] = tau and in[2 p + 1] = theta.  limit[p]: the largest speed known to be stable.
 template <int EQ>
-__global__ void __launch_bounds__(32) k_vn_bisect(int64_t npairs, VnPair *pairs, int start, int iterations,
-                                                  double u_hi, double tol) {
+__global__ void __launch_bounds__(32) k_vn_bisect(int64_t npairs, VnPair *pairs, const double *in, double *limit, int start,
+                                                  int iterations, double u_hi, double tol) {
     for (int64_t p = blockIdx.x; p < npairs; p += gridDim.x) {
         VnPair *P = pairs + p;
-        double lo = P->lo, hi = P->hi, trial = P->trial;
-        int done = P->done, level = P->level;
+        const double tau = in[2 * p], theta = in[2 * p + 1];
+        double lo = 0.0, hi = u_hi, trial = u_hi;
+        int done = 0, level = 0;
+        if (!start) {
+            lo = P->lo;
+            hi = P->hi;
+            trial = P->trial;
+            done = P->done;
+            level = P->level;
+        }
         if (!start && !done) {
             const bool stable = __longlong_as_double((long long)P->worst) <= 1.0 + tol;
             int next = 0, last = 0;  // the look-ahead's trials that follow
@@ -511,13 +520,20 @@ __global__ void __launch_bounds__(32) k_vn_bisect(int64_t npairs, VnPair *pairs,
             P->level = level;
             P->done = done;
             P->worst = 0;
-            if (P->cand) P->look = P->cand;
+            if (start) {
+                P->tau = tau;
+                P->theta = theta;
+                P->look = 0;
+            } else if (P->cand) {
+                P->look = P->cand;
+            }
             P->cand = 0;
+            limit[p] = lo;
         }
         if (threadIdx.x < kN && !done) {
             double st, ct, row[9];
-            sincos(P->theta, &st, &ct);
-            vn_row<EQ, false>(P->tau, 1.0, trial * ct, trial * st, threadIdx.x, row);
+            sincos(theta, &st, &ct);
+            vn_row<EQ, false>(tau, 1.0, trial * ct, trial * st, threadIdx.x, row);
             for (int j = 0; j < 9; ++j) P->A[9 * threadIdx.x + j] = row[j];
         }
         __syncwarp();
@@ -569,22 +585,8 @@ cudaError_t vn_eigs(int eq, int bulk, int64_t count, const double *params, doubl
 
 size_t vn_limit_bytes(int64_t npairs) { return sizeof(VnPair) * (size_t)npairs; }
 
-void vn_limit_fill(void *host, int64_t npairs, const double *nu, const double *theta, double u_hi) {
-    VnPair *P = static_cast<VnPair *>(host);
-    for (int64_t p = 0; p < npairs; ++p) {
-        P[p] = VnPair{};
-        P[p].tau = 0.5 + 3.0 * nu[p];
-        P[p].theta = theta[p];
-        P[p].hi = P[p].trial = u_hi;
-    }
-}
-
-void vn_limit_read(const void *host, int64_t npairs, double *umax) {
-    for (int64_t p = 0; p < npairs; ++p) umax[p] = static_cast<const VnPair *>(host)[p].lo;
-}
-
 template <int EQ, int G>
-static cudaError_t vn_limit_g(int64_t npairs, VnPair *P, int nk, double u_hi, int iterations, double tol,
+static cudaError_t vn_limit_g(int64_t npairs, VnPair *P, const double *in, double *limit, int nk, double u_hi, int iterations, double tol,
                                int32_t *status, cudaStream_t s) {
     constexpr int per = kVnThreads / G;
     const int gb = grid_n(npairs);
@@ -595,27 +597,27 @@ static cudaError_t vn_limit_g(int64_t npairs, VnPair *P, int nk, double u_hi, in
     const int64_t looks = (kVnLooks + per - 1) / per, sweep = ((int64_t)nk * nk + per - 1) / per;
     const bool ahead = 8 * looks <= sweep || npairs * (looks + sweep) <= 608;
     const int gr = grid_n(ahead ? npairs * (sweep + looks) : (npairs * nk * nk + per - 1) / per);
-    k_vn_bisect<EQ><<<gb, 32, 0, s>>>(npairs, P, 1, iterations, u_hi, tol);
+    k_vn_bisect<EQ><<<gb, 32, 0, s>>>(npairs, P, in, limit, 1, iterations, u_hi, tol);
     for (int it = 0; it <= iterations; ++it) {  // every round decides at least one trial of a pair
         k_vn_round<G, EQ><<<gr, kVnThreads, 0, s>>>(npairs, P, nk, tol, ahead, status);
-        k_vn_bisect<EQ><<<gb, 32, 0, s>>>(npairs, P, 0, iterations, u_hi, tol);
+        k_vn_bisect<EQ><<<gb, 32, 0, s>>>(npairs, P, in, limit, 0, iterations, u_hi, tol);
     }
     return cudaGetLastError();
 }
 
 template <int EQ>
-static cudaError_t vn_limit_eq(int64_t npairs, VnPair *P, int nk, double u_hi, int iterations, double tol,
+static cudaError_t vn_limit_eq(int64_t npairs, VnPair *P, const double *in, double *limit, int nk, double u_hi, int iterations, double tol,
                                int32_t *status, cudaStream_t s) {
-    if (vn_lanes(npairs * nk * nk) == 4) return vn_limit_g<EQ, 4>(npairs, P, nk, u_hi, iterations, tol, status, s);
-    return vn_limit_g<EQ, 1>(npairs, P, nk, u_hi, iterations, tol, status, s);
+    if (vn_lanes(npairs * nk * nk) == 4) return vn_limit_g<EQ, 4>(npairs, P, in, limit, nk, u_hi, iterations, tol, status, s);
+    return vn_limit_g<EQ, 1>(npairs, P, in, limit, nk, u_hi, iterations, tol, status, s);
 }
 
-cudaError_t vn_limit(int eq, int64_t npairs, void *pairs, int nk, double u_hi, int iterations, double tol,
+cudaError_t vn_limit(int eq, int64_t npairs, void *pairs, const double *in, double *limit, int nk, double u_hi, int iterations, double tol,
                      int32_t *status, cudaStream_t s) {
     VnPair *P = static_cast<VnPair *>(pairs);
-    if (eq == EQ_ENT) return vn_limit_eq<EQ_ENT>(npairs, P, nk, u_hi, iterations, tol, status, s);
-    if (eq == EQ_POLY2) return vn_limit_eq<EQ_POLY2>(npairs, P, nk, u_hi, iterations, tol, status, s);
-    if (eq == EQ_PROD) return vn_limit_eq<EQ_PROD>(npairs, P, nk, u_hi, iterations, tol, status, s);
+    if (eq == EQ_ENT) return vn_limit_eq<EQ_ENT>(npairs, P, in, limit, nk, u_hi, iterations, tol, status, s);
+    if (eq == EQ_POLY2) return vn_limit_eq<EQ_POLY2>(npairs, P, in, limit, nk, u_hi, iterations, tol, status, s);
+    if (eq == EQ_PROD) return vn_limit_eq<EQ_PROD>(npairs, P, in, limit, nk, u_hi, iterations, tol, status, s);
     return cudaErrorInvalidValue;
 }
 

@@ -167,12 +167,10 @@ cudaError_t vn_eigs(int eq, int bulk, int64_t count, const double *params, doubl
 // trials lead to after an unstable swept one (2, 4, .. 32), and after a stable one (3, 6, .. 48).
 constexpr int kVnLooks = 10;
 constexpr int vn_look_node(int q) { return q < kVnLooks / 2 ? 2 << q : 3 << (q - kVnLooks / 2); }
-// Stability-limit search: vn_limit_bytes of state per call, filled and read on the host, all
-// trials enqueued by vn_limit.
+// Stability-limit search, all trials enqueued: in[npairs][2] = tau and theta, limit[npairs] the result,
+// pairs vn_limit_bytes of device memory.
 size_t vn_limit_bytes(int64_t npairs);
-void vn_limit_fill(void *host, int64_t npairs, const double *nu, const double *theta, double u_hi);
-void vn_limit_read(const void *host, int64_t npairs, double *umax);
-cudaError_t vn_limit(int eq, int64_t npairs, void *pairs, int nk, double u_hi, int iterations, double tol,
-                     int32_t *status, cudaStream_t s);
+cudaError_t vn_limit(int eq, int64_t npairs, void *pairs, const double *in, double *limit, int nk, double u_hi, int iterations,
+                     double tol, int32_t *status, cudaStream_t s);
 
 }  // namespace lbmh
