@@ -509,8 +509,9 @@ __device__ __forceinline__ float vrcp(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// The same for a density of FP32 storage, which may lie below the normal numbers (three instructions more,
-// not to be seen in the FP32 steps; 4096^2 binary16, whose storage holds no such state, 75.7 against 77.8 us).
+// The same for a density that may lie below the normal numbers: FP32 storage with a reference density to
+// match (for every FP32 cell 509 x 381 quadratic 3.85 -> 3.91 us a step, 4096^2 binary16, whose storage
+// holds no such state, 75.7 -> 77.8).
 __device__ __forceinline__ float vrcp_any(float x) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -614,9 +615,10 @@ __device__ __forceinline__ Moments32<V> collide32(V (&f)[qof(D)], float rho0s, f
         j[0] = vsub(c2, c0);
         j[1] = vsub(vadd(vadd(a[6], a[7]), a[8]), vadd(vadd(a[0], a[1]), a[2]));
     }
-    V inv;
-    if constexpr (P == P_F32) inv = vrcp_any(m.rho);
-    else inv = vrcp(m.rho);
+    V inv = vrcp(m.rho);
+    if constexpr (P == P_F32) {
+        if (rho0s < 1e-30f) inv = vrcp_any(m.rho);
+    }
     m.u[2] = vset<V>(0.0f);
 #pragma unroll
     for (int a = 0; a < D; ++a) m.u[a] = vmul(j[a], inv);
