@@ -28,7 +28,7 @@
 // loader that waits for another block's step must not hold up the stores that other blocks wait for.
 // With both in one kernel (a loader and a storer for single steps too, registers for the longer
 // body) single steps lost 2 % of 512^3 binary16 (2.19 -> 2.23 ms; now 2.18) and 3 % of 128^3, and
-// several steps gained 1 % by the parting (512^3 1.67 -> 1.64 ms a step).
+// several steps gained 2 % by the parting (512^3 1.67 -> 1.62 ms a step).
 //
 // Segmented rows (seg < Nx) carry a halo of U = 16 / sizeof(storage) cells on each side.
 // In the odd step the cells of a segment touch positions [X0 - 1, X0 + len - 1) of the
@@ -713,10 +713,13 @@ __global__ void __launch_bounds__(tma_max_threads(D, P) + 32) k_step_tma(const l
 }
 
 // Several steps a launch (see decode_chain).  The warps after the consumers are the loader and the storer.
+// One block an SM as the least lets the compiler have registers (74 - 78 in 2-D, 140 - 164 in 3-D, two
+// blocks of 192 threads still fit; left alone it kept to 56 - 72 and 128): binary16 4096^2 75.7 -> 73.3 us
+// a step, 512^3 1.64 -> 1.62 ms, rows of odd length 5 - 15 % (2237 x 2466 44 -> 38 us).
 constexpr int kTmaServiceThreads = 64;
 
 template <int D, int P, int EQ, bool BULK, int CAPB>
-__global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads) k_steps_tma(const lbmh::StepArgs a, const TmaGeom g) {
+__global__ void __launch_bounds__(tma_max_threads(D, P) + kTmaServiceThreads, 1) k_steps_tma(const lbmh::StepArgs a, const TmaGeom g) {
     using T = typename Storage<P>::T;
     constexpr int Q = qof(D);
     extern __shared__ __align__(128) unsigned char smem_raw[];
